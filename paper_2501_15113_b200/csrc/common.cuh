@@ -12,7 +12,7 @@ namespace taskkv {
 
 constexpr int kDecodeChunk = 512;                 // rows of one split-K decode item
 constexpr int kGatherRows = 64;                   // rows of one gather item
-constexpr int kScoreChunk = 1024;                 // keys of one window-score work item (CUDA-core path)
+constexpr int kScoreChunk = 256;                  // keys of one window-score work item (CUDA-core path)
 constexpr int kTcChunk = 2048;                    // fewest keys of one window-score work item (tensor-core path)
 constexpr int kTcParts = 8;                       // partial-statistic slots per work item (one per epilogue warp)
 constexpr float kLog2e = 1.4426950408889634f;
@@ -199,11 +199,12 @@ __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepco
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <class... KArgs, class... Args>
-cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned grid, unsigned block, cudaStream_t s, Args... args) {
+cudaError_t launch_dependent_smem(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                                  Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid, 1, 1);
   cfg.blockDim = dim3(block, 1, 1);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -211,6 +212,10 @@ cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned grid, unsigned b
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <class... KArgs, class... Args>
+cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned grid, unsigned block, cudaStream_t s, Args... args) {
+  return launch_dependent_smem(kernel, grid, block, 0, s, args...);
 }
 #endif
 

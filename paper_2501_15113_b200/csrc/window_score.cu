@@ -3,156 +3,253 @@
 //   C[j] = mean over the unit's G*L window rows of the normalised weights.
 //
 // Generic two-pass path on the CUDA cores (fp32 accumulate), used for fp32
-// inputs and as the reference implementation for bf16:
-//   pass 1  per (unit, 1024-key chunk): row maxima and exp-sums  -> partial stats
-//   reduce  per unit: combine chunks -> (row max, 1 / row sum)
+// inputs and for bf16 with a number of window rows the tensor-core path does not take:
+//   pass 1  per (unit, 256-key chunk): row maxima and exp-sums  -> partial stats
+//   reduce  per unit: combine chunks -> (row max, 1 / row sum); units of up to 32 chunks need no launch for it,
+//           their pass-2 blocks combine the chunks themselves
 //   pass 2  per (unit, chunk): recompute S, C[j] = sum_i exp(s_ij - max_i) / Z_i / rows
 // Scores are kept in log2 units (scaled by log2(e)/sqrt(d)) so exp is one ex2.
+//
+// Bound by the fp32 FMA rate (2 * rows * d flop per key and pass), so each pass is a register-tiled product: a thread
+// holds KPT keys x RPT rows (8x8 at 128 rows), fed by 16-byte shared-memory reads along d, and keeps its own running
+// (max, sum) per row, so that lanes meet once per chunk instead of twice per row and tile.  32 units of 6001 keys, 64
+// rows, d = 64, fp32 (3.1 GFLOP in both passes): with one key per thread and a warp reduction per row and tile
+// 0.57 + 0.32 ms, this form 0.12 + 0.10 ms; the whole compression with four decode steps 1.06 -> 0.42 ms.
 #include "common.cuh"
 
 namespace taskkv {
 
 namespace {
 
-constexpr int kTile = 128;      // keys per tile, one per thread
-constexpr int kRowBlock = 16;   // window rows accumulated in registers at a time
+constexpr int kTile = 128;      // keys per tile
+constexpr int kBlock = 256;     // threads
+constexpr int kDepth = 64;      // elements of d staged in shared memory at a time
+constexpr int kPitch = kDepth + 4;   // floats per staged key row: 16-byte reads of consecutive rows hit all banks
+constexpr int kFoldChunks = 32; // units of up to this many chunks are folded by the pass-2 blocks
 
-template <typename T, int D>
-struct WinSmem {
-  static constexpr int kRowBytes = D * (int)sizeof(T) + 16;  // +16: conflict-free 16-byte row reads
+// How a block's 256 threads cover 128 keys x ROWS window rows.
+template <int ROWS>
+struct WinTile {
+  static constexpr int RPT = ROWS == 128 ? 8 : 4;
+  static constexpr int NTY = ROWS / RPT;
+  static constexpr int NTX = kBlock / NTY;
+  static constexpr int KPT = kTile / NTX;
+  static constexpr int PARTS = kBlock / ROWS;    // threads that share a row's fold over the chunks
 };
 
-template <typename T, int D, int PASS>
-__global__ void __launch_bounds__(kTile) window_pass_kernel(DeviceProblem p, UnitRange ur) {
-  const int u = ur.unit(blockIdx.y);
+template <int D, int ROWS>
+constexpr size_t win_smem() {
+  return ((size_t)ROWS * (D + 4) + (size_t)kTile * kPitch + 2 * (size_t)ROWS) * sizeof(float);
+}
+
+// (max, sum) pairs in log2 units: a <- a + b.
+__device__ __forceinline__ void fold_pair(float2& a, const float2 b) {
+  if (b.x > -INFINITY) {
+    const float M = fmaxf(a.x, b.x);
+    a.y = a.y * exp2f(a.x - M) + b.y * exp2f(b.x - M);
+    a.x = M;
+  }
+}
+
+// (row max, 1 / row sum) of every row of unit u from its chunks' partials, by the whole block, into out[ROWS] (shared
+// memory); tmp: kBlock pairs.  The order is fixed by the unit's own length.
+template <int ROWS>
+__device__ void fold_unit(const DeviceProblem& p, int u, int chunks, float2* tmp, float2* out) {
+  constexpr int PARTS = WinTile<ROWS>::PARTS;
+  const int row = threadIdx.x % ROWS, part = threadIdx.x / ROWS;
+  const float2* src = reinterpret_cast<const float2*>(p.stat_part) + (size_t)u * p.chunks_max * p.rows_pad + row;
+  float2 a = make_float2(-INFINITY, 0.f);
+  if (row < p.rows) {
+    for (int c = part; c < chunks; c += 4 * PARTS) {
+      float2 o[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        o[i] = c + i * PARTS < chunks ? src[(size_t)(c + i * PARTS) * p.rows_pad] : make_float2(-INFINITY, 0.f);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) fold_pair(a, o[i]);
+    }
+  }
+  tmp[threadIdx.x] = a;
+  __syncthreads();
+  if (part == 0) {
+#pragma unroll
+    for (int q = 1; q < PARTS; ++q) fold_pair(a, tmp[q * ROWS + row]);
+    out[row] = (row < p.rows && a.y > 0.f) ? make_float2(a.x, 1.0f / a.y) : make_float2(0.f, 0.f);
+  }
+  __syncthreads();
+}
+
+// fold: pass 2 combines the chunks itself (p.stat is not used).
+template <typename T, int D, int ROWS, int PASS>
+__global__ void __launch_bounds__(kBlock) window_pass_kernel(DeviceProblem p, UnitRange ur, int grid_chunks, int fold) {
+  using W = WinTile<ROWS>;
+  constexpr int RPT = W::RPT, NTY = W::NTY, NTX = W::NTX, KPT = W::KPT;
+  constexpr int VN = Vec16<T>::N;
+  constexpr int VPR = kDepth / VN;                       // 16-byte vectors of one key row of a stage
+  constexpr int VPT = kTile * VPR / kBlock;              // vectors per thread and stage
+  constexpr int QP = D + 4;
+  extern __shared__ __align__(16) float win_mem[];
+  float* Qs = win_mem;                                                  // [ROWS][D + 4]
+  float* Ks = Qs + ROWS * QP;                                           // [kTile][kPitch]; later scratch
+  float2* st = reinterpret_cast<float2*>(Ks + kTile * kPitch);          // [ROWS]  pass 2: (max, 1 / sum)
+
+  const int u = ur.unit(blockIdx.x / grid_chunks);
+  const int chunk = blockIdx.x % grid_chunks;
   const int N = p.unit_N[u];
-  const int key0 = blockIdx.x * kScoreChunk;
+  const int key0 = chunk * kScoreChunk;
   if (key0 >= N) return;
   const int key_end = min(N, key0 + kScoreChunk);
-  const int rows = p.rows, rows_pad = p.rows_pad, L = p.L;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int L = p.L;
+  const int tid = threadIdx.x, tx = tid % NTX, ty = tid / NTX;
 
-  extern __shared__ __align__(16) unsigned char smem[];
-  float* Qs = reinterpret_cast<float*>(smem);                       // [rows_pad][D]
-  unsigned char* Ks = smem + (size_t)rows_pad * D * sizeof(float);  // [kTile][kRowBytes]
-  float2* st = reinterpret_cast<float2*>(Ks + kTile * WinSmem<T, D>::kRowBytes);  // [rows_pad][4]
-
-  // Q rows of the unit's G heads: [rows][d] contiguous, converted to fp32 once.
-  const T* q = static_cast<const T*>(p.q_ptr[u]);
-  for (int i = tid; i < rows_pad * D; i += kTile) Qs[i] = (i < rows * D) ? to_float(q[i]) : 0.f;
-  for (int i = tid; i < rows_pad * 4; i += kTile) {
-    if (PASS == 1) {
-      st[i] = make_float2(-INFINITY, 0.f);
-    } else if (i < rows_pad) {
-      // pass 2: st[row] = (row max, 1/Z)
-      st[i] = (i < rows) ? reinterpret_cast<const float2*>(p.stat)[(size_t)u * rows_pad + i]
-                         : make_float2(0.f, 0.f);
+  // a stage is kDepth elements of 128 key rows; its global loads are issued before the stage before it is used
+  const unsigned char* kbase = static_cast<const unsigned char*>(p.k_ptr[u]);
+  const int stages = (key_end - key0 + kTile - 1) / kTile * (D / kDepth);
+  uint4 pre[VPT];
+  auto fetch = [&](int s) {
+    const int t0 = key0 + s / (D / kDepth) * kTile, d0 = s % (D / kDepth) * kDepth;
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+      const int v = tid + i * kBlock, r = v / VPR, c = v % VPR;
+      pre[i] = t0 + r < N ? *reinterpret_cast<const uint4*>(kbase + ((size_t)(t0 + r) * D + d0) * sizeof(T) + (size_t)c * 16)
+                          : make_uint4(0, 0, 0, 0);
+    }
+  };
+  fetch(0);
+  // Q rows of the unit's G heads: [rows][d] contiguous, converted to fp32 once
+  const uint4* q = static_cast<const uint4*>(p.q_ptr[u]);
+  for (int v = tid; v < ROWS * (D / VN); v += kBlock) {
+    const int r = v / (D / VN), c = v % (D / VN);
+    float f[VN];
+    Vec16<T>::unpack(r < p.rows ? q[v] : make_uint4(0, 0, 0, 0), f);
+#pragma unroll
+    for (int h = 0; h < VN; h += 4) *reinterpret_cast<float4*>(Qs + r * QP + c * VN + h) = make_float4(f[h], f[h + 1], f[h + 2], f[h + 3]);
+  }
+  if (PASS == 2) {
+    grid_dependency_wait();                              // the statistics come from the launch before
+    if (fold) {
+      fold_unit<ROWS>(p, u, (N + kScoreChunk - 1) / kScoreChunk, reinterpret_cast<float2*>(Ks), st);
+    } else {
+      for (int i = tid; i < ROWS; i += kBlock)
+        st[i] = i < p.rows ? reinterpret_cast<const float2*>(p.stat)[(size_t)u * p.rows_pad + i] : make_float2(0.f, 0.f);
     }
   }
 
   const float scale2 = kLog2e * rsqrtf((float)D);
-  constexpr int VN = Vec16<T>::N;
-  constexpr int VPR = D / VN;  // 16-byte vectors per key row
-  const unsigned char* kbase = static_cast<const unsigned char*>(p.k_ptr[u]);
-  const unsigned char* krow = Ks + tid * WinSmem<T, D>::kRowBytes;
-
-  for (int t0 = key0; t0 < key_end; t0 += kTile) {
-    __syncthreads();  // previous tile consumed (and Q/state initialised on the first trip)
-    for (int v = tid; v < kTile * VPR; v += kTile) {
-      const int r = v / VPR, c = v % VPR;
-      uint4 raw = make_uint4(0, 0, 0, 0);
-      if (t0 + r < N)
-        raw = *reinterpret_cast<const uint4*>(kbase + ((size_t)(t0 + r) * D) * sizeof(T) + (size_t)c * 16);
-      *reinterpret_cast<uint4*>(Ks + r * WinSmem<T, D>::kRowBytes + c * 16) = raw;
+  // last key the thread's rows may see: window row (row % L) sits at position N - L + (row % L)
+  int pos[RPT];
+  float m[RPT], z[RPT];                                  // pass 1: running max and sum; pass 2: the row's pair
+#pragma unroll
+  for (int j = 0; j < RPT; ++j) {
+    const int row = ty + NTY * j;
+    pos[j] = row < p.rows ? N - L + row % L : -1;
+    m[j] = -INFINITY;
+    z[j] = 0.f;
+  }
+  float acc[KPT][RPT];
+  for (int s = 0; s < stages; ++s) {
+    __syncthreads();                                     // the previous stage's readers (and the fold) are done
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+      const int v = tid + i * kBlock, r = v / VPR, c = v % VPR;
+      float f[VN];
+      Vec16<T>::unpack(pre[i], f);
+#pragma unroll
+      for (int h = 0; h < VN; h += 4) *reinterpret_cast<float4*>(Ks + r * kPitch + c * VN + h) = make_float4(f[h], f[h + 1], f[h + 2], f[h + 3]);
     }
+    if (s + 1 < stages) fetch(s + 1);
     __syncthreads();
-
-    const int j = t0 + tid;       // this thread's key
-    float csum = 0.f;
-    for (int rb = 0; rb < rows_pad; rb += kRowBlock) {
-      float acc[kRowBlock];
+    const int t0 = key0 + s / (D / kDepth) * kTile, d0 = s % (D / kDepth) * kDepth;
+    if (d0 == 0) {
 #pragma unroll
-      for (int i = 0; i < kRowBlock; ++i) acc[i] = 0.f;
+      for (int i = 0; i < KPT; ++i)
+#pragma unroll
+        for (int j = 0; j < RPT; ++j) acc[i][j] = 0.f;
+    }
 #pragma unroll 2
-      for (int dd = 0; dd < D; dd += VN) {
-        float kf[VN];
-        Vec16<T>::unpack(*reinterpret_cast<const uint4*>(krow + dd * sizeof(T)), kf);
+    for (int dd = 0; dd < kDepth; dd += 4) {
+      float4 kf[KPT];
 #pragma unroll
-        for (int i = 0; i < kRowBlock; ++i) {
-          const float4* qp = reinterpret_cast<const float4*>(Qs + (rb + i) * D + dd);
+      for (int i = 0; i < KPT; ++i) kf[i] = *reinterpret_cast<const float4*>(Ks + (tx + NTX * i) * kPitch + dd);
 #pragma unroll
-          for (int h = 0; h < VN / 4; ++h) {
-            const float4 qv = qp[h];
-            acc[i] = fmaf(qv.x, kf[4 * h + 0], acc[i]);
-            acc[i] = fmaf(qv.y, kf[4 * h + 1], acc[i]);
-            acc[i] = fmaf(qv.z, kf[4 * h + 2], acc[i]);
-            acc[i] = fmaf(qv.w, kf[4 * h + 3], acc[i]);
-          }
-        }
-      }
+      for (int j = 0; j < RPT; ++j) {
+        const float4 qv = *reinterpret_cast<const float4*>(Qs + (ty + NTY * j) * QP + d0 + dd);
 #pragma unroll
-      for (int i = 0; i < kRowBlock; ++i) {
-        const int row = rb + i;
-        // window row (row % L) sits at position N - L + (row % L)
-        const bool visible = (row < rows) && (j < N) && (j <= N - L + (row % L));
-        const float s2 = acc[i] * scale2;
-        if (PASS == 1) {
-          const float sv = visible ? s2 : -INFINITY;
-          const float m = warp_max(sv);
-          const float e = (visible && m > -INFINITY) ? exp2f(sv - m) : 0.f;
-          const float z = warp_sum(e);
-          if (lane == 0 && row < rows && m > -INFINITY) {
-            float2 o = st[row * 4 + warp];
-            const float M = fmaxf(o.x, m);
-            o.y = o.y * exp2f(o.x - M) + z * exp2f(m - M);
-            o.x = M;
-            st[row * 4 + warp] = o;
-          }
-        } else {
-          if (visible) {
-            const float2 ms = st[row];
-            csum += exp2f(s2 - ms.x) * ms.y;
-          }
+        for (int i = 0; i < KPT; ++i) {
+          acc[i][j] = fmaf(qv.x, kf[i].x, acc[i][j]);
+          acc[i][j] = fmaf(qv.y, kf[i].y, acc[i][j]);
+          acc[i][j] = fmaf(qv.z, kf[i].z, acc[i][j]);
+          acc[i][j] = fmaf(qv.w, kf[i].w, acc[i][j]);
         }
       }
     }
-    if (PASS == 2 && j < N) p.C[p.c_off[u] + j] = csum * (1.0f / (float)rows);
+    if (d0 + kDepth < D) continue;                       // (D = 128) the other half of the products comes next
+    if (PASS == 1) {
+#pragma unroll
+      for (int j = 0; j < RPT; ++j) {
+        float x[KPT], mt = -INFINITY;
+#pragma unroll
+        for (int i = 0; i < KPT; ++i) {
+          x[i] = t0 + tx + NTX * i <= pos[j] ? acc[i][j] * scale2 : -INFINITY;
+          mt = fmaxf(mt, x[i]);
+        }
+        if (mt > m[j]) {
+          z[j] *= exp2f(m[j] - mt);
+          m[j] = mt;
+        }
+        if (m[j] > -INFINITY) {
+#pragma unroll
+          for (int i = 0; i < KPT; ++i) z[j] += exp2f(x[i] - m[j]);
+        }
+      }
+    } else {
+      float cs[KPT];
+#pragma unroll
+      for (int i = 0; i < KPT; ++i) cs[i] = 0.f;
+#pragma unroll
+      for (int j = 0; j < RPT; ++j) {
+        const float2 ms = st[ty + NTY * j];
+#pragma unroll
+        for (int i = 0; i < KPT; ++i)
+          if (t0 + tx + NTX * i <= pos[j]) cs[i] += exp2f(acc[i][j] * scale2 - ms.x) * ms.y;
+      }
+      __syncthreads();                                   // every thread is done with this tile's keys
+#pragma unroll
+      for (int i = 0; i < KPT; ++i) Ks[ty * kTile + tx + NTX * i] = cs[i];
+      __syncthreads();
+      if (tid < kTile && t0 + tid < N) {
+        float c = 0.f;
+#pragma unroll
+        for (int y = 0; y < NTY; ++y) c += Ks[y * kTile + tid];
+        p.C[p.c_off[u] + t0 + tid] = c * (1.0f / (float)p.rows);
+      }
+    }
   }
 
   if (PASS == 1) {
+    grid_launch_dependents();
     __syncthreads();
-    for (int row = tid; row < rows_pad; row += kTile) {
-      float M = -INFINITY;
-      for (int w = 0; w < 4; ++w) M = fmaxf(M, st[row * 4 + w].x);
-      float z = 0.f;
-      for (int w = 0; w < 4; ++w) {
-        const float2 o = st[row * 4 + w];
-        if (o.x > -INFINITY) z += o.y * exp2f(o.x - M);
-      }
-      reinterpret_cast<float2*>(p.stat_part)[((size_t)u * p.chunks_max + blockIdx.x) * rows_pad + row] =
-          make_float2(M, z);
+    float2* red = reinterpret_cast<float2*>(Ks);         // [ROWS][NTX + 1]
+#pragma unroll
+    for (int j = 0; j < RPT; ++j) red[(ty + NTY * j) * (NTX + 1) + tx] = make_float2(m[j], z[j]);
+    __syncthreads();
+    if (tid < p.rows) {
+      float2 a = make_float2(-INFINITY, 0.f);
+      for (int x = 0; x < NTX; ++x) fold_pair(a, red[tid * (NTX + 1) + x]);
+      reinterpret_cast<float2*>(p.stat_part)[((size_t)u * p.chunks_max + chunk) * p.rows_pad + tid] = a;
     }
   }
 }
 
-// Combine the chunk partials of one unit: (max, sum) -> (max, 1/sum) per window row.
-__global__ void window_reduce_kernel(DeviceProblem p, UnitRange ur) {
+// The fold as a launch of its own, for units of many chunks: every pass-2 block would read all of them again.
+template <int ROWS>
+__global__ void __launch_bounds__(kBlock) window_reduce_kernel(DeviceProblem p, UnitRange ur) {
+  __shared__ float2 tmp[kBlock], out[ROWS];
   const int u = ur.unit(blockIdx.x);
-  const int row = threadIdx.x;
-  if (row >= p.rows_pad) return;
-  const int N = p.unit_N[u];
-  const int chunks = (N + kScoreChunk - 1) / kScoreChunk;
-  const float2* part = reinterpret_cast<const float2*>(p.stat_part) + (size_t)u * p.chunks_max * p.rows_pad;
-  float M = -INFINITY;
-  for (int c = 0; c < chunks; ++c) M = fmaxf(M, part[(size_t)c * p.rows_pad + row].x);
-  float z = 0.f;
-  for (int c = 0; c < chunks; ++c) {
-    const float2 o = part[(size_t)c * p.rows_pad + row];
-    if (o.x > -INFINITY) z += o.y * exp2f(o.x - M);
-  }
-  float2 out = make_float2(0.f, 0.f);
-  if (row < p.rows && z > 0.f) out = make_float2(M, 1.0f / z);
-  reinterpret_cast<float2*>(p.stat)[(size_t)u * p.rows_pad + row] = out;
+  grid_dependency_wait();
+  grid_launch_dependents();
+  fold_unit<ROWS>(p, u, (p.unit_N[u] + kScoreChunk - 1) / kScoreChunk, tmp, out);
+  for (int i = threadIdx.x; i < p.rows; i += kBlock) reinterpret_cast<float2*>(p.stat)[(size_t)u * p.rows_pad + i] = out[i];
 }
 
 // Caller-supplied normalisers lse_i = ln sum_j exp(s_ij) of the window rows, in place of pass 1.  A unit's G*L rows
@@ -167,18 +264,21 @@ __global__ void lse_to_stat_kernel(DeviceProblem p, int u0, const float* __restr
   else reinterpret_cast<float2*>(p.stat)[u * p.rows_pad + row] = make_float2(v, 1.0f);
 }
 
-template <typename T, int D>
-cudaError_t launch_generic(const DeviceProblem& p, int max_N, const WindowHostInfo& h, cudaStream_t s, int layer0,
-                           int n_layers) {
-  const size_t smem = (size_t)p.rows_pad * D * sizeof(float) + (size_t)kTile * WinSmem<T, D>::kRowBytes +
-                      (size_t)p.rows_pad * 4 * sizeof(float2);
+template <typename T, int D, int ROWS>
+cudaError_t launch_generic_rows(const DeviceProblem& p, int max_N, const WindowHostInfo& h, cudaStream_t s, int layer0,
+                                int n_layers) {
+  constexpr size_t smem = win_smem<D, ROWS>();
+  static_assert((size_t)kTile * kPitch >= 2 * (size_t)ROWS * (WinTile<ROWS>::NTX + 1), "pass 1's pairs reuse the key tile");
   cudaError_t e;
-  e = cudaFuncSetAttribute(window_pass_kernel<T, D, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = cudaFuncSetAttribute(window_pass_kernel<T, D, ROWS, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(window_pass_kernel<T, D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = cudaFuncSetAttribute(window_pass_kernel<T, D, ROWS, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const UnitRange ur = layer_range(p, h.batch, layer0, n_layers);
-  const dim3 grid((max_N + kScoreChunk - 1) / kScoreChunk, ur.blocks);
+  const int chunks = (max_N + kScoreChunk - 1) / kScoreChunk;
+  const int64_t grid = (int64_t)chunks * ur.blocks;
+  if (grid > 0x7fffffff) return cudaErrorInvalidConfiguration;
+  const int fold = !h.lse && chunks <= kFoldChunks ? 1 : 0;
   if (h.lse) {
     const int per_seq = p.R * p.n_kv;
     const size_t lse_skip = (size_t)(layer0 - h.base_layer) * p.n_heads * p.L;
@@ -189,18 +289,30 @@ cudaError_t launch_generic(const DeviceProblem& p, int max_N, const WindowHostIn
   } else {
     {
       LaunchScope ls(K_WINDOW_STATS, s);
-      window_pass_kernel<T, D, 1><<<grid, kTile, smem, s>>>(p, ur);
+      window_pass_kernel<T, D, ROWS, 1><<<(unsigned)grid, kBlock, smem, s>>>(p, ur, chunks, 0);
     }
-    {
+    if (!fold) {
       LaunchScope ls(K_WINDOW_REDUCE, s);
-      window_reduce_kernel<<<ur.blocks, p.rows_pad, 0, s>>>(p, ur);
+      e = launch_dependent(window_reduce_kernel<ROWS>, (unsigned)ur.blocks, kBlock, s, p, ur);
+      if (e != cudaSuccess) return e;
     }
   }
   {
     LaunchScope ls(K_WINDOW_SCORES, s);
-    window_pass_kernel<T, D, 2><<<grid, kTile, smem, s>>>(p, ur);
+    if (h.lse) window_pass_kernel<T, D, ROWS, 2><<<(unsigned)grid, kBlock, smem, s>>>(p, ur, chunks, 0);
+    else e = launch_dependent_smem(window_pass_kernel<T, D, ROWS, 2>, (unsigned)grid, kBlock, smem, s, p, ur, chunks, fold);
+    if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
+}
+
+template <typename T, int D>
+cudaError_t launch_generic(const DeviceProblem& p, int max_N, const WindowHostInfo& h, cudaStream_t s, int layer0,
+                           int n_layers) {
+  if (p.rows <= 16) return launch_generic_rows<T, D, 16>(p, max_N, h, s, layer0, n_layers);
+  if (p.rows <= 32) return launch_generic_rows<T, D, 32>(p, max_N, h, s, layer0, n_layers);
+  if (p.rows <= 64) return launch_generic_rows<T, D, 64>(p, max_N, h, s, layer0, n_layers);
+  return launch_generic_rows<T, D, 128>(p, max_N, h, s, layer0, n_layers);
 }
 
 }  // namespace

@@ -167,6 +167,16 @@ def test_shapes_and_edge_cases(case):
     run_workload(wl)
 
 
+# (query heads per KV head, window) -> 8, 16, 24, 48, 96 and 128 window rows; key counts around the 128-key tile, the
+# 256-key chunk and the 8192 keys up to which pass 2 folds the chunks' statistics itself.  (Four KV heads: two are always
+# equally far from their mean, so which of them is promoted would be a tie.)
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("G,L,d,N", [(1, 8, 64, 129), (2, 8, 128, 255), (1, 24, 64, 257), (2, 24, 128, 511),
+                                     (4, 24, 64, 8192), (4, 24, 128, 8193), (8, 16, 64, 384), (8, 16, 128, 9001)])
+def test_cuda_core_window_scores(G, L, d, N, dtype):
+    run_workload(small("winrows", n=4 * G, n_kv=4, d=d, N=N, L=L, s1=4, s2=32, k=40, dtype=dtype, nh=0, t=64, steps=1))
+
+
 def test_every_head_heterogeneous_is_full_attention():
     """force_class = 1: the cache is the whole K/V and decode is textbook attention."""
     wl = small("full", n=8, n_kv=4, d=128, N=1111, L=32, s1=4, s2=64, k=50, dtype="bf16")
