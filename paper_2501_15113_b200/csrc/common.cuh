@@ -158,8 +158,10 @@ cudaError_t launch_window_scores(const DeviceProblem& p, int dtype, int max_N, c
 bool window_tc_supported(const DeviceProblem& p, int dtype);
 cudaError_t launch_window_scores_tc(const DeviceProblem& p, const WindowHostInfo& h, cudaStream_t s, int layer0 = 0,
                                     int n_layers = -1);
-cudaError_t launch_window_prefix(const DeviceProblem& p, const void* q, const void* k, int heads, int group, int N,
-                                 cudaStream_t s);
+// Column sums of the causal attention matrix per 128-row block: q [heads][N][d], k [heads / group][N][d] ->
+// scores [heads][64 nb (nb + 1)], nb = ceil(N / 128), block b of a head at offset 64 b (b + 1).
+cudaError_t launch_prefix_scores(const void* q, const void* k, int d, int heads, int group, int N, float* scores,
+                                 int32_t* status, cudaStream_t s);
 bool window_res_supported(const DeviceProblem& p, const WindowHostInfo& h);
 // layers [layer0, layer0 + n_layers) of every sequence; n_layers < 0: all of them
 cudaError_t launch_window_scores_res(const DeviceProblem& p, const WindowHostInfo& h, cudaStream_t s, int layer0 = 0,

@@ -88,11 +88,6 @@ struct TcArgs {
   int n_local;              // units per sequence (layers * kv heads)
   int chunk_keys;           // keys per work item (multiple of 128)
   int steps;                // items of the busiest CTA
-  // Prefix mode (the column sums of the full causal attention matrix, Eq. 1-2 of Sec. III-A): unit lu stands for the
-  // 128 query rows [128 b, 128 b + 128) of query head lu / prefix_blocks, b = lu % prefix_blocks, as a window
-  // over the first 128 (b + 1) keys of that head's KV head.  0: every unit has its own N keys and rows.
-  int prefix_blocks;
-  int group;                // query heads per KV head (prefix mode)
   int u0[kMaxSeq];          // first unit of each sequence
   int N[kMaxSeq];           // sequence length
   int chunks[kMaxSeq];      // work items per unit
@@ -117,17 +112,9 @@ __device__ __forceinline__ Item decode_item(const TcArgs& a, int k, int rows) {
   it.lu = local / a.chunks[it.seq];
   it.ch = local % a.chunks[it.seq];
   const int N = a.N[it.seq];
-  if (a.prefix_blocks > 0) {
-    const int head = it.lu / a.prefix_blocks, b = it.lu % a.prefix_blocks;
-    it.N = (b + 1) * kTile;                 // may run past the sequence end: those rows and keys are neutralised
-    it.krow0 = (head / a.group) * N;
-    it.qrow0 = head * N + b * kTile;
-    it.valid = it.valid && it.ch * a.chunk_keys < it.N;
-  } else {
-    it.N = N;
-    it.krow0 = it.lu * N;
-    it.qrow0 = it.lu * rows;
-  }
+  it.N = N;
+  it.krow0 = it.lu * N;
+  it.qrow0 = it.lu * rows;
   return it;
 }
 
@@ -345,10 +332,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
     if (a.pass == 2) fetch_stats(0);
     for (int k = 0; k < a.steps && ok; ++k) {
       const Item it = decode_item(a, k, rows);
-      if (!it.valid) {
-        if (a.pass == 2) fetch_stats(k + 1);   // (prefix mode skips items in mid-run: keep the prefetch one ahead)
-        continue;
-      }
+      if (!it.valid) continue;
       const int u = a.u0[it.seq] + it.lu;
       const int N = it.N;
       const int key0 = it.ch * a.chunk_keys;
@@ -549,7 +533,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
 // launch), its neighbours reading the neighbouring rows of the same slot (coalesced); four slots are loaded ahead of
 // the dependent max / sum updates.
 __global__ void __launch_bounds__(128) window_tc_reduce_kernel(DeviceProblem p, UnitRange ur, int chunk_keys,
-                                                               int parts, int n_real) {
+                                                               int parts) {
   const int u = ur.unit(blockIdx.x);
   const int slots = (p.unit_N[u] + chunk_keys - 1) / chunk_keys * parts;
   const float2* part = reinterpret_cast<const float2*>(p.stat_part) + (size_t)u * p.chunks_max * p.rows_pad;
@@ -573,10 +557,7 @@ __global__ void __launch_bounds__(128) window_tc_reduce_kernel(DeviceProblem p, 
   }
   for (; c < slots; ++c) fold(part[(size_t)c * p.rows_pad + row]);
   // one offset per row: score * scale - (max + log2(sum) + log2(rows)) is log2 of the row's share of C
-  // prefix mode (n_real > 0): a query row at or beyond the end of the sequence does not exist; an infinite
-  // offset takes it out of every column sum
-  const bool absent = n_real > 0 && p.unit_N[u] - p.rows + row >= n_real;
-  p.stat[(size_t)u * (2 * p.rows_pad) + row] = (z > 0.f && !absent) ? M + log2f(z) + log2f((float)p.rows) : INFINITY;
+  p.stat[(size_t)u * (2 * p.rows_pad) + row] = z > 0.f ? M + log2f(z) + log2f((float)p.rows) : INFINITY;
 }
 
 // Keys per work item.  Every item costs a Q load and, in pass 2, a statistics load, so long items are
@@ -615,8 +596,6 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
     for (int i = 0; i < nb; ++i) keys += (int64_t)per_seq * h.seq_lens[b0 + i];
     a.n_seq = nb;
     a.n_local = per_seq;
-    a.prefix_blocks = 0;
-    a.group = 1;
     a.chunk_keys = pick_chunk(keys, n_sm);
     a.item_off[0] = 0;
     for (int i = 0; i < kMaxSeq; ++i) {
@@ -657,7 +636,7 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
       {
         LaunchScope ls(K_WINDOW_REDUCE, s);
         const UnitRange ur{b0 * per_seq_all + first, per_seq, per_seq_all, nb * per_seq};
-        window_tc_reduce_kernel<<<nb * per_seq, 128, 0, s>>>(p, ur, a.chunk_keys, parts, 0);
+        window_tc_reduce_kernel<<<nb * per_seq, 128, 0, s>>>(p, ur, a.chunk_keys, parts);
       }
     }
     a.pass = 2;
@@ -671,72 +650,11 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
   return cudaSuccess;
 }
 
-// Prefix mode: p describes heads * blocks virtual units of 128 window rows (rows = L = 128; unit_N, c_off, stat,
-// stat_part sized for them); q is [heads][N][d], k is [heads / group][N][d].
-template <int D>
-cudaError_t launch_prefix_d(const DeviceProblem& p, const void* q, const void* k, int heads, int group, int N,
-                            cudaStream_t s) {
-  int dev = 0, n_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-  if (n_sm <= 0) n_sm = 148;
-  const TcLayout lay = make_layout(D, p.rows);
-  if (lay.stages < 2) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(window_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, lay.total);
-  if (e != cudaSuccess) return e;
-  const int blocks = (N + kTile - 1) / kTile;
-  TcMaps maps;
-  TcArgs a;
-  a.n_seq = 1;
-  a.n_local = heads * blocks;
-  a.prefix_blocks = blocks;
-  a.group = group;
-  a.chunk_keys = kTcChunk;
-  a.item_off[0] = 0;
-  for (int i = 0; i < kMaxSeq; ++i) {
-    if (i > 0) {
-      maps.k[i] = maps.k[0];
-      maps.q[i] = maps.q[0];
-    } else {
-      if (!make_tensor_map_2d(&maps.k[i], k, D, (uint64_t)(heads / group) * (uint64_t)N, kTile)) return cudaErrorUnknown;
-      if (!make_tensor_map_2d(&maps.q[i], q, D, (uint64_t)heads * (uint64_t)N, p.rows)) return cudaErrorUnknown;
-    }
-    a.u0[i] = 0;
-    a.N[i] = N;
-    a.chunks[i] = (blocks * kTile + a.chunk_keys - 1) / a.chunk_keys;
-    a.item_off[i + 1] = a.item_off[i] + (i == 0 ? a.n_local * a.chunks[i] : 0);
-  }
-  const int n1 = a.item_off[1];
-  const int grid = n1 < n_sm ? n1 : n_sm;
-  a.steps = (n1 + grid - 1) / grid;
-  a.pass = 1;
-  {
-    LaunchScope ls(K_WINDOW_TC, s);
-    window_tc_kernel<D><<<grid, kThreads, lay.total, s>>>(maps, p, a, lay);
-  }
-  {
-    LaunchScope ls(K_WINDOW_REDUCE, s);
-    const UnitRange ur{0, a.n_local, a.n_local, a.n_local};
-    window_tc_reduce_kernel<<<a.n_local, 128, 0, s>>>(p, ur, a.chunk_keys, 2, N);
-  }
-  a.pass = 2;
-  {
-    LaunchScope ls(K_WINDOW_TC, s);
-    window_tc_kernel<D><<<grid, kThreads, lay.total, s>>>(maps, p, a, lay);
-  }
-  return cudaGetLastError();
-}
-
 }  // namespace
 
 bool window_tc_supported(const DeviceProblem& p, int dtype) {
   return dtype == TASKKV_BF16 && (p.rows == 32 || p.rows == 64 || p.rows == 128) && p.L <= p.rows &&
          encode_fn() != nullptr;
-}
-
-cudaError_t launch_window_prefix(const DeviceProblem& p, const void* q, const void* k, int heads, int group, int N,
-                                 cudaStream_t s) {
-  return p.d == 64 ? launch_prefix_d<64>(p, q, k, heads, group, N, s) : launch_prefix_d<128>(p, q, k, heads, group, N, s);
 }
 
 cudaError_t launch_window_scores_tc(const DeviceProblem& p, const WindowHostInfo& h, cudaStream_t s, int layer0,
