@@ -22,9 +22,10 @@ struct HostPlan {
   taskkv_plan_info info;
   int64_t c_total = 0;
   int32_t max_N = 0, min_N = 0;
-  int32_t chunks_max = 0, rows = 0, rows_pad = 0, idx_stride = 0;
+  int32_t chunks_max = 0, rows = 0, rows_pad = 0, idx_stride = 0, dec_chunk = 0;
   std::vector<int32_t> seq_lens, mid, nhet;     // [B], [B*R] middle budget of a (sequence, layer), [B*R]
   std::vector<int32_t> full;                    // [B*R] full-cache heads
+  std::vector<int32_t> full_model;              // [B*R] the same over all shards
   std::vector<int64_t> layer_items;             // [R] split-K decode items of a layer over all sequences, at capacity
   // where each (sequence, layer) block starts: pool rows (block b * R + r), gather and decode work items (block
   // r * B + b, layer-major); one entry more than blocks
@@ -62,6 +63,24 @@ int32_t mid_budget_impl(double budget_tokens, int32_t N, int32_t h_full, int32_t
   if (k < 0) k = 0;
   if (k > room) k = room;
   return (int32_t)k;
+}
+
+// Rows per split-K decode item.  Half a thousand rows an item is best where the cache fills the GPU with items anyway; a
+// cache that has fewer than two per SM gets smaller ones (a warp walks its share of an item 16 rows at a time, one
+// trip to memory after the other).  Counted over the retained rows of the model's heads, so that a head shard, a paged
+// cache or another reserve for appended tokens cut the same units alike and give the same bits.
+int32_t pick_decode_chunk(const HostPlan& hp, const taskkv_params* p, int n_model) {
+  const int B = p->batch, R = p->n_layers, s = p->sink + p->recent;
+  for (int32_t chunk = kDecodeChunk;; chunk /= 2) {
+    int64_t items = 0;
+    for (int b = 0; b < B; ++b)
+      for (int r = 0; r < R; ++r) {
+        const int64_t N = hp.seq_lens[b], h = hp.full_model[(size_t)b * R + r];
+        const int64_t kept = N > s ? s + std::min<int64_t>(hp.mid[(size_t)b * R + r], N - s) : N;
+        items += h * ((N + chunk - 1) / chunk) + (n_model - h) * ((kept + chunk - 1) / chunk);
+      }
+    if (items >= 2 * 148 || chunk <= kDecodeChunkMin) return chunk;
+  }
 }
 
 taskkv_status make_plan(const taskkv_params* p, HostPlan& hp, int32_t page_rows = 0) {
@@ -106,6 +125,7 @@ taskkv_status make_plan(const taskkv_params* p, HostPlan& hp, int32_t page_rows 
   }
   hp.nhet.resize((size_t)B * R);
   hp.full.resize((size_t)B * R);
+  hp.full_model.resize((size_t)B * R);
   for (int b = 0; b < B; ++b)
     for (int r = 0; r < R; ++r) {
       int f = p->n_hetero ? p->n_hetero[(size_t)b * R + r] : hetero_count_impl(n_model, p->beta, p->m_top, R, r);
@@ -117,6 +137,7 @@ taskkv_status make_plan(const taskkv_params* p, HostPlan& hp, int32_t page_rows 
       if (p->force_class == 0) h = 0;
       // a shard plans for as many of the layer's full-cache heads as it has heads (which ones it gets is data dependent)
       hp.full[(size_t)b * R + r] = std::min(h, nkv);
+      hp.full_model[(size_t)b * R + r] = h;
       // a budget given as a fraction of the full cache: Eq. 17 per (sequence, layer), with the heads that really
       // keep everything (the device computes the same number for its own table, see budget_kernel)
       if (p->budget_frac > 0.f)
@@ -133,6 +154,7 @@ taskkv_status make_plan(const taskkv_params* p, HostPlan& hp, int32_t page_rows 
   hp.kept_len.assign((size_t)B * R, 0);
   hp.pages_compress = 0;
   hp.page_stride = 0;
+  hp.dec_chunk = pick_decode_chunk(hp, p, n_model);
   std::vector<int64_t> blk_g((size_t)B * R, 0), blk_d((size_t)B * R, 0);   // per block b * R + r
   for (int b = 0; b < B; ++b) {
     const int64_t N = hp.seq_lens[b];
@@ -152,8 +174,8 @@ taskkv_status make_plan(const taskkv_params* p, HostPlan& hp, int32_t page_rows 
       kept_rows += h * N + (nkv - h) * kept;
       blk_g[br] = h * ((N + kGatherRows - 1) / kGatherRows) + (nkv - h) * ((kept + kGatherRows - 1) / kGatherRows);
       gitems += blk_g[br];
-      const int64_t li = h * ((N + mn + kDecodeChunk - 1) / kDecodeChunk) +
-                         (nkv - h) * ((kept + mn + kDecodeChunk - 1) / kDecodeChunk);
+      const int64_t li = h * ((N + mn + hp.dec_chunk - 1) / hp.dec_chunk) +
+                         (nkv - h) * ((kept + mn + hp.dec_chunk - 1) / hp.dec_chunk);
       blk_d[br] = li;
       ditems += li;
       hp.layer_items[(size_t)r] += li;
@@ -531,6 +553,9 @@ void fill_device_problem(taskkv_cache* c) {
   for (int32_t m : hp.mid) d.max_mid = m > d.max_mid ? m : d.max_mid;
   if (d.max_mid > hp.max_N) d.max_mid = hp.max_N;
   d.max_new = p.max_new_tokens;
+  d.dec_chunk = hp.dec_chunk;
+  d.max_prompt = hp.max_N;
+  d.max_cap = hp.max_N + p.max_new_tokens;
   d.idx_stride = hp.idx_stride;
   d.chunks_max = hp.chunks_max;
   d.pool_rows = hp.info.pool_rows;

@@ -10,7 +10,8 @@
 
 namespace taskkv {
 
-constexpr int kDecodeChunk = 512;                 // rows of one split-K decode item
+constexpr int kDecodeChunk = 512;                 // most rows of one split-K decode item
+constexpr int kDecodeChunkMin = 64;               // fewest
 constexpr int kGatherRows = 64;                   // rows of one gather item
 constexpr int kScoreChunk = 256;                  // keys of one window-score work item (CUDA-core path)
 constexpr int kTcChunk = 2048;                    // fewest keys of one window-score work item (tensor-core path)
@@ -53,6 +54,8 @@ struct DeviceProblem {
   // n_kv + h stands for layer view_l0 + r'.  q, k_new, v_new, out and `lengths` are indexed by view unit.
   int32_t view_l0, view_nl, view_U;
   int32_t max_new;
+  int32_t dec_chunk;    // rows of one split-K decode item of this cache
+  int32_t max_prompt, max_cap;   // most rows a unit holds right after compression, most it can grow to
   float budget_frac;    // > 0: the middle budget follows Eq. 17 from this fraction of the full cache
   // Head sharding: this problem holds KV heads [kv_first, kv_first + n_kv) of a model with n_kv_model per layer.
   // Eq. 8 / Eq. 16 / Eq. 17 count over the model's heads; the separator then reads every head's semantic vector

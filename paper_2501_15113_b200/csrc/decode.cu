@@ -2,15 +2,19 @@
 // head, no mask): o_a = softmax(q_a K_u^T / sqrt(d)) V_u over the len_u rows of
 // the KV head's segment, for the G query heads that share it.
 //
-// Split-K: a unit's rows are cut into work items of kDecodeChunk (512) rows, numbered once at
+// Split-K: a unit's rows are cut into work items of dec_chunk rows (512, fewer in small caches), numbered once at
 // compression for every unit at its capacity (so a 32768-row full head and a 772-row pruned head
 // load the SMs alike; items beyond a segment's current length are skipped).  Each item produces an un-normalised partial
 // (running max, sum, weighted V) per head with an online softmax in fp32; one
 // combine pass merges a unit's partials.  K/V rows are read once, as 16-byte
 // vectors, by all G heads.
+#include <cooperative_groups.h>
+
 #include <type_traits>
 
 #include "common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace taskkv {
 
@@ -56,102 +60,29 @@ struct PageWalk {
     }
   }
 };
+// One work item of the scalar path: rows [rbeg, rend) of unit u for the G heads of view unit vu (row new_r, if it is
+// among them, comes from kn_row / vn_row).  Leaves every row sub-group's running max, sum and weighted V in shared
+// memory.  AHEAD: the next iteration's rows are requested before this one's are used, for grids that leave the SMs
+// few warps; the arithmetic is the same.
 template <typename T, int D, int G, bool PAGED>
-__global__ void __launch_bounds__(kAttnThreads) decode_attn_kernel(DeviceProblem p, const T* __restrict__ q,
-                                                                   const int32_t* __restrict__ lengths,
-                                                                   const unsigned char* __restrict__ k_new,
-                                                                   const unsigned char* __restrict__ v_new,
-                                                                   T* __restrict__ out, int early) {
-  constexpr int EPL = 16 / (int)sizeof(T);          // elements per lane (one 16-byte vector)
-  constexpr int LPR = D / EPL;                      // lanes per row
-  constexpr int RPW = 32 / LPR;                     // rows per warp instruction
-  constexpr int NSG = kAttnWarps * RPW;             // row sub-groups per block
-  constexpr int ROW_BYTES = D * (int)sizeof(T);
-
-  __shared__ float sm_m[NSG][G];
-  __shared__ float sm_l[NSG][G];
-  __shared__ __align__(16) float sm_acc[NSG][G][D];
-  __shared__ int s_unit, s_rbeg;
-  __shared__ int s_direct;     // >= 0: the item is its unit's only one, the output goes to view unit s_direct
-
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int sg = lane / LPR, sl = lane % LPR;
-  const int gsg = warp * RPW + sg;
-  // the view's layers are a contiguous range of layer-major indices, hence of work items
-  const int w0 = p.view_l0 * lm_batch(p) * p.n_kv;
-  // (from the host's table of block starts: it does not depend on which layers have been compressed so far)
-  const int item0 = p.dec_base[p.view_l0 * lm_batch(p)], item1 = p.dec_base[(p.view_l0 + p.view_nl) * lm_batch(p)];
-  const float scale2 = kLog2e * rsqrtf((float)D);
-
-  // The table of work items is written when the cache is planned, not by the kernel before this one in the
-  // stream: the block's first item is looked up before the wait, under that kernel's tail.
-  int wi_first = 0;
-  if (warp == 0 && item0 + (int)blockIdx.x < item1)
-    wi_first = w0 + upper_unit_warp(p.dec_off + w0, p.view_U, item0 + (int)blockIdx.x, lane);
-  // `early` (set by the host when the kernel before this one in the stream cannot be one that writes these units'
-  // lengths or page tables: see launch_decode): the first item's unit data is read before the wait as well, and the
-  // wait comes just before the block first touches what the caller's kernels produce (q, the new token's rows) or
-  // writes anything.  (A block all of whose items are beyond their segments' lengths leaves without waiting.)
-  bool waited = false;
-  auto wait_once = [&]() {
-    if (!waited) {
-      grid_dependency_wait();
-      grid_launch_dependents();
-      waited = true;
-    }
+struct ScalarItem {
+  static constexpr int EPL = 16 / (int)sizeof(T);          // elements per lane (one 16-byte vector)
+  static constexpr int LPR = D / EPL;                      // lanes per row
+  static constexpr int RPW = 32 / LPR;                     // rows per warp instruction
+  static constexpr int NSG = kAttnWarps * RPW;             // row sub-groups per block
+  static constexpr int ROW_BYTES = D * (int)sizeof(T);
+  struct Smem {
+    float m[NSG][G], l[NSG][G];
+    __align__(16) float acc[NSG][G][D];
   };
-  if (!early) wait_once();
-  for (int item = item0 + blockIdx.x; item < item1; item += gridDim.x) {
-    __syncthreads();                                // previous item's shared state consumed
-    if (warp == 0) {
-      const int wi = item == item0 + (int)blockIdx.x ? wi_first
-                                                     : w0 + upper_unit_warp(p.dec_off + w0, p.view_U, item, lane);
-      if (lane == 0) {
-        s_unit = wi;
-        s_rbeg = (item - p.dec_off[wi]) * kDecodeChunk;
-      }
-    }
-    __syncthreads();
-    const int w = s_unit;
-    const LmUnit lu = lm_unit(p, w);
-    const int vu = lu.v;                            // view unit: index into q and lengths
-    const int u = lu.u;                             // unit: index into the cache
-    int len = p.len[u];
-    // fused step: the new token's row sits at index len; it is read from k_new / v_new and the item that holds
-    // it also stores it in the segment (the length itself is raised by the combine pass)
-    const int new_r = (k_new != nullptr && len < p.cap[u]) ? len : -1;
-    if (new_r >= 0) ++len;
-    if (lengths) len = min(max(lengths[vu], 0), len);
-    const int rbeg = s_rbeg;
-    if (rbeg >= len) continue;                      // an item of the reserve beyond the segment's length
-    const int rend = min(len, rbeg + kDecodeChunk);
-    if (tid == 0) s_direct = len <= kDecodeChunk ? vu : -1;     // read back after the row loop (no register held)
-    const int64_t seg = p.seg_off[u];
-    const unsigned char* kn_row = k_new + (size_t)vu * ROW_BYTES;
-    const unsigned char* vn_row = v_new + (size_t)vu * ROW_BYTES;
-    wait_once();
-    if (new_r >= rbeg && new_r < rend) {
-      bool have_page = true;
-      if (PAGED && new_r % p.page_rows == 0) {
-        // the appended row opens a new page: one comes off the pool (only this block touches the unit's new row)
-        if (tid == 0) {
-          const int at = pool_pop(p, 1);
-          if (at >= 0) p.page_tab[(size_t)u * p.page_stride + new_r / p.page_rows] = p.pool_free[at];
-          s_unit = at;                              // (the unit index has been read by everybody)
-        }
-        __syncthreads();
-        have_page = s_unit >= 0;                    // an empty pool: status ESTATE, the row is not stored
-      }
-      if (have_page && tid < ROW_BYTES / 16) {
-        const size_t drow = pool_row(p, u, seg, new_r);
-        unsigned char* kd = static_cast<unsigned char*>(p.k_pool) + drow * ROW_BYTES + tid * 16;
-        unsigned char* vd = static_cast<unsigned char*>(p.v_pool) + drow * ROW_BYTES + tid * 16;
-        *reinterpret_cast<uint4*>(kd) = *reinterpret_cast<const uint4*>(kn_row + tid * 16);
-        *reinterpret_cast<uint4*>(vd) = *reinterpret_cast<const uint4*>(vn_row + tid * 16);
-      }
-    }
-    ItemPages ip{0, 0};
-    if (PAGED) ip = item_pages(p, u, rbeg, lane);
+  template <bool AHEAD>
+  __device__ __forceinline__ static void run(const DeviceProblem& p, const T* __restrict__ q, int vu, int64_t seg, int rbeg,
+                                             int rend, int new_r, const unsigned char* kn_row, const unsigned char* vn_row,
+                                             const ItemPages& ip, Smem& sm) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int sg = lane / LPR, sl = lane % LPR;
+    const int gsg = warp * RPW + sg;
+    const float scale2 = kLog2e * rsqrtf((float)D);
     const unsigned char* kp = static_cast<const unsigned char*>(p.k_pool) + (PAGED ? 0 : (size_t)seg * ROW_BYTES) + sl * 16;
     const unsigned char* vp = static_cast<const unsigned char*>(p.v_pool) + (PAGED ? 0 : (size_t)seg * ROW_BYTES) + sl * 16;
 
@@ -176,7 +107,7 @@ __global__ void __launch_bounds__(kAttnThreads) decode_attn_kernel(DeviceProblem
     auto rows_loop = [&](auto has_new) {
     PageWalk pw{0, 0};
     if (PAGED) pw.start(p, ip, rbeg);
-    for (int base = rbeg; base < rend; base += NSG * kUnroll) {   // warp-uniform trip count
+    auto load = [&](int base, uint4 (&kraw)[kUnroll], uint4 (&vraw)[kUnroll]) {
       const int r0 = base + gsg;
       // pool row of row `base` minus base: adding a row index of this iteration gives its pool row
       size_t rowoff = 0;
@@ -184,7 +115,6 @@ __global__ void __launch_bounds__(kAttnThreads) decode_attn_kernel(DeviceProblem
         rowoff = pw.where(p, ip, base);
         pw.advance(p, NSG * kUnroll);
       }
-      uint4 kraw[kUnroll], vraw[kUnroll];
       // one 64-bit address per array and iteration; the unrolled loads differ by compile-time offsets
       const unsigned char* kb = kp + (rowoff + (size_t)r0) * ROW_BYTES;
       const unsigned char* vb = vp + (rowoff + (size_t)r0) * ROW_BYTES;
@@ -201,6 +131,9 @@ __global__ void __launch_bounds__(kAttnThreads) decode_attn_kernel(DeviceProblem
           vraw[i] = make_uint4(0, 0, 0, 0);
         }
       }
+    };
+    auto use = [&](int base, const uint4 (&kraw)[kUnroll], const uint4 (&vraw)[kUnroll]) {
+      const int r0 = base + gsg;
       float s[kUnroll][G];
 #pragma unroll
       for (int i = 0; i < kUnroll; ++i) {
@@ -251,46 +184,35 @@ __global__ void __launch_bounds__(kAttnThreads) decode_attn_kernel(DeviceProblem
 #pragma unroll
           for (int e = 0; e < EPL; ++e) acc[g][e] = fmaf(pw[i][g], vf[e], acc[g][e]);
       }
+    };
+    constexpr int kStep = NSG * kUnroll;
+    if constexpr (AHEAD) {
+      uint4 k0[kUnroll], v0[kUnroll], k1[kUnroll], v1[kUnroll];
+      load(rbeg, k0, v0);
+      for (int base = rbeg; base < rend; base += 2 * kStep) {     // warp-uniform trip count
+        if (base + kStep < rend) load(base + kStep, k1, v1);
+        use(base, k0, v0);
+        if (base + 2 * kStep < rend) load(base + 2 * kStep, k0, v0);
+        if (base + kStep < rend) use(base + kStep, k1, v1);
+      }
+    } else {
+      for (int base = rbeg; base < rend; base += kStep) {         // warp-uniform trip count
+        uint4 kraw[kUnroll], vraw[kUnroll];
+        load(base, kraw, vraw);
+        use(base, kraw, vraw);
+      }
     }
-
     };
     if (new_r >= rbeg && new_r < rend) rows_loop(std::true_type{}); else rows_loop(std::false_type{});
 
-    // merge the block's sub-groups
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      if (sl == 0) { sm_m[gsg][g] = m[g]; sm_l[gsg][g] = l[g]; }
+      if (sl == 0) { sm.m[gsg][g] = m[g]; sm.l[gsg][g] = l[g]; }
 #pragma unroll
-      for (int e = 0; e < EPL; ++e) sm_acc[gsg][g][sl * EPL + e] = acc[g][e];
-    }
-    __syncthreads();
-    for (int i = tid; i < G * D; i += kAttnThreads) {
-      const int g = i / D, dd = i % D;
-      float M = -INFINITY;
-#pragma unroll
-      for (int x = 0; x < NSG; ++x) M = fmaxf(M, sm_m[x][g]);
-      float a = 0.f, ll = 0.f;
-#pragma unroll
-      for (int x = 0; x < NSG; ++x) {
-        const float mx = sm_m[x][g];
-        const float w = (mx == -INFINITY) ? 0.f : exp2f(mx - M);
-        a = fmaf(w, sm_acc[x][g][dd], a);
-        ll = fmaf(w, sm_l[x][g], ll);
-      }
-      if (s_direct >= 0) {
-        // the unit's only item: this is Eq. 1 over the whole segment (what the combine pass would make of one
-        // partial, bit for bit); the combine pass skips such units
-        store_out(out + ((size_t)s_direct * G + g) * D + dd, ll > 0.f ? a / ll : 0.f);
-        continue;
-      }
-      p.part_acc[((size_t)item * G + g) * D + dd] = a;
-      if (dd == 0) {
-        p.part_ml[((size_t)item * G + g) * 2 + 0] = M;
-        p.part_ml[((size_t)item * G + g) * 2 + 1] = ll;
-      }
+      for (int e = 0; e < EPL; ++e) sm.acc[gsg][g][sl * EPL + e] = acc[g][e];
     }
   }
-}
+};
 
 // ---------------------------------------------------------------------------------------------
 // Grouped-query variant for bf16 (G >= 2 query heads per KV head): with several heads per row the
@@ -325,105 +247,29 @@ __device__ __forceinline__ uint32_t word_of(const uint4& v, int i) {
   return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w;
 }
 
+// One work item of the warp-mma path (see ScalarItem): the sub-groups are the block's four warps.
 template <int D, int G, bool PAGED>
-__global__ void __launch_bounds__(kAttnThreads, 4) decode_attn_mma_kernel(DeviceProblem p,
-                                                                       const __nv_bfloat16* __restrict__ q,
-                                                                       const int32_t* __restrict__ lengths,
-                                                                       const unsigned char* __restrict__ k_new,
-                                                                       const unsigned char* __restrict__ v_new,
-                                                                       __nv_bfloat16* __restrict__ out, int early) {
-  constexpr int ROW_BYTES = D * 2;
-  constexpr int KC = D / 16;            // k-chunks of the first product
-  constexpr int KP = D / 32;            // 16-byte pieces of a K row per lane
-  constexpr int MB = D / 16;            // m-blocks (16 d each) of the second product
-  constexpr int VP = D / 64;            // 16-byte pieces of a V row per lane
-  constexpr int kBlk = 16;              // cache rows per warp iteration
-
-  __shared__ float sm_m[kAttnWarps][G];
-  __shared__ float sm_l[kAttnWarps][G];
-  __shared__ __align__(16) float sm_acc[kAttnWarps][G][D];
-  __shared__ int s_unit, s_rbeg;
-  __shared__ int s_direct;     // >= 0: the item is its unit's only one, the output goes to view unit s_direct
-
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int g = lane >> 2, t = lane & 3;
-  // the view's layers are a contiguous range of layer-major indices, hence of work items
-  const int w0 = p.view_l0 * lm_batch(p) * p.n_kv;
-  // (from the host's table of block starts: it does not depend on which layers have been compressed so far)
-  const int item0 = p.dec_base[p.view_l0 * lm_batch(p)], item1 = p.dec_base[(p.view_l0 + p.view_nl) * lm_batch(p)];
-  const float scale2 = kLog2e * rsqrtf((float)D);
-  // d of accumulator row (mb, hf) of this lane's two output rows: e = hf * MB + mb, piece e / 8, element e % 8
-  auto pd = [&](int mb, int hf, int gg) { const int e = hf * MB + mb; return (e >> 3) * 64 + gg * 8 + (e & 7); };
-
-  // The table of work items is written when the cache is planned, not by the kernel before this one in the
-  // stream: the block's first item is looked up before the wait, under that kernel's tail.
-  int wi_first = 0;
-  if (warp == 0 && item0 + (int)blockIdx.x < item1)
-    wi_first = w0 + upper_unit_warp(p.dec_off + w0, p.view_U, item0 + (int)blockIdx.x, lane);
-  // `early` (set by the host when the kernel before this one in the stream cannot be one that writes these units'
-  // lengths or page tables: see launch_decode): the first item's unit data is read before the wait as well, and the
-  // wait comes just before the block first touches what the caller's kernels produce (q, the new token's rows) or
-  // writes anything.  (A block all of whose items are beyond their segments' lengths leaves without waiting.)
-  bool waited = false;
-  auto wait_once = [&]() {
-    if (!waited) {
-      grid_dependency_wait();
-      grid_launch_dependents();
-      waited = true;
-    }
+struct MmaItem {
+  static constexpr int NSG = kAttnWarps;
+  static constexpr int ROW_BYTES = D * 2;
+  static constexpr int KC = D / 16;            // k-chunks of the first product
+  static constexpr int KP = D / 32;            // 16-byte pieces of a K row per lane
+  static constexpr int MB = D / 16;            // m-blocks (16 d each) of the second product
+  static constexpr int VP = D / 64;            // 16-byte pieces of a V row per lane
+  static constexpr int kBlk = 16;              // cache rows per warp iteration
+  struct Smem {
+    float m[NSG][G], l[NSG][G];
+    __align__(16) float acc[NSG][G][D];
   };
-  if (!early) wait_once();
-  for (int item = item0 + blockIdx.x; item < item1; item += gridDim.x) {
-    __syncthreads();
-    if (warp == 0) {
-      const int wi = item == item0 + (int)blockIdx.x ? wi_first
-                                                     : w0 + upper_unit_warp(p.dec_off + w0, p.view_U, item, lane);
-      if (lane == 0) {
-        s_unit = wi;
-        s_rbeg = (item - p.dec_off[wi]) * kDecodeChunk;
-      }
-    }
-    __syncthreads();
-    const int w = s_unit;
-    const LmUnit lu = lm_unit(p, w);
-    const int vu = lu.v;                            // view unit: index into q and lengths
-    const int u = lu.u;                             // unit: index into the cache
-    int len = p.len[u];
-    // fused step: the new token's row sits at index len; it is read from k_new / v_new and the item that holds
-    // it also stores it in the segment (the length itself is raised by the combine pass)
-    const int new_r = (k_new != nullptr && len < p.cap[u]) ? len : -1;
-    if (new_r >= 0) ++len;
-    if (lengths) len = min(max(lengths[vu], 0), len);
-    const int rbeg = s_rbeg;
-    if (rbeg >= len) continue;                      // an item of the reserve beyond the segment's length
-    const int rend = min(len, rbeg + kDecodeChunk);
-    if (tid == 0) s_direct = len <= kDecodeChunk ? vu : -1;     // read back after the row loop (no register held)
-    const int64_t seg = p.seg_off[u];
-    const unsigned char* kn_row = k_new + (size_t)vu * ROW_BYTES;
-    const unsigned char* vn_row = v_new + (size_t)vu * ROW_BYTES;
-    wait_once();
-    if (new_r >= rbeg && new_r < rend) {
-      bool have_page = true;
-      if (PAGED && new_r % p.page_rows == 0) {
-        // the appended row opens a new page: one comes off the pool (only this block touches the unit's new row)
-        if (tid == 0) {
-          const int at = pool_pop(p, 1);
-          if (at >= 0) p.page_tab[(size_t)u * p.page_stride + new_r / p.page_rows] = p.pool_free[at];
-          s_unit = at;                              // (the unit index has been read by everybody)
-        }
-        __syncthreads();
-        have_page = s_unit >= 0;                    // an empty pool: status ESTATE, the row is not stored
-      }
-      if (have_page && tid < ROW_BYTES / 16) {
-        const size_t drow = pool_row(p, u, seg, new_r);
-        unsigned char* kd = static_cast<unsigned char*>(p.k_pool) + drow * ROW_BYTES + tid * 16;
-        unsigned char* vd = static_cast<unsigned char*>(p.v_pool) + drow * ROW_BYTES + tid * 16;
-        *reinterpret_cast<uint4*>(kd) = *reinterpret_cast<const uint4*>(kn_row + tid * 16);
-        *reinterpret_cast<uint4*>(vd) = *reinterpret_cast<const uint4*>(vn_row + tid * 16);
-      }
-    }
-    ItemPages ip{0, 0};
-    if (PAGED) ip = item_pages(p, u, rbeg, lane);
+  template <bool AHEAD>
+  __device__ __forceinline__ static void run(const DeviceProblem& p, const __nv_bfloat16* __restrict__ q, int vu, int64_t seg,
+                                             int rbeg, int rend, int new_r, const unsigned char* kn_row,
+                                             const unsigned char* vn_row, const ItemPages& ip, Smem& sm) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int g = lane >> 2, t = lane & 3;
+    const float scale2 = kLog2e * rsqrtf((float)D);
+    // d of accumulator row (mb, hf) of this lane's two output rows: e = hf * MB + mb, piece e / 8, element e % 8
+    auto pd = [&](int mb, int hf, int gg) { const int e = hf * MB + mb; return (e >> 3) * 64 + gg * 8 + (e & 7); };
     const unsigned char* kp = static_cast<const unsigned char*>(p.k_pool);
     const unsigned char* vp = static_cast<const unsigned char*>(p.v_pool);
 
@@ -449,12 +295,12 @@ __global__ void __launch_bounds__(kAttnThreads, 4) decode_attn_mma_kernel(Device
     auto rows_loop = [&](auto has_new) {
     PageWalk pw{0, 0};
     if (PAGED) pw.start(p, ip, rbeg + warp * kBlk);
-    // kb, vb: this lane's first K and V vector of the current 16-row block; the unrolled loads differ from them by
+    // kb, vb: this lane's first K and V vector of the next 16-row block to load; the unrolled loads differ from them by
     // compile-time offsets.  Contiguous layout: row r of the unit is pool row seg + r, the pointers step from block
     // to block; paged: they are set from the block's page.
     const unsigned char* kb = kp + ((size_t)seg + (size_t)(rbeg + warp * kBlk)) * ROW_BYTES + klane;
     const unsigned char* vb = vp + ((size_t)seg + (size_t)(rbeg + warp * kBlk)) * ROW_BYTES + vlane;
-    for (int blk = rbeg + warp * kBlk; blk < rend; blk += kAttnWarps * kBlk) {   // warp-uniform
+    auto load = [&](int blk, uint4 (&kraw)[2][KP], uint4 (&vraw)[4][VP]) {
       if (PAGED) {
         // pool row of row `blk` minus blk: adding a row index of this 16-row block gives its pool row
         const size_t rowoff = pw.where(p, ip, blk);
@@ -462,7 +308,6 @@ __global__ void __launch_bounds__(kAttnThreads, 4) decode_attn_mma_kernel(Device
         kb = kp + (rowoff + (size_t)blk) * ROW_BYTES + klane;
         vb = vp + (rowoff + (size_t)blk) * ROW_BYTES + vlane;
       }
-      uint4 kraw[2][KP], vraw[4][VP];
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         const int r = blk + 8 * j + g;
@@ -483,6 +328,12 @@ __global__ void __launch_bounds__(kAttnThreads, 4) decode_attn_mma_kernel(Device
                                                                       : vb + ((x & 1) + 8 * (x >> 1)) * ROW_BYTES + i * 128)
                                 : make_uint4(0, 0, 0, 0);
       }
+      if (!PAGED) {
+        kb += kAttnWarps * kBlk * ROW_BYTES;
+        vb += kAttnWarps * kBlk * ROW_BYTES;
+      }
+    };
+    auto use = [&](int blk, const uint4 (&kraw)[2][KP], const uint4 (&vraw)[4][VP]) {
       // S^T for the two 8-row halves of the block
       float sc[2][4];
 #pragma unroll
@@ -538,51 +389,172 @@ __global__ void __launch_bounds__(kAttnThreads, 4) decode_attn_mma_kernel(Device
         }
         mma_bf16_16816(o[mb], a[0], a[1], a[2], a[3], pb0, pb1);
       }
-      if (!PAGED) {
-        kb += kAttnWarps * kBlk * ROW_BYTES;
-        vb += kAttnWarps * kBlk * ROW_BYTES;
+    };
+    constexpr int kStep = kAttnWarps * kBlk;
+    const int first = rbeg + warp * kBlk;
+    if constexpr (AHEAD) {
+      uint4 k0[2][KP], v0[4][VP], k1[2][KP], v1[4][VP];
+      if (first < rend) load(first, k0, v0);
+      for (int blk = first; blk < rend; blk += 2 * kStep) {       // warp-uniform
+        if (blk + kStep < rend) load(blk + kStep, k1, v1);
+        use(blk, k0, v0);
+        if (blk + 2 * kStep < rend) load(blk + 2 * kStep, k0, v0);
+        if (blk + kStep < rend) use(blk + kStep, k1, v1);
+      }
+    } else {
+      for (int blk = first; blk < rend; blk += kStep) {           // warp-uniform
+        uint4 kraw[2][KP], vraw[4][VP];
+        load(blk, kraw, vraw);
+        use(blk, kraw, vraw);
       }
     }
-
     };
     if (new_r >= rbeg && new_r < rend) rows_loop(std::true_type{}); else rows_loop(std::false_type{});
 
-    // merge the four warps (same partial format as the scalar kernel)
     l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
     l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
-    if (t == 0 && g < G) { sm_m[warp][g] = m_run; sm_l[warp][g] = l_run; }
+    if (t == 0 && g < G) { sm.m[warp][g] = m_run; sm.l[warp][g] = l_run; }
 #pragma unroll
     for (int mb = 0; mb < MB; ++mb)
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const int head = 2 * t + (e & 1);
-        if (head < G) sm_acc[warp][head][pd(mb, e >> 1, g)] = o[mb][e];
+        if (head < G) sm.acc[warp][head][pd(mb, e >> 1, g)] = o[mb][e];
       }
+  }
+};
+
+template <typename T, int D, int G, bool PAGED>
+using Item = typename std::conditional<sizeof(T) == 2, MmaItem<D, G, PAGED>, ScalarItem<T, D, G, PAGED>>::type;
+
+// Merges the sub-groups an item left in shared memory: emit(head, d, weighted V, max, sum) for this thread's elements.
+template <int NSG, int D, int G, class Smem, class Emit>
+__device__ __forceinline__ void merge_item(const Smem& sm, const Emit& emit) {
+  for (int i = threadIdx.x; i < G * D; i += kAttnThreads) {
+    const int hh = i / D, dd = i % D;
+    float M = -INFINITY;
+#pragma unroll
+    for (int x = 0; x < NSG; ++x) M = fmaxf(M, sm.m[x][hh]);
+    float a = 0.f, ll = 0.f;
+#pragma unroll
+    for (int x = 0; x < NSG; ++x) {
+      const float mx = sm.m[x][hh];
+      const float w = (mx == -INFINITY) ? 0.f : exp2f(mx - M);
+      a = fmaf(w, sm.acc[x][hh][dd], a);
+      ll = fmaf(w, sm.l[x][hh], ll);
+    }
+    emit(hh, dd, a, M, ll);
+  }
+}
+
+// The new token's K and V rows into the segment of unit u at row new_r, by the block whose work item holds that row
+// (only it touches the unit's new row).  s_word: a shared word free for use here.
+template <int ROW_BYTES, bool PAGED>
+__device__ __forceinline__ void store_new_row(const DeviceProblem& p, int u, int64_t seg, int new_r,
+                                              const unsigned char* kn_row, const unsigned char* vn_row, int* s_word) {
+  const int tid = threadIdx.x;
+  bool have_page = true;
+  if (PAGED && new_r % p.page_rows == 0) {
+    // the appended row opens a new page: one comes off the pool
+    if (tid == 0) {
+      const int at = pool_pop(p, 1);
+      if (at >= 0) p.page_tab[(size_t)u * p.page_stride + new_r / p.page_rows] = p.pool_free[at];
+      *s_word = at;
+    }
     __syncthreads();
-    for (int i = tid; i < G * D; i += kAttnThreads) {
-      const int hh = i / D, dd = i % D;
-      float M = -INFINITY;
-#pragma unroll
-      for (int x = 0; x < kAttnWarps; ++x) M = fmaxf(M, sm_m[x][hh]);
-      float a = 0.f, ll = 0.f;
-#pragma unroll
-      for (int x = 0; x < kAttnWarps; ++x) {
-        const float mx = sm_m[x][hh];
-        const float w = (mx == -INFINITY) ? 0.f : exp2f(mx - M);
-        a = fmaf(w, sm_acc[x][hh][dd], a);
-        ll = fmaf(w, sm_l[x][hh], ll);
+    have_page = *s_word >= 0;                       // an empty pool: status ESTATE, the row is not stored
+  }
+  if (have_page && tid < ROW_BYTES / 16) {
+    const size_t drow = pool_row(p, u, seg, new_r);
+    unsigned char* kd = static_cast<unsigned char*>(p.k_pool) + drow * ROW_BYTES + tid * 16;
+    unsigned char* vd = static_cast<unsigned char*>(p.v_pool) + drow * ROW_BYTES + tid * 16;
+    *reinterpret_cast<uint4*>(kd) = *reinterpret_cast<const uint4*>(kn_row + tid * 16);
+    *reinterpret_cast<uint4*>(vd) = *reinterpret_cast<const uint4*>(vn_row + tid * 16);
+  }
+}
+
+template <typename T, int D, int G, bool PAGED>
+__global__ void __launch_bounds__(kAttnThreads, sizeof(T) == 2 ? 4 : 1)
+decode_attn_kernel(DeviceProblem p, const T* __restrict__ q, const int32_t* __restrict__ lengths,
+                   const unsigned char* __restrict__ k_new, const unsigned char* __restrict__ v_new, T* __restrict__ out,
+                   int early) {
+  using It = Item<T, D, G, PAGED>;
+  constexpr int ROW_BYTES = It::ROW_BYTES;
+  __shared__ typename It::Smem sm;
+  __shared__ int s_unit, s_rbeg, s_word;
+  __shared__ int s_direct;     // >= 0: the item is its unit's only one, the output goes to view unit s_direct
+
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // the view's layers are a contiguous range of layer-major indices, hence of work items
+  const int w0 = p.view_l0 * lm_batch(p) * p.n_kv;
+  // (from the host's table of block starts: it does not depend on which layers have been compressed so far)
+  const int item0 = p.dec_base[p.view_l0 * lm_batch(p)], item1 = p.dec_base[(p.view_l0 + p.view_nl) * lm_batch(p)];
+
+  // The table of work items is written when the cache is planned, not by the kernel before this one in the
+  // stream: the block's first item is looked up before the wait, under that kernel's tail.
+  int wi_first = 0;
+  if (warp == 0 && item0 + (int)blockIdx.x < item1)
+    wi_first = w0 + upper_unit_warp(p.dec_off + w0, p.view_U, item0 + (int)blockIdx.x, lane);
+  // `early` (set by the host when the kernel before this one in the stream cannot be one that writes these units'
+  // lengths or page tables: see launch_decode): the first item's unit data is read before the wait as well, and the
+  // wait comes just before the block first touches what the caller's kernels produce (q, the new token's rows) or
+  // writes anything.  (A block all of whose items are beyond their segments' lengths leaves without waiting.)
+  bool waited = false;
+  auto wait_once = [&]() {
+    if (!waited) {
+      grid_dependency_wait();
+      grid_launch_dependents();
+      waited = true;
+    }
+  };
+  if (!early) wait_once();
+  for (int item = item0 + blockIdx.x; item < item1; item += gridDim.x) {
+    __syncthreads();
+    if (warp == 0) {
+      const int wi = item == item0 + (int)blockIdx.x ? wi_first
+                                                     : w0 + upper_unit_warp(p.dec_off + w0, p.view_U, item, lane);
+      if (lane == 0) {
+        s_unit = wi;
+        s_rbeg = (item - p.dec_off[wi]) * p.dec_chunk;
       }
+    }
+    __syncthreads();
+    const int w = s_unit;
+    const LmUnit lu = lm_unit(p, w);
+    const int vu = lu.v;                            // view unit: index into q and lengths
+    const int u = lu.u;                             // unit: index into the cache
+    int len = p.len[u];
+    // fused step: the new token's row sits at index len; it is read from k_new / v_new and the item that holds
+    // it also stores it in the segment (the length itself is raised by the combine pass)
+    const int new_r = (k_new != nullptr && len < p.cap[u]) ? len : -1;
+    if (new_r >= 0) ++len;
+    if (lengths) len = min(max(lengths[vu], 0), len);
+    const int rbeg = s_rbeg;
+    if (rbeg >= len) continue;                      // an item of the reserve beyond the segment's length
+    const int rend = min(len, rbeg + p.dec_chunk);
+    if (tid == 0) s_direct = len <= p.dec_chunk ? vu : -1;     // read back after the row loop (no register held)
+    const int64_t seg = p.seg_off[u];
+    const unsigned char* kn_row = k_new + (size_t)vu * ROW_BYTES;
+    const unsigned char* vn_row = v_new + (size_t)vu * ROW_BYTES;
+    wait_once();
+    if (new_r >= rbeg && new_r < rend) store_new_row<ROW_BYTES, PAGED>(p, u, seg, new_r, kn_row, vn_row, &s_word);
+    ItemPages ip{0, 0};
+    if (PAGED) ip = item_pages(p, u, rbeg, lane);
+    It::template run<false>(p, q, vu, seg, rbeg, rend, new_r, kn_row, vn_row, ip, sm);
+    __syncthreads();
+    merge_item<It::NSG, D, G>(sm, [&](int hh, int dd, float a, float M, float ll) {
       if (s_direct >= 0) {
-        // the unit's only item: Eq. 1 over the whole segment, as in the scalar kernel
+        // the unit's only item: this is Eq. 1 over the whole segment (what the combine pass would make of one
+        // partial, bit for bit); the combine pass skips such units
         store_out(out + ((size_t)s_direct * G + hh) * D + dd, ll > 0.f ? a / ll : 0.f);
-        continue;
+        return;
       }
       p.part_acc[((size_t)item * G + hh) * D + dd] = a;
       if (dd == 0) {
         p.part_ml[((size_t)item * G + hh) * 2 + 0] = M;
         p.part_ml[((size_t)item * G + hh) * 2 + 1] = ll;
       }
-    }
+    });
   }
 }
 
@@ -620,7 +592,7 @@ __global__ void __launch_bounds__(kCombineThreads, PRE > 0 ? 4 : 6) decode_combi
   len = len_next;
   if (lengths) len = min(max(lengths[u], 0), len);
   // the unit's items that hold rows (the table also numbers the reserve for appended tokens)
-  const int i0 = p.dec_off[lm_index(p, unit)], i1 = i0 + (len + kDecodeChunk - 1) / kDecodeChunk;
+  const int i0 = p.dec_off[lm_index(p, unit)], i1 = i0 + (len + p.dec_chunk - 1) / p.dec_chunk;
   grid_dependency_wait();
   grid_launch_dependents();
   if (i1 - i0 != 1) {                                   // a unit of one item has its output from the attention kernel
@@ -704,11 +676,196 @@ __global__ void __launch_bounds__(kCombineThreads, PRE > 0 ? 4 : 6) decode_combi
   }
 }
 
+// Asks for rows [r0, r1) of a work item (K by warp 0, V by warp 1) to be brought into L2.  A hint only: nothing is
+// ordered by it, and it may be given before the rows' writers are known to be complete.
+template <int ROW_BYTES, bool PAGED>
+__device__ __forceinline__ void prefetch_item(const DeviceProblem& p, const ItemPages& ip, int64_t seg, int r0, int r1) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp > 1) return;
+  const unsigned char* pool = static_cast<const unsigned char*>(warp == 0 ? p.k_pool : p.v_pool);
+  size_t row = (size_t)seg + (size_t)r0;
+  if (PAGED) {
+    const int pg = ip.first + lane;                        // lanes 0..7: one page each
+    r0 = max(r0, pg * p.page_rows);
+    r1 = lane < 8 ? min(r1, (pg + 1) * p.page_rows) : r0;
+    row = (size_t)ip.mine * p.page_rows + (size_t)(r0 - pg * p.page_rows);
+  } else if (lane > 0) {
+    return;
+  }
+  if (r1 > r0)
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(pool + row * ROW_BYTES), "r"((r1 - r0) * ROW_BYTES)
+                 : "memory");
+}
+
+// The whole of a small call in one launch: a thread-block cluster of cs CTAs owns a unit, its CTAs take the unit's work
+// items (rank, rank + cs), push their partial results into the cluster's shared memory, and every CTA merges its share
+// of the outputs after one cluster barrier.  The items, their arithmetic and the order in which they are merged are
+// those of the two kernels above, so the results are theirs bit for bit.
+// Bound by latency (a layer of a 4096-token, 32-head prompt holds 21 MB, 3.2 us of HBM time; two launches 17.2 us, this
+// one 13.9; one fp32 layer of 8 heads x 512 rows 16.6 and 6.4 us, there with items of 64 rows instead of 512): it saves the second launch, the
+// trip of the partial results through L2 and the search for the block's work item; an item's rows are requested into
+// L2 as a whole when it starts, and where the registers allow it (d = 64, fp32) the warps, few to an SM here, load the
+// next rows before they use the present ones.
+constexpr int kClusterSlots = 2;         // items per CTA
+constexpr int kClusterMax = 16;          // CTAs per cluster
+constexpr int kClusterItems = kClusterSlots * kClusterMax;
+static_assert(kClusterItems <= 32, "one lane per item in the merge");
+
+template <typename T, int D, int G, bool PAGED>
+__global__ void __launch_bounds__(kAttnThreads, 2)
+decode_cluster_kernel(DeviceProblem p, const T* __restrict__ q, const int32_t* __restrict__ lengths,
+                      const unsigned char* __restrict__ k_new, const unsigned char* __restrict__ v_new,
+                      T* __restrict__ out, int early) {
+  using It = Item<T, D, G, PAGED>;
+  constexpr int ROW_BYTES = It::ROW_BYTES;
+  constexpr bool kAhead = sizeof(T) == 4 || D == 64;
+  __shared__ typename It::Smem sm;
+  __shared__ float s_part[kClusterSlots * G * D];        // [item][this CTA's share of the G * D outputs]
+  __shared__ float2 s_ml[G][kClusterItems];              // (max, sum) of every item
+  __shared__ float s_w[G][kClusterItems], s_L[G];
+  __shared__ int s_word;
+  cg::cluster_group cl = cg::this_cluster();
+  const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int v = (int)blockIdx.x / cs, u = view_unit(p, v);
+  const int share = G * D / cs;
+  cl.sync();                                             // every CTA is there before anything is pushed to it
+  if (!early) { grid_dependency_wait(); grid_launch_dependents(); }
+  int len = p.len[u];
+  const bool fused = k_new != nullptr;
+  const bool grown = fused && len < p.cap[u];
+  const int len_next = len + (grown ? 1 : 0), new_r = grown ? len : -1;
+  const int64_t seg = p.seg_off[u];
+  len = len_next;
+  if (lengths) len = min(max(lengths[v], 0), len);
+  const int n = (len + p.dec_chunk - 1) / p.dec_chunk;
+  const int old_len = new_r >= 0 ? min(len, new_r) : len;   // rows that are in the segment already
+  if (!PAGED) prefetch_item<ROW_BYTES, PAGED>(p, ItemPages{0, 0}, seg, rank * p.dec_chunk, min(old_len, (rank + 1) * p.dec_chunk));
+  if (early) { grid_dependency_wait(); grid_launch_dependents(); }
+  for (int j = rank; j < n; j += cs) {
+    const int rbeg = j * p.dec_chunk, rend = min(len, rbeg + p.dec_chunk);
+    const unsigned char* kn_row = k_new + (size_t)v * ROW_BYTES;
+    const unsigned char* vn_row = v_new + (size_t)v * ROW_BYTES;
+    if (new_r >= rbeg && new_r < rend) store_new_row<ROW_BYTES, PAGED>(p, u, seg, new_r, kn_row, vn_row, &s_word);
+    ItemPages ip{0, 0};
+    if (PAGED) {
+      ip = item_pages(p, u, rbeg, lane);
+      prefetch_item<ROW_BYTES, PAGED>(p, ip, seg, rbeg, min(rend, old_len));
+    }
+    __syncthreads();                                     // the previous item's sub-groups have been merged
+    It::template run<kAhead>(p, q, v, seg, rbeg, rend, new_r, kn_row, vn_row, ip, sm);
+    __syncthreads();
+    merge_item<It::NSG, D, G>(sm, [&](int hh, int dd, float a, float M, float ll) {
+      if (n == 1) {
+        store_out(out + ((size_t)v * G + hh) * D + dd, ll > 0.f ? a / ll : 0.f);
+        return;
+      }
+      const int i = hh * D + dd, owner = i / share;
+      *cl.map_shared_rank(&s_part[j * share + (i - owner * share)], owner) = a;
+      if (dd < cs) *cl.map_shared_rank(&s_ml[hh][j], dd) = make_float2(M, ll);
+    });
+  }
+  cl.sync();                                             // all items are in; every CTA has read the length
+  if (n != 1) {
+    for (int hh = warp; hh < G; hh += kAttnWarps) {
+      const float2 o = lane < n ? s_ml[hh][lane] : make_float2(-INFINITY, 0.f);
+      const float M = warp_max(o.x);
+      const float w = (o.x == -INFINITY) ? 0.f : exp2f(o.x - M);
+      s_w[hh][lane] = w;
+      const float L = warp_sum(fmaf(w, o.y, 0.f));
+      if (lane == 0) s_L[hh] = L;
+    }
+    __syncthreads();
+    for (int i = tid; i < share; i += kAttnThreads) {
+      const int hh = (rank * share + i) / D;
+      float a = 0.f;
+      for (int w = 0; w < kCombineWarps; ++w) {          // the order of the combine kernel's warps
+        float acc = 0.f;
+        for (int j = w; j < n; j += kCombineWarps) acc = fmaf(s_w[hh][j], s_part[j * share + i], acc);
+        a += acc;
+      }
+      const float L = s_L[hh];
+      store_out(out + (size_t)v * G * D + rank * share + i, L > 0.f ? a / L : 0.f);
+    }
+  }
+  if (fused && rank == 0 && tid == 0) {
+    // (a recorded device error freezes the lengths of a paged cache, as in the combine kernel)
+    if (!grown) set_status(p.status, TASKKV_ESTATE);
+    else if (!PAGED || *reinterpret_cast<volatile int32_t*>(p.status) == 0) p.len[u] = len_next;
+  }
+}
+
+// Whether the device co-schedules a cluster of cs CTAs of this kernel (16 is above the portable size).
+template <typename T, int D, int G, bool PAGED>
+bool cluster16_fits() {
+  static const bool ok = [] {
+    if (cudaFuncSetAttribute(decode_cluster_kernel<T, D, G, PAGED>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+        cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kClusterMax, 1, 1);
+    cfg.blockDim = dim3(kAttnThreads, 1, 1);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = kClusterMax;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, decode_cluster_kernel<T, D, G, PAGED>, &cfg) != cudaSuccess) n = 0;
+    cudaGetLastError();
+    return n > 0;
+  }();
+  return ok;
+}
+
+// CTAs per unit for the one-launch form, 0 if the call is not small enough for it.  A unit gets a CTA per item of the
+// longest prompt (the tokens appended since may give a CTA a second one), and all CTAs of the call fit on the GPU
+// together, two to an SM: beyond that the call is bound by HBM, and the persistent attention kernel with its
+// deal of equal items is the better one.
+int cluster_size(const DeviceProblem& p) {
+  const int items_cap = (p.max_cap + p.dec_chunk - 1) / p.dec_chunk, items = (p.max_prompt + p.dec_chunk - 1) / p.dec_chunk;
+  if (items_cap > kClusterItems) return 0;
+  int cs = 1;
+  while (cs < items || kClusterSlots * cs < items_cap) cs *= 2;
+  if (cs > kClusterMax || cs > p.G * p.d || (int64_t)p.view_U * cs > 148 * 2) return 0;
+  return cs;
+}
+
+template <typename T, int D, int G, bool PAGED>
+cudaError_t launch_cluster(const DeviceProblem& p, int cs, const T* q, const int32_t* lengths, const unsigned char* kn,
+                           const unsigned char* vn, T* out, cudaStream_t s, int early) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(p.view_U * cs), 1, 1);
+  cfg.blockDim = dim3(kAttnThreads, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cs;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  LaunchScope ls(K_DECODE_ATTN, s);
+  return cudaLaunchKernelEx(&cfg, decode_cluster_kernel<T, D, G, PAGED>, p, q, lengths, kn, vn, out, early);
+}
+
 template <typename T, int D, int G>
 cudaError_t launch_typed(const DeviceProblem& p, const void* q, const int32_t* lengths, const void* k_new,
                          const void* v_new, void* out, cudaStream_t s, int early) {
   const unsigned char* kn = static_cast<const unsigned char*>(k_new);
   const unsigned char* vn = static_cast<const unsigned char*>(v_new);
+  const int cs = cluster_size(p);
+  if (cs > 0 && (cs <= 8 || (p.page_rows > 0 ? cluster16_fits<T, D, G, true>() : cluster16_fits<T, D, G, false>()))) {
+    const T* qt = static_cast<const T*>(q);
+    return p.page_rows > 0 ? launch_cluster<T, D, G, true>(p, cs, qt, lengths, kn, vn, static_cast<T*>(out), s, early)
+                           : launch_cluster<T, D, G, false>(p, cs, qt, lengths, kn, vn, static_cast<T*>(out), s, early);
+  }
   // persistent blocks: 16 per SM (measured best on B200 with 512-row items)
   int64_t grid = p.max_items < 148 * 16 ? p.max_items : 148 * 16;
   if (grid < 1) grid = 1;
@@ -717,12 +874,12 @@ cudaError_t launch_typed(const DeviceProblem& p, const void* q, const int32_t* l
     LaunchScope ls(K_DECODE_ATTN, s);
     if (p.page_rows > 0) {
       if constexpr (sizeof(T) == 2)
-        e = launch_dependent(decode_attn_mma_kernel<D, G, true>, (unsigned)grid, kAttnThreads, s, p, static_cast<const T*>(q), lengths, kn, vn, static_cast<T*>(out), early);
+        e = launch_dependent(decode_attn_kernel<T, D, G, true>, (unsigned)grid, kAttnThreads, s, p, static_cast<const T*>(q), lengths, kn, vn, static_cast<T*>(out), early);
       else
         e = launch_dependent(decode_attn_kernel<T, D, G, true>, (unsigned)grid, kAttnThreads, s, p, static_cast<const T*>(q), lengths, kn, vn, static_cast<T*>(out), early);
     } else {
       if constexpr (sizeof(T) == 2)
-        e = launch_dependent(decode_attn_mma_kernel<D, G, false>, (unsigned)grid, kAttnThreads, s, p, static_cast<const T*>(q), lengths, kn, vn, static_cast<T*>(out), early);
+        e = launch_dependent(decode_attn_kernel<T, D, G, false>, (unsigned)grid, kAttnThreads, s, p, static_cast<const T*>(q), lengths, kn, vn, static_cast<T*>(out), early);
       else
         e = launch_dependent(decode_attn_kernel<T, D, G, false>, (unsigned)grid, kAttnThreads, s, p, static_cast<const T*>(q), lengths, kn, vn, static_cast<T*>(out), early);
     }

@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(128) separator_plan_kernel(DeviceProblem p, in
     p.cap[u] = cap;
     s_cap[tid] = cap;
     s_git[tid] = (len + kGatherRows - 1) / kGatherRows;
-    s_dit[tid] = (cap + kDecodeChunk - 1) / kDecodeChunk;
+    s_dit[tid] = (cap + p.dec_chunk - 1) / p.dec_chunk;
   }
   __syncthreads();
   if (tid < nl) {

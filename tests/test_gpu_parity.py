@@ -167,6 +167,53 @@ def test_shapes_and_edge_cases(case):
     run_workload(wl)
 
 
+# Small decode calls run as one launch of clusters (up to 16 CTAs a unit, up to two items a CTA), larger ones as attention
+# and combine kernels; the same cache is decoded whole (the kernels) and layer by layer (the clusters), or the other way
+# round, and gives the same bits.  Prompt lengths around the items' 64 ... 512 rows; grown past one item boundary.
+@pytest.mark.parametrize("kw", [dict(n=4, n_kv=4, d=64, seq_lens=[127], R=1, dtype="f32"),
+                                dict(n=8, n_kv=4, d=128, seq_lens=[513, 300], R=2, dtype="f32"),
+                                dict(n=32, n_kv=32, d=128, seq_lens=[4095], R=10, dtype="bf16"),
+                                dict(n=32, n_kv=32, d=64, seq_lens=[4090], R=10, dtype="bf16"),
+                                dict(n=32, n_kv=4, d=128, seq_lens=[8190], R=20, dtype="bf16"),
+                                dict(n=8, n_kv=4, d=64, seq_lens=[2047, 900], R=3, dtype="bf16")])
+@pytest.mark.parametrize("page_rows", [0, 64])
+def test_cluster_decode_equals_the_two_kernels_bit_for_bit(kw, page_rows):
+    tk = _tk()
+    wl = small("cldec", N=0, L=16, s1=4, s2=64, k=300, nh=1, steps=4, **kw)
+    qs, ks, vs = W.materialize(wl, DEV)
+    params = tk.params_from_workload(wl, max_new_tokens=8)
+    R = wl.n_layers
+
+    def compress():
+        if not page_rows:
+            return tk.taskkv_compress_ex(params, qs, ks, vs), None
+        info, pages = tk.taskkv_plan_paged(params, page_rows)
+        pool = tk.Pool(page_rows, pages + int(info.n_units), wl.head_dim, wl.dtype, DEV)
+        return tk.taskkv_compress_paged(params, qs, ks, vs, pool), pool
+
+    (a, pa), (b, pb) = compress(), compress()
+    P = _parity()
+    for s in range(4):
+        q, kn, vn = W.gen_decode_step(wl, s, DEV)
+        whole = a.taskkv_decode_step(q, kn, vn)
+        parts = [b.taskkv_decode_step_ex(*(x[:, r:r + 1].contiguous() for x in (q, kn, vn)), r, 1) for r in range(R)]
+        assert torch.equal(whole, torch.cat(parts, dim=1))
+        again = [b.taskkv_decode_ex(q[:, r:r + 1].contiguous(), r, 1) for r in range(R)]   # the row just appended included
+        assert torch.equal(whole, torch.cat(again, dim=1))
+    assert a.status() == 0 and b.status() == 0 and a.lengths().tolist() == b.lengths().tolist()
+    # the first layer of sequence 0 against 64-bit attention over the rows the cache holds
+    G, d = wl.group, wl.head_dim
+    for h in range(wl.n_kv_heads):
+        kc, vc = b.pool_rows("k", h).double(), b.pool_rows("v", h).double()
+        sc = q[0, 0, h * G:(h + 1) * G].double().cpu() @ kc.T / d ** 0.5
+        want = torch.softmax(sc, -1) @ vc
+        assert (whole[0, 0, h * G:(h + 1) * G].double().cpu() - want).abs().max() < P.TOL_OUT[wl.dtype]
+    for c, p in ((a, pa), (b, pb)):
+        c.close()
+        if p:
+            p.close()
+
+
 # (query heads per KV head, window) -> 8, 16, 24, 48, 96 and 128 window rows; key counts around the 128-key tile, the
 # 256-key chunk and the 8192 keys up to which pass 2 folds the chunks' statistics itself.  (Four KV heads: two are always
 # equally far from their mean, so which of them is promoted would be a tie.)
