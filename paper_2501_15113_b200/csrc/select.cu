@@ -3,13 +3,12 @@
 //   the k middle activations: top-k of the average-pooled scores over the
 //   intermediate positions [s1, N - s2) (Sec. IV-B, pooling of Sec. V-D), written
 //   with the sinks and the recent window as the unit's ascending index list.
-// Both selections find the exact k-th largest order-preserving 32-bit key by bisection
-// over the key bits, followed by an ordered compaction; of equal scores the lower
-// position wins.  Up to 32768 positions the keys live in the registers of one block
-// (select_fast_kernel), up to 262144 in those of a thread-block cluster
-// (select_cluster_kernel); longer units, or other pooling kernels, stream them from L2
-// once per bisection step until few enough survive to be collected in shared memory
-// (select_kernel).
+// Both selections find the exact k-th largest order-preserving 32-bit key, followed by an
+// ordered compaction; of equal scores the lower position wins.  Up to 32768 positions the keys
+// live in the registers of one block (select_fast_kernel), up to 262144 in those of a
+// thread-block cluster (select_cluster_kernel), and the key is found by histograms over a
+// shrinking range; longer units, or other pooling kernels, stream the keys from L2 once per
+// bisection step until few enough survive to be collected in shared memory (select_kernel).
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -293,115 +292,145 @@ __global__ void __launch_bounds__(kThreads) select_kernel(DeviceProblem p, UnitR
 
 
 // ---------------------------------------------------------------------------
-// Register-resident variant for N <= 32768 (and pooling kernel 1 or 7): every
-// thread keeps 32 consecutive scores in registers, so a selection is a bisection
-// over the 32 key bits -- each step is 32 compares per thread plus one block-wide
-// count -- and the ordered compaction is a single block scan.  Same results as
-// the radix path: exact k-th key, lower position first among equal keys, pooled
-// sums added in ascending position.
-constexpr int kEpt = 32;
+// Register-resident variant for N <= 32768 (and pooling kernel 1 or 7): every thread keeps EPT consecutive scores in
+// registers (2, 8 or 32, the fewest that hold the sequence), and a selection is a histogram over the range of the keys,
+// refined inside the bin that holds the k-th largest until few candidates are left, which are then ranked directly.
+// Same results as the streaming path: exact k-th key, lower position first among equal keys, pooled sums added in
+// ascending position.
+constexpr int kEptMax = 32;
+constexpr int kBins = 2 * kThreads;    // bins of one refinement: two per thread in the scan
+constexpr int kBinBits = 11;
+static_assert(kBins == 1 << kBinBits, "a refinement settles kBinBits bits of the keys' range");
+constexpr int kFew = 256;              // candidates that are ranked against one another instead of refined further
 
-struct FastSmem {
-  int cnt[2][kWarps];
+struct HistSmem {
+  int hist[kBins];
+  __align__(16) uint32_t list[kFew + 4];
   uint32_t mn[kWarps], mx[kWarps];
-  int scan[kWarps];
-  int scan_tot;
-  int list_n;          // keys collected for the narrow phase of the bisection
-  uint32_t list_thr;   // its result
+  int wsum[kWarps];
+  int bin, above, count;   // the bin that holds the wanted key, how many candidates lie above it and in it
+  int list_n;
+  uint32_t thr;
+  int need;
 };
-constexpr int kNarrow = 1023;  // the bisection runs over all keys until at most this many lie in the undecided range
 
-__device__ __forceinline__ int block_count_ge(const uint32_t (&key)[kEpt], uint32_t cand, int* slot) {
-  int c = 0;
+// The candidates of one refinement are counted in h (this thread's two bins of the histogram from the top down: bins
+// kBins - 1 - 2 tid and kBins - 2 - 2 tid): finds the bin that holds the rem-th largest.  Two block barriers.
+__device__ __forceinline__ void find_bin(HistSmem& hs, int c_hi, int c_lo, int rem) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int sum = c_hi + c_lo;
+  int incl = sum;
 #pragma unroll
-  for (int e = 0; e < kEpt; ++e) c += (key[e] >= cand) ? 1 : 0;
-  c = __reduce_add_sync(0xffffffffu, c);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) slot[warp] = c;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) hs.wsum[warp] = incl;
   __syncthreads();
-  return __reduce_add_sync(0xffffffffu, slot[lane]);
+  const int before = __reduce_add_sync(0xffffffffu, lane < warp ? hs.wsum[lane] : 0);
+  const int excl = before + incl - sum;
+  if (excl < rem && rem <= excl + sum) {
+    const bool first = rem <= excl + c_hi;
+    hs.bin = kBins - 1 - 2 * tid - (first ? 0 : 1);
+    hs.above = excl + (first ? 0 : c_hi);
+    hs.count = first ? c_hi : c_lo;
+  }
+  __syncthreads();
+}
+
+// The rem-th largest of the n <= kFew collected candidates (hs.list, padded with zeros to a multiple of four) and how
+// many equal to it belong to the first rem.  Between two block barriers.
+__device__ __forceinline__ void rank_few(HistSmem& hs, int n, int rem, uint32_t& thr, int& need_eq) {
+  if ((int)threadIdx.x < n) {
+    const uint32_t mine = hs.list[threadIdx.x];
+    int gt = 0, eq = 0;
+    for (int i = 0; i < n; i += 4) {
+      const uint4 v = *reinterpret_cast<const uint4*>(hs.list + i);
+      gt += (int)(v.x > mine) + (int)(v.y > mine) + (int)(v.z > mine) + (int)(v.w > mine);
+      eq += (int)(v.x == mine) + (int)(v.y == mine) + (int)(v.z == mine) + (int)(v.w == mine);
+    }
+    if (gt < rem && rem <= gt + eq) {       // threads that hold the same key write the same two words
+      hs.thr = mine;
+      hs.need = rem - gt;
+    }
+  }
+  __syncthreads();
+  thr = hs.thr;
+  need_eq = hs.need;
+}
+
+// Range of candidates [base, limit] of one refinement: bins of 2^shift consecutive keys.
+__device__ __forceinline__ int bin_shift(uint32_t base, uint32_t limit) {
+  return max(0, 32 - __clz((int)(limit - base)) - kBinBits);
+}
+__device__ __forceinline__ void narrow_range(uint32_t& base, uint32_t& limit, int bin, int shift) {
+  base += (uint32_t)bin << shift;
+  const uint32_t w = (1u << shift) - 1u;
+  if (limit - base > w) limit = base + w;
 }
 
 // k-th largest key (1 <= want <= number of non-zero keys) and how many keys equal to it belong to the top `want`.
-// Every step over all keys also tells how many keys still lie in the undecided range [t, t + 2^(bit+1)); once
-// they are few, they are collected into `list` (shared memory, `cap` entries, any order) and one warp settles
-// the remaining bits on them.  With many near-equal scores that moment may never come and the bisection simply
-// stays on all keys.  The result is the same key either way.
-__device__ void block_bisect(FastSmem& fs, const uint32_t (&key)[kEpt], int want, uint32_t* list, int cap,
-                             uint32_t& thr, int& need_eq) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // bits above the highest bit in which the non-zero keys differ are common to the answer
+// A refinement costs one shared-memory atomic per candidate and three block barriers; the first has at most 32768
+// candidates, and on scores that are not all alike it leaves a few dozen.  Bisection over the key bits, 32 scores per
+// thread whatever the length, took 291 us for 1024 units of 32768 keys (now 210), 261 for 1024 of 4096 (92), 45 for 8 of
+// 8191 (19); the cluster form 548 us for 256 units of 131072 keys (361).
+template <int EPT>
+__device__ void block_select(HistSmem& hs, const uint32_t (&key)[EPT], int want, uint32_t& thr, int& need_eq) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t lo = 0xffffffffu, hi = 0u;
 #pragma unroll
-  for (int e = 0; e < kEpt; ++e)
+  for (int e = 0; e < EPT; ++e)
     if (key[e]) { lo = min(lo, key[e]); hi = max(hi, key[e]); }
   lo = __reduce_min_sync(0xffffffffu, lo);
   hi = __reduce_max_sync(0xffffffffu, hi);
-  if (lane == 0) { fs.mn[warp] = lo; fs.mx[warp] = hi; }
-  if (threadIdx.x == 0) fs.list_n = 0;
+  if (lane == 0) { hs.mn[warp] = lo; hs.mx[warp] = hi; }
+  if (tid == 0) hs.list_n = 0;
+  hs.hist[tid] = 0;
+  hs.hist[tid + kThreads] = 0;
   __syncthreads();
-  lo = __reduce_min_sync(0xffffffffu, fs.mn[lane]);
-  hi = __reduce_max_sync(0xffffffffu, fs.mx[lane]);
-  const uint32_t diff = lo ^ hi;
-  int bit = diff ? 31 - __clz(diff) : -1;
-  uint32_t t = diff ? (hi & ~((2u << bit) - 1u)) : hi;
-  int par = 0;
-  int above = 0;           // keys >= t + 2^(bit+1): the last count that fell short of `want`
-  int at_least = 1 << 30;  // keys >= t: the last count that reached `want` (unknown before the first one)
-  const int narrow = min(cap, kNarrow);
-  for (; bit >= 0 && at_least - above > narrow; --bit) {
-    const uint32_t cand = t | (1u << bit);
-    const int c = block_count_ge(key, cand, fs.cnt[par]);
-    if (c >= want) { t = cand; at_least = c; } else above = c;
-    par ^= 1;
-  }
-  if (bit >= 0) {
-    const uint32_t top = t + (2u << bit);            // end of the undecided range (0 if it wraps: no upper bound)
-    const int alive = at_least - above;
-    {
+  uint32_t base = __reduce_min_sync(0xffffffffu, hs.mn[lane]), limit = __reduce_max_sync(0xffffffffu, hs.mx[lane]);
+  int rem = want;
+  while (base != limit) {
+    const int shift = bin_shift(base, limit);
 #pragma unroll
-      for (int e = 0; e < kEpt; ++e)
-        if (key[e] >= t && (top == 0u || key[e] < top)) list[atomicAdd(&fs.list_n, 1)] = key[e];
+    for (int e = 0; e < EPT; ++e)
+      if (key[e] >= base && key[e] <= limit) atomicAdd(&hs.hist[(key[e] - base) >> shift], 1);
+    __syncthreads();
+    int* mine = &hs.hist[kBins - 2 - 2 * tid];
+    const int c_lo = mine[0], c_hi = mine[1];
+    mine[0] = 0;
+    mine[1] = 0;
+    find_bin(hs, c_hi, c_lo, rem);
+    rem -= hs.above;
+    narrow_range(base, limit, hs.bin, shift);
+    const int n = hs.count;
+    if (base != limit && n <= kFew) {
+#pragma unroll
+      for (int e = 0; e < EPT; ++e)
+        if (key[e] >= base && key[e] <= limit) hs.list[atomicAdd(&hs.list_n, 1)] = key[e];
+      if (tid < 4) hs.list[n + tid] = 0u;
       __syncthreads();
-      // every thread takes one collected key (there are at most as many as threads); two bits per step: the
-      // counts above the three thresholds travel packed in one word (10 bits each hold a count <= 1023)
-      static_assert(kNarrow <= kThreads && kNarrow < (1 << 10), "one key per thread, three counts per word");
-      const uint32_t mine = (int)threadIdx.x < alive ? list[threadIdx.x] : 0u;
-      const int want2 = want - above;                 // rank inside the collected keys
-      while (bit >= 0) {
-        const uint32_t b_hi = 1u << bit, b_lo = bit > 0 ? 1u << (bit - 1) : 0u;
-        const uint32_t c10 = t | b_hi, c11 = c10 | b_lo, c01 = t | b_lo;
-        int v = (int)(mine >= c10) | ((int)(mine >= c11) << 10) | ((int)(b_lo != 0u && mine >= c01) << 20);
-        v = __reduce_add_sync(0xffffffffu, v);
-        if (lane == 0) fs.cnt[par][warp] = v;
-        __syncthreads();
-        v = __reduce_add_sync(0xffffffffu, fs.cnt[par][lane]);
-        par ^= 1;
-        const int n10 = v & 0x3ff, n11 = (v >> 10) & 0x3ff, n01 = (v >> 20) & 0x3ff;
-        if (b_lo != 0u && n11 >= want2) t = c11;
-        else if (n10 >= want2) t = c10;
-        else if (b_lo != 0u && n01 >= want2) t = c01;
-        bit -= 2;
-      }
+      rank_few(hs, n, rem, thr, need_eq);
+      __syncthreads();
+      return;
     }
   }
-  const int n_gt = (t == 0xffffffffu) ? 0 : block_count_ge(key, t + 1u, fs.cnt[par]);
-  thr = t;
-  need_eq = want - n_gt;
+  thr = base;
+  need_eq = rem;
   __syncthreads();
 }
 
-// Ordered compaction of this thread's 32 consecutive positions [base, base + 32): emit(rank, position) for every
+// Ordered compaction of this thread's EPT consecutive positions [base, base + EPT): emit(rank, position) for every
 // key above thr and for the first need_eq keys equal to it (lower position first).  The comparisons are made once,
 // into two bit masks; the selected keys are few per thread, so the emitting loop walks set bits only.
-template <class Emit>
-__device__ void block_compact_regs(FastSmem& fs, const uint32_t (&key)[kEpt], int base, uint32_t thr, int need_eq,
+template <int EPT, class Emit>
+__device__ void block_compact_regs(HistSmem& fs, const uint32_t (&key)[EPT], int base, uint32_t thr, int need_eq,
                                    const Emit& emit) {
-  static_assert(kEpt == 32, "one mask bit per key");
+  static_assert(EPT <= 32, "one mask bit per key");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t m_gt = 0u, m_ge = 0u;
 #pragma unroll
-  for (int e = 0; e < kEpt; ++e) {
+  for (int e = 0; e < EPT; ++e) {
     m_gt |= (uint32_t)(key[e] > thr) << e;
     m_ge |= (uint32_t)(key[e] >= thr) << e;
   }
@@ -413,9 +442,9 @@ __device__ void block_compact_regs(FastSmem& fs, const uint32_t (&key)[kEpt], in
     const int y = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += y;
   }
-  if (lane == 31) fs.scan[warp] = incl;
+  if (lane == 31) fs.wsum[warp] = incl;
   __syncthreads();
-  int wp = fs.scan[lane];
+  int wp = fs.wsum[lane];
   int wi = wp;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -435,9 +464,9 @@ __device__ void block_compact_regs(FastSmem& fs, const uint32_t (&key)[kEpt], in
   __syncthreads();
 }
 
-template <typename T, int D, int POOL_HALF>
+template <typename T, int D, int POOL_HALF, int EPT>
 __global__ void __launch_bounds__(kThreads, 1) select_fast_kernel(DeviceProblem p, UnitRange ur) {
-  __shared__ FastSmem fs;
+  __shared__ HistSmem fs;
   __shared__ int sel[TASKKV_MAX_TOP_T];
   __shared__ float selw[TASKKV_MAX_TOP_T];
   __shared__ float red[kWarps][D];
@@ -446,30 +475,29 @@ __global__ void __launch_bounds__(kThreads, 1) select_fast_kernel(DeviceProblem 
   const int N = p.unit_N[u];
   const float* C = p.C + p.c_off[u];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int base = tid * kEpt;
+  const int base = tid * EPT;
 
   // only the keys are kept (a key maps back to its score exactly); key 0 marks "no element"
-  uint32_t key[kEpt];
-  if (base + kEpt <= N && ((reinterpret_cast<uintptr_t>(C + base) & 15) == 0)) {
+  uint32_t key[EPT];
+  if (EPT >= 4 && base + EPT <= N && ((reinterpret_cast<uintptr_t>(C + base) & 15) == 0)) {
 #pragma unroll
-    for (int e = 0; e < kEpt; e += 4) {
+    for (int e = 0; e + 4 <= EPT; e += 4) {
       const float4 v = *reinterpret_cast<const float4*>(C + base + e);
       key[e] = ordered_key(v.x); key[e + 1] = ordered_key(v.y);
       key[e + 2] = ordered_key(v.z); key[e + 3] = ordered_key(v.w);
     }
   } else {
 #pragma unroll
-    for (int e = 0; e < kEpt; ++e) key[e] = (base + e < N) ? ordered_key(C[base + e]) : 0u;
+    for (int e = 0; e < EPT; ++e) key[e] = (base + e < N) ? ordered_key(C[base + e]) : 0u;
   }
 
   // ---- Eq. 14: I = top-min(t, N) of C
   const int t = min(p.top_t, N);
   uint32_t thr;
   int need_eq;
-  uint32_t* scratch = reinterpret_cast<uint32_t*>(&red[0][0]);   // free until the semantic vector is summed
-  block_bisect(fs, key, t, scratch, kWarps * D, thr, need_eq);
+  block_select<EPT>(fs, key, t, thr, need_eq);
   int* topt = p.topt + (size_t)u * p.top_t;
-  block_compact_regs(fs, key, base, thr, need_eq, [&](int pos, int j) {
+  block_compact_regs<EPT>(fs, key, base, thr, need_eq, [&](int pos, int j) {
     sel[pos] = j;
     selw[pos] = C[j];
     topt[pos] = j;
@@ -482,6 +510,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_fast_kernel(DeviceProblem 
 #pragma unroll
   for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
   const T* V = static_cast<const T*>(p.v_ptr[u]);
+#pragma unroll 8    // eight rows in flight: a row is a trip to HBM
   for (int i = warp; i < t; i += kWarps) {
     const float w = selw[i];
     const T* row = V + (size_t)sel[i] * D + lane * EPL;
@@ -518,17 +547,17 @@ __global__ void __launch_bounds__(kThreads, 1) select_fast_kernel(DeviceProblem 
 
   // pooled window sums in ascending position: ext = [3 left neighbours][32 own][3 right neighbours]
   if (POOL_HALF > 0) {
-    float ext[kEpt + 2 * POOL_HALF];
+    float ext[EPT + 2 * POOL_HALF];
 #pragma unroll
     for (int h = 0; h < POOL_HALF; ++h) {
-      const int jl = base - POOL_HALF + h, jr = base + kEpt + h;
+      const int jl = base - POOL_HALF + h, jr = base + EPT + h;
       ext[h] = (jl >= 0 && jl < N) ? C[jl] : 0.f;
-      ext[POOL_HALF + kEpt + h] = (jr < N) ? C[jr] : 0.f;
+      ext[POOL_HALF + EPT + h] = (jr < N) ? C[jr] : 0.f;
     }
 #pragma unroll
-    for (int e = 0; e < kEpt; ++e) ext[POOL_HALF + e] = (base + e < N) ? key_score(key[e]) : 0.f;
+    for (int e = 0; e < EPT; ++e) ext[POOL_HALF + e] = (base + e < N) ? key_score(key[e]) : 0.f;
 #pragma unroll
-    for (int e = 0; e < kEpt; ++e) {
+    for (int e = 0; e < EPT; ++e) {
       float sum = 0.f;
 #pragma unroll
       for (int o = 0; o <= 2 * POOL_HALF; ++o) sum += ext[e + o];
@@ -537,14 +566,14 @@ __global__ void __launch_bounds__(kThreads, 1) select_fast_kernel(DeviceProblem 
     }
   } else {
 #pragma unroll
-    for (int e = 0; e < kEpt; ++e) {
+    for (int e = 0; e < EPT; ++e) {
       const int j = base + e;
       if (!(j >= lo && j < hi)) key[e] = 0u;
     }
   }
   __syncthreads();
-  block_bisect(fs, key, kmid, scratch, kWarps * D, thr, need_eq);
-  block_compact_regs(fs, key, base, thr, need_eq, [&](int pos, int j) { idx[s1 + pos] = j; });
+  block_select<EPT>(fs, key, kmid, thr, need_eq);
+  block_compact_regs<EPT>(fs, key, base, thr, need_eq, [&](int pos, int j) { idx[s1 + pos] = j; });
 }
 
 // ---------------------------------------------------------------------------
@@ -557,44 +586,23 @@ __global__ void __launch_bounds__(kThreads, 1) select_fast_kernel(DeviceProblem 
 constexpr int kMaxCS = 8;
 
 struct ClusterSmem {
-  int cnt[2][kMaxCS][kWarps];
-  int loc[2][kWarps];        // block-local counts of the narrow phase (peers never write here)
+  HistSmem h;                // this CTA's own counts; the list holds the candidates of the whole cluster
   uint32_t mn[kMaxCS][kWarps], mx[kMaxCS][kWarps];
+  uint32_t stage[kFew];      // this CTA's own candidates
   int tot[2][kMaxCS][2];     // per compaction and CTA: keys above the threshold, keys equal to it
-  int scan[kWarps];
-  int list_n;                // survivors received from all CTAs
-  int loc_n;                 // this CTA's own survivors
+  int loc_n;                 // this CTA's own candidates
   int base[kMaxCS];          // where they go in each CTA's list
 };
 
-// Sum over the whole cluster of one int per warp (v: this warp's value, already reduced over the warp).
-__device__ __forceinline__ int cluster_sum(cg::cluster_group& cl, ClusterSmem& cs, int cs_n, int rank, int par, int v) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane < cs_n) cl.map_shared_rank(&cs.cnt[par][rank][warp], lane)[0] = v;
-  cl.sync();
-  int acc = 0;
-  for (int r = 0; r < cs_n; ++r) acc += cs.cnt[par][r][lane];
-  return __reduce_add_sync(0xffffffffu, acc);
-}
-
-__device__ __forceinline__ int cluster_count_ge(cg::cluster_group& cl, ClusterSmem& cs, int cs_n, int rank, int par,
-                                                const uint32_t (&key)[kEpt], uint32_t cand) {
-  int c = 0;
-#pragma unroll
-  for (int e = 0; e < kEpt; ++e) c += (key[e] >= cand) ? 1 : 0;
-  c = __reduce_add_sync(0xffffffffu, c);
-  return cluster_sum(cl, cs, cs_n, rank, par, c);
-}
-
-// block_bisect over the keys of the whole cluster.  For the narrow phase every CTA sends its surviving keys to all
-// CTAs (at most kNarrow in the whole cluster, so at most one per thread), and each settles the rest on its own copy.
-// `list` must hold 2 (kNarrow + 1) words.
-__device__ void cluster_bisect(cg::cluster_group& cl, ClusterSmem& cs, int cs_n, int rank, const uint32_t (&key)[kEpt],
-                               int want, uint32_t* list, int cap, uint32_t& thr, int& need_eq) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// block_select over the keys of the whole cluster: every CTA adds up the CTAs' histograms for itself, so that all of
+// them refine the same range; the last few candidates are sent to all CTAs, and each ranks its own copy.
+__device__ void cluster_select(cg::cluster_group& cl, ClusterSmem& cs, int cs_n, int rank, const uint32_t (&key)[kEptMax],
+                               int want, uint32_t& thr, int& need_eq) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  HistSmem& hs = cs.h;
   uint32_t lo = 0xffffffffu, hi = 0u;
 #pragma unroll
-  for (int e = 0; e < kEpt; ++e)
+  for (int e = 0; e < kEptMax; ++e)
     if (key[e]) { lo = min(lo, key[e]); hi = max(hi, key[e]); }
   lo = __reduce_min_sync(0xffffffffu, lo);
   hi = __reduce_max_sync(0xffffffffu, hi);
@@ -602,88 +610,70 @@ __device__ void cluster_bisect(cg::cluster_group& cl, ClusterSmem& cs, int cs_n,
     cl.map_shared_rank(&cs.mn[rank][warp], lane)[0] = lo;
     cl.map_shared_rank(&cs.mx[rank][warp], lane)[0] = hi;
   }
-  if (threadIdx.x == 0) { cs.list_n = 0; cs.loc_n = 0; }
+  if (tid == 0) { hs.list_n = 0; cs.loc_n = 0; }
+  hs.hist[tid] = 0;
+  hs.hist[tid + kThreads] = 0;
   cl.sync();
   lo = 0xffffffffu; hi = 0u;
   for (int r = 0; r < cs_n; ++r) { lo = min(lo, cs.mn[r][lane]); hi = max(hi, cs.mx[r][lane]); }
-  lo = __reduce_min_sync(0xffffffffu, lo);
-  hi = __reduce_max_sync(0xffffffffu, hi);
-  const uint32_t diff = lo ^ hi;
-  int bit = diff ? 31 - __clz(diff) : -1;
-  uint32_t t = diff ? (hi & ~((2u << bit) - 1u)) : hi;
-  int par = 0;
-  int above = 0;
-  int at_least = 1 << 30;
-  const int narrow = min(cap - (kNarrow + 1), kNarrow);   // lower half of `list`: the cluster's survivors; upper half: staging
-  for (; bit >= 0 && at_least - above > narrow; --bit) {
-    const uint32_t cand = t | (1u << bit);
-    const int c = cluster_count_ge(cl, cs, cs_n, rank, par, key, cand);
-    if (c >= want) { t = cand; at_least = c; } else above = c;
-    par ^= 1;
-  }
-  if (bit >= 0) {
-    const uint32_t top = t + (2u << bit);            // end of the undecided range (0 if it wraps: no upper bound)
-    const int alive = at_least - above;              // survivors in the whole cluster: at most one per thread
-    // this CTA's survivors are staged in the upper half of `list`, then copied into every CTA's lower half at an
-    // offset reserved with one remote atomic per CTA (any order: only counts matter)
-    uint32_t* stage = list + kNarrow + 1;
+  uint32_t base = __reduce_min_sync(0xffffffffu, lo), limit = __reduce_max_sync(0xffffffffu, hi);
+  int rem = want;
+  while (base != limit) {
+    const int shift = bin_shift(base, limit);
 #pragma unroll
-    for (int e = 0; e < kEpt; ++e)
-      if (key[e] >= t && (top == 0u || key[e] < top)) stage[atomicAdd(&cs.loc_n, 1)] = key[e];
-    __syncthreads();
-    const int n_loc = cs.loc_n;
-    if ((int)threadIdx.x < cs_n) cs.base[threadIdx.x] = atomicAdd(cl.map_shared_rank(&cs.list_n, threadIdx.x), n_loc);
-    __syncthreads();
-    for (int r = 0; r < cs_n; ++r) {
-      uint32_t* dst = cl.map_shared_rank(list, r) + cs.base[r];
-      for (int i = threadIdx.x; i < n_loc; i += kThreads) dst[i] = stage[i];
-    }
+    for (int e = 0; e < kEptMax; ++e)
+      if (key[e] >= base && key[e] <= limit) atomicAdd(&hs.hist[(key[e] - base) >> shift], 1);
     cl.sync();
-    // from here on every CTA settles the remaining bits on its own copy, with block barriers only
-    const uint32_t mine = (int)threadIdx.x < alive ? list[threadIdx.x] : 0u;
-    const int want2 = want - above;                  // rank inside the collected keys
-    int lpar = 0;
-    while (bit >= 0) {
-      const uint32_t b_hi = 1u << bit, b_lo = bit > 0 ? 1u << (bit - 1) : 0u;
-      const uint32_t c10 = t | b_hi, c11 = c10 | b_lo, c01 = t | b_lo;
-      int v = (int)(mine >= c10) | ((int)(mine >= c11) << 10) | ((int)(b_lo != 0u && mine >= c01) << 20);
-      v = __reduce_add_sync(0xffffffffu, v);
-      if (lane == 0) cs.loc[lpar][warp] = v;
-      __syncthreads();
-      v = __reduce_add_sync(0xffffffffu, cs.loc[lpar][lane]);
-      lpar ^= 1;
-      const int n10 = v & 0x3ff, n11 = (v >> 10) & 0x3ff, n01 = (v >> 20) & 0x3ff;
-      if (b_lo != 0u && n11 >= want2) t = c11;
-      else if (n10 >= want2) t = c10;
-      else if (b_lo != 0u && n01 >= want2) t = c01;
-      bit -= 2;
+    int2* mine = reinterpret_cast<int2*>(&hs.hist[kBins - 2 - 2 * tid]);
+    int c_lo = 0, c_hi = 0;
+    for (int r = 0; r < cs_n; ++r) {
+      const int2 c = *cl.map_shared_rank(mine, r);
+      c_lo += c.x;
+      c_hi += c.y;
     }
-    // keys above the threshold: those above the undecided range plus the survivors above it (no pass over all keys)
-    int g = __reduce_add_sync(0xffffffffu, (int)(mine > t));
-    if (lane == 0) cs.loc[lpar][warp] = g;
+    find_bin(hs, c_hi, c_lo, rem);
+    rem -= hs.above;
+    narrow_range(base, limit, hs.bin, shift);
+    const int n = hs.count;
+    if (base != limit && n <= kFew) {
+      // own candidates first into `stage`, then into every CTA's list at an offset reserved with one remote atomic per
+      // CTA (any order: only counts matter)
+#pragma unroll
+      for (int e = 0; e < kEptMax; ++e)
+        if (key[e] >= base && key[e] <= limit) cs.stage[atomicAdd(&cs.loc_n, 1)] = key[e];
+      if (tid < 4) hs.list[n + tid] = 0u;
+      __syncthreads();
+      const int n_loc = cs.loc_n;
+      if (tid < cs_n) cs.base[tid] = atomicAdd(cl.map_shared_rank(&hs.list_n, tid), n_loc);
+      __syncthreads();
+      for (int r = 0; r < cs_n; ++r) {
+        uint32_t* dst = cl.map_shared_rank(hs.list, r) + cs.base[r];
+        for (int i = tid; i < n_loc; i += kThreads) dst[i] = cs.stage[i];
+      }
+      cl.sync();
+      rank_few(hs, n, rem, thr, need_eq);
+      __syncthreads();
+      return;
+    }
+    cl.sync();                                        // the peers have read this CTA's counts
+    *mine = make_int2(0, 0);
     __syncthreads();
-    g = __reduce_add_sync(0xffffffffu, cs.loc[lpar][lane]);
-    thr = t;
-    need_eq = want - (above + g);
-    __syncthreads();
-    return;
   }
-  const int n_gt = (t == 0xffffffffu) ? 0 : cluster_count_ge(cl, cs, cs_n, rank, par, key, t + 1u);
-  thr = t;
-  need_eq = want - n_gt;
+  thr = base;
+  need_eq = rem;
   __syncthreads();
 }
 
 // block_compact_regs with the ranks continued across the CTAs of the cluster (`which` names the totals' slot).
 template <class Emit>
 __device__ void cluster_compact_regs(cg::cluster_group& cl, ClusterSmem& cs, int cs_n, int rank, int which,
-                                     const uint32_t (&key)[kEpt], int base, uint32_t thr, int need_eq,
+                                     const uint32_t (&key)[kEptMax], int base, uint32_t thr, int need_eq,
                                      const Emit& emit) {
-  static_assert(kEpt == 32, "one mask bit per key");
+  static_assert(kEptMax == 32, "one mask bit per key");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t m_gt = 0u, m_ge = 0u;
 #pragma unroll
-  for (int e = 0; e < kEpt; ++e) {
+  for (int e = 0; e < kEptMax; ++e) {
     m_gt |= (uint32_t)(key[e] > thr) << e;
     m_ge |= (uint32_t)(key[e] >= thr) << e;
   }
@@ -695,9 +685,9 @@ __device__ void cluster_compact_regs(cg::cluster_group& cl, ClusterSmem& cs, int
     const int y = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += y;
   }
-  if (lane == 31) cs.scan[warp] = incl;
+  if (lane == 31) cs.h.wsum[warp] = incl;
   __syncthreads();
-  int wp = cs.scan[lane];
+  int wp = cs.h.wsum[lane];
   int wi = wp;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -740,27 +730,26 @@ __global__ void __launch_bounds__(kThreads, 1) select_cluster_kernel(DeviceProbl
   const int N = p.unit_N[u];
   const float* C = p.C + p.c_off[u];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int base = (rank * kThreads + tid) * kEpt;
+  const int base = (rank * kThreads + tid) * kEptMax;
 
-  uint32_t key[kEpt];
-  if (base + kEpt <= N && ((reinterpret_cast<uintptr_t>(C + base) & 15) == 0)) {
+  uint32_t key[kEptMax];
+  if (base + kEptMax <= N && ((reinterpret_cast<uintptr_t>(C + base) & 15) == 0)) {
 #pragma unroll
-    for (int e = 0; e < kEpt; e += 4) {
+    for (int e = 0; e < kEptMax; e += 4) {
       const float4 v = *reinterpret_cast<const float4*>(C + base + e);
       key[e] = ordered_key(v.x); key[e + 1] = ordered_key(v.y);
       key[e + 2] = ordered_key(v.z); key[e + 3] = ordered_key(v.w);
     }
   } else {
 #pragma unroll
-    for (int e = 0; e < kEpt; ++e) key[e] = (base + e < N) ? ordered_key(C[base + e]) : 0u;
+    for (int e = 0; e < kEptMax; ++e) key[e] = (base + e < N) ? ordered_key(C[base + e]) : 0u;
   }
 
   // ---- Eq. 14: I = top-min(t, N) of C; every CTA receives the whole list
   const int t = min(p.top_t, N);
   uint32_t thr;
   int need_eq;
-  uint32_t* scratch = reinterpret_cast<uint32_t*>(&red[0][0]);   // free until the semantic vector is summed
-  cluster_bisect(cl, cs, cs_n, rank, key, t, scratch, kWarps * D, thr, need_eq);
+  cluster_select(cl, cs, cs_n, rank, key, t, thr, need_eq);
   int* topt = p.topt + (size_t)u * p.top_t;
   cluster_compact_regs(cl, cs, cs_n, rank, 0, key, base, thr, need_eq, [&](int pos, int j) {
     const float w = C[j];
@@ -780,6 +769,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_cluster_kernel(DeviceProbl
 #pragma unroll
   for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
   const T* V = static_cast<const T*>(p.v_ptr[u]);
+#pragma unroll 4
   for (int i = rank * kWarps + warp; i < t; i += cs_n * kWarps) {
     const float w = selw[i];
     const T* row = V + (size_t)sel[i] * D + lane * EPL;
@@ -821,17 +811,17 @@ __global__ void __launch_bounds__(kThreads, 1) select_cluster_kernel(DeviceProbl
   if (kmid == 0) return;
 
   if (POOL_HALF > 0) {
-    float ext[kEpt + 2 * POOL_HALF];
+    float ext[kEptMax + 2 * POOL_HALF];
 #pragma unroll
     for (int h = 0; h < POOL_HALF; ++h) {
-      const int jl = base - POOL_HALF + h, jr = base + kEpt + h;
+      const int jl = base - POOL_HALF + h, jr = base + kEptMax + h;
       ext[h] = (jl >= 0 && jl < N) ? C[jl] : 0.f;
-      ext[POOL_HALF + kEpt + h] = (jr < N) ? C[jr] : 0.f;
+      ext[POOL_HALF + kEptMax + h] = (jr < N) ? C[jr] : 0.f;
     }
 #pragma unroll
-    for (int e = 0; e < kEpt; ++e) ext[POOL_HALF + e] = (base + e < N) ? key_score(key[e]) : 0.f;
+    for (int e = 0; e < kEptMax; ++e) ext[POOL_HALF + e] = (base + e < N) ? key_score(key[e]) : 0.f;
 #pragma unroll
-    for (int e = 0; e < kEpt; ++e) {
+    for (int e = 0; e < kEptMax; ++e) {
       float sum = 0.f;
 #pragma unroll
       for (int o = 0; o <= 2 * POOL_HALF; ++o) sum += ext[e + o];
@@ -840,13 +830,13 @@ __global__ void __launch_bounds__(kThreads, 1) select_cluster_kernel(DeviceProbl
     }
   } else {
 #pragma unroll
-    for (int e = 0; e < kEpt; ++e) {
+    for (int e = 0; e < kEptMax; ++e) {
       const int j = base + e;
       if (!(j >= lo && j < hi)) key[e] = 0u;
     }
   }
   __syncthreads();
-  cluster_bisect(cl, cs, cs_n, rank, key, kmid, scratch, kWarps * D, thr, need_eq);
+  cluster_select(cl, cs, cs_n, rank, key, kmid, thr, need_eq);
   cluster_compact_regs(cl, cs, cs_n, rank, 1, key, base, thr, need_eq, [&](int pos, int j) { idx[s1 + pos] = j; });
 }
 
@@ -900,10 +890,18 @@ cudaError_t launch_cluster(const DeviceProblem& p, const UnitRange& ur, int cs_n
   return p.pool_w == 7 ? launch_cluster_k<T, D, 3>(p, ur, cs_n, s) : launch_cluster_k<T, D, 0>(p, ur, cs_n, s);
 }
 
+// The fewest scores per thread that hold the longest sequence of the call: a thread's share of every pass over the
+// keys is what a short unit's selection costs, beside the barriers.
+template <typename T, int D, int EPT>
+void launch_fast_ept(const DeviceProblem& p, const UnitRange& ur, cudaStream_t s) {
+  if (p.pool_w == 7) select_fast_kernel<T, D, 3, EPT><<<ur.blocks, kThreads, 0, s>>>(p, ur);
+  else select_fast_kernel<T, D, 0, EPT><<<ur.blocks, kThreads, 0, s>>>(p, ur);
+}
 template <typename T, int D>
-void launch_fast(const DeviceProblem& p, const UnitRange& ur, cudaStream_t s) {
-  if (p.pool_w == 7) select_fast_kernel<T, D, 3><<<ur.blocks, kThreads, 0, s>>>(p, ur);
-  else select_fast_kernel<T, D, 0><<<ur.blocks, kThreads, 0, s>>>(p, ur);
+void launch_fast(const DeviceProblem& p, const UnitRange& ur, int max_N, cudaStream_t s) {
+  if (max_N <= 2 * kThreads) launch_fast_ept<T, D, 2>(p, ur, s);
+  else if (max_N <= 8 * kThreads) launch_fast_ept<T, D, 8>(p, ur, s);
+  else launch_fast_ept<T, D, kEptMax>(p, ur, s);
 }
 
 }  // namespace
@@ -912,17 +910,17 @@ cudaError_t launch_select(const DeviceProblem& p, int dtype, int max_N, cudaStre
   LaunchScope ls(K_SELECT, s);
   const UnitRange ur = range ? *range : UnitRange{0, p.U, p.U, p.U};
   if (ur.blocks <= 0) return cudaSuccess;
-  if (max_N <= kThreads * kEpt && (p.pool_w == 7 || p.pool_w == 1)) {
+  if (max_N <= kThreads * kEptMax && (p.pool_w == 7 || p.pool_w == 1)) {
     if (dtype == TASKKV_F32) {
-      if (p.d == 64) launch_fast<float, 64>(p, ur, s); else launch_fast<float, 128>(p, ur, s);
+      if (p.d == 64) launch_fast<float, 64>(p, ur, max_N, s); else launch_fast<float, 128>(p, ur, max_N, s);
     } else {
-      if (p.d == 64) launch_fast<__nv_bfloat16, 64>(p, ur, s); else launch_fast<__nv_bfloat16, 128>(p, ur, s);
+      if (p.d == 64) launch_fast<__nv_bfloat16, 64>(p, ur, max_N, s); else launch_fast<__nv_bfloat16, 128>(p, ur, max_N, s);
     }
     return cudaGetLastError();
   }
-  if (max_N <= kMaxCS * kThreads * kEpt && (p.pool_w == 7 || p.pool_w == 1)) {
+  if (max_N <= kMaxCS * kThreads * kEptMax && (p.pool_w == 7 || p.pool_w == 1)) {
     int cs_n = 2;
-    while (cs_n * kThreads * kEpt < max_N) cs_n *= 2;
+    while (cs_n * kThreads * kEptMax < max_N) cs_n *= 2;
     const bool fits = dtype == TASKKV_F32
                           ? (p.d == 64 ? cluster_supported<float, 64>(p, cs_n) : cluster_supported<float, 128>(p, cs_n))
                           : (p.d == 64 ? cluster_supported<__nv_bfloat16, 64>(p, cs_n)

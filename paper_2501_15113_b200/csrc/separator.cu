@@ -30,17 +30,21 @@ __global__ void __launch_bounds__(128) separator_plan_kernel(DeviceProblem p, in
 
   if (tid < d) {
     double s = 0.0;
+#pragma unroll 8
     for (int h = 0; h < n; ++h) s += (double)sem[h * d + tid];
     center[tid] = s / (double)n;
   }
   __syncthreads();
-  if (tid < n) {
+  // a warp per head: one thread's chain of d double-precision additions was most of this kernel's 8 us
+  for (int h = tid >> 5; h < n; h += 4) {
     double s = 0.0;
-    for (int x = 0; x < d; ++x) {
-      const double o = (double)sem[tid * d + x] - center[x];
+    for (int x = tid & 31; x < d; x += 32) {
+      const double o = (double)sem[h * d + x] - center[x];
       s += o * o;
     }
-    dist[tid] = sqrt(s);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((tid & 31) == 0) dist[h] = sqrt(s);
   }
   __syncthreads();
 

@@ -444,6 +444,33 @@ def test_cluster_select_equal_scores_keep_the_lower_positions():
     cache.close()
 
 
+# Register-resident selection: 2, 8 or 32 scores per thread (up to 2048, 8192, 32768 positions), clusters beyond.  Scores
+# of one magnitude (one refinement of the histogram), scores spread over hundreds of octaves by a few heavy keys (several),
+# and all scores equal (the whole range is one bin to the end): positions alone decide.
+@pytest.mark.parametrize("N", [700, 2048, 2049, 8192, 8193, 32768, 32769])
+@pytest.mark.parametrize("scores", ["flat", "heavy", "equal"])
+def test_register_selection_sizes(N, scores):
+    k, s1, s2 = N // 3, 4, 32
+    wl = small("regsel", n=4, n_kv=4, d=64, N=N, L=32, s1=s1, s2=s2, k=k, dtype="bf16", nh=0, steps=1, promote=False)
+    if scores != "equal":
+        if scores == "heavy":
+            wl.heavy_keys, wl.heavy_scale = 6, 60.0
+        run_workload(wl)
+        return
+    tk = _tk()
+    qs, ks, vs = W.materialize(wl, DEV)
+    ks[0][0][:] = ks[0][0][:, 0:1].clone()
+    cache = tk.taskkv_compress_ex(tk.params_from_workload(wl, max_new_tokens=0), qs, ks, vs)
+    assert cache.status() == 0
+    topt, idx = cache.query(tk.Q_TOPT), cache.query(tk.Q_INDICES)
+    want = list(range(s1 + k)) + list(range(N - s2, N))
+    for u in range(4):
+        assert topt[u].tolist() == list(range(256))
+        # the zeros beside the sequence make the pooled sums of its first three positions smaller; they are sinks
+        assert idx[u, :s1 + k + s2].tolist() == want
+    cache.close()
+
+
 def test_mistral_shaped_ragged_batch():
     """Config 4 scaled down: a ragged batch with a different number of heterogeneous heads per sequence."""
     from paper_2501_15113_b200 import configs
