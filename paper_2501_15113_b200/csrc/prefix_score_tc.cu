@@ -5,14 +5,15 @@
 // column sums, so that nothing is exchanged between CTAs and the second walk finds its keys in L2.
 //   warp 0          TMA producer: K tiles of 128 keys (four stages), the block's Q rows (two buffers, one block ahead)
 //   warps 1, 6      tcgen05.mma issuers, alternate tiles; four accumulators of 128 columns in TMEM
-//   warps 2-5, 7-10 two epilogue groups, alternate tiles
+//   warps 2-5, 7-18 four epilogue groups, every fourth tile each
 // First walk: D[row, key] = Q K^T, a TMEM lane is a query row and keeps its own running (max, sum); the two groups'
 // pairs meet in shared memory.  Second walk: D[key, row] = K Q^T, a lane is a key and sums its column.
 // Bound by the special-function unit: two exponentials per score at 16 a cycle and SM, 2048 cycles per tile and block.
 // Blocks are dealt out longest first, in both directions alternately, so that every CTA gets the same number of tiles;
 // the heads go in groups whose keys fit well into L2.  32 heads x 16384 rows, d = 128, both walks: as two launches of
 // the window kernel over (block, 2048 keys) items 4.19 ms (a CTA met the same two of a block's eight key ranges again
-// and again, a third more tiles for some than on average), like this 2.98 ms, 1600 cycles per tile and walk.
+// and again, a third more tiles for some than on average), like this with two epilogue groups 2.98 ms, with four 2.76 ms,
+// 1480 cycles per tile and walk: with two warps to a scheduler the special-function unit idles while they hand over.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -26,8 +27,10 @@ namespace {
 
 constexpr int kTile = 128;          // keys per tile, query rows per block
 constexpr int kStages = 4;          // K tiles in flight (even: a stage always has the same issuer)
-constexpr int kEpiWarps = 8;
-constexpr int kThreads = 352;
+constexpr int kGroups = 4;          // epilogue groups of four warps, one per accumulator
+constexpr int kEpiWarps = 4 * kGroups;
+constexpr int kThreads = (3 + kEpiWarps) * 32;
+constexpr int kCols = 32;           // accumulator columns per tensor-memory load
 constexpr uint32_t kTmemCols = 512;
 
 struct PrefixMaps {
@@ -67,7 +70,7 @@ inline PrefixLayout make_prefix_layout(int D) {
   l.tile_bytes = D / 64 * kTile * 128;
   l.off_q = kStages * l.tile_bytes;
   l.off_stat = l.off_q + 2 * l.tile_bytes;
-  l.off_off = l.off_stat + 2 * 2 * kTile * (int)sizeof(float2);
+  l.off_off = l.off_stat + 2 * kGroups * kTile * (int)sizeof(float2);
   l.off_bars = l.off_off + kEpiWarps * kTile * (int)sizeof(float);
   l.total = l.off_bars + 512 + 1024;
   return l;
@@ -85,8 +88,8 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char* sK = smem;                                         // [stages][KB][128 keys][128 B]
   unsigned char* sQ = smem + lay.off_q;                             // [2][KB][128 rows][128 B]
-  float2* sStat = reinterpret_cast<float2*>(smem + lay.off_stat);   // [2 blocks][2 groups][128 rows]
-  float* sOff = reinterpret_cast<float*>(smem + lay.off_off);       // [8 warps][128 rows]
+  float2* sStat = reinterpret_cast<float2*>(smem + lay.off_stat);   // [2 blocks][groups][128 rows]
+  float* sOff = reinterpret_cast<float*>(smem + lay.off_off);       // [epilogue warps][128 rows]
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + lay.off_bars);
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + B_COUNT);
   volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
@@ -207,7 +210,7 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
     }
   } else {
     // ------------------------------------------------------------ epilogue
-    const int ew = warp < 6 ? warp - 2 : warp - 3;  // 0..7
+    const int ew = warp < 6 ? warp - 2 : warp - 3;  // 0..15
     const int grp = ew >> 2;
     const int quad = warp & 3;                      // TMEM lane quadrant this warp may read
     const int row = quad * 32 + lane;               // first walk: this thread's query row; second: its key
@@ -227,25 +230,25 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
       // ---- first walk: the row's running max and sum over the tiles of this group
       float m_run = -INFINITY, z_run = 0.f;
       for (int t = 0; t < T; ++t, ++n) {
-        if ((n & 1) != grp) continue;
+        if ((n & (kGroups - 1)) != grp) continue;
         const int acc = n & 3;
         ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_TFULL + acc), (uint32_t)((n >> 2) & 1), s_abort));
         if (!ok) break;
         tc_fence_after();
         const bool tail = t == T - 1;               // row i sees the first i + 1 keys of the block's last tile
 #pragma unroll
-        for (int cg = 0; cg < 2; ++cg) {
-          uint32_t r[64];
-          tc_ld64(lane_addr + (uint32_t)(acc * 128 + cg * 64), r);
+        for (int c0 = 0; c0 < kTile; c0 += kCols) {
+          uint32_t r[kCols];
+          tc_ld32(lane_addr + (uint32_t)(acc * 128 + c0), r);
           tc_wait_ld();
           if (tail) {
 #pragma unroll
-            for (int i = 0; i < 64; ++i)
-              if (cg * 64 + i > row) r[i] = __float_as_uint(-INFINITY);
+            for (int i = 0; i < kCols; ++i)
+              if (c0 + i > row) r[i] = __float_as_uint(-INFINITY);
           }
           float cm4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-          for (int i = 0; i < 64; ++i) cm4[i & 3] = fmaxf(cm4[i & 3], __uint_as_float(r[i]));
+          for (int i = 0; i < kCols; ++i) cm4[i & 3] = fmaxf(cm4[i & 3], __uint_as_float(r[i]));
           const float cm = fmaxf(fmaxf(cm4[0], cm4[1]), fmaxf(cm4[2], cm4[3]));
           if (cm > m_run) {
             z_run *= ex2((m_run - cm) * scale2);
@@ -255,7 +258,7 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
             const float ms = -m_run * scale2;
             float zs[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int i = 0; i < 64; ++i) zs[i & 3] += ex2(fmaf(__uint_as_float(r[i]), scale2, ms));
+            for (int i = 0; i < kCols; ++i) zs[i & 3] += ex2(fmaf(__uint_as_float(r[i]), scale2, ms));
             z_run += (zs[0] + zs[1]) + (zs[2] + zs[3]);
           }
         }
@@ -265,7 +268,7 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
       // ---- the groups' pairs of every row -> one offset per row: max + log2(sum) + log2(128).  A query row beyond the
       // end of the sequence does not exist: an infinite offset takes it out of every column sum
       const int buf = k & 1;
-      sStat[(buf * 2 + grp) * kTile + row] = make_float2(m_run * scale2, z_run);
+      sStat[(buf * kGroups + grp) * kTile + row] = make_float2(m_run * scale2, z_run);
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR(B_STAT + buf));
       ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_STAT + buf), (uint32_t)((k >> 1) & 1), s_abort));
@@ -273,16 +276,21 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int i = q * 32 + lane;
-        const float2 u = sStat[(buf * 2) * kTile + i], v = sStat[(buf * 2 + 1) * kTile + i];
-        const float M = fmaxf(u.x, v.x);
-        const float z = (u.x > -INFINITY ? u.y * exp2f(u.x - M) : 0.f) + (v.x > -INFINITY ? v.y * exp2f(v.x - M) : 0.f);
+        float M = -INFINITY, z = 0.f;
+#pragma unroll
+        for (int g = 0; g < kGroups; ++g) M = fmaxf(M, sStat[(buf * kGroups + g) * kTile + i].x);
+#pragma unroll
+        for (int g = 0; g < kGroups; ++g) {
+          const float2 o = sStat[(buf * kGroups + g) * kTile + i];
+          if (o.x > -INFINITY) z += o.y * exp2f(o.x - M);
+        }
         myOff[i] = (z > 0.f && x.b * kTile + i < a.N) ? M + log2f(z) + 7.f : INFINITY;
       }
       __syncwarp();
       // ---- second walk: this thread's key, summed over the rows
       float* out = a.scores + (int64_t)x.head * 64 * a.nb * (a.nb + 1) + (int64_t)64 * x.b * (x.b + 1);
       for (int t = 0; t < T; ++t, ++n) {
-        if ((n & 1) != grp) continue;
+        if ((n & (kGroups - 1)) != grp) continue;
         const int acc = n & 3;
         ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_TFULL + acc), (uint32_t)((n >> 2) & 1), s_abort));
         if (!ok) break;
@@ -290,18 +298,18 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
         const bool tail = t == T - 1;
         float cs[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int c0 = 0; c0 < kTile; c0 += 64) {
-          uint32_t r[64];
-          tc_ld64(lane_addr + (uint32_t)(acc * 128 + c0), r);
+        for (int c0 = 0; c0 < kTile; c0 += kCols) {
+          uint32_t r[kCols];
+          tc_ld32(lane_addr + (uint32_t)(acc * 128 + c0), r);
           tc_wait_ld();
           if (tail) {                               // key i is seen by rows i .. 127 of the block
 #pragma unroll
-            for (int i = 0; i < 64; ++i)
+            for (int i = 0; i < kCols; ++i)
               if (c0 + i < row) r[i] = __float_as_uint(-INFINITY);
           }
           const float4* off4 = reinterpret_cast<const float4*>(myOff + c0);
 #pragma unroll
-          for (int i = 0; i < 64; i += 4) {
+          for (int i = 0; i < kCols; i += 4) {
             const float4 off = off4[i >> 2];
             cs[0] += ex2(fmaf(__uint_as_float(r[i]), scale2, -off.x));
             cs[1] += ex2(fmaf(__uint_as_float(r[i + 1]), scale2, -off.y));
