@@ -476,6 +476,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_fast_kernel(DeviceProblem 
   const float* C = p.C + p.c_off[u];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int base = tid * EPT;
+  grid_dependency_wait();
 
   // only the keys are kept (a key maps back to its score exactly); key 0 marks "no element"
   uint32_t key[EPT];
@@ -731,6 +732,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_cluster_kernel(DeviceProbl
   const float* C = p.C + p.c_off[u];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int base = (rank * kThreads + tid) * kEptMax;
+  grid_dependency_wait();
 
   uint32_t key[kEptMax];
   if (base + kEptMax <= N && ((reinterpret_cast<uintptr_t>(C + base) & 15) == 0)) {
@@ -847,13 +849,15 @@ cudaError_t launch_cluster_k(const DeviceProblem& p, const UnitRange& ur, int cs
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = s;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = (unsigned)cs_n;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)cs_n;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, select_cluster_kernel<T, D, POOL_HALF>, p, ur);
 }
 
@@ -894,8 +898,9 @@ cudaError_t launch_cluster(const DeviceProblem& p, const UnitRange& ur, int cs_n
 // keys is what a short unit's selection costs, beside the barriers.
 template <typename T, int D, int EPT>
 void launch_fast_ept(const DeviceProblem& p, const UnitRange& ur, cudaStream_t s) {
-  if (p.pool_w == 7) select_fast_kernel<T, D, 3, EPT><<<ur.blocks, kThreads, 0, s>>>(p, ur);
-  else select_fast_kernel<T, D, 0, EPT><<<ur.blocks, kThreads, 0, s>>>(p, ur);
+  // (an error stays with the runtime, where launch_select picks it up)
+  if (p.pool_w == 7) launch_dependent(select_fast_kernel<T, D, 3, EPT>, (unsigned)ur.blocks, kThreads, s, p, ur);
+  else launch_dependent(select_fast_kernel<T, D, 0, EPT>, (unsigned)ur.blocks, kThreads, s, p, ur);
 }
 template <typename T, int D>
 void launch_fast(const DeviceProblem& p, const UnitRange& ur, int max_N, cudaStream_t s) {

@@ -86,13 +86,23 @@ struct TcArgs {
   int pass;                 // 1 = row statistics, 2 = scores
   int n_seq;                // sequences in this launch
   int n_local;              // units per sequence (layers * kv heads)
-  int chunk_keys;           // keys per work item (multiple of 128)
+  int chunk_keys;           // keys per work item (multiple of 512)
+  int fine;                 // 128 rows, items shorter than 2048 keys: pass 1 stores every 512 keys
   int steps;                // items of the busiest CTA
   int u0[kMaxSeq];          // first unit of each sequence
   int N[kMaxSeq];           // sequence length
   int chunks[kMaxSeq];      // work items per unit
   int item_off[kMaxSeq + 1];
 };
+
+// Running (max, sum) pairs in log2 units: a <- a + b.
+__device__ __forceinline__ void fold_stat(float2& a, const float2 b) {
+  if (b.x > -INFINITY) {
+    const float M = fmaxf(a.x, b.x);
+    a.y = a.y * exp2f(a.x - M) + b.y * exp2f(b.x - M);
+    a.x = M;
+  }
+}
 
 struct Item {
   int seq, lu, ch;
@@ -201,6 +211,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
   const float scale2 = kLog2e * rsqrtf((float)D);
+  grid_dependency_wait();       // the setup above runs under the tail of the kernel before this one
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (whole warp, one lane issues)
@@ -352,10 +363,43 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
       // Which of the item's tiles this group takes depends on how many tiles the CTA has seen before (n): with n even
       // at the item's start it is the even ones.  The partial statistics below are filed under that parity, not under
       // the group, so that a slot always holds the same tiles (and keys) whatever else the CTA worked on before:
-      // results do not depend on how a problem is cut into launches.
+      // results do not depend on how a problem is cut into launches -- nor on the length of the items: what is stored
+      // covers 16 tiles of the unit, and with 128 rows those are folded from four parts of 4 tiles each, here (long
+      // items) or, where items are shorter than 16 tiles (a.fine), from the stored parts by the reduction.
       const int par = grp ^ (n & 1);                 // parity, within the item, of the tiles this warp takes
+      const int sub_shift = rows == 128 ? 2 : 4;     // log2 of the tiles per part
+      int sub = 0;                                   // the part this warp is working on, counted from the item's first
+      float2 group = make_float2(-INFINITY, 0.f);
+      auto end_part = [&]() {
+        // slot (part of the unit, part of the warps): (tile parity, lane quadrant); with 128 rows a quadrant is a set of
+        // rows, so there it is the tile parity alone
+        float2* base = reinterpret_cast<float2*>(p.stat_part) + (size_t)u * p.chunks_max * p.rows_pad;
+        const int tile0 = key0 / kTile;
+        if (rows == 128) {
+          const float2 mine = make_float2(m_run[0] * scale2, z_run[0]);
+          if (a.fine) {
+            base[(size_t)(((tile0 >> 2) + sub) * 2 + par) * p.rows_pad + quad * 32 + lane] = mine;
+          } else {
+            fold_stat(group, mine);
+            if ((sub & 3) == 3 || sub == ((ntiles + 3) >> 2) - 1) {
+              base[(size_t)(((tile0 >> 4) + (sub >> 2)) * 2 + par) * p.rows_pad + quad * 32 + lane] = group;
+              group = make_float2(-INFINITY, 0.f);
+            }
+          }
+        } else {
+#pragma unroll
+          for (int rg = 0; rg < 4; ++rg)
+            if (rg * 32 < rows)
+              base[(size_t)(((tile0 >> 4) + sub) * kTcParts + par * 4 + quad) * p.rows_pad + rg * 32 + lane] =
+                  make_float2(m_run[rg] * scale2, z_run[rg]);
+        }
+#pragma unroll
+        for (int rg = 0; rg < 4; ++rg) { m_run[rg] = -INFINITY; z_run[rg] = 0.f; }
+        ++sub;
+      };
       for (int t = 0; t < ntiles; ++t, ++n) {
         if ((n & 1) != grp) continue;
+        if (a.pass == 1 && (t >> sub_shift) != sub) end_part();
         const int acc = n & 3;
         const uint32_t accphase = (uint32_t)((n >> 2) & 1);
         ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_TFULL + acc), accphase, s_abort));
@@ -499,18 +543,9 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
       }
       if (!ok) break;
       if (a.pass == 1) {
-        // the warp's partial of this item: slot (chunk, part), part = (tile parity, lane quadrant); with 128 rows a
-        // quadrant is a set of rows, so there part = tile parity
-        float2* slot = reinterpret_cast<float2*>(p.stat_part) +
-                       ((size_t)u * p.chunks_max + (size_t)it.ch * (rows == 128 ? 2 : kTcParts)) * p.rows_pad;
-        if (rows == 128) {
-          slot[(size_t)par * p.rows_pad + quad * 32 + lane] = make_float2(m_run[0] * scale2, z_run[0]);
-        } else {
-#pragma unroll
-          for (int rg = 0; rg < 4; ++rg)
-            if (rg * 32 < rows)
-              slot[(size_t)(par * 4 + quad) * p.rows_pad + rg * 32 + lane] = make_float2(m_run[rg] * scale2, z_run[rg]);
-        }
+        // the last part, and an empty one should it hold no tile of this group
+        const int subs = (ntiles + (1 << sub_shift) - 1) >> sub_shift;
+        while (sub < subs) end_part();
       }
     }
   }
@@ -528,43 +563,61 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
   if (tid == 0 && *s_abort) set_status(p.status, TASKKV_ETIMEOUT);
 }
 
-// Folds the partial statistics of one unit: slots (item, warp) of pass 1 -> one offset per row.
-// One block per unit, one thread per row: the thread walks the unit's slots in order (a fixed order whatever the
-// launch), its neighbours reading the neighbouring rows of the same slot (coalesced); four slots are loaded ahead of
-// the dependent max / sum updates.
-__global__ void __launch_bounds__(128) window_tc_reduce_kernel(DeviceProblem p, UnitRange ur, int chunk_keys,
-                                                               int parts) {
+// Folds the partial statistics of one unit -> one offset per row.  One block per unit; 1024 / rows threads share a row,
+// each taking every (1024 / rows)-th slot in order with four loads ahead of the dependent updates, and their results are
+// joined in order: the outcome depends on the unit's own length alone.
+__global__ void __launch_bounds__(1024) window_tc_reduce_kernel(DeviceProblem p, UnitRange ur, int fine) {
+  __shared__ float2 tmp[1024];
   const int u = ur.unit(blockIdx.x);
-  const int slots = (p.unit_N[u] + chunk_keys - 1) / chunk_keys * parts;
-  const float2* part = reinterpret_cast<const float2*>(p.stat_part) + (size_t)u * p.chunks_max * p.rows_pad;
-  const int row = threadIdx.x;
-  if (row >= p.rows) return;
-  float M = -INFINITY, z = 0.f;
-  auto fold = [&](const float2 o) {
-    if (o.x > -INFINITY) {
-      const float Mn = fmaxf(M, o.x);
-      z = z * exp2f(M - Mn) + o.y * exp2f(o.x - Mn);
-      M = Mn;
+  const int N = p.unit_N[u];
+  const int slots = (N + 16 * kTile - 1) / (16 * kTile) * (p.rows == 128 ? 2 : kTcParts);
+  const int rows = p.rows, P = 1024 / rows;
+  const int row = threadIdx.x % rows, part = threadIdx.x / rows;
+  const float2* src = reinterpret_cast<const float2*>(p.stat_part) + (size_t)u * p.chunks_max * p.rows_pad + row;
+  float2 acc = make_float2(-INFINITY, 0.f);
+  grid_dependency_wait();
+  if (fine) {
+    // 128 rows: slot (group, parity) is folded from up to four stored parts
+    const int parts = (N + 4 * kTile - 1) / (4 * kTile);
+    for (int c = part; c < slots; c += P) {
+      float2 o[4], g = make_float2(-INFINITY, 0.f);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int q = (c >> 1) * 4 + i;
+        o[i] = q < parts ? src[(size_t)(q * 2 + (c & 1)) * p.rows_pad] : make_float2(-INFINITY, 0.f);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) fold_stat(g, o[i]);
+      fold_stat(acc, g);
     }
-  };
-  int c = 0;
-  for (; c + 4 <= slots; c += 4) {
-    float2 o[4];
+  } else {
+    for (int c = part; c < slots; c += 4 * P) {
+      float2 o[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) o[i] = part[(size_t)(c + i) * p.rows_pad + row];
+      for (int i = 0; i < 4; ++i)
+        o[i] = c + i * P < slots ? src[(size_t)(c + i * P) * p.rows_pad] : make_float2(-INFINITY, 0.f);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) fold(o[i]);
+      for (int i = 0; i < 4; ++i) fold_stat(acc, o[i]);
+    }
   }
-  for (; c < slots; ++c) fold(part[(size_t)c * p.rows_pad + row]);
-  // one offset per row: score * scale - (max + log2(sum) + log2(rows)) is log2 of the row's share of C
-  p.stat[(size_t)u * (2 * p.rows_pad) + row] = z > 0.f ? M + log2f(z) + log2f((float)p.rows) : INFINITY;
+  tmp[threadIdx.x] = acc;
+  __syncthreads();
+  if (part == 0) {
+    for (int q = 1; q < P; ++q) fold_stat(acc, tmp[q * rows + row]);
+    // one offset per row: score * scale - (max + log2(sum) + log2(rows)) is log2 of the row's share of C
+    p.stat[(size_t)u * (2 * p.rows_pad) + row] = acc.y > 0.f ? acc.x + log2f(acc.y) + log2f((float)rows) : INFINITY;
+  }
 }
 
-// Keys per work item.  Every item costs a Q load and, in pass 2, a statistics load, so long items are
-// better as long as the CTAs still get a dozen items each; short inputs keep 2048-key items.
-inline int pick_chunk(int64_t units_times_keys, int n_sm) {
-  const int big = 2 * kTcChunk;
-  return units_times_keys / big >= (int64_t)12 * n_sm ? big : kTcChunk;
+// Keys per work item.  Every item costs a Q load and, in pass 2, a statistics load, so long items are better as long as
+// the CTAs still get a dozen items each; a launch with fewer takes shorter ones, down to the 512 keys of one partial
+// (2048 with fewer than 128 rows, in pass 1), so that a single layer of a short prompt still reaches every SM: 8 units of
+// 8191 keys, 128 rows, took 23.2 us a pass on 32 CTAs of 16 tiles, 15.3 on 128 of 4.
+inline int pick_chunk(int64_t units_times_keys, int n_sm, int least) {
+  if (units_times_keys / 4096 >= (int64_t)12 * n_sm) return 4096;
+  int chunk = 2048;
+  while (chunk > least && units_times_keys / chunk < (int64_t)3 * n_sm) chunk /= 2;
+  return chunk;
 }
 
 template <int D>
@@ -586,7 +639,6 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
   const int per_seq = n_layers * p.n_kv;
   const int skip = (layer0 - h.base_layer) * p.n_kv;   // units between what h.q / h.k point at and the first one
   if (per_seq <= 0) return cudaSuccess;
-  const int parts = p.rows == 128 ? 2 : kTcParts;
   // up to kMaxSeq sequences per pair of launches
   for (int b0 = 0; b0 < h.batch; b0 += kMaxSeq) {
     const int nb = h.batch - b0 < kMaxSeq ? h.batch - b0 : kMaxSeq;
@@ -596,8 +648,6 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
     for (int i = 0; i < nb; ++i) keys += (int64_t)per_seq * h.seq_lens[b0 + i];
     a.n_seq = nb;
     a.n_local = per_seq;
-    a.chunk_keys = pick_chunk(keys, n_sm);
-    a.item_off[0] = 0;
     for (int i = 0; i < kMaxSeq; ++i) {
       const int b = b0 + (i < nb ? i : 0);                  // unused slots repeat the first sequence
       const int N = h.seq_lens[b];
@@ -613,12 +663,21 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
       }
       a.u0[i] = b * per_seq_all + first;
       a.N[i] = N;
-      a.chunks[i] = (N + a.chunk_keys - 1) / a.chunk_keys;
-      a.item_off[i + 1] = a.item_off[i] + (i < nb ? per_seq * a.chunks[i] : 0);
     }
-    const int n1 = a.item_off[nb];
-    const int grid = n1 < n_sm ? n1 : n_sm;
-    a.steps = (n1 + grid - 1) / grid;
+    auto launch_pass = [&](int pass, int least) -> cudaError_t {
+      a.pass = pass;
+      a.chunk_keys = pick_chunk(keys, n_sm, least);
+      a.fine = pass == 1 && p.rows == 128 && a.chunk_keys < 16 * kTile ? 1 : 0;
+      a.item_off[0] = 0;
+      for (int i = 0; i < kMaxSeq; ++i) {
+        a.chunks[i] = (a.N[i] + a.chunk_keys - 1) / a.chunk_keys;
+        a.item_off[i + 1] = a.item_off[i] + (i < nb ? per_seq * a.chunks[i] : 0);
+      }
+      const int items = a.item_off[nb], grid = items < n_sm ? items : n_sm;
+      a.steps = (items + grid - 1) / grid;
+      LaunchScope ls(K_WINDOW_TC, s);
+      return launch_dependent_smem(window_tc_kernel<D>, (unsigned)grid, kThreads, (size_t)smem, s, maps, p, a, lay);
+    };
     if (h.lse) {
       // the caller already has the rows' normalisers: no pass 1
       const size_t lse_skip = (size_t)(layer0 - h.base_layer) * p.n_heads * p.L;
@@ -628,22 +687,15 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
         if (e != cudaSuccess) return e;
       }
     } else {
-      a.pass = 1;
-      {
-        LaunchScope ls(K_WINDOW_TC, s);
-        window_tc_kernel<D><<<grid, kThreads, smem, s>>>(maps, p, a, lay);
-      }
-      {
-        LaunchScope ls(K_WINDOW_REDUCE, s);
-        const UnitRange ur{b0 * per_seq_all + first, per_seq, per_seq_all, nb * per_seq};
-        window_tc_reduce_kernel<<<nb * per_seq, 128, 0, s>>>(p, ur, a.chunk_keys, parts);
-      }
+      e = launch_pass(1, p.rows == 128 ? 4 * kTile : kTcChunk);
+      if (e != cudaSuccess) return e;
+      LaunchScope ls(K_WINDOW_REDUCE, s);
+      const UnitRange ur{b0 * per_seq_all + first, per_seq, per_seq_all, nb * per_seq};
+      e = launch_dependent(window_tc_reduce_kernel, (unsigned)(nb * per_seq), 1024, s, p, ur, a.fine);
+      if (e != cudaSuccess) return e;
     }
-    a.pass = 2;
-    {
-      LaunchScope ls(K_WINDOW_TC, s);
-      window_tc_kernel<D><<<grid, kThreads, smem, s>>>(maps, p, a, lay);
-    }
+    e = launch_pass(2, 4 * kTile);
+    if (e != cudaSuccess) return e;
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
