@@ -736,10 +736,12 @@ taskkv_status taskkv_compress_lse(const taskkv_params* p, const void* const* q_w
 
 namespace {
 // Plans the problem, takes or allocates the memory, and puts the tables and a clean state on the device (enqueued
-// on `s`); no layer is compressed yet.
+// on `s`); no layer is compressed yet.  With q_win, k, v the per-unit input pointers of every layer go up with the
+// other tables in the same copy.
 taskkv_status cache_create_impl(const taskkv_params* p, void* cache_mem, size_t cache_bytes, void* workspace_mem,
                                 size_t workspace_bytes, cudaStream_t s, taskkv_cache** out_cache,
-                                taskkv_pool* pool = nullptr) {
+                                taskkv_pool* pool = nullptr, const void* const* q_win = nullptr,
+                                const void* const* k = nullptr, const void* const* v = nullptr) {
   if (!p || !out_cache) return TASKKV_EINVAL;
   *out_cache = nullptr;
   taskkv_cache* c = new (std::nothrow) taskkv_cache();
@@ -790,6 +792,7 @@ taskkv_status cache_create_impl(const taskkv_params* p, void* cache_mem, size_t 
   }
   fill_device_problem(c);
   fill_tables(c);
+  if (q_win) set_layer_pointers(c, 0, p->n_layers, q_win, k, v);
   // the tables, then zeros over everything between them and the pools: status word, lengths, capacities, offsets,
   // classes, work lists (a layer that has not been compressed yet has length 0 everywhere)
   cudaError_t e = cudaMemcpyAsync(c->cache_mem, c->meta.data(), c->hp.meta_bytes, cudaMemcpyHostToDevice, s);
@@ -806,13 +809,6 @@ taskkv_status cache_create_impl(const taskkv_params* p, void* cache_mem, size_t 
   }
   *out_cache = c;
   return TASKKV_OK;
-}
-
-// Uploads the per-unit input pointer tables (three adjacent arrays of the table area).
-cudaError_t upload_pointers(taskkv_cache* c, cudaStream_t s) {
-  const HostPlan& hp = c->hp;
-  return cudaMemcpyAsync(static_cast<unsigned char*>(c->cache_mem) + hp.o_qp, c->meta.data() + hp.o_qp,
-                         hp.meta_bytes - hp.o_qp, cudaMemcpyHostToDevice, s);
 }
 
 bool pointers_ok(const taskkv_params* p, const void* const* q_win, const void* const* k, const void* const* v,
@@ -834,15 +830,15 @@ taskkv_status compress_impl(const taskkv_params* p, const void* const* q_win, co
   if (p->shard_kv_heads > 0) return TASKKV_EINVAL;      // a shard needs the other shards' vectors: begin / finish
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   taskkv_cache* c = nullptr;
-  const taskkv_status st = cache_create_impl(p, cache_mem, cache_bytes, workspace_mem, workspace_bytes, s, &c, pool);
+  const taskkv_status st = cache_create_impl(p, cache_mem, cache_bytes, workspace_mem, workspace_bytes, s, &c, pool,
+                                             q_win, k, v);
   if (st != TASKKV_OK) return st;
   if (pool) {
     pool->free_host -= c->hp.pages_compress;
     c->pages_held = c->hp.pages_compress;
     ++pool->caches;
   }
-  set_layer_pointers(c, 0, p->n_layers, q_win, k, v);
-  cudaError_t e = upload_pointers(c, s);
+  cudaError_t e = cudaSuccess;
   WindowHostInfo wh;
   wh.batch = p->batch;
   wh.seq_lens = c->hp.seq_lens.data();
@@ -973,10 +969,10 @@ taskkv_status taskkv_compress_shard_begin(const taskkv_params* p, const void* co
   if (p->batch < 1 || p->shard_kv_heads < 1 || !pointers_ok(p, q_win, k, v, window_lse)) return TASKKV_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   taskkv_cache* c = nullptr;
-  const taskkv_status st = cache_create_impl(p, cache_mem, cache_bytes, workspace_mem, workspace_bytes, s, &c);
+  const taskkv_status st =
+      cache_create_impl(p, cache_mem, cache_bytes, workspace_mem, workspace_bytes, s, &c, nullptr, q_win, k, v);
   if (st != TASKKV_OK) return st;
-  set_layer_pointers(c, 0, p->n_layers, q_win, k, v);
-  cudaError_t e = upload_pointers(c, s);
+  cudaError_t e = cudaSuccess;
   WindowHostInfo wh;
   wh.batch = p->batch;
   wh.seq_lens = c->hp.seq_lens.data();
