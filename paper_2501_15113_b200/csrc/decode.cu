@@ -697,6 +697,89 @@ __device__ __forceinline__ void prefetch_item(const DeviceProblem& p, const Item
                  : "memory");
 }
 
+// The merge for calls whose units have at most 32 partial results each: a warp per (view unit, query head), eight to a
+// block, one partial's (max, sum) per lane and no block barrier.  The sums are formed in the order of the kernel above
+// (its warp w adds partials w, w + 8, ...), so the results are the same bits.  Where units are short the block per head
+// of that kernel is launch and barriers: 384 units x 4 heads of at most 12 partials, the step 65.7 -> 61.0 us; a single
+// layer of units of 25 partials, three rounds for a warp, is 0.3 us slower than with a block per head.
+template <typename T, int D, int G>
+__global__ void __launch_bounds__(kCombineThreads) decode_combine_few_kernel(DeviceProblem p,
+                                                                             const int32_t* __restrict__ lengths,
+                                                                             int fused_step, T* __restrict__ out) {
+  constexpr int EPL = D / 32;
+  using Vec = typename std::conditional<EPL == 4, float4, float2>::type;
+  const int lane = threadIdx.x & 31;
+  const int vg = (int)blockIdx.x * kCombineWarps + (threadIdx.x >> 5);
+  const bool there = vg < p.view_U * G;
+  const int u = there ? vg / G : 0, g = vg % G;         // u: view unit
+  const int unit = view_unit(p, u);
+  // read before the wait, as in the kernel above
+  int len = p.len[unit];
+  const bool grown = fused_step && len < p.cap[unit];
+  const int len_next = len + (grown ? 1 : 0);
+  len = len_next;
+  if (lengths) len = min(max(lengths[u], 0), len);
+  const int i0 = p.dec_off[lm_index(p, unit)], n = (len + p.dec_chunk - 1) / p.dec_chunk;
+  grid_dependency_wait();
+  grid_launch_dependents();
+  if (!there) return;
+  if (n != 1) {                                         // a unit of one item has its output from the attention kernel
+    const float2 v = lane < n ? reinterpret_cast<const float2*>(p.part_ml)[(size_t)(i0 + lane) * G + g]
+                              : make_float2(-INFINITY, 0.f);
+    const float* src = p.part_acc + ((size_t)i0 * G + g) * D + lane * EPL;
+    Vec first[kCombineWarps];                           // requested together with the pairs
+#pragma unroll
+    for (int j = 0; j < kCombineWarps; ++j)
+      if (j < n) first[j] = *reinterpret_cast<const Vec*>(src + (size_t)j * G * D);
+    const float M = warp_max(v.x);
+    const float w = (v.x == -INFINITY) ? 0.f : exp2f(v.x - M);
+    const float L = warp_sum(fmaf(w, v.y, 0.f));
+    float acc[kCombineWarps][EPL];
+    auto add = [&](float (&a)[EPL], float wgt, const Vec& t) {
+      a[0] = fmaf(wgt, t.x, a[0]);
+      a[1] = fmaf(wgt, t.y, a[1]);
+      if constexpr (EPL == 4) {
+        a[2] = fmaf(wgt, t.z, a[2]);
+        a[3] = fmaf(wgt, t.w, a[3]);
+      }
+    };
+#pragma unroll
+    for (int j = 0; j < kCombineWarps; ++j) {
+#pragma unroll
+      for (int e = 0; e < EPL; ++e) acc[j][e] = 0.f;
+      const float wj = __shfl_sync(0xffffffffu, w, j);
+      if (j < n) add(acc[j], wj, first[j]);
+    }
+    for (int j0 = kCombineWarps; j0 < n; j0 += kCombineWarps) {
+      Vec t[kCombineWarps];
+#pragma unroll
+      for (int j = 0; j < kCombineWarps; ++j)
+        if (j0 + j < n) t[j] = *reinterpret_cast<const Vec*>(src + (size_t)(j0 + j) * G * D);
+#pragma unroll
+      for (int j = 0; j < kCombineWarps; ++j) {
+        const float wj = __shfl_sync(0xffffffffu, w, j0 + j);
+        if (j0 + j < n) add(acc[j], wj, t[j]);
+      }
+    }
+    T* o = out + ((size_t)u * G + g) * D + lane * EPL;
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) {
+      float a = 0.f;
+#pragma unroll
+      for (int j = 0; j < kCombineWarps; ++j) a += acc[j][e];
+      store_out(o + e, L > 0.f ? a / L : 0.f);
+    }
+  }
+  if (fused_step && lane == 0) {
+    // the last of the unit's G warps raises the length, as above
+    if (atomicAdd(&p.step_cnt[unit], 1) == G - 1) {
+      p.step_cnt[unit] = 0;
+      if (grown) { if (p.page_rows == 0 || *p.status == 0) p.len[unit] = len_next; }
+      else set_status(p.status, TASKKV_ESTATE);
+    }
+  }
+}
+
 // The whole of a small call in one launch: a thread-block cluster of cs CTAs owns a unit, its CTAs take the unit's work
 // items (rank, rank + cs), push their partial results into the cluster's shared memory, and every CTA merges its share
 // of the outputs after one cluster barrier.  The items, their arithmetic and the order in which they are merged are
@@ -887,13 +970,19 @@ cudaError_t launch_typed(const DeviceProblem& p, const void* q, const int32_t* l
   if (e != cudaSuccess) return e;
   {
     LaunchScope ls(K_DECODE_COMBINE, s);
-    // up to 16 blocks per SM: the variant that loads ahead (its blocks are resident within a few waves)
-    if ((int64_t)p.view_U * G <= 148 * 16)
+    const int fused = k_new != nullptr ? 1 : 0;
+    // units of at most 16 items each (32, if a block per head would be more than the GPU holds at once): a warp per head.
+    // Otherwise a block per head; up to 16 of them per SM the variant that loads ahead (its blocks are resident within a
+    // few waves)
+    if ((int64_t)p.max_cap <= (int64_t)((int64_t)p.view_U * G > 148 * 4 ? 32 : 16) * p.dec_chunk)
+      e = launch_dependent(decode_combine_few_kernel<T, D, G>, (unsigned)((p.view_U * G + kCombineWarps - 1) / kCombineWarps),
+                           kCombineThreads, s, p, lengths, fused, static_cast<T*>(out));
+    else if ((int64_t)p.view_U * G <= 148 * 16)
       e = launch_dependent(decode_combine_kernel<T, D, G, 8>, (unsigned)(p.view_U * G), kCombineThreads, s, p, lengths,
-                           k_new != nullptr ? 1 : 0, static_cast<T*>(out));
+                           fused, static_cast<T*>(out));
     else
       e = launch_dependent(decode_combine_kernel<T, D, G, 0>, (unsigned)(p.view_U * G), kCombineThreads, s, p, lengths,
-                           k_new != nullptr ? 1 : 0, static_cast<T*>(out));
+                           fused, static_cast<T*>(out));
   }
   return e;
 }

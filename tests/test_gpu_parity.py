@@ -193,6 +193,12 @@ def test_cluster_decode_equals_the_two_kernels_bit_for_bit(kw, page_rows):
 
     (a, pa), (b, pb) = compress(), compress()
     P = _parity()
+    if not page_rows and R > 1:
+        # a reserve of 32 items makes the whole call's merge the block per head, not the warp per head
+        far = tk.taskkv_compress_ex(tk.params_from_workload(wl, max_new_tokens=32 * 512), qs, ks, vs)
+        q, _, _ = W.gen_decode_step(wl, 9, DEV)
+        assert torch.equal(far.taskkv_decode(q), a.taskkv_decode(q))
+        far.close()
     for s in range(4):
         q, kn, vn = W.gen_decode_step(wl, s, DEV)
         whole = a.taskkv_decode_step(q, kn, vn)
