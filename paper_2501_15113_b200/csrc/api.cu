@@ -554,6 +554,8 @@ void fill_device_problem(taskkv_cache* c) {
   if (d.max_mid > hp.max_N) d.max_mid = hp.max_N;
   d.max_new = p.max_new_tokens;
   d.dec_chunk = hp.dec_chunk;
+  d.dec_shift = 0;
+  while ((1 << d.dec_shift) < hp.dec_chunk) ++d.dec_shift;
   d.max_prompt = hp.max_N;
   d.max_cap = hp.max_N + p.max_new_tokens;
   d.idx_stride = hp.idx_stride;

@@ -54,7 +54,8 @@ struct DeviceProblem {
   // n_kv + h stands for layer view_l0 + r'.  q, k_new, v_new, out and `lengths` are indexed by view unit.
   int32_t view_l0, view_nl, view_U;
   int32_t max_new;
-  int32_t dec_chunk;    // rows of one split-K decode item of this cache
+  int32_t dec_chunk;    // rows of one split-K decode item of this cache: a power of two, log2 in dec_shift
+  int32_t dec_shift;
   int32_t max_prompt, max_cap;   // most rows a unit holds right after compression, most it can grow to
   float budget_frac;    // > 0: the middle budget follows Eq. 17 from this fraction of the full cache
   // Head sharding: this problem holds KV heads [kv_first, kv_first + n_kv) of a model with n_kv_model per layer.

@@ -592,7 +592,7 @@ __global__ void __launch_bounds__(kCombineThreads, PRE > 0 ? 4 : 6) decode_combi
   len = len_next;
   if (lengths) len = min(max(lengths[u], 0), len);
   // the unit's items that hold rows (the table also numbers the reserve for appended tokens)
-  const int i0 = p.dec_off[lm_index(p, unit)], i1 = i0 + (len + p.dec_chunk - 1) / p.dec_chunk;
+  const int i0 = p.dec_off[lm_index(p, unit)], i1 = i0 + ((len + p.dec_chunk - 1) >> p.dec_shift);
   grid_dependency_wait();
   grid_launch_dependents();
   if (i1 - i0 != 1) {                                   // a unit of one item has its output from the attention kernel
@@ -719,7 +719,7 @@ __global__ void __launch_bounds__(kCombineThreads) decode_combine_few_kernel(Dev
   const int len_next = len + (grown ? 1 : 0);
   len = len_next;
   if (lengths) len = min(max(lengths[u], 0), len);
-  const int i0 = p.dec_off[lm_index(p, unit)], n = (len + p.dec_chunk - 1) / p.dec_chunk;
+  const int i0 = p.dec_off[lm_index(p, unit)], n = (len + p.dec_chunk - 1) >> p.dec_shift;
   grid_dependency_wait();
   grid_launch_dependents();
   if (!there) return;
@@ -821,7 +821,7 @@ decode_cluster_kernel(DeviceProblem p, const T* __restrict__ q, const int32_t* _
   const int64_t seg = p.seg_off[u];
   len = len_next;
   if (lengths) len = min(max(lengths[v], 0), len);
-  const int n = (len + p.dec_chunk - 1) / p.dec_chunk;
+  const int n = (len + p.dec_chunk - 1) >> p.dec_shift;
   const int old_len = new_r >= 0 ? min(len, new_r) : len;   // rows that are in the segment already
   if (!PAGED) prefetch_item<ROW_BYTES, PAGED>(p, ItemPages{0, 0}, seg, rank * p.dec_chunk, min(old_len, (rank + 1) * p.dec_chunk));
   if (early) { grid_dependency_wait(); grid_launch_dependents(); }
