@@ -10,6 +10,14 @@ namespace taskkv {
 
 // 2-D bf16 tensor [rows_total][d], box of 64 elements x box_rows rows, 128-byte swizzle (host; window_score_tc.cu).
 bool make_tensor_map_2d(CUtensorMap* map, const void* base, int d, uint64_t rows_total, int box_rows);
+// 3-D bf16 tensor [units][rows][d], box of 64 elements x box_rows rows of one unit, 128-byte swizzle; box_rows may be more
+// than a unit has, the rows beyond it are filled with zeros.
+bool make_tensor_map_units(CUtensorMap* map, const void* base, int d, int rows, uint64_t units, int box_rows);
+// Window rows of the tensor-core kernels: the MMA's N (and a TMEM tile's columns) is 32, 64 or 128; a window of another
+// size runs as the next larger one, its missing rows being zero queries that weigh nothing (compression and one step, 32
+// heads x 4 layers x 20001 keys with 16 rows: 1.10 ms on the CUDA cores, 0.33 like this; 4 KV heads x 8 layers x 6001 keys
+// with 96 rows 0.43 and 0.10).
+__host__ __device__ inline int tc_rows(int rows) { return rows <= 32 ? 32 : rows <= 64 ? 64 : 128; }
 
 namespace tc {
 
@@ -72,6 +80,12 @@ static __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorM
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
       ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
+      : "memory");
+}
+static __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar)
       : "memory");
 }
 static __device__ __forceinline__ void tc_alloc(uint32_t smem_dst, uint32_t cols) {

@@ -3,7 +3,7 @@
 //   C[j] = mean over the unit's G*L window rows of the normalised weights.
 //
 // Generic two-pass path on the CUDA cores (fp32 accumulate), used for fp32
-// inputs and for bf16 with a number of window rows the tensor-core path does not take:
+// inputs (bf16 runs on the tensor cores; it comes here only where the driver has no tensor maps to give):
 //   pass 1  per (unit, 256-key chunk): row maxima and exp-sums  -> partial stats
 //   reduce  per unit: combine chunks -> (row max, 1 / row sum); units of up to 32 chunks need no launch for it,
 //           their pass-2 blocks combine the chunks themselves
@@ -253,14 +253,18 @@ __global__ void __launch_bounds__(kBlock) window_reduce_kernel(DeviceProblem p, 
 }
 
 // Caller-supplied normalisers lse_i = ln sum_j exp(s_ij) of the window rows, in place of pass 1.  A unit's G*L rows
-// are contiguous in [R][n][L].  Tensor-core path: one offset per row, lse * log2(e) + log2(rows); here: the pair
+// are contiguous in [R][n][L].  Tensor-core path: one offset per row, lse * log2(e) + log2(rows),
+// up to 32 rows the pair (lse * log2(e), 1 / rows), one array after the other; here: the pair
 // (reference, 1 / sum relative to it) = (lse * log2(e), 1).
 __global__ void lse_to_stat_kernel(DeviceProblem p, int u0, const float* __restrict__ lse, int tc_format) {
   const int lu = blockIdx.x, row = threadIdx.x;
   if (row >= p.rows) return;
   const float v = lse[(size_t)lu * p.rows + row] * kLog2e;
   const size_t u = (size_t)(u0 + lu);
-  if (tc_format) p.stat[u * (2 * p.rows_pad) + row] = v + log2f((float)p.rows);
+  if (tc_format && p.rows <= 32) {
+    p.stat[u * (2 * p.rows_pad) + row] = v;
+    p.stat[u * (2 * p.rows_pad) + p.rows_pad + row] = 1.0f / (float)p.rows;
+  } else if (tc_format) p.stat[u * (2 * p.rows_pad) + row] = v + log2f((float)p.rows);
   else reinterpret_cast<float2*>(p.stat)[u * p.rows_pad + row] = make_float2(v, 1.0f);
 }
 
@@ -327,7 +331,7 @@ cudaError_t launch_lse_to_stat(const DeviceProblem& p, int u0, int n_units, cons
 cudaError_t launch_window_scores(const DeviceProblem& p, int dtype, int max_N, const WindowHostInfo& h,
                                  cudaStream_t s, int layer0, int n_layers) {
   if (n_layers < 0) { layer0 = 0; n_layers = p.R; }
-  // bf16 with 32 / 64 / 128 window rows runs on the tensor cores; everything else here
+  // bf16 runs on the tensor cores; everything else here
   if (window_tc_supported(p, dtype)) return launch_window_scores_tc(p, h, s, layer0, n_layers);
   if (dtype == TASKKV_F32) {
     return p.d == 64 ? launch_generic<float, 64>(p, max_N, h, s, layer0, n_layers)

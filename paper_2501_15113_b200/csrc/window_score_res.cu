@@ -1,6 +1,6 @@
 // Observation-window scores (Eq. 12, Eq. 13) with K read once: the raw scores of a whole unit stay in
-// tensor memory between the two steps of the softmax.  For bf16 inputs with G*L = 32 window rows and
-// sequences of up to 16 x 2048 keys.
+// tensor memory between the two steps of the softmax.  For bf16 inputs with G*L <= 32 window rows (fewer than 32 are
+// filled up with zero rows, whose terms are masked) and sequences of up to 16 x 2048 keys.
 //
 // Eq. 13 sums the rows of the window's softmax, so every row's normaliser (over all N keys) is needed before
 // any column can be finished.  The two-launch kernel of window_score_tc.cu reads K a second time for that.
@@ -48,7 +48,7 @@ constexpr uint32_t kTmemCols = 512;
 
 struct ResMaps {
   CUtensorMap k[kMaxSeq];   // [units * N][d] of each sequence
-  CUtensorMap q[kMaxSeq];   // [units * 32][d]
+  CUtensorMap q[kMaxSeq];   // [units][window rows][d]
 };
 struct ResArgs {
   int n_seq;                // sequences in this launch
@@ -191,8 +191,8 @@ window_res_kernel(const __grid_constant__ ResMaps maps, DeviceProblem p, const _
       if (elect_one()) {
         mbar_expect_tx(BAR(B_QFULL + qb), (uint32_t)lay.q_block_bytes);
         for (int kb = 0; kb < KB; ++kb)
-          tma_load_2d(smem_u32(sQ + (size_t)qb * lay.q_block_bytes + (size_t)kb * kRows * 128), &maps.q[it.seq],
-                      kb * 64, it.lu * kRows, BAR(B_QFULL + qb));
+          tma_load_3d(smem_u32(sQ + (size_t)qb * lay.q_block_bytes + (size_t)kb * kRows * 128), &maps.q[it.seq],
+                      kb * 64, 0, it.lu, BAR(B_QFULL + qb));
       }
       __syncwarp();
       qphase[qb] ^= 1;
@@ -271,6 +271,7 @@ window_res_kernel(const __grid_constant__ ResMaps maps, DeviceProblem p, const _
     float* myRef = sRef + ew * kRows;
     float* myW = sOff + ew * kRows;
     uint32_t fphase = 0;                            // bit t: phase of TFULL[t] to wait for
+    const uint32_t row_mask = p.rows >= 32 ? 0xffffffffu : (1u << p.rows) - 1u;   // rows the window has
     int nu = 0;                                     // units this CTA has been through
     bool ok = true;
     for (int k = 0; k < a.steps && ok; ++k) {
@@ -285,12 +286,12 @@ window_res_kernel(const __grid_constant__ ResMaps maps, DeviceProblem p, const _
       // bit i: window row i may see this thread's key of tile t (Eq. 12: key <= N - L + i % L, and a key at all)
       auto in_tail = [&](int t) { return (it.t0 + t) * kTile + kTile - 1 > N - L; };   // some key masked for some row
       auto visible_rows = [&](int t) -> uint32_t {
-        if (!in_tail(t)) return 0xffffffffu;
+        if (!in_tail(t)) return row_mask;
         const int j = key_of(t);
         uint32_t vm = 0;
 #pragma unroll
         for (int i = 0; i < 32; ++i) vm |= (uint32_t)(j < N && j <= N - L + sMod[i]) << i;
-        return vm;
+        return vm & row_mask;
       };
 
       // ---- step 1: every score becomes e = exp2(s - c_row) in place; per-thread row sums of e.
@@ -426,17 +427,16 @@ window_res_kernel(const __grid_constant__ ResMaps maps, DeviceProblem p, const _
       ok = __all_sync(0xffffffffu, mbar_wait_cluster(BAR(B_X + buf), uphase, s_abort));
       if (!ok) break;
       {
-        // lane = row: the T pairs -> the row's offset max + log2(sum) + log2(rows); a stored e of this warp then
-        // weighs exp2(c - offset) in C
+        // lane = row: the T pairs -> the row's max and sum; a stored e of this warp weighs exp2(c - max) / (sum rows) in C
         float M = -INFINITY, Z = 0.f;
         for (int r = 0; r < team; ++r) M = fmaxf(M, sX[(buf * kMaxTeam + r) * kRows + lane].x);
         for (int r = 0; r < team; ++r) {
           const float2 o = sX[(buf * kMaxTeam + r) * kRows + lane];
           if (o.x > -INFINITY) Z += o.y * ex2(o.x - M);
         }
-        const float off = M + lg2(Z) + 5.f;         // log2(32 rows)
         __syncwarp();
-        myW[lane] = (Z > 0.f && my_c > -INFINITY) ? ex2(my_c - off) : 0.f;
+        // (one division instead of a logarithm in the exponent: an offset of 20 carries a rounding of 1e-6)
+        myW[lane] = (Z > 0.f && my_c > -INFINITY) ? ex2(my_c - M) / (Z * (float)p.rows) : 0.f;
         __syncwarp();
       }
 
@@ -550,10 +550,9 @@ cudaError_t launch_res_d(const DeviceProblem& p, const WindowHostInfo& h, cudaSt
           // h.k[b], h.q[b] point at layer h.base_layer
           const size_t skip = (size_t)(first - h.base_layer * p.n_kv);
           const char* kb = static_cast<const char*>(h.k[b]) + skip * (size_t)N * D * sizeof(__nv_bfloat16);
-          const char* qb = static_cast<const char*>(h.q[b]) + skip * kRows * D * sizeof(__nv_bfloat16);
+          const char* qb = static_cast<const char*>(h.q[b]) + skip * p.rows * D * sizeof(__nv_bfloat16);
           if (!make_tensor_map_2d(&maps.k[i], kb, D, (uint64_t)per_seq * (uint64_t)N, kTile)) return cudaErrorUnknown;
-          if (!make_tensor_map_2d(&maps.q[i], qb, D, (uint64_t)per_seq * (uint64_t)kRows, kRows))
-            return cudaErrorUnknown;
+          if (!make_tensor_map_units(&maps.q[i], qb, D, p.rows, (uint64_t)per_seq, kRows)) return cudaErrorUnknown;
         }
         a.u0[i] = b * per_seq_all + first;
         a.N[i] = N;
@@ -588,10 +587,10 @@ cudaError_t launch_res_d(const DeviceProblem& p, const WindowHostInfo& h, cudaSt
 
 }  // namespace
 
-// Whether the single-read kernel takes this problem: 32 window rows, every sequence within 16 CTAs x 16 tiles, and a
+// Whether the single-read kernel takes this problem: at most 32 window rows, every sequence within 16 CTAs x 16 tiles, and a
 // device that co-schedules enough clusters of every size in use to fill three quarters of its SMs.
 bool window_res_supported(const DeviceProblem& p, const WindowHostInfo& h) {
-  if (p.rows != kRows || p.L > kRows || h.lse != nullptr) return false;
+  if (p.rows > kRows || h.lse != nullptr) return false;
   int dev = 0, n_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);

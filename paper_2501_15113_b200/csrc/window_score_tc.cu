@@ -1,5 +1,5 @@
 // Observation-window scores (Eq. 12, Eq. 13) on the 5th-generation tensor cores,
-// for bf16 inputs with G*L in {32, 64, 128} window rows.
+// for bf16 inputs.  Kernels for 32, 64 and 128 window rows (G*L); other windows are filled up with zero rows.
 //
 // The contraction S = Q_win K^T is 2*G*L*d flop per key (32-128 flop per byte of
 // K): too much for the CUDA cores next to an HBM-rate K stream, little for
@@ -65,6 +65,18 @@ bool make_tensor_map_2d(CUtensorMap* map, const void* base, int d, uint64_t rows
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool make_tensor_map_units(CUtensorMap* map, const void* base, int d, int rows, uint64_t units, int box_rows) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  const cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)rows, (cuuint64_t)units};
+  const cuuint64_t strides[2] = {(cuuint64_t)d * 2, (cuuint64_t)rows * d * 2};
+  const cuuint32_t box[3] = {64u, (cuuint32_t)box_rows, 1u};
+  const cuuint32_t estr[3] = {1u, 1u, 1u};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 namespace {
 
 constexpr int kTile = 128;          // keys per tile (UMMA M in pass 2, key sub-tiles in pass 1)
@@ -80,7 +92,7 @@ constexpr uint32_t kTmemCols = 512; // four accumulators of up to 128 columns
 constexpr int kMaxSeq = 8;
 struct TcMaps {
   CUtensorMap k[kMaxSeq];   // [units * N][d] of each sequence
-  CUtensorMap q[kMaxSeq];   // [units * rows][d]
+  CUtensorMap q[kMaxSeq];   // [units][window rows][d]
 };
 struct TcArgs {
   int pass;                 // 1 = row statistics, 2 = scores
@@ -107,10 +119,10 @@ __device__ __forceinline__ void fold_stat(float2& a, const float2 b) {
 struct Item {
   int seq, lu, ch;
   int N;                    // keys of the unit
-  int krow0, qrow0;         // first row of the unit in the K and Q tensor maps
+  int krow0;                // first row of the unit in the K tensor map
   bool valid;
 };
-__device__ __forceinline__ Item decode_item(const TcArgs& a, int k, int rows) {
+__device__ __forceinline__ Item decode_item(const TcArgs& a, int k) {
   Item it;
   const int i = (int)blockIdx.x + k * (int)gridDim.x;
   it.valid = i < a.item_off[a.n_seq];
@@ -124,7 +136,6 @@ __device__ __forceinline__ Item decode_item(const TcArgs& a, int k, int rows) {
   const int N = a.N[it.seq];
   it.N = N;
   it.krow0 = it.lu * N;
-  it.qrow0 = it.lu * rows;
   return it;
 }
 
@@ -164,7 +175,11 @@ enum : int {
   B_FULL = 0, B_EMPTY = 8, B_QFULL = 16, B_QEMPTY = 18, B_TFULL = 20, B_TEMPTY = 24, B_COUNT = 28
 };
 
-template <int D>
+// ROWS (32, 64 or 128: columns of an accumulator) is a template argument also for the sake of registers: with 128 rows the
+// gather of another chunk of layers shares the SMs with this kernel, and how many of its blocks (6144 registers) fit beside
+// a CTA is decided here.  One kernel for all row counts took 168 registers a thread, which leaves room for one gather block:
+// 7.0 -> 7.5 ms for 32 layers of 131072 keys; this one takes 128, room for three.
+template <int D, int ROWS>
 __global__ void __launch_bounds__(kThreads, 1)
 window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __grid_constant__ TcArgs a,
                  TcLayout lay) {
@@ -183,7 +198,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
   volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int rows = p.rows;                  // 32, 64 or 128
+  constexpr int rows = ROWS;                // the window's own rows: p.rows
   const int L = p.L;
   const int S = lay.stages;
   const uint32_t bar0 = smem_u32(bars);
@@ -220,7 +235,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
       uint32_t phase = 0, qphase[2] = {0, 0};
       bool ok = true;
       for (int k = 0; k < a.steps && ok; ++k) {
-        const Item it = decode_item(a, k, rows);
+        const Item it = decode_item(a, k);
         if (!it.valid) continue;
         const int N = it.N;
         const int key0 = it.ch * a.chunk_keys;
@@ -230,8 +245,8 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
         if (elect_one()) {
           mbar_expect_tx(BAR(B_QFULL + qb), (uint32_t)lay.q_block_bytes);
           for (int kb = 0; kb < KB; ++kb)
-            tma_load_2d(smem_u32(sQ + (size_t)qb * lay.q_block_bytes + (size_t)kb * rows * 128), &maps.q[it.seq],
-                        kb * 64, it.qrow0, BAR(B_QFULL + qb));
+            tma_load_3d(smem_u32(sQ + (size_t)qb * lay.q_block_bytes + (size_t)kb * rows * 128), &maps.q[it.seq],
+                        kb * 64, 0, it.lu, BAR(B_QFULL + qb));
         }
         __syncwarp();
         qphase[qb] ^= 1;
@@ -276,7 +291,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
       const uint64_t desc_hi = smem_desc(0);    // everything but the start address
       bool ok = true;
       for (int k = 0; k < a.steps && ok; ++k) {
-        const Item it = decode_item(a, k, rows);
+        const Item it = decode_item(a, k);
         if (!it.valid) continue;
         const int N = it.N;
         const int key0 = it.ch * a.chunk_keys;
@@ -325,7 +340,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
     const int ew = warp < 6 ? warp - 2 : warp - 3;  // 0..7
     const int grp = ew >> 2;
     const int quad = warp & 3;                      // TMEM lane quadrant this warp may read
-    float* myStat = reinterpret_cast<float*>(sStat) + ew * rows;
+    float* myStat = reinterpret_cast<float*>(sStat) + ew * 2 * rows;
     float* myT = sTrans + ew * (32 * 33);
     int n = 0;
     bool ok = true;
@@ -334,15 +349,23 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
     const float* stat_g = p.stat;
     float pre[4];
     auto fetch_stats = [&](int k) {
-      const Item nx = decode_item(a, k, rows);
+      const Item nx = decode_item(a, k);
+      const float* st = stat_g + (size_t)(a.u0[nx.seq] + nx.lu) * (2 * p.rows_pad);
+      if (rows == 32) {
+        // the row's maximum and the weight 1 / (sum rows): with few rows to average over, the rounding of one offset that
+        // holds both would show in the result
+        const bool there = nx.valid && lane < p.rows;
+        pre[0] = there ? st[lane] : 0.f;
+        pre[1] = there ? st[p.rows_pad + lane] : 0.f;
+        return;
+      }
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        pre[q] = (nx.valid && q * 32 + lane < rows) ? stat_g[(size_t)(a.u0[nx.seq] + nx.lu) * (2 * p.rows_pad) + q * 32 + lane]
-                                                    : 0.f;
+        pre[q] = (nx.valid && q * 32 + lane < p.rows) ? st[q * 32 + lane] : INFINITY;   // a row that is not there weighs nothing
     };
     if (a.pass == 2) fetch_stats(0);
     for (int k = 0; k < a.steps && ok; ++k) {
-      const Item it = decode_item(a, k, rows);
+      const Item it = decode_item(a, k);
       if (!it.valid) continue;
       const int u = a.u0[it.seq] + it.lu;
       const int N = it.N;
@@ -356,7 +379,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
         __syncwarp();                       // the previous item's readers of myStat are done
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-          if (q * 32 + lane < rows) myStat[q * 32 + lane] = pre[q];
+          if (q * 32 + lane < (rows == 32 ? 64 : rows)) myStat[q * 32 + lane] = pre[q];
         __syncwarp();
         fetch_stats(k + 1);                 // in flight while this item's tiles are worked on
       }
@@ -376,20 +399,21 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
         float2* base = reinterpret_cast<float2*>(p.stat_part) + (size_t)u * p.chunks_max * p.rows_pad;
         const int tile0 = key0 / kTile;
         if (rows == 128) {
+          const bool there = quad * 32 + lane < p.rows;
           const float2 mine = make_float2(m_run[0] * scale2, z_run[0]);
           if (a.fine) {
-            base[(size_t)(((tile0 >> 2) + sub) * 2 + par) * p.rows_pad + quad * 32 + lane] = mine;
+            if (there) base[(size_t)(((tile0 >> 2) + sub) * 2 + par) * p.rows_pad + quad * 32 + lane] = mine;
           } else {
             fold_stat(group, mine);
             if ((sub & 3) == 3 || sub == ((ntiles + 3) >> 2) - 1) {
-              base[(size_t)(((tile0 >> 4) + (sub >> 2)) * 2 + par) * p.rows_pad + quad * 32 + lane] = group;
+              if (there) base[(size_t)(((tile0 >> 4) + (sub >> 2)) * 2 + par) * p.rows_pad + quad * 32 + lane] = group;
               group = make_float2(-INFINITY, 0.f);
             }
           }
         } else {
 #pragma unroll
           for (int rg = 0; rg < 4; ++rg)
-            if (rg * 32 < rows)
+            if (rg * 32 + lane < p.rows)
               base[(size_t)(((tile0 >> 4) + sub) * kTcParts + par * 4 + quad) * p.rows_pad + rg * 32 + lane] =
                   make_float2(m_run[rg] * scale2, z_run[rg]);
         }
@@ -505,6 +529,33 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
                 cs[3] += ex2(fmaf(__uint_as_float(r[c + 3]), scale2, -off.w));
               }
             }
+          } else if (rows == 32) {
+            uint32_t r[32];
+            tc_ld32(taddr, r);
+            tc_wait_ld();
+            const float4* mx4 = reinterpret_cast<const float4*>(myStat);
+            const float4* wt4 = reinterpret_cast<const float4*>(myStat + 32);
+            uint32_t vm = 0xffffffffu;              // bit c: window row c sees this thread's key
+            if (tail) {
+              const int need = j < N ? j - (N - L) : L;        // the residue c % L the row must reach (L: none does)
+              int res = 0;
+              vm = 0;
+#pragma unroll
+              for (int c = 0; c < 32; ++c) {
+                vm |= (uint32_t)(need <= res) << c;
+                res = (res + 1 == L) ? 0 : res + 1;
+              }
+            }
+#pragma unroll
+            for (int c = 0; c < 32; c += 4) {
+              const float4 mx = mx4[c >> 2], w = wt4[c >> 2];
+              const float m4[4] = {mx.x, mx.y, mx.z, mx.w}, w4[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const float e = ex2(fmaf(__uint_as_float(r[c + i]), scale2, -m4[i]));
+                cs[i] = fmaf((vm >> (c + i)) & 1u ? e : 0.f, w4[i], cs[i]);
+              }
+            }
           } else
           for (int c0 = 0; c0 < rows; c0 += 32) {
             uint32_t r[32];
@@ -563,20 +614,22 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
   if (tid == 0 && *s_abort) set_status(p.status, TASKKV_ETIMEOUT);
 }
 
-// Folds the partial statistics of one unit -> one offset per row.  One block per unit; 1024 / rows threads share a row,
-// each taking every (1024 / rows)-th slot in order with four loads ahead of the dependent updates, and their results are
+// Folds the partial statistics of one unit -> one offset per row.  One block per unit; 8 to 32 threads share a row, each
+// taking every 8th to 32nd slot in order with four loads ahead of the dependent updates, and their results are
 // joined in order: the outcome depends on the unit's own length alone.
 __global__ void __launch_bounds__(1024) window_tc_reduce_kernel(DeviceProblem p, UnitRange ur, int fine) {
   __shared__ float2 tmp[1024];
   const int u = ur.unit(blockIdx.x);
   const int N = p.unit_N[u];
-  const int slots = (N + 16 * kTile - 1) / (16 * kTile) * (p.rows == 128 ? 2 : kTcParts);
-  const int rows = p.rows, P = 1024 / rows;
+  const int rows = tc_rows(p.rows), P = 1024 / rows;
+  const int slots = (N + 16 * kTile - 1) / (16 * kTile) * (rows == 128 ? 2 : kTcParts);
   const int row = threadIdx.x % rows, part = threadIdx.x / rows;
   const float2* src = reinterpret_cast<const float2*>(p.stat_part) + (size_t)u * p.chunks_max * p.rows_pad + row;
   float2 acc = make_float2(-INFINITY, 0.f);
+  const bool there = row < p.rows;
   grid_dependency_wait();
-  if (fine) {
+  if (!there) {
+  } else if (fine) {
     // 128 rows: slot (group, parity) is folded from up to four stored parts
     const int parts = (N + 4 * kTile - 1) / (4 * kTile);
     for (int c = part; c < slots; c += P) {
@@ -602,10 +655,16 @@ __global__ void __launch_bounds__(1024) window_tc_reduce_kernel(DeviceProblem p,
   }
   tmp[threadIdx.x] = acc;
   __syncthreads();
-  if (part == 0) {
+  if (part == 0 && there) {
     for (int q = 1; q < P; ++q) fold_stat(acc, tmp[q * rows + row]);
-    // one offset per row: score * scale - (max + log2(sum) + log2(rows)) is log2 of the row's share of C
-    p.stat[(size_t)u * (2 * p.rows_pad) + row] = acc.y > 0.f ? acc.x + log2f(acc.y) + log2f((float)rows) : INFINITY;
+    float* st = p.stat + (size_t)u * (2 * p.rows_pad);
+    if (rows == 32) {
+      st[row] = acc.y > 0.f ? acc.x : 0.f;
+      st[p.rows_pad + row] = acc.y > 0.f ? 1.0f / (acc.y * (float)p.rows) : 0.f;
+    } else {
+      // one offset per row: score * scale - (max + log2(sum) + log2(rows)) is log2 of the row's share of C
+      st[row] = acc.y > 0.f ? acc.x + log2f(acc.y) + log2f((float)p.rows) : INFINITY;
+    }
   }
 }
 
@@ -620,7 +679,7 @@ inline int pick_chunk(int64_t units_times_keys, int n_sm, int least) {
   return chunk;
 }
 
-template <int D>
+template <int D, int ROWS>
 cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStream_t s, int layer0, int n_layers) {
   static int n_sm = 0;
   if (n_sm == 0) {
@@ -629,10 +688,11 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (n_sm <= 0) n_sm = 148;
   }
-  const TcLayout lay = make_layout(D, p.rows);
+  constexpr int rows = ROWS;
+  const TcLayout lay = make_layout(D, rows);
   if (lay.stages < 2) return cudaErrorInvalidValue;
   const int smem = lay.total;
-  cudaError_t e = cudaFuncSetAttribute(window_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(window_tc_kernel<D, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const int per_seq_all = p.R * p.n_kv;
   const int first = layer0 * p.n_kv;               // the launch covers units [first, first + per_seq) of every sequence
@@ -658,8 +718,7 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
         const char* kb = static_cast<const char*>(h.k[b]) + (size_t)skip * (size_t)N * D * sizeof(__nv_bfloat16);
         const char* qb = static_cast<const char*>(h.q[b]) + (size_t)skip * p.rows * D * sizeof(__nv_bfloat16);
         if (!make_tensor_map_2d(&maps.k[i], kb, D, (uint64_t)per_seq * (uint64_t)N, kTile)) return cudaErrorUnknown;
-        if (!make_tensor_map_2d(&maps.q[i], qb, D, (uint64_t)per_seq * (uint64_t)p.rows, p.rows))
-          return cudaErrorUnknown;
+        if (!make_tensor_map_units(&maps.q[i], qb, D, p.rows, (uint64_t)per_seq, rows)) return cudaErrorUnknown;
       }
       a.u0[i] = b * per_seq_all + first;
       a.N[i] = N;
@@ -667,7 +726,7 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
     auto launch_pass = [&](int pass, int least) -> cudaError_t {
       a.pass = pass;
       a.chunk_keys = pick_chunk(keys, n_sm, least);
-      a.fine = pass == 1 && p.rows == 128 && a.chunk_keys < 16 * kTile ? 1 : 0;
+      a.fine = pass == 1 && rows == 128 && a.chunk_keys < 16 * kTile ? 1 : 0;
       a.item_off[0] = 0;
       for (int i = 0; i < kMaxSeq; ++i) {
         a.chunks[i] = (a.N[i] + a.chunk_keys - 1) / a.chunk_keys;
@@ -676,7 +735,7 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
       const int items = a.item_off[nb], grid = items < n_sm ? items : n_sm;
       a.steps = (items + grid - 1) / grid;
       LaunchScope ls(K_WINDOW_TC, s);
-      return launch_dependent_smem(window_tc_kernel<D>, (unsigned)grid, kThreads, (size_t)smem, s, maps, p, a, lay);
+      return launch_dependent_smem(window_tc_kernel<D, ROWS>, (unsigned)grid, kThreads, (size_t)smem, s, maps, p, a, lay);
     };
     if (h.lse) {
       // the caller already has the rows' normalisers: no pass 1
@@ -687,7 +746,7 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
         if (e != cudaSuccess) return e;
       }
     } else {
-      e = launch_pass(1, p.rows == 128 ? 4 * kTile : kTcChunk);
+      e = launch_pass(1, rows == 128 ? 4 * kTile : kTcChunk);
       if (e != cudaSuccess) return e;
       LaunchScope ls(K_WINDOW_REDUCE, s);
       const UnitRange ur{b0 * per_seq_all + first, per_seq, per_seq_all, nb * per_seq};
@@ -705,8 +764,7 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
 }  // namespace
 
 bool window_tc_supported(const DeviceProblem& p, int dtype) {
-  return dtype == TASKKV_BF16 && (p.rows == 32 || p.rows == 64 || p.rows == 128) && p.L <= p.rows &&
-         encode_fn() != nullptr;
+  return dtype == TASKKV_BF16 && p.rows <= 128 && encode_fn() != nullptr;
 }
 
 cudaError_t launch_window_scores_tc(const DeviceProblem& p, const WindowHostInfo& h, cudaStream_t s, int layer0,
@@ -714,7 +772,11 @@ cudaError_t launch_window_scores_tc(const DeviceProblem& p, const WindowHostInfo
   if (n_layers < 0) { layer0 = 0; n_layers = p.R; }
   // 32 window rows and sequences short enough for a unit's scores to stay in tensor memory: K is read once
   if (window_res_supported(p, h)) return launch_window_scores_res(p, h, s, layer0, n_layers);
-  return p.d == 64 ? launch_tc_d<64>(p, h, s, layer0, n_layers) : launch_tc_d<128>(p, h, s, layer0, n_layers);
+  switch (tc_rows(p.rows)) {
+    case 32: return p.d == 64 ? launch_tc_d<64, 32>(p, h, s, layer0, n_layers) : launch_tc_d<128, 32>(p, h, s, layer0, n_layers);
+    case 64: return p.d == 64 ? launch_tc_d<64, 64>(p, h, s, layer0, n_layers) : launch_tc_d<128, 64>(p, h, s, layer0, n_layers);
+    default: return p.d == 64 ? launch_tc_d<64, 128>(p, h, s, layer0, n_layers) : launch_tc_d<128, 128>(p, h, s, layer0, n_layers);
+  }
 }
 
 }  // namespace taskkv

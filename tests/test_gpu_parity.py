@@ -220,13 +220,15 @@ def test_cluster_decode_equals_the_two_kernels_bit_for_bit(kw, page_rows):
             p.close()
 
 
-# (query heads per KV head, window) -> 8, 16, 24, 48, 96 and 128 window rows; key counts around the 128-key tile, the
+# (query heads per KV head, window) -> 8 to 128 window rows: on the CUDA cores (fp32), or as the next larger tensor-core
+# tile with zero rows (bf16; up to 32768 keys the single-read kernel takes up to 32 rows); key counts around the 128-key tile, the
 # 256-key chunk and the 8192 keys up to which pass 2 folds the chunks' statistics itself.  (Four KV heads: two are always
 # equally far from their mean, so which of them is promoted would be a tie.)
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("G,L,d,N", [(1, 8, 64, 129), (2, 8, 128, 255), (1, 24, 64, 257), (2, 24, 128, 511),
-                                     (4, 24, 64, 8192), (4, 24, 128, 8193), (8, 16, 64, 384), (8, 16, 128, 9001)])
-def test_cuda_core_window_scores(G, L, d, N, dtype):
+                                     (4, 24, 64, 8192), (4, 24, 128, 8193), (8, 16, 64, 384), (8, 16, 128, 9001),
+                                     (1, 16, 64, 32769), (2, 16, 128, 33000)])
+def test_windows_of_every_size(G, L, d, N, dtype):
     run_workload(small("winrows", n=4 * G, n_kv=4, d=d, N=N, L=L, s1=4, s2=32, k=40, dtype=dtype, nh=0, t=64, steps=1))
 
 
@@ -1098,7 +1100,9 @@ def test_random_shapes(seed):
     dict(n=4, n_kv=4, d=128, N=2341, L=32, s1=4, s2=64, k=100, dtype="bf16"),            # tensor-core path, 32 rows
     dict(n=8, n_kv=2, d=128, N=0, L=32, s1=4, s2=64, k=150, dtype="bf16", R=2, seq_lens=[3000, 1777], nh=1),  # 128 rows
     dict(n=4, n_kv=4, d=64, N=1500, L=16, s1=4, s2=32, k=77, dtype="f32"),               # CUDA-core path
-], ids=["tc32", "tc128_ragged", "f32"])
+    dict(n=4, n_kv=4, d=64, N=1500, L=9, s1=4, s2=32, k=77, dtype="bf16"),               # 9 rows in a tile of 32
+    dict(n=8, n_kv=4, d=128, N=1500, L=24, s1=4, s2=32, k=77, dtype="bf16"),             # 48 rows in a tile of 64
+], ids=["tc32", "tc128_ragged", "f32", "tc9", "tc48"])
 def test_compress_with_supplied_window_lse(case):
     """With the window rows' log-sum-exp handed in (here: the oracle's, rounded to fp32) pass 1 is skipped; scores,
     selections, classes, rows and decode outputs must match the oracle exactly as in the full computation."""
