@@ -146,7 +146,7 @@ taskkv_status taskkv_plan(const taskkv_params* p, taskkv_plan_info* out);
  * Streams: all work is ordered after what `stream` holds at the call and is
  * complete, for every later operation on `stream`, when the call's last kernel is.
  * For large bf16 problems the steps of different chunks of layers overlap on
- * streams the library owns (with 32 window rows the selection of one chunk
+ * streams the library owns (with up to 32 window rows the selection of one chunk
  * beside the window scores of the next; with more window rows the gather of
  * one chunk beside window scores and selection of the next; two streams per
  * device, created by the first such call: make that call before capturing
