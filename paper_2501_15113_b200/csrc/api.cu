@@ -39,7 +39,7 @@ struct HostPlan {
   size_t o_ptab = 0;
   // byte offsets inside the cache memory
   size_t o_unit_N, o_unit_mid, o_nhet, o_c_off, o_seg_base, o_gbase, o_dbase, o_qp, o_kp, o_vp, meta_bytes;
-  size_t o_status, o_len, o_cap, o_seg, o_cls, o_dist, o_sem, o_idx, o_goff, o_doff, o_step, o_pacc, o_pml, o_kpool,
+  size_t o_status, o_len, o_cap, o_seg, o_cls, o_dist, o_sem, o_idx, o_goff, o_doff, o_ditem, o_step, o_pacc, o_pml, o_kpool,
       o_vpool;
   // inside the workspace
   size_t w_C, w_pool, w_spart, w_stat, w_topt;
@@ -236,6 +236,7 @@ taskkv_status make_plan(const taskkv_params* p, HostPlan& hp, int32_t page_rows 
   hp.o_idx = take((size_t)U * hp.idx_stride * 4);
   hp.o_goff = take((U + 1) * 4);
   hp.o_doff = take((U + 1) * 4);
+  hp.o_ditem = take((size_t)ditems * 8);
   hp.o_step = take(U * 4);
   hp.o_pacc = take((size_t)ditems * G * d * 4);
   hp.o_pml = take((size_t)ditems * G * 2 * 4);
@@ -549,6 +550,8 @@ void fill_device_problem(taskkv_cache* c) {
   d.view_l0 = 0;
   d.view_nl = p.n_layers;
   d.view_U = (int32_t)hp.info.n_units;
+  d.item0 = 0;
+  d.item1 = (int32_t)hp.info.max_decode_items;
   d.max_mid = 0;
   for (int32_t m : hp.mid) d.max_mid = m > d.max_mid ? m : d.max_mid;
   if (d.max_mid > hp.max_N) d.max_mid = hp.max_N;
@@ -586,6 +589,7 @@ void fill_device_problem(taskkv_cache* c) {
   d.idx = reinterpret_cast<int32_t*>(cm + hp.o_idx);
   d.gather_off = reinterpret_cast<int32_t*>(cm + hp.o_goff);
   d.dec_off = reinterpret_cast<int32_t*>(cm + hp.o_doff);
+  d.dec_item = reinterpret_cast<int2*>(cm + hp.o_ditem);
   d.step_cnt = reinterpret_cast<int32_t*>(cm + hp.o_step);
   d.part_acc = reinterpret_cast<float*>(cm + hp.o_pacc);
   d.part_ml = reinterpret_cast<float*>(cm + hp.o_pml);
@@ -1133,6 +1137,8 @@ bool layer_view(const taskkv_cache* c, int32_t layer_begin, int32_t layer_count,
   int64_t items = 0;
   for (int32_t r = layer_begin; r < layer_begin + layer_count; ++r) items += c->hp.layer_items[(size_t)r];
   out->max_items = items;
+  out->item0 = c->hp.dec_base[(size_t)layer_begin * c->prm.batch];
+  out->item1 = c->hp.dec_base[(size_t)(layer_begin + layer_count) * c->prm.batch];
   return true;
 }
 }  // namespace

@@ -53,6 +53,7 @@ struct DeviceProblem {
   // Append and decode address a range of layers of every sequence ("view"): view unit v = (b * view_nl + r') *
   // n_kv + h stands for layer view_l0 + r'.  q, k_new, v_new, out and `lengths` are indexed by view unit.
   int32_t view_l0, view_nl, view_U;
+  int32_t item0, item1;       // decode work items of the view
   int32_t max_new;
   int32_t dec_chunk;    // rows of one split-K decode item of this cache: a power of two, log2 in dec_shift
   int32_t dec_shift;
@@ -94,6 +95,8 @@ struct DeviceProblem {
   int32_t* idx;               // [U][idx_stride]
   int32_t* gather_off;        // [U+1] gather work items, indexed layer-major like dec_off
   int32_t* dec_off;           // [U+1] decode work items, indexed by w = (r * B + b) * n_kv + h
+  int2* dec_item;             // [items] decode work item -> (unit index w of dec_off plus one, first row); (0, 0): the item's
+                              // layer has not been compressed
   int32_t* step_cnt;          // [U] combine blocks of a unit that finished the current fused step (0 between calls)
   void* k_pool;
   void* v_pool;
@@ -299,18 +302,8 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-// Largest index i in [0, n) with off[i] <= x, for a non-decreasing off[0..n]
-// with off[0] <= x < off[n].
-__device__ __forceinline__ int upper_unit(const int32_t* off, int n, int x) {
-  int lo = 0, hi = n;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (off[mid] <= x) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-
-// The same by all 32 lanes of a converged warp: 32 probes per round, so 1024 entries take two dependent loads instead
+// Largest index i in [0, n) with off[i] <= x, for a non-decreasing off[0..n] with off[0] <= x < off[n], by all 32 lanes of
+// a converged warp: 32 probes per round, so 1024 entries take two dependent loads instead
 // of ten.  Every lane returns the index.
 __device__ __forceinline__ int upper_unit_warp(const int32_t* off, int n, int x, int lane) {
   int lo = 0, hi = n;                                   // off[lo] <= x < off[hi]

@@ -481,20 +481,15 @@ decode_attn_kernel(DeviceProblem p, const T* __restrict__ q, const int32_t* __re
   using It = Item<T, D, G, PAGED>;
   constexpr int ROW_BYTES = It::ROW_BYTES;
   __shared__ typename It::Smem sm;
-  __shared__ int s_unit, s_rbeg, s_word;
+  __shared__ int s_word;
   __shared__ int s_direct;     // >= 0: the item is its unit's only one, the output goes to view unit s_direct
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // the view's layers are a contiguous range of layer-major indices, hence of work items
-  const int w0 = p.view_l0 * lm_batch(p) * p.n_kv;
-  // (from the host's table of block starts: it does not depend on which layers have been compressed so far)
-  const int item0 = p.dec_base[p.view_l0 * lm_batch(p)], item1 = p.dec_base[(p.view_l0 + p.view_nl) * lm_batch(p)];
-
+  const int tid = threadIdx.x, lane = tid & 31;
   // The table of work items is written when the cache is planned, not by the kernel before this one in the
-  // stream: the block's first item is looked up before the wait, under that kernel's tail.
-  int wi_first = 0;
-  if (warp == 0 && item0 + (int)blockIdx.x < item1)
-    wi_first = w0 + upper_unit_warp(p.dec_off + w0, p.view_U, item0 + (int)blockIdx.x, lane);
+  // stream: the block's first entry is read before the wait, under that kernel's tail.  (With a search of the units'
+  // offsets in its place 384 units of 1500 to 6000 rows took 60.9 us instead of 59.4, 1024 units of 32768 rows 473 and 470.)
+  const int item_first = p.item0 + (int)blockIdx.x;
+  const int2 at_first = item_first < p.item1 ? p.dec_item[item_first] : make_int2(0, 0);
   // `early` (set by the host when the kernel before this one in the stream cannot be one that writes these units'
   // lengths or page tables: see launch_decode): the first item's unit data is read before the wait as well, and the
   // wait comes just before the block first touches what the caller's kernels produce (q, the new token's rows) or
@@ -508,18 +503,11 @@ decode_attn_kernel(DeviceProblem p, const T* __restrict__ q, const int32_t* __re
     }
   };
   if (!early) wait_once();
-  for (int item = item0 + blockIdx.x; item < item1; item += gridDim.x) {
-    __syncthreads();
-    if (warp == 0) {
-      const int wi = item == item0 + (int)blockIdx.x ? wi_first
-                                                     : w0 + upper_unit_warp(p.dec_off + w0, p.view_U, item, lane);
-      if (lane == 0) {
-        s_unit = wi;
-        s_rbeg = (item - p.dec_off[wi]) * p.dec_chunk;
-      }
-    }
-    __syncthreads();
-    const int w = s_unit;
+  for (int item = item_first; item < p.item1; item += gridDim.x) {
+    __syncthreads();                                // previous item's shared state consumed
+    const int2 at = item == item_first ? at_first : p.dec_item[item];
+    if (at.x == 0) continue;                        // an item of a layer that is not in yet
+    const int w = at.x - 1, rbeg = at.y;
     const LmUnit lu = lm_unit(p, w);
     const int vu = lu.v;                            // view unit: index into q and lengths
     const int u = lu.u;                             // unit: index into the cache
@@ -529,7 +517,6 @@ decode_attn_kernel(DeviceProblem p, const T* __restrict__ q, const int32_t* __re
     const int new_r = (k_new != nullptr && len < p.cap[u]) ? len : -1;
     if (new_r >= 0) ++len;
     if (lengths) len = min(max(lengths[vu], 0), len);
-    const int rbeg = s_rbeg;
     if (rbeg >= len) continue;                      // an item of the reserve beyond the segment's length
     const int rend = min(len, rbeg + p.dec_chunk);
     if (tid == 0) s_direct = len <= p.dec_chunk ? vu : -1;     // read back after the row loop (no register held)

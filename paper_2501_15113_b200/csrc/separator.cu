@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(128) separator_plan_kernel(DeviceProblem p, in
   __syncthreads();
 
   // ---- plan of this block's units (the problem's own heads)
-  __shared__ int s_cap[TASKKV_MAX_KV_HEADS], s_git[TASKKV_MAX_KV_HEADS], s_dit[TASKKV_MAX_KV_HEADS];
+  __shared__ int s_cap[TASKKV_MAX_KV_HEADS], s_git[TASKKV_MAX_KV_HEADS], s_dit[TASKKV_MAX_KV_HEADS], s_dat[TASKKV_MAX_KV_HEADS];
   const int B = lm_batch(p);
   const int lm_block = r_lay * B + b_seq;
   int len = 0;
@@ -108,6 +108,7 @@ __global__ void __launch_bounds__(128) separator_plan_kernel(DeviceProblem p, in
     p.seg_off[u] = p.seg_base[br] + rows_before;
     p.gather_off[w] = p.gather_base[lm_block] + git_before;
     p.dec_off[w] = p.dec_base[lm_block] + dit_before;
+    s_dat[tid] = p.dec_base[lm_block] + dit_before;
     if (tid == nl - 1) {
       // The block must end exactly where the host placed the next one.  (A shard cannot know how many of the layer's
       // full-cache heads it will hold, so its blocks are sized for the most it can get and may end early: rows and
@@ -127,6 +128,16 @@ __global__ void __launch_bounds__(128) separator_plan_kernel(DeviceProblem p, in
         p.dec_off[p.U] = p.dec_base[lm_block + 1];
       }
     }
+  }
+  // the items' own table, so that an attention block finds its unit with one load; what a shard's block leaves unused
+  // before the next block's first item points beyond every segment
+  __syncthreads();
+  {
+    const int end = p.dec_base[lm_block + 1], last = s_dat[nl - 1] + s_dit[nl - 1];
+    for (int h = 0; h < nl; ++h)
+      for (int i = tid; i < s_dit[h] && s_dat[h] + i < end; i += 128)
+        p.dec_item[s_dat[h] + i] = make_int2(lm_block * nl + h + 1, i * p.dec_chunk);
+    for (int i = last + tid; i < end; i += 128) p.dec_item[i] = make_int2(lm_block * nl + nl, 0x7fffffff);
   }
   // ---- paged cache: the block takes the pages of its units' retained rows off the pool in one step (growth takes
   // pages later, one at a time) and deals them out in unit order

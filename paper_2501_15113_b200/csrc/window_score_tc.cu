@@ -357,11 +357,11 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
         const bool there = nx.valid && lane < p.rows;
         pre[0] = there ? st[lane] : 0.f;
         pre[1] = there ? st[p.rows_pad + lane] : 0.f;
-        return;
-      }
+      } else {
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        pre[q] = (nx.valid && q * 32 + lane < p.rows) ? st[q * 32 + lane] : INFINITY;   // a row that is not there weighs nothing
+        for (int q = 0; q < 4; ++q)               // a row that is not there weighs nothing
+          pre[q] = (nx.valid && q * 32 + lane < p.rows) ? st[q * 32 + lane] : INFINITY;
+      }
     };
     if (a.pass == 2) fetch_stats(0);
     for (int k = 0; k < a.steps && ok; ++k) {
