@@ -16,6 +16,11 @@ namespace taskkv {
 
 namespace {
 
+// A distance as it is ranked: non-finite scores (an infinite key element) make a layer's vectors and distances NaN,
+// which compares false with everything; all heads would then be the farthest and the nearest at once, keep every row, and
+// the layer's segments would not fit where the host placed them.  NaN ranks as the farthest instead.
+__device__ __forceinline__ double rank_of(double dist) { return dist == dist ? dist : (double)INFINITY; }
+
 __global__ void __launch_bounds__(128) separator_plan_kernel(DeviceProblem p, int layer0, int n_layers) {
   grid_dependency_wait();
   __shared__ double center[128];
@@ -56,9 +61,12 @@ __global__ void __launch_bounds__(128) separator_plan_kernel(DeviceProblem p, in
 
   if (tid < n) {
     // rank among all heads, farthest first, lower index first on equal distance
-    const double me = dist[tid];
+    const double me = rank_of(dist[tid]);
     int rank = 0;
-    for (int h = 0; h < n; ++h) rank += (dist[h] > me) || (dist[h] == me && h < tid);
+    for (int h = 0; h < n; ++h) {
+      const double other = rank_of(dist[h]);
+      rank += (other > me) || (other == me && h < tid);
+    }
     cls[tid] = rank < f ? TASKKV_CLASS_HETERO : TASKKV_CLASS_NON_HETERO;
   }
   __syncthreads();
@@ -66,10 +74,12 @@ __global__ void __launch_bounds__(128) separator_plan_kernel(DeviceProblem p, in
   if (tid < n) {
     c = cls[tid];
     if (promote && c == TASKKV_CLASS_NON_HETERO) {
-      const double me = dist[tid];
+      const double me = rank_of(dist[tid]);
       int nearer = 0;
-      for (int h = 0; h < n; ++h)
-        if (cls[h] == TASKKV_CLASS_NON_HETERO) nearer += (dist[h] < me) || (dist[h] == me && h < tid);
+      for (int h = 0; h < n; ++h) {
+        const double other = rank_of(dist[h]);
+        if (cls[h] == TASKKV_CLASS_NON_HETERO) nearer += (other < me) || (other == me && h < tid);
+      }
       if (nearer == 0) c = TASKKV_CLASS_CENTER;
     }
     if (tid >= h0 && tid < h0 + nl) {      // this problem's own heads

@@ -248,6 +248,46 @@ def test_every_head_heterogeneous_is_full_attention():
     assert err < 2e-2
 
 
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), -float("inf")])
+@pytest.mark.parametrize("page_rows", [0, 64])
+def test_non_finite_values_leave_the_plan_as_it_is(value, page_rows):
+    """A semantic vector that is not finite makes its layer's distances NaN or infinite (the center is the mean).  The heads are
+    still ranked one after the other: as many keep everything as the host planned for, and the other layer sees nothing."""
+    tk = _tk()
+    wl = small("nonfinite", n=8, n_kv=8, d=64, N=700, L=16, s1=4, s2=32, k=40, dtype="f32", R=2, nh=2)
+    qs, ks, vs = W.materialize(wl, DEV)
+    params = tk.params_from_workload(wl, max_new_tokens=3)
+
+    def compress():
+        if not page_rows:
+            return tk.taskkv_compress_ex(params, qs, ks, vs), None
+        pool = tk.Pool(page_rows, int(tk.taskkv_plan_paged(params, page_rows)[1]), wl.head_dim, wl.dtype, DEV)
+        return tk.taskkv_compress_paged(params, qs, ks, vs, pool), pool
+
+    def facts(cache):
+        return (cache.classes().reshape(2, 8), cache.lengths().reshape(2, 8), cache.query(tk.Q_DIST).reshape(2, 8))
+
+    cache, pool = compress()
+    cls0, len0, dist0 = facts(cache)
+    cache.close()
+    if pool:
+        pool.close()
+    vs[0][0, 5] = value                         # every V row of one head of layer 0
+    cache, pool = compress()
+    cls, lens, dist = facts(cache)
+    assert cache.status() == 0
+    assert not np.isfinite(dist[0]).any() and np.array_equal(dist[1], dist0[1])
+    assert sorted(cls[0].tolist()) == sorted(cls0[0].tolist()) and np.array_equal(cls[1], cls0[1])
+    assert sorted(lens[0].tolist()) == sorted(len0[0].tolist()) and np.array_equal(lens[1], len0[1])
+    assert int(lens.sum()) == cache.info.retained_rows
+    if not page_rows:
+        off, cap = cache.query(tk.Q_OFFSETS), cache.query(tk.Q_CAPACITY)
+        assert np.array_equal(np.diff(off), cap) and off[-1] == cache.info.pool_rows
+    cache.close()
+    if pool:
+        pool.close()
+
+
 def test_decode_prefix_lengths():
     """A caller-supplied lengths array attends over a prefix of every segment."""
     tk, P = _tk(), _parity()
