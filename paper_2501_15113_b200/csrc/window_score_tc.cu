@@ -513,7 +513,9 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
         } else {
           const int j = tbase + quad * 32 + lane;   // this thread's key
           float cs[4] = {0.f, 0.f, 0.f, 0.f};   // four interleaved chains (FMA latency)
-          if (rows >= 64 && !tail) {
+          // A row that the window does not have is a zero query, and its score at a key with an infinite element is NaN:
+          // such rows are left out, not given a weight of zero.
+          if (rows >= 64 && !tail && p.rows == rows) {
             // 64 columns per TMEM load: half the load / wait round trips of the 32-column walk below
             for (int c0 = 0; c0 < rows; c0 += 64) {
               uint32_t r[64];
@@ -535,16 +537,17 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
             tc_wait_ld();
             const float4* mx4 = reinterpret_cast<const float4*>(myStat);
             const float4* wt4 = reinterpret_cast<const float4*>(myStat + 32);
-            uint32_t vm = 0xffffffffu;              // bit c: window row c sees this thread's key
+            uint32_t vm = p.rows >= 32 ? 0xffffffffu : (1u << p.rows) - 1u;   // bit c: window row c sees this thread's key
             if (tail) {
               const int need = j < N ? j - (N - L) : L;        // the residue c % L the row must reach (L: none does)
               int res = 0;
-              vm = 0;
+              uint32_t seen = 0;
 #pragma unroll
               for (int c = 0; c < 32; ++c) {
-                vm |= (uint32_t)(need <= res) << c;
+                seen |= (uint32_t)(need <= res) << c;
                 res = (res + 1 == L) ? 0 : res + 1;
               }
+              vm &= seen;
             }
 #pragma unroll
             for (int c = 0; c < 32; c += 4) {
@@ -557,7 +560,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
               }
             }
           } else
-          for (int c0 = 0; c0 < rows; c0 += 32) {
+          for (int c0 = 0; c0 < p.rows; c0 += 32) {
             uint32_t r[32];
             tc_ld32(taddr + (uint32_t)c0, r);
             tc_wait_ld();
@@ -566,10 +569,10 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
 #pragma unroll
               for (int c = 0; c < 32; c += 4) {
                 const float4 off = st4[c >> 2];
-                cs[0] += ex2(fmaf(__uint_as_float(r[c]), scale2, -off.x));
-                cs[1] += ex2(fmaf(__uint_as_float(r[c + 1]), scale2, -off.y));
-                cs[2] += ex2(fmaf(__uint_as_float(r[c + 2]), scale2, -off.z));
-                cs[3] += ex2(fmaf(__uint_as_float(r[c + 3]), scale2, -off.w));
+                const float o4[4] = {off.x, off.y, off.z, off.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                  if (c0 + c + i < p.rows) cs[i] += ex2(fmaf(__uint_as_float(r[c + i]), scale2, -o4[i]));
               }
             } else {
               // window row c0 + c sees keys up to N - L + (c0 + c) % L.  The residue is counted along (one
@@ -579,7 +582,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
 #pragma unroll
               for (int c = 0; c < 32; ++c) {
                 const float off = myStat[c0 + c];
-                const bool vis = (j < N) && (need <= res);
+                const bool vis = (j < N) && (need <= res) && (c0 + c < p.rows);
                 if (vis) cs[c & 3] += ex2(fmaf(__uint_as_float(r[c]), scale2, -off));
                 res = (res + 1 == L) ? 0 : res + 1;
               }

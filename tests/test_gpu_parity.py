@@ -232,6 +232,33 @@ def test_windows_of_every_size(G, L, d, N, dtype):
     run_workload(small("winrows", n=4 * G, n_kv=4, d=d, N=N, L=L, s1=4, s2=32, k=40, dtype=dtype, nh=0, t=64, steps=1))
 
 
+# A key with an infinite element that every window row scores -inf weighs nothing, whatever fills the window's tile up: a zero
+# query times infinity is NaN.  (G, L): 9 rows in the single-read kernel and in a tile of 32, 48 in one of 64, 96 in one of
+# 128, and full tiles; with and without the caller's normalisers (which take the two-pass kernel's second pass alone).
+@pytest.mark.parametrize("lse", [False, True])
+@pytest.mark.parametrize("G,L,d,N", [(1, 9, 64, 3000), (1, 9, 64, 32900), (2, 24, 128, 3000), (4, 24, 64, 3000), (1, 32, 64, 3000),
+                                     (2, 32, 64, 3000), (4, 32, 128, 3000)])
+def test_key_that_every_window_row_scores_minus_infinity(G, L, d, N, lse):
+    tk = _tk()
+    wl = small("infkey", n=4 * G, n_kv=4, d=d, N=N, L=L, s1=4, s2=32, k=40, dtype="bf16", nh=0, t=64, steps=1, promote=False)
+    qs, ks, vs = W.materialize(wl, DEV)
+    qs[0][0][..., 3] = qs[0][0][..., 3].abs() + 0.5
+    dead = [5, 200, N // 2, N - L - 1, N - 2]       # whole tiles and the causally masked one
+    ks[0][0][:, dead, 3] = -float("inf")
+    s = torch.einsum("hrd,hjd->hrj", qs[0][0].double().view(4, G * L, d), ks[0][0].double()) / d ** 0.5
+    last = N - L + torch.arange(G * L, device=DEV) % L
+    s.masked_fill_(torch.arange(N, device=DEV)[None] > last[:, None], -float("inf"))
+    want = torch.softmax(s, -1).mean(1).cpu().numpy()
+    given = [torch.logsumexp(s, -1).float().view(1, 4 * G, L).contiguous()] if lse else None
+    cache = tk.taskkv_compress_ex(tk.params_from_workload(wl, max_new_tokens=0), qs, ks, vs, window_lse=given)
+    got = cache.query(tk.Q_SCORES).reshape(4, -1)[:, :N]
+    assert cache.status() == 0
+    assert np.all(got[:, dead] == 0.0)
+    # fp32 scores of up to ~10 in the exponent and sums of fp32 terms: a few units of 2^-20
+    assert np.abs(got / np.where(want > 0, want, 1) - (want > 0)).max() < 1e-5
+    cache.close()
+
+
 def test_every_head_heterogeneous_is_full_attention():
     """force_class = 1: the cache is the whole K/V and decode is textbook attention."""
     wl = small("full", n=8, n_kv=4, d=128, N=1111, L=32, s1=4, s2=64, k=50, dtype="bf16")
