@@ -390,11 +390,11 @@ struct SideStream {
   bool ok = false, tried = false;
 };
 std::mutex g_side_mu;
-SideStream g_side[64];
+SideStream g_side[kMaxDevices];
 
 SideStream* side_stream() {   // call with g_side_mu held
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
   SideStream& ss = g_side[dev];
   if (!ss.tried) {
     ss.tried = true;

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "per_device.h"
 #include "taskkv.h"
 
 namespace taskkv {
@@ -206,6 +207,20 @@ __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepco
 // of tables this grid does not write -- under this grid's tail.  Called after this kernel's own wait, so that by the
 // time a dependent block runs, everything before this grid in the stream is complete.
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+inline int current_device() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) cudaGetLastError();
+  return dev;
+}
+inline int sm_count() {
+  static PerDevice<> known;
+  const int dev = current_device();
+  return known.get(dev, 0, [dev] {
+    int n = 0;
+    return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0 ? n : 148;
+  });
+}
 
 template <class... KArgs, class... Args>
 cudaError_t launch_dependent_smem(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,

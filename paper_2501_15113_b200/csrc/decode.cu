@@ -865,14 +865,16 @@ decode_cluster_kernel(DeviceProblem p, const T* __restrict__ q, const int32_t* _
   }
 }
 
-// Whether the device co-schedules a cluster of cs CTAs of this kernel (16 is above the portable size).
+// Whether the device co-schedules a cluster of 16 CTAs of this kernel (above the portable size, which the kernel's
+// attribute allows on the devices where it was set).
 template <typename T, int D, int G, bool PAGED>
 bool cluster16_fits() {
-  static const bool ok = [] {
+  static PerDevice<> known;
+  return known.get(current_device(), 0, [] {
     if (cudaFuncSetAttribute(decode_cluster_kernel<T, D, G, PAGED>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
         cudaSuccess) {
       cudaGetLastError();
-      return false;
+      return 0;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kClusterMax, 1, 1);
@@ -887,9 +889,8 @@ bool cluster16_fits() {
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, decode_cluster_kernel<T, D, G, PAGED>, &cfg) != cudaSuccess) n = 0;
     cudaGetLastError();
-    return n > 0;
-  }();
-  return ok;
+    return n > 0 ? 1 : 0;
+  }) > 0;
 }
 
 // CTAs per unit for the one-launch form, 0 if the call is not small enough for it.  A unit gets a CTA per item of the

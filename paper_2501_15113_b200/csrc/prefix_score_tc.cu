@@ -338,10 +338,7 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
 template <int D>
 cudaError_t launch_prefix_d(const void* q, const void* k, int heads, int group, int N, float* scores, int32_t* status,
                             cudaStream_t s) {
-  int dev = 0, n_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-  if (n_sm <= 0) n_sm = 148;
+  const int n_sm = sm_count();
   const PrefixLayout lay = make_prefix_layout(D);
   cudaError_t e = cudaFuncSetAttribute(prefix_score_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, lay.total);
   if (e != cudaSuccess) return e;

@@ -861,11 +861,11 @@ cudaError_t launch_cluster_k(const DeviceProblem& p, const UnitRange& ur, int cs
   return cudaLaunchKernelEx(&cfg, select_cluster_kernel<T, D, POOL_HALF>, p, ur);
 }
 
-// Whether the device can co-schedule at least one cluster of cs_n such CTAs (asked once per cluster size).
+// Whether the device can co-schedule at least one cluster of cs_n such CTAs (asked once per device and cluster size).
 template <typename T, int D, int POOL_HALF>
 bool cluster_fits(int cs_n) {
-  static int cached[kMaxCS + 1] = {0};      // 0 unknown, 1 yes, -1 no
-  if (cached[cs_n] == 0) {
+  static PerDevice<kMaxCS + 1> known;
+  return known.get(current_device(), cs_n, [cs_n] {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)cs_n, 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
@@ -879,9 +879,8 @@ bool cluster_fits(int cs_n) {
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, select_cluster_kernel<T, D, POOL_HALF>, &cfg) != cudaSuccess) n = 0;
     cudaGetLastError();
-    cached[cs_n] = n > 0 ? 1 : -1;
-  }
-  return cached[cs_n] > 0;
+    return n > 0 ? 1 : 0;
+  }) > 0;
 }
 
 template <typename T, int D>

@@ -483,32 +483,31 @@ window_res_kernel(const __grid_constant__ ResMaps maps, DeviceProblem p, const _
   if (tid == 0 && *s_abort) set_status(p.status, TASKKV_ETIMEOUT);
 }
 
-// Clusters of `team` CTAs of this kernel that the device runs at once (0: the cluster size is not available).
+// Clusters of `team` CTAs of this kernel that the device runs at once (0: the cluster size is not available).  The
+// kernel's attributes are set on the device along with the question.
 template <int D>
 int max_clusters(int team, int smem) {
-  static int cached[kMaxTeam + 1] = {0};
-  static bool known[kMaxTeam + 1] = {false};
-  if (known[team]) return cached[team];
-  known[team] = true;
-  int n = 0;
-  if (cudaFuncSetAttribute(window_res_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
-      cudaFuncSetAttribute(window_res_kernel<D>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(team, 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = team;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, window_res_kernel<D>, &cfg) != cudaSuccess) n = 0;
-  }
-  cudaGetLastError();
-  cached[team] = n;
-  return n;
+  static PerDevice<kMaxTeam + 1> known;
+  return known.get(current_device(), team, [team, smem] {
+    int n = 0;
+    if (cudaFuncSetAttribute(window_res_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+        cudaFuncSetAttribute(window_res_kernel<D>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(team, 1, 1);
+      cfg.blockDim = dim3(kThreads, 1, 1);
+      cfg.dynamicSmemBytes = smem;
+      cudaLaunchAttribute attr;
+      attr.id = cudaLaunchAttributeClusterDimension;
+      attr.val.clusterDim.x = team;
+      attr.val.clusterDim.y = 1;
+      attr.val.clusterDim.z = 1;
+      cfg.attrs = &attr;
+      cfg.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&n, window_res_kernel<D>, &cfg) != cudaSuccess) n = 0;
+    }
+    cudaGetLastError();
+    return n;
+  });
 }
 
 inline int team_for(int max_tiles) {
@@ -594,9 +593,7 @@ cudaError_t launch_res_d(const DeviceProblem& p, const WindowHostInfo& h, cudaSt
 // device that co-schedules enough clusters of every size in use to fill three quarters of its SMs.
 bool window_res_supported(const DeviceProblem& p, const WindowHostInfo& h) {
   if (p.rows > kRows || h.lse != nullptr) return false;
-  int dev = 0, n_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  const int n_sm = sm_count();
   const int smem = make_layout(p.d).total;
   bool checked[kMaxTeam + 1] = {false};
   for (int b = 0; b < h.batch; ++b) {

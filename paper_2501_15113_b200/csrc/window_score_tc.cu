@@ -682,13 +682,7 @@ inline int pick_chunk(int64_t units_times_keys, int n_sm, int least) {
 
 template <int D, int ROWS>
 cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStream_t s, int layer0, int n_layers) {
-  static int n_sm = 0;
-  if (n_sm == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (n_sm <= 0) n_sm = 148;
-  }
+  const int n_sm = sm_count();
   constexpr int rows = ROWS;
   const TcLayout lay = make_layout(D, rows);
   if (lay.stages < 2) return cudaErrorInvalidValue;

@@ -209,3 +209,56 @@ def test_plan_of_a_paged_cache_counts_pages_per_unit(tk):
     shard = tk.Params(**dict(kw, n_heads=4, n_kv_heads=4, shard_kv_heads=8, shard_first=0))
     with pytest.raises(tk.TaskKVError):
         tk.taskkv_plan_paged(shard, 64)
+
+
+# ---------------------------------------------------------------- answers that belong to a device
+PER_DEVICE_PROGRAM = r"""
+#include <cstdio>
+#include <thread>
+#include <vector>
+#include "per_device.h"
+using namespace taskkv;
+int main() {
+  static PerDevice<3> known;
+  std::atomic<int> asked{0};
+  // a device's answer is its own, asked for once: 0 and 1 among them, each key by itself
+  auto get = [&](int dev, int key) { return known.get(dev, key, [&] { ++asked; return dev * 10 + key; }); };
+  for (int round = 0; round < 3; ++round)
+    for (int dev = 0; dev < kMaxDevices; ++dev)
+      for (int key = 0; key < 3; ++key)
+        if (get(dev, key) != dev * 10 + key) return 1;
+  if (asked != 3 * kMaxDevices) return 2;
+  // beyond the table (or with no device at all): asked every time, nothing kept
+  for (int dev : {-1, kMaxDevices}) { get(dev, 0); if (get(dev, 2) != dev * 10 + 2) return 3; }
+  if (asked != 3 * kMaxDevices + 4) return 4;
+  // threads on different devices
+  static PerDevice<> other;
+  std::atomic<int> wrong{0};
+  std::vector<std::thread> ts;
+  for (int t = 0; t < 8; ++t)
+    ts.emplace_back([&, t] {
+      for (int i = 0; i < 2000; ++i)
+        if (other.get((t + i) % 5, 0, [&] { return (t + i) % 5 == 3 ? 0 : 16; }) != ((t + i) % 5 == 3 ? 0 : 16)) ++wrong;
+    });
+  for (auto& t : ts) t.join();
+  return wrong ? 5 : 0;
+}
+"""
+
+
+def test_answers_are_kept_per_device(tmp_path):
+    import subprocess
+    src = tmp_path / "per_device.cpp"
+    src.write_text(PER_DEVICE_PROGRAM)
+    exe = tmp_path / "per_device"
+    subprocess.run(["g++", "-std=c++17", "-O1", "-pthread", "-I", os.path.join(ROOT, "paper_2501_15113_b200", "csrc"),
+                    str(src), "-o", str(exe)], check=True)
+    assert subprocess.run([str(exe)]).returncode == 0
+
+
+def test_no_host_function_keeps_a_device_answer_for_the_whole_process():
+    """A plain function-local static would hold the first device's answer for every other device."""
+    d = os.path.join(ROOT, "paper_2501_15113_b200", "csrc")
+    for f in sorted(os.listdir(d)):
+        for n, line in enumerate(open(os.path.join(d, f)).read().split("\n"), 1):
+            assert not re.match(r"\s+static (const )?(int|bool|size_t|int64_t) \w+", line), f"{f}:{n}: {line.strip()}"

@@ -220,6 +220,24 @@ def test_cluster_decode_equals_the_two_kernels_bit_for_bit(kw, page_rows):
             p.close()
 
 
+@pytest.mark.skipif(torch.cuda.device_count() < 2, reason="needs a second CUDA device")
+def test_second_device_of_a_process_decodes_with_clusters_of_sixteen():
+    """Units of 9 to 16 items run in clusters above the portable size, which a function attribute allows device by device."""
+    tk = _tk()
+    wl = small("twodev", n=8, n_kv=8, d=64, N=1000, L=16, s1=4, s2=32, k=300, dtype="f32", nh=1, steps=1)
+    qs, ks, vs = W.materialize(wl, DEV)
+    q, kn, vn = W.gen_decode_step(wl, 0, DEV)
+    outs = []
+    for dev in range(2):
+        with torch.cuda.device(dev):
+            to = lambda ts: [t.to(f"cuda:{dev}") for t in ts]
+            cache = tk.taskkv_compress_ex(tk.params_from_workload(wl, max_new_tokens=4), to(qs), to(ks), to(vs))
+            outs.append(cache.taskkv_decode_step(*to([q, kn, vn])).cpu())
+            assert cache.status() == 0
+            cache.close()
+    assert torch.equal(outs[0], outs[1])
+
+
 # (query heads per KV head, window) -> 8 to 128 window rows: on the CUDA cores (fp32), or as the next larger tensor-core
 # tile with zero rows (bf16; up to 32768 keys the single-read kernel takes up to 32 rows); key counts around the 128-key tile, the
 # 256-key chunk and the 8192 keys up to which pass 2 folds the chunks' statistics itself.  (Four KV heads: two are always
