@@ -493,7 +493,8 @@ decode_attn_kernel(DeviceProblem p, const T* __restrict__ q, const int32_t* __re
   // `early` (set by the host when the kernel before this one in the stream cannot be one that writes these units'
   // lengths or page tables: see launch_decode): the first item's unit data is read before the wait as well, and the
   // wait comes just before the block first touches what the caller's kernels produce (q, the new token's rows) or
-  // writes anything.  (A block all of whose items are beyond their segments' lengths leaves without waiting.)
+  // writes anything.  A block none of whose items holds rows waits before it leaves: were that so for the whole grid, the
+  // merge, which waits for this grid alone, and whatever follows it could overtake the kernels before this one.
   bool waited = false;
   auto wait_once = [&]() {
     if (!waited) {
@@ -543,6 +544,7 @@ decode_attn_kernel(DeviceProblem p, const T* __restrict__ q, const int32_t* __re
       }
     });
   }
+  wait_once();
 }
 
 // One block per (view unit, query head of the group): merge the unit's partials.  First the block finds

@@ -333,6 +333,39 @@ def test_non_finite_values_leave_the_plan_as_it_is(value, page_rows):
         pool.close()
 
 
+def test_decode_of_a_layer_that_is_not_in_yet_keeps_its_place_in_the_stream():
+    """None of the attention blocks of such a call has rows to read; what it writes (zeros) still comes after the step before
+    it, and the step after it still reads the lengths that one left.  (Units of 40 items: attention and merge kernels.)"""
+    tk = _tk()
+    wl = small("order", n=8, n_kv=8, d=128, N=20000, L=32, s1=4, s2=64, k=300, dtype="bf16", R=2, nh=2, steps=1)
+    qs, ks, vs = W.materialize(wl, DEV)
+    steps = 60
+    params = tk.params_from_workload(wl, max_new_tokens=steps + 1)
+
+    def one_layer_of_two():
+        c = tk.taskkv_cache_create(params, DEV)
+        c.taskkv_compress_layer(0, [qs[0][0]], [ks[0][0]], [vs[0][0]])
+        return c
+
+    mixed, alone = one_layer_of_two(), one_layer_of_two()
+    inputs = [[x[:, :1].contiguous() for x in W.gen_decode_step(wl, s, DEV)] for s in range(4)]
+    both = torch.ones(steps, *inputs[0][0].shape, dtype=torch.bfloat16, device=DEV)
+    torch.cuda.synchronize()
+    for s in range(steps):
+        q, kn, vn = inputs[s % 4]
+        mixed.taskkv_decode_step_ex(q, kn, vn, 0, 1, out=both[s])
+        mixed.taskkv_decode_ex(q, 1, 1, out=both[s])                       # the same buffer: zeros in the end
+    got = mixed.taskkv_decode_step_ex(q, kn, vn, 0, 1)
+    assert not both.any()
+    for s in range(steps):
+        alone.taskkv_decode_step_ex(*inputs[s % 4], 0, 1)
+        torch.cuda.synchronize()
+    assert torch.equal(got, alone.taskkv_decode_step_ex(q, kn, vn, 0, 1))
+    assert mixed.lengths().tolist() == alone.lengths().tolist() and mixed.status() == alone.status() == 0
+    mixed.close()
+    alone.close()
+
+
 def test_decode_prefix_lengths():
     """A caller-supplied lengths array attends over a prefix of every segment."""
     tk, P = _tk(), _parity()
