@@ -22,7 +22,7 @@ struct HostPlan {
   taskkv_plan_info info;
   int64_t c_total = 0;
   int32_t max_N = 0, min_N = 0;
-  int32_t chunks_max = 0, rows = 0, rows_pad = 0, idx_stride = 0, dec_chunk = 0;
+  int32_t chunks_max = 0, rows = 0, rows_pad = 0, idx_stride = 0, dec_shift = 0, dec_tail = 0;
   std::vector<int32_t> seq_lens, mid, nhet;     // [B], [B*R] middle budget of a (sequence, layer), [B*R]
   std::vector<int32_t> full;                    // [B*R] full-cache heads
   std::vector<int32_t> full_model;              // [B*R] the same over all shards
@@ -65,22 +65,38 @@ int32_t mid_budget_impl(double budget_tokens, int32_t N, int32_t h_full, int32_t
   return (int32_t)k;
 }
 
-// Rows per split-K decode item.  Half a thousand rows an item is best where the cache fills the GPU with items anyway; a
-// cache that has fewer than two per SM gets smaller ones (a warp walks its share of an item 16 rows at a time, one
-// trip to memory after the other).  Counted over the retained rows of the model's heads, so that a head shard, a paged
-// cache or another reserve for appended tokens cut the same units alike and give the same bits.
-int32_t pick_decode_chunk(const HostPlan& hp, const taskkv_params* p, int n_model) {
+// Split-K decode items of the model's heads, cut by 2^shift and 2^tail rows (UnitItems), `grown` rows after compression.
+int64_t decode_items(const HostPlan& hp, const taskkv_params* p, int n_model, int shift, int tail, int64_t grown) {
   const int B = p->batch, R = p->n_layers, s = p->sink + p->recent;
-  for (int32_t chunk = kDecodeChunk;; chunk /= 2) {
-    int64_t items = 0;
-    for (int b = 0; b < B; ++b)
-      for (int r = 0; r < R; ++r) {
-        const int64_t N = hp.seq_lens[b], h = hp.full_model[(size_t)b * R + r];
-        const int64_t kept = N > s ? s + std::min<int64_t>(hp.mid[(size_t)b * R + r], N - s) : N;
-        items += h * ((N + chunk - 1) / chunk) + (n_model - h) * ((kept + chunk - 1) / chunk);
-      }
-    if (items >= 2 * 148 || chunk <= kDecodeChunkMin) return chunk;
-  }
+  int64_t items = 0;
+  for (int b = 0; b < B; ++b)
+    for (int r = 0; r < R; ++r) {
+      const int64_t N = hp.seq_lens[b], h = hp.full_model[(size_t)b * R + r];
+      const int64_t kept = N > s ? s + std::min<int64_t>(hp.mid[(size_t)b * R + r], N - s) : N;
+      items += h * UnitItems<int64_t>(N, shift, tail).count(N + grown) +
+               (n_model - h) * UnitItems<int64_t>(kept, shift, tail).count(kept + grown);
+    }
+  return items;
+}
+// Rows per item.  Half a thousand rows an item is best where the cache fills the GPU with items anyway; a cache that has
+// fewer than two per SM gets smaller ones (a warp walks its share of an item 16 rows at a time, one trip to memory after
+// the other).  Counted over the retained rows of the model's heads, so that a head shard, a paged cache or another
+// reserve for appended tokens cut the retained rows of the same units alike and give the same bits.
+// The rows appended beyond them are cut alike as long as the cache has at most eight items per SM at its capacity, and
+// into larger items, 512 rows in the end, where the reserve is larger: its items are walked at every step, filled or not,
+// and each takes memory for its partial results.  A whole call in us right after compression and 4000 rows later, with
+// 512 rows an item throughout, with equal items throughout, and like this:
+//   32 bf16 units of 1000 rows, room for 4096 more   11.4, 15.7    8.9, 17.8    7.3, 15.2
+//   the same, room for 65536 more                    16.0, 24.8   38.8, 48.8   11.0, 24.6
+//   16 fp32 units of 1000 rows, room for 4096 more   17.0, 19.2    7.9, 13.6   (equal items)
+void pick_decode_items(HostPlan& hp, const taskkv_params* p, int n_model) {
+  int least = 0, most = 0;
+  while ((1 << least) < kDecodeChunkMin) ++least;
+  while ((1 << most) < kDecodeChunk) ++most;
+  hp.dec_shift = most;
+  while (hp.dec_shift > least && decode_items(hp, p, n_model, hp.dec_shift, hp.dec_shift, 0) < 2 * 148) --hp.dec_shift;
+  hp.dec_tail = hp.dec_shift;
+  while (hp.dec_tail < most && decode_items(hp, p, n_model, hp.dec_shift, hp.dec_tail, p->max_new_tokens) > 8 * 148) ++hp.dec_tail;
 }
 
 taskkv_status make_plan(const taskkv_params* p, HostPlan& hp, int32_t page_rows = 0) {
@@ -154,7 +170,7 @@ taskkv_status make_plan(const taskkv_params* p, HostPlan& hp, int32_t page_rows 
   hp.kept_len.assign((size_t)B * R, 0);
   hp.pages_compress = 0;
   hp.page_stride = 0;
-  hp.dec_chunk = pick_decode_chunk(hp, p, n_model);
+  pick_decode_items(hp, p, n_model);
   std::vector<int64_t> blk_g((size_t)B * R, 0), blk_d((size_t)B * R, 0);   // per block b * R + r
   for (int b = 0; b < B; ++b) {
     const int64_t N = hp.seq_lens[b];
@@ -174,8 +190,8 @@ taskkv_status make_plan(const taskkv_params* p, HostPlan& hp, int32_t page_rows 
       kept_rows += h * N + (nkv - h) * kept;
       blk_g[br] = h * ((N + kGatherRows - 1) / kGatherRows) + (nkv - h) * ((kept + kGatherRows - 1) / kGatherRows);
       gitems += blk_g[br];
-      const int64_t li = h * ((N + mn + hp.dec_chunk - 1) / hp.dec_chunk) +
-                         (nkv - h) * ((kept + mn + hp.dec_chunk - 1) / hp.dec_chunk);
+      const int64_t li = h * UnitItems<int64_t>(N, hp.dec_shift, hp.dec_tail).count(N + mn) +
+                         (nkv - h) * UnitItems<int64_t>(kept, hp.dec_shift, hp.dec_tail).count(kept + mn);
       blk_d[br] = li;
       ditems += li;
       hp.layer_items[(size_t)r] += li;
@@ -556,11 +572,12 @@ void fill_device_problem(taskkv_cache* c) {
   for (int32_t m : hp.mid) d.max_mid = m > d.max_mid ? m : d.max_mid;
   if (d.max_mid > hp.max_N) d.max_mid = hp.max_N;
   d.max_new = p.max_new_tokens;
-  d.dec_chunk = hp.dec_chunk;
-  d.dec_shift = 0;
-  while ((1 << d.dec_shift) < hp.dec_chunk) ++d.dec_shift;
-  d.max_prompt = hp.max_N;
-  d.max_cap = hp.max_N + p.max_new_tokens;
+  d.dec_chunk = 1 << hp.dec_shift;
+  d.dec_shift = (int16_t)hp.dec_shift;
+  d.dec_tail = (int16_t)hp.dec_tail;
+  const UnitItems<int64_t> longest(hp.max_N, hp.dec_shift, hp.dec_tail);
+  d.items_kept = (int32_t)longest.n_kept;
+  d.items_cap = (int32_t)longest.count((int64_t)hp.max_N + p.max_new_tokens);
   d.idx_stride = hp.idx_stride;
   d.chunks_max = hp.chunks_max;
   d.pool_rows = hp.info.pool_rows;

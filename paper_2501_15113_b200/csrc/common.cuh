@@ -13,6 +13,7 @@ namespace taskkv {
 
 constexpr int kDecodeChunk = 512;                 // most rows of one split-K decode item
 constexpr int kDecodeChunkMin = 64;               // fewest
+constexpr int kDecodeFewItems = 32;               // most items of a unit that a cluster takes or one warp merges
 constexpr int kGatherRows = 64;                   // rows of one gather item
 constexpr int kScoreChunk = 256;                  // keys of one window-score work item (CUDA-core path)
 constexpr int kTcChunk = 2048;                    // fewest keys of one window-score work item (tensor-core path)
@@ -56,9 +57,11 @@ struct DeviceProblem {
   int32_t view_l0, view_nl, view_U;
   int32_t item0, item1;       // decode work items of the view
   int32_t max_new;
-  int32_t dec_chunk;    // rows of one split-K decode item of this cache: a power of two, log2 in dec_shift
-  int32_t dec_shift;
-  int32_t max_prompt, max_cap;   // most rows a unit holds right after compression, most it can grow to
+  // Split-K decode items (see UnitItems): their rows within what a unit holds after compression, log2 of them there and
+  // beyond; the most items a unit has after compression and at its capacity.
+  int32_t dec_chunk;
+  int16_t dec_shift, dec_tail;
+  int32_t items_kept, items_cap;
   float budget_frac;    // > 0: the middle budget follows Eq. 17 from this fraction of the full cache
   // Head sharding: this problem holds KV heads [kv_first, kv_first + n_kv) of a model with n_kv_model per layer.
   // Eq. 8 / Eq. 16 / Eq. 17 count over the model's heads; the separator then reads every head's semantic vector
@@ -96,8 +99,8 @@ struct DeviceProblem {
   int32_t* idx;               // [U][idx_stride]
   int32_t* gather_off;        // [U+1] gather work items, indexed layer-major like dec_off
   int32_t* dec_off;           // [U+1] decode work items, indexed by w = (r * B + b) * n_kv + h
-  int2* dec_item;             // [items] decode work item -> (unit index w of dec_off plus one, first row); (0, 0): the item's
-                              // layer has not been compressed
+  int2* dec_item;             // [items] decode work item -> (unit index w of dec_off plus one, first row | log2 of its rows: a
+                              // first row is a multiple of 64); (0, 0): the item's layer has not been compressed
   int32_t* step_cnt;          // [U] combine blocks of a unit that finished the current fused step (0 between calls)
   void* k_pool;
   void* v_pool;
@@ -201,6 +204,26 @@ cudaError_t launch_decode(const DeviceProblem& p, int dtype, const void* q, cons
 // the launch attribute the wait returns at once.)  This takes the launch latency out of chains of short dependent
 // kernels: attention -> combine -> attention of a layer-by-layer decode loop, separator -> plan -> gather.
 #ifdef __CUDACC__
+// How a unit's rows are cut into decode items: rows [0, begin(n_kept)), the retained ones filled up to a whole item, into
+// items of 2^shift rows, the rest of the reserve for appended tokens into items of 2^tail.
+// (Int: 64 bits where a capacity is planned that may be more than the device's 32-bit counts take.)
+template <class Int = int>
+struct UnitItems {
+  Int n_kept;
+  int shift, tail;
+  __host__ __device__ UnitItems(Int kept, int shift_, int tail_)
+      : n_kept(((kept > 0 ? kept : 0) + (1 << shift_) - 1) >> shift_), shift(shift_), tail(tail_) {}
+  __host__ __device__ Int begin(Int j) const {                    // first row of item j
+    const Int over = j - n_kept;
+    return over <= 0 ? j << shift : (n_kept << shift) + (over << tail);
+  }
+  __host__ __device__ int log_rows(Int j) const { return j < n_kept ? shift : tail; }
+  __host__ __device__ Int count(Int rows) const {                 // items that hold rows [0, rows)
+    const Int over = rows - (n_kept << shift);
+    return over <= 0 ? (rows + (1 << shift) - 1) >> shift : n_kept + ((over + (1 << tail) - 1) >> tail);
+  }
+};
+
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel in the stream (if launched with launch_dependent()) become resident once every block of this
 // grid has got here or exited: its blocks then run whatever they do before their own grid_dependency_wait() -- reads

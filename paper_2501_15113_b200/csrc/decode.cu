@@ -2,7 +2,7 @@
 // head, no mask): o_a = softmax(q_a K_u^T / sqrt(d)) V_u over the len_u rows of
 // the KV head's segment, for the G query heads that share it.
 //
-// Split-K: a unit's rows are cut into work items of dec_chunk rows (512, fewer in small caches), numbered once at
+// Split-K: a unit's rows are cut into work items of 512 rows (fewer in small caches: UnitItems), numbered once at
 // compression for every unit at its capacity (so a 32768-row full head and a 772-row pruned head
 // load the SMs alike; items beyond a segment's current length are skipped).  Each item produces an un-normalised partial
 // (running max, sum, weighted V) per head with an online softmax in fp32; one
@@ -424,6 +424,14 @@ struct MmaItem {
   }
 };
 
+// Work items that hold the first `len` rows of a unit.  (Where the reserve is cut like the rest, the usual case, its first
+// row does not matter and the unit's capacity is not read.)
+template <bool TAIL>
+__device__ __forceinline__ int unit_item_count(const DeviceProblem& p, int unit, int len) {
+  if (!TAIL || p.dec_tail == p.dec_shift) return (len + p.dec_chunk - 1) >> p.dec_shift;
+  return UnitItems<>(p.cap[unit] - p.max_new, p.dec_shift, p.dec_tail).count(len);
+}
+
 template <typename T, int D, int G, bool PAGED>
 using Item = typename std::conditional<sizeof(T) == 2, MmaItem<D, G, PAGED>, ScalarItem<T, D, G, PAGED>>::type;
 
@@ -508,7 +516,7 @@ decode_attn_kernel(DeviceProblem p, const T* __restrict__ q, const int32_t* __re
     __syncthreads();                                // previous item's shared state consumed
     const int2 at = item == item_first ? at_first : p.dec_item[item];
     if (at.x == 0) continue;                        // an item of a layer that is not in yet
-    const int w = at.x - 1, rbeg = at.y;
+    const int w = at.x - 1, rbeg = at.y & ~63;
     const LmUnit lu = lm_unit(p, w);
     const int vu = lu.v;                            // view unit: index into q and lengths
     const int u = lu.u;                             // unit: index into the cache
@@ -519,7 +527,7 @@ decode_attn_kernel(DeviceProblem p, const T* __restrict__ q, const int32_t* __re
     if (new_r >= 0) ++len;
     if (lengths) len = min(max(lengths[vu], 0), len);
     if (rbeg >= len) continue;                      // an item of the reserve beyond the segment's length
-    const int rend = min(len, rbeg + p.dec_chunk);
+    const int rend = min(len, rbeg + (1 << (at.y & 63)));
     if (tid == 0) s_direct = len <= p.dec_chunk ? vu : -1;     // read back after the row loop (no register held)
     const int64_t seg = p.seg_off[u];
     const unsigned char* kn_row = k_new + (size_t)vu * ROW_BYTES;
@@ -559,8 +567,9 @@ constexpr int kCombineStage = 1024;     // partial results weighted per round (o
 // 16-byte loads in it (a long unit has over a hundred partials and one block: its latency is the kernel's).
 // PRE: partial outputs a warp loads ahead of the weights (8: 64 registers, four blocks per SM (the lean one: six), for grids that are
 // resident at once anyway -- it takes two round trips to L2 off the merge; 0: the lean variant for many thousands of
-// blocks, most of them with nothing to merge).
-template <typename T, int D, int G, int PRE>
+// blocks, most of them with nothing to merge).  TAIL: the reserve's items are larger than the others (a template argument,
+// since a branch here costs a single layer's merge 0.2 to 0.4 us: 9.1 -> 9.5 for 8 units of up to 8000 rows).
+template <typename T, int D, int G, int PRE, bool TAIL>
 __global__ void __launch_bounds__(kCombineThreads, PRE > 0 ? 4 : 6) decode_combine_kernel(DeviceProblem p,
                                                                          const int32_t* __restrict__ lengths,
                                                                          int fused_step, T* __restrict__ out) {
@@ -581,7 +590,7 @@ __global__ void __launch_bounds__(kCombineThreads, PRE > 0 ? 4 : 6) decode_combi
   len = len_next;
   if (lengths) len = min(max(lengths[u], 0), len);
   // the unit's items that hold rows (the table also numbers the reserve for appended tokens)
-  const int i0 = p.dec_off[lm_index(p, unit)], i1 = i0 + ((len + p.dec_chunk - 1) >> p.dec_shift);
+  const int i0 = p.dec_off[lm_index(p, unit)], i1 = i0 + unit_item_count<TAIL>(p, unit, len);
   grid_dependency_wait();
   grid_launch_dependents();
   if (i1 - i0 != 1) {                                   // a unit of one item has its output from the attention kernel
@@ -708,7 +717,7 @@ __global__ void __launch_bounds__(kCombineThreads) decode_combine_few_kernel(Dev
   const int len_next = len + (grown ? 1 : 0);
   len = len_next;
   if (lengths) len = min(max(lengths[u], 0), len);
-  const int i0 = p.dec_off[lm_index(p, unit)], n = (len + p.dec_chunk - 1) >> p.dec_shift;
+  const int i0 = p.dec_off[lm_index(p, unit)], n = unit_item_count<true>(p, unit, len);
   grid_dependency_wait();
   grid_launch_dependents();
   if (!there) return;
@@ -781,7 +790,7 @@ __global__ void __launch_bounds__(kCombineThreads) decode_combine_few_kernel(Dev
 constexpr int kClusterSlots = 2;         // items per CTA
 constexpr int kClusterMax = 16;          // CTAs per cluster
 constexpr int kClusterItems = kClusterSlots * kClusterMax;
-static_assert(kClusterItems <= 32, "one lane per item in the merge");
+static_assert(kClusterItems == kDecodeFewItems, "one lane per item in the merge");
 
 template <typename T, int D, int G, bool PAGED>
 __global__ void __launch_bounds__(kAttnThreads, 2)
@@ -895,16 +904,16 @@ bool cluster16_fits() {
   }) > 0;
 }
 
-// CTAs per unit for the one-launch form, 0 if the call is not small enough for it.  A unit gets a CTA per item of the
-// longest prompt (the tokens appended since may give a CTA a second one), and all CTAs of the call fit on the GPU
-// together, two to an SM: beyond that the call is bound by HBM, and the persistent attention kernel with its
-// deal of equal items is the better one.
+// CTAs per unit for the one-launch form, 0 if the call is not small enough for it or its items are not all of one size (a
+// reserve that is cut into longer ones is more than 32 items a unit where this form would be the faster one).  A unit gets a
+// CTA per item of the longest prompt (the tokens appended since may give a CTA a second one), and all CTAs of the call
+// fit on the GPU together, two to an SM: beyond that the call is bound by HBM, and the persistent attention kernel with
+// its deal of equal items is the better one.
 int cluster_size(const DeviceProblem& p) {
-  const int items_cap = (p.max_cap + p.dec_chunk - 1) / p.dec_chunk, items = (p.max_prompt + p.dec_chunk - 1) / p.dec_chunk;
-  if (items_cap > kClusterItems) return 0;
+  if (p.items_cap > kClusterItems || p.dec_tail != p.dec_shift) return 0;
   int cs = 1;
-  while (cs < items || kClusterSlots * cs < items_cap) cs *= 2;
-  if (cs > kClusterMax || cs > p.G * p.d || (int64_t)p.view_U * cs > 148 * 2) return 0;
+  while (cs < p.items_kept || kClusterSlots * cs < p.items_cap) cs *= 2;
+  if (cs > kClusterMax || (int64_t)p.view_U * cs > 148 * 2) return 0;
   return cs;
 }
 
@@ -964,14 +973,17 @@ cudaError_t launch_typed(const DeviceProblem& p, const void* q, const int32_t* l
     // units of at most 16 items each (32, if a block per head would be more than the GPU holds at once): a warp per head.
     // Otherwise a block per head; up to 16 of them per SM the variant that loads ahead (its blocks are resident within a
     // few waves)
-    if ((int64_t)p.max_cap <= (int64_t)((int64_t)p.view_U * G > 148 * 4 ? 32 : 16) * p.dec_chunk)
+    if (p.items_cap <= ((int64_t)p.view_U * G > 148 * 4 ? kDecodeFewItems : kDecodeFewItems / 2))
       e = launch_dependent(decode_combine_few_kernel<T, D, G>, (unsigned)((p.view_U * G + kCombineWarps - 1) / kCombineWarps),
                            kCombineThreads, s, p, lengths, fused, static_cast<T*>(out));
+    else if (p.dec_tail != p.dec_shift)      // (fewer than 296 items after compression, so fewer units than that)
+      e = launch_dependent(decode_combine_kernel<T, D, G, 8, true>, (unsigned)(p.view_U * G), kCombineThreads, s, p, lengths,
+                           fused, static_cast<T*>(out));
     else if ((int64_t)p.view_U * G <= 148 * 16)
-      e = launch_dependent(decode_combine_kernel<T, D, G, 8>, (unsigned)(p.view_U * G), kCombineThreads, s, p, lengths,
+      e = launch_dependent(decode_combine_kernel<T, D, G, 8, false>, (unsigned)(p.view_U * G), kCombineThreads, s, p, lengths,
                            fused, static_cast<T*>(out));
     else
-      e = launch_dependent(decode_combine_kernel<T, D, G, 0>, (unsigned)(p.view_U * G), kCombineThreads, s, p, lengths,
+      e = launch_dependent(decode_combine_kernel<T, D, G, 0, false>, (unsigned)(p.view_U * G), kCombineThreads, s, p, lengths,
                            fused, static_cast<T*>(out));
   }
   return e;

@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(128) separator_plan_kernel(DeviceProblem p, in
 
   // ---- plan of this block's units (the problem's own heads)
   __shared__ int s_cap[TASKKV_MAX_KV_HEADS], s_git[TASKKV_MAX_KV_HEADS], s_dit[TASKKV_MAX_KV_HEADS], s_dat[TASKKV_MAX_KV_HEADS];
+  __shared__ int s_len[TASKKV_MAX_KV_HEADS];
   const int B = lm_batch(p);
   const int lm_block = r_lay * B + b_seq;
   int len = 0;
@@ -107,7 +108,8 @@ __global__ void __launch_bounds__(128) separator_plan_kernel(DeviceProblem p, in
     p.cap[u] = cap;
     s_cap[tid] = cap;
     s_git[tid] = (len + kGatherRows - 1) / kGatherRows;
-    s_dit[tid] = (cap + p.dec_chunk - 1) / p.dec_chunk;
+    s_len[tid] = len;
+    s_dit[tid] = UnitItems<>(len, p.dec_shift, p.dec_tail).count(cap);
   }
   __syncthreads();
   if (tid < nl) {
@@ -144,10 +146,12 @@ __global__ void __launch_bounds__(128) separator_plan_kernel(DeviceProblem p, in
   __syncthreads();
   {
     const int end = p.dec_base[lm_block + 1], last = s_dat[nl - 1] + s_dit[nl - 1];
-    for (int h = 0; h < nl; ++h)
+    for (int h = 0; h < nl; ++h) {
+      const UnitItems<> it(s_len[h], p.dec_shift, p.dec_tail);
       for (int i = tid; i < s_dit[h] && s_dat[h] + i < end; i += 128)
-        p.dec_item[s_dat[h] + i] = make_int2(lm_block * nl + h + 1, i * p.dec_chunk);
-    for (int i = last + tid; i < end; i += 128) p.dec_item[i] = make_int2(lm_block * nl + nl, 0x7fffffff);
+        p.dec_item[s_dat[h] + i] = make_int2(lm_block * nl + h + 1, it.begin(i) | it.log_rows(i));
+    }
+    for (int i = last + tid; i < end; i += 128) p.dec_item[i] = make_int2(lm_block * nl + nl, 0x7fffffc0);
   }
   // ---- paged cache: the block takes the pages of its units' retained rows off the pool in one step (growth takes
   // pages later, one at a time) and deals them out in unit order

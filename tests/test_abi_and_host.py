@@ -211,6 +211,25 @@ def test_plan_of_a_paged_cache_counts_pages_per_unit(tk):
         tk.taskkv_plan_paged(shard, 64)
 
 
+# (kv heads, rows, reserve) of one fp32 layer with every head whole -> rows per item of the prompt and of the reserve: short
+# items where the cache has fewer than two per SM, the reserve cut alike up to eight per SM, longer beyond
+@pytest.mark.parametrize("n,N,reserve,chunk,tail", [
+    (8, 512, 16, 64, 64), (8, 512, 8960, 64, 64), (8, 512, 8961, 64, 128), (8, 512, 20000, 64, 256), (8, 512, 65536, 64, 512),
+    (8, 500, 8972, 64, 64), (8, 500, 8973, 64, 128), (32, 1000, 4096, 64, 256), (32, 1000, 16384, 64, 512), (32, 3000, 0, 256, 256),
+    (32, 3000, 4000, 256, 256), (32, 3000, 100000, 256, 512), (32, 20000, 100000, 512, 512)])
+def test_decode_items_of_a_reserve(tk, n, N, reserve, chunk, tail):
+    params = tk.Params(n_layers=1, n_heads=n, n_kv_heads=n, head_dim=64, seq_lens=[N], sink=4, recent=32, mid_budget=32,
+                       window=16, dtype="f32", force_class=1, max_new_tokens=reserve)
+    kept = -(-N // chunk)
+    over = max(0, N + reserve - kept * chunk)
+    per_unit = -(-(N + reserve) // chunk) if over == 0 else kept + -(-over // tail)
+    info = tk.taskkv_plan(params)
+    assert int(info.max_decode_items) == n * per_unit
+    # what the items take beside the rows: an entry of the table, 64 + 2 floats of partial results; the rest does not depend on them
+    rows = 2 * int(info.pool_rows) * 64 * 4
+    assert abs(int(info.cache_bytes) - rows - n * per_unit * (8 + 66 * 4)) < 40000
+
+
 # ---------------------------------------------------------------- answers that belong to a device
 PER_DEVICE_PROGRAM = r"""
 #include <cstdio>

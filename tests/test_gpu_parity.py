@@ -220,6 +220,57 @@ def test_cluster_decode_equals_the_two_kernels_bit_for_bit(kw, page_rows):
             p.close()
 
 
+# A small cache cuts its retained rows into items of 64 rows and a large reserve into longer ones (here 128 and 512): appended
+# rows on both sides of the change and of an item's end, whole, layer by layer and against 64-bit attention over the rows the
+# cache holds.
+@pytest.mark.parametrize("kw,reserve,items", [(dict(n=8, n_kv=8, d=64, seq_lens=[500], R=5, dtype="f32"), 2000, (8, 128)),
+                                              (dict(n=8, n_kv=4, d=128, seq_lens=[700, 450], R=3, dtype="bf16"), 20000, (11, 512))])
+@pytest.mark.parametrize("page_rows", [0, 64])
+def test_rows_appended_into_a_large_reserve_of_a_small_cache(kw, reserve, items, page_rows):
+    tk, P = _tk(), _parity()
+    wl = small("reserve", N=0, L=16, s1=4, s2=64, k=300, nh=1, steps=4, **kw)
+    qs, ks, vs = W.materialize(wl, DEV)
+    params = tk.params_from_workload(wl, max_new_tokens=reserve)
+    R, G, d, N = wl.n_layers, wl.group, wl.head_dim, wl.seq_lens[0]
+
+    def compress():
+        if not page_rows:
+            return tk.taskkv_compress_ex(params, qs, ks, vs), None
+        info, pages = tk.taskkv_plan_paged(params, page_rows)
+        pool = tk.Pool(page_rows, pages + 12 * int(info.n_units), d, wl.dtype, DEV)
+        return tk.taskkv_compress_paged(params, qs, ks, vs, pool), pool
+
+    (a, pa), (b, pb) = compress(), compress()
+    kept, tail = items
+    edge = kept * 64 - N                         # appended rows that the longest unit's last short item still takes
+    assert kept == -(-N // 64) and edge >= 0
+    appended = 0
+    for stop in (2, edge, edge + 1, edge + tail, edge + tail + 1):
+        if stop < appended:
+            continue
+        while appended < stop:
+            _, kn, vn = W.gen_decode_step(wl, appended % 7, DEV)
+            a.taskkv_append(kn, vn)
+            b.taskkv_append(kn, vn)
+            appended += 1
+        q, kn, vn = W.gen_decode_step(wl, 8, DEV)
+        whole = a.taskkv_decode_step(q, kn, vn)
+        parts = [b.taskkv_decode_step_ex(*(x[:, r:r + 1].contiguous() for x in (q, kn, vn)), r, 1) for r in range(R)]
+        appended += 1
+        assert torch.equal(whole, torch.cat(parts, dim=1)) and torch.equal(whole, a.taskkv_decode(q))
+        for h in range(wl.n_kv_heads):
+            kc, vc = a.pool_rows("k", h).double(), a.pool_rows("v", h).double()
+            want = torch.softmax(q[0, 0, h * G:(h + 1) * G].double().cpu() @ kc.T / d ** 0.5, -1) @ vc
+            assert (whole[0, 0, h * G:(h + 1) * G].double().cpu() - want).abs().max() < P.TOL_OUT[wl.dtype]
+    lens = a.lengths()
+    assert int(lens.max()) == N + appended and lens.tolist() == b.lengths().tolist()
+    assert a.status() == 0 and b.status() == 0
+    for c, pool in ((a, pa), (b, pb)):
+        c.close()
+        if pool:
+            pool.close()
+
+
 @pytest.mark.skipif(torch.cuda.device_count() < 2, reason="needs a second CUDA device")
 def test_second_device_of_a_process_decodes_with_clusters_of_sixteen():
     """Units of 9 to 16 items run in clusters above the portable size, which a function attribute allows device by device."""
