@@ -6,7 +6,7 @@
 // gives its column sums C_b[j] = (1/128) sum_{i in block b} A[i, j].  Then
 //   C[j] = 128 / (G N) * sum over the G query heads of the KV head, and over the blocks b >= j / 128, of C_b[j]
 //   v    = sum_j C[j] V[j, :]
-// with fixed summation orders.  K of a head (N d 2 bytes) is re-read once per block and stays in L2 meanwhile.
+// with fixed summation orders.  K of a head (N d 2 bytes) is walked twice per block and stays in L2 meanwhile.
 #include <algorithm>
 
 #include "common.cuh"
@@ -85,7 +85,7 @@ ExactLayout exact_layout(int64_t hb, int nb, int G, int N, int d, int slices) {
 }
 
 struct ExactShape {
-  int N, d, G, nb, chunks, slices;
+  int N, d, G, nb, slices;
   int64_t q_heads;
   bool ok;
 };
@@ -98,17 +98,19 @@ ExactShape exact_shape(int32_t n_layers, int32_t n_heads, int32_t n_kv_heads, in
   x.d = head_dim;
   x.G = n_heads / n_kv_heads;
   x.nb = (x.N + kBlockRows - 1) / kBlockRows;
-  x.chunks = (x.nb * kBlockRows + kTcChunk - 1) / kTcChunk;
   x.slices = (x.N + kSliceKeys - 1) / kSliceKeys;
   x.q_heads = (int64_t)n_layers * n_heads;
-  x.ok = (int64_t)x.nb * x.G * x.chunks <= (1 << 24);
+  // the longest sequences with many query heads to a KV head are refused: the least a batch can be, one KV group, is then
+  // more than 2^28 tiles of 128 rows x 128 keys
+  x.ok = (int64_t)x.nb * x.G * ((x.nb + 15) / 16) <= (1 << 24);
   return x;
 }
-// Most query heads per batch: whole KV groups, a work-item count that fits an int, scratch within `budget` bytes
-// (0 if not even one group fits).
+// Most query heads per batch: whole KV groups, as many as a launch takes (grid dimension y of the sums: a KV head each;
+// blocks of 128 query rows in one launch of the prefix kernel), scratch within `budget` bytes (0 if not even one group fits).
 int64_t exact_heads_per_batch(const ExactShape& x, size_t budget) {
   int64_t hb = x.q_heads;
-  while (hb > x.G && hb * x.nb * x.chunks > (1 << 30)) hb -= x.G;
+  hb = std::min<int64_t>(hb, (int64_t)65535 * x.G);
+  hb = std::max<int64_t>(x.G, std::min<int64_t>(hb, 0x3fffffff / x.nb / x.G * x.G));
   while (hb > x.G && exact_layout(hb, x.nb, x.G, x.N, x.d, x.slices).total > budget)
     hb = std::max<int64_t>(x.G, hb / 2 / x.G * x.G);
   return exact_layout(hb, x.nb, x.G, x.N, x.d, x.slices).total <= budget ? hb : 0;

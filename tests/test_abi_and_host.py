@@ -230,6 +230,21 @@ def test_decode_items_of_a_reserve(tk, n, N, reserve, chunk, tail):
     assert abs(int(info.cache_bytes) - rows - n * per_unit * (8 + 66 * 4)) < 40000
 
 
+@pytest.mark.parametrize("heads,kv", [(1, 1), (8, 2)])
+def test_exact_semantic_batches_stay_within_a_launch(tk, heads, kv):
+    """The sums' launches take a KV head per block along y, 65535 at most: what a longer list of heads needs as scratch is
+    that of a batch of so many (here one whose scratch would fit the library's own budget at once)."""
+    most = 65535 // kv * kv
+    full = int(tk.lib.taskkv_exact_semantic_bytes(most // kv, heads, kv, 64, 128))
+    assert full > 0
+    for layers in (70000 // kv, 140000 // kv):
+        got = int(tk.lib.taskkv_exact_semantic_bytes(layers, heads, kv, 64, 128))
+        assert full <= got <= full * 65535 / most + 4096
+    # one KV group of the longest sequences: accepted and refused as before
+    assert int(tk.lib.taskkv_exact_semantic_bytes(1, 4, 1, 128, 1 << 20)) > 0
+    assert int(tk.lib.taskkv_exact_semantic_bytes(1, 8, 1, 128, 1 << 20)) == 0
+
+
 # ---------------------------------------------------------------- answers that belong to a device
 PER_DEVICE_PROGRAM = r"""
 #include <cstdio>
