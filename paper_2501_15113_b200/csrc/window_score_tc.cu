@@ -176,8 +176,9 @@ enum : int {
 // ROWS (32, 64 or 128: columns of an accumulator) is a template argument also for the sake of registers: with 128 rows the
 // gather of another chunk of layers shares the SMs with this kernel, and how many of its blocks (6144 registers) fit beside
 // a CTA is decided here.  One kernel for all row counts took 168 registers a thread, which leaves room for one gather block:
-// 7.0 -> 7.5 ms for 32 layers of 131072 keys; this one takes 128, room for three.
-template <int D, int ROWS>
+// 7.0 -> 7.5 ms for 32 layers of 131072 keys; this one takes 128, room for three.  FILLED: the window has ROWS rows; the
+// masks of the others cost full windows 0.5 us a layer of 8191 keys if they are only known at run time.
+template <int D, int ROWS, bool FILLED>
 __global__ void __launch_bounds__(kThreads, 1)
 window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __grid_constant__ TcArgs a,
                  TcLayout lay) {
@@ -513,7 +514,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
           float cs[4] = {0.f, 0.f, 0.f, 0.f};   // four interleaved chains (FMA latency)
           // A row that the window does not have is a zero query, and its score at a key with an infinite element is NaN:
           // such rows are left out, not given a weight of zero.
-          if (rows >= 64 && !tail && p.rows == rows) {
+          if (rows >= 64 && !tail && FILLED) {
             // 64 columns per TMEM load: half the load / wait round trips of the 32-column walk below
             for (int c0 = 0; c0 < rows; c0 += 64) {
               uint32_t r[64];
@@ -535,7 +536,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
             tc_wait_ld();
             const float4* mx4 = reinterpret_cast<const float4*>(myStat);
             const float4* wt4 = reinterpret_cast<const float4*>(myStat + 32);
-            uint32_t vm = p.rows >= 32 ? 0xffffffffu : (1u << p.rows) - 1u;   // bit c: window row c sees this thread's key
+            uint32_t vm = FILLED ? 0xffffffffu : (1u << p.rows) - 1u;   // bit c: window row c sees this thread's key
             if (tail) {
               const int need = j < N ? j - (N - L) : L;        // the residue c % L the row must reach (L: none does)
               int res = 0;
@@ -558,7 +559,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
               }
             }
           } else
-          for (int c0 = 0; c0 < p.rows; c0 += 32) {
+          for (int c0 = 0; c0 < (FILLED ? rows : p.rows); c0 += 32) {
             uint32_t r[32];
             tc_ld32(taddr + (uint32_t)c0, r);
             tc_wait_ld();
@@ -570,7 +571,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
                 const float o4[4] = {off.x, off.y, off.z, off.w};
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                  if (c0 + c + i < p.rows) cs[i] += ex2(fmaf(__uint_as_float(r[c + i]), scale2, -o4[i]));
+                  if (FILLED || c0 + c + i < p.rows) cs[i] += ex2(fmaf(__uint_as_float(r[c + i]), scale2, -o4[i]));
               }
             } else {
               // window row c0 + c sees keys up to N - L + (c0 + c) % L.  The residue is counted along (one
@@ -580,7 +581,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
 #pragma unroll
               for (int c = 0; c < 32; ++c) {
                 const float off = myStat[c0 + c];
-                const bool vis = (j < N) && (need <= res) && (c0 + c < p.rows);
+                const bool vis = (j < N) && (need <= res) && (FILLED || c0 + c < p.rows);
                 if (vis) cs[c & 3] += ex2(fmaf(__uint_as_float(r[c]), scale2, -off));
                 res = (res + 1 == L) ? 0 : res + 1;
               }
@@ -680,14 +681,14 @@ inline int pick_chunk(int64_t units_times_keys, int n_sm, int least) {
   return chunk;
 }
 
-template <int D, int ROWS>
+template <int D, int ROWS, bool FILLED>
 cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStream_t s, int layer0, int n_layers) {
   const int n_sm = sm_count();
   constexpr int rows = ROWS;
   const TcLayout lay = make_layout(D, rows);
   if (lay.stages < 2) return cudaErrorInvalidValue;
   const int smem = lay.total;
-  cudaError_t e = cudaFuncSetAttribute(window_tc_kernel<D, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(window_tc_kernel<D, ROWS, FILLED>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const int per_seq_all = p.R * p.n_kv;
   const int first = layer0 * p.n_kv;               // the launch covers units [first, first + per_seq) of every sequence
@@ -730,7 +731,7 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
       const int items = a.item_off[nb], grid = items < n_sm ? items : n_sm;
       a.steps = (items + grid - 1) / grid;
       LaunchScope ls(K_WINDOW_TC, s);
-      return launch_dependent_smem(window_tc_kernel<D, ROWS>, (unsigned)grid, kThreads, (size_t)smem, s, maps, p, a, lay);
+      return launch_dependent_smem(window_tc_kernel<D, ROWS, FILLED>, (unsigned)grid, kThreads, (size_t)smem, s, maps, p, a, lay);
     };
     if (h.lse) {
       // the caller already has the rows' normalisers: no pass 1
@@ -756,6 +757,13 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
   return cudaSuccess;
 }
 
+template <int ROWS>
+cudaError_t launch_tc_rows(const DeviceProblem& p, const WindowHostInfo& h, cudaStream_t s, int layer0, int n_layers) {
+  if (p.rows == ROWS)
+    return p.d == 64 ? launch_tc_d<64, ROWS, true>(p, h, s, layer0, n_layers) : launch_tc_d<128, ROWS, true>(p, h, s, layer0, n_layers);
+  return p.d == 64 ? launch_tc_d<64, ROWS, false>(p, h, s, layer0, n_layers) : launch_tc_d<128, ROWS, false>(p, h, s, layer0, n_layers);
+}
+
 }  // namespace
 
 bool window_tc_supported(const DeviceProblem& p, int dtype) {
@@ -768,9 +776,9 @@ cudaError_t launch_window_scores_tc(const DeviceProblem& p, const WindowHostInfo
   // 32 window rows and sequences short enough for a unit's scores to stay in tensor memory: K is read once
   if (window_res_supported(p, h)) return launch_window_scores_res(p, h, s, layer0, n_layers);
   switch (tc_rows(p.rows)) {
-    case 32: return p.d == 64 ? launch_tc_d<64, 32>(p, h, s, layer0, n_layers) : launch_tc_d<128, 32>(p, h, s, layer0, n_layers);
-    case 64: return p.d == 64 ? launch_tc_d<64, 64>(p, h, s, layer0, n_layers) : launch_tc_d<128, 64>(p, h, s, layer0, n_layers);
-    default: return p.d == 64 ? launch_tc_d<64, 128>(p, h, s, layer0, n_layers) : launch_tc_d<128, 128>(p, h, s, layer0, n_layers);
+    case 32: return launch_tc_rows<32>(p, h, s, layer0, n_layers);
+    case 64: return launch_tc_rows<64>(p, h, s, layer0, n_layers);
+    default: return launch_tc_rows<128>(p, h, s, layer0, n_layers);
   }
 }
 
