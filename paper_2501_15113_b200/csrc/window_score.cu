@@ -2,8 +2,7 @@
 //   S = Q_win K^T / sqrt(d), causal mask on the last L keys, row softmax,
 //   C[j] = mean over the unit's G*L window rows of the normalised weights.
 //
-// Generic two-pass path on the CUDA cores (fp32 accumulate), used for fp32
-// inputs (bf16 runs on the tensor cores; it comes here only where the driver has no tensor maps to give):
+// Two-pass path on the CUDA cores for fp32 inputs (bf16 runs on the tensor cores):
 //   pass 1  per (unit, 256-key chunk): row maxima and exp-sums  -> partial stats
 //   reduce  per unit: combine chunks -> (row max, 1 / row sum); units of up to 32 chunks need no launch for it,
 //           their pass-2 blocks combine the chunks themselves
@@ -80,10 +79,11 @@ __device__ void fold_unit(const DeviceProblem& p, int u, int chunks, float2* tmp
 }
 
 // fold: pass 2 combines the chunks itself (p.stat is not used).
-template <typename T, int D, int ROWS, int PASS>
+template <int D, int ROWS, int PASS>
 __global__ void __launch_bounds__(kBlock) window_pass_kernel(DeviceProblem p, UnitRange ur, int grid_chunks, int fold) {
   using W = WinTile<ROWS>;
   constexpr int RPT = W::RPT, NTY = W::NTY, NTX = W::NTX, KPT = W::KPT;
+  using T = float;
   constexpr int VN = Vec16<T>::N;
   constexpr int VPR = kDepth / VN;                       // 16-byte vectors of one key row of a stage
   constexpr int VPT = kTile * VPR / kBlock;              // vectors per thread and stage
@@ -268,15 +268,15 @@ __global__ void lse_to_stat_kernel(DeviceProblem p, int u0, const float* __restr
   else reinterpret_cast<float2*>(p.stat)[u * p.rows_pad + row] = make_float2(v, 1.0f);
 }
 
-template <typename T, int D, int ROWS>
+template <int D, int ROWS>
 cudaError_t launch_generic_rows(const DeviceProblem& p, int max_N, const WindowHostInfo& h, cudaStream_t s, int layer0,
                                 int n_layers) {
   constexpr size_t smem = win_smem<D, ROWS>();
   static_assert((size_t)kTile * kPitch >= 2 * (size_t)ROWS * (WinTile<ROWS>::NTX + 1), "pass 1's pairs reuse the key tile");
   cudaError_t e;
-  e = cudaFuncSetAttribute(window_pass_kernel<T, D, ROWS, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = cudaFuncSetAttribute(window_pass_kernel<D, ROWS, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(window_pass_kernel<T, D, ROWS, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = cudaFuncSetAttribute(window_pass_kernel<D, ROWS, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const UnitRange ur = layer_range(p, h.batch, layer0, n_layers);
   const int chunks = (max_N + kScoreChunk - 1) / kScoreChunk;
@@ -293,7 +293,7 @@ cudaError_t launch_generic_rows(const DeviceProblem& p, int max_N, const WindowH
   } else {
     {
       LaunchScope ls(K_WINDOW_STATS, s);
-      window_pass_kernel<T, D, ROWS, 1><<<(unsigned)grid, kBlock, smem, s>>>(p, ur, chunks, 0);
+      window_pass_kernel<D, ROWS, 1><<<(unsigned)grid, kBlock, smem, s>>>(p, ur, chunks, 0);
     }
     if (!fold) {
       LaunchScope ls(K_WINDOW_REDUCE, s);
@@ -303,20 +303,20 @@ cudaError_t launch_generic_rows(const DeviceProblem& p, int max_N, const WindowH
   }
   {
     LaunchScope ls(K_WINDOW_SCORES, s);
-    if (h.lse) window_pass_kernel<T, D, ROWS, 2><<<(unsigned)grid, kBlock, smem, s>>>(p, ur, chunks, 0);
-    else e = launch_dependent_smem(window_pass_kernel<T, D, ROWS, 2>, (unsigned)grid, kBlock, smem, s, p, ur, chunks, fold);
+    if (h.lse) window_pass_kernel<D, ROWS, 2><<<(unsigned)grid, kBlock, smem, s>>>(p, ur, chunks, 0);
+    else e = launch_dependent_smem(window_pass_kernel<D, ROWS, 2>, (unsigned)grid, kBlock, smem, s, p, ur, chunks, fold);
     if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
 }
 
-template <typename T, int D>
+template <int D>
 cudaError_t launch_generic(const DeviceProblem& p, int max_N, const WindowHostInfo& h, cudaStream_t s, int layer0,
                            int n_layers) {
-  if (p.rows <= 16) return launch_generic_rows<T, D, 16>(p, max_N, h, s, layer0, n_layers);
-  if (p.rows <= 32) return launch_generic_rows<T, D, 32>(p, max_N, h, s, layer0, n_layers);
-  if (p.rows <= 64) return launch_generic_rows<T, D, 64>(p, max_N, h, s, layer0, n_layers);
-  return launch_generic_rows<T, D, 128>(p, max_N, h, s, layer0, n_layers);
+  if (p.rows <= 16) return launch_generic_rows<D, 16>(p, max_N, h, s, layer0, n_layers);
+  if (p.rows <= 32) return launch_generic_rows<D, 32>(p, max_N, h, s, layer0, n_layers);
+  if (p.rows <= 64) return launch_generic_rows<D, 64>(p, max_N, h, s, layer0, n_layers);
+  return launch_generic_rows<D, 128>(p, max_N, h, s, layer0, n_layers);
 }
 
 }  // namespace
@@ -331,14 +331,9 @@ cudaError_t launch_lse_to_stat(const DeviceProblem& p, int u0, int n_units, cons
 cudaError_t launch_window_scores(const DeviceProblem& p, int dtype, int max_N, const WindowHostInfo& h,
                                  cudaStream_t s, int layer0, int n_layers) {
   if (n_layers < 0) { layer0 = 0; n_layers = p.R; }
-  // bf16 runs on the tensor cores; everything else here
   if (window_tc_supported(p, dtype)) return launch_window_scores_tc(p, h, s, layer0, n_layers);
-  if (dtype == TASKKV_F32) {
-    return p.d == 64 ? launch_generic<float, 64>(p, max_N, h, s, layer0, n_layers)
-                     : launch_generic<float, 128>(p, max_N, h, s, layer0, n_layers);
-  }
-  return p.d == 64 ? launch_generic<__nv_bfloat16, 64>(p, max_N, h, s, layer0, n_layers)
-                   : launch_generic<__nv_bfloat16, 128>(p, max_N, h, s, layer0, n_layers);
+  if (dtype != TASKKV_F32) return cudaErrorNotSupported;      // bf16 without the driver's tensor maps
+  return p.d == 64 ? launch_generic<64>(p, max_N, h, s, layer0, n_layers) : launch_generic<128>(p, max_N, h, s, layer0, n_layers);
 }
 
 }  // namespace taskkv
