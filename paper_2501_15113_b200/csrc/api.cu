@@ -94,9 +94,9 @@ void pick_decode_items(HostPlan& hp, const taskkv_params* p, int n_model) {
   while ((1 << least) < kDecodeChunkMin) ++least;
   while ((1 << most) < kDecodeChunk) ++most;
   hp.dec_shift = most;
-  while (hp.dec_shift > least && decode_items(hp, p, n_model, hp.dec_shift, hp.dec_shift, 0) < 2 * 148) --hp.dec_shift;
+  while (hp.dec_shift > least && decode_items(hp, p, n_model, hp.dec_shift, hp.dec_shift, 0) < 2 * kSms) --hp.dec_shift;
   hp.dec_tail = hp.dec_shift;
-  while (hp.dec_tail < most && decode_items(hp, p, n_model, hp.dec_shift, hp.dec_tail, p->max_new_tokens) > 8 * 148) ++hp.dec_tail;
+  while (hp.dec_tail < most && decode_items(hp, p, n_model, hp.dec_shift, hp.dec_tail, p->max_new_tokens) > 8 * kSms) ++hp.dec_tail;
 }
 
 taskkv_status make_plan(const taskkv_params* p, HostPlan& hp, int32_t page_rows = 0) {
@@ -219,8 +219,8 @@ taskkv_status make_plan(const taskkv_params* p, HostPlan& hp, int32_t page_rows 
   hp.c_total = c_total;
   hp.rows = G * p->window;
   hp.rows_pad = (hp.rows + 15) / 16 * 16;
-  // partial-statistic slots per unit: one per 1024-key chunk on the CUDA-core path, one per epilogue warp and
-  // work item on the tensor-core path
+  // partial-statistic slots per unit: one per 256-key chunk on the CUDA-core path, one per epilogue warp and 2048 keys on
+  // the tensor-core path
   {
     const int generic = (hp.max_N + kScoreChunk - 1) / kScoreChunk;
     const int tc = (hp.max_N + kTcChunk - 1) / kTcChunk * kTcParts;

@@ -16,8 +16,9 @@ constexpr int kDecodeChunkMin = 64;               // fewest
 constexpr int kDecodeFewItems = 32;               // most items of a unit that a cluster takes or one warp merges
 constexpr int kGatherRows = 64;                   // rows of one gather item
 constexpr int kScoreChunk = 256;                  // keys of one window-score work item (CUDA-core path)
-constexpr int kTcChunk = 2048;                    // fewest keys of one window-score work item (tensor-core path)
-constexpr int kTcParts = 8;                       // partial-statistic slots per work item (one per epilogue warp)
+constexpr int kTcChunk = 2048;                    // keys that one set of partial statistics covers (tensor-core path)
+constexpr int kTcParts = 8;                       // partial statistics per set (one per epilogue warp)
+constexpr int kSms = 148;                         // SMs of a B200: what plans, made without a device, and grids count with
 constexpr float kLog2e = 1.4426950408889634f;
 
 // kernel ids for launch counting / timing
@@ -241,7 +242,7 @@ inline int sm_count() {
   const int dev = current_device();
   return known.get(dev, 0, [dev] {
     int n = 0;
-    return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0 ? n : 148;
+    return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0 ? n : kSms;
   });
 }
 

@@ -913,7 +913,7 @@ int cluster_size(const DeviceProblem& p) {
   if (p.items_cap > kClusterItems || p.dec_tail != p.dec_shift) return 0;
   int cs = 1;
   while (cs < p.items_kept || kClusterSlots * cs < p.items_cap) cs *= 2;
-  if (cs > kClusterMax || (int64_t)p.view_U * cs > 148 * 2) return 0;
+  if (cs > kClusterMax || (int64_t)p.view_U * cs > 2 * kSms) return 0;
   return cs;
 }
 
@@ -949,22 +949,16 @@ cudaError_t launch_typed(const DeviceProblem& p, const void* q, const int32_t* l
                            : launch_cluster<T, D, G, false>(p, cs, qt, lengths, kn, vn, static_cast<T*>(out), s, early);
   }
   // persistent blocks: 16 per SM (measured best on B200 with 512-row items)
-  int64_t grid = p.max_items < 148 * 16 ? p.max_items : 148 * 16;
+  int64_t grid = p.max_items < 16 * kSms ? p.max_items : 16 * kSms;
   if (grid < 1) grid = 1;
   cudaError_t e;
   {
     LaunchScope ls(K_DECODE_ATTN, s);
-    if (p.page_rows > 0) {
-      if constexpr (sizeof(T) == 2)
-        e = launch_dependent(decode_attn_kernel<T, D, G, true>, (unsigned)grid, kAttnThreads, s, p, static_cast<const T*>(q), lengths, kn, vn, static_cast<T*>(out), early);
-      else
-        e = launch_dependent(decode_attn_kernel<T, D, G, true>, (unsigned)grid, kAttnThreads, s, p, static_cast<const T*>(q), lengths, kn, vn, static_cast<T*>(out), early);
-    } else {
-      if constexpr (sizeof(T) == 2)
-        e = launch_dependent(decode_attn_kernel<T, D, G, false>, (unsigned)grid, kAttnThreads, s, p, static_cast<const T*>(q), lengths, kn, vn, static_cast<T*>(out), early);
-      else
-        e = launch_dependent(decode_attn_kernel<T, D, G, false>, (unsigned)grid, kAttnThreads, s, p, static_cast<const T*>(q), lengths, kn, vn, static_cast<T*>(out), early);
-    }
+    const T* qt = static_cast<const T*>(q);
+    e = p.page_rows > 0 ? launch_dependent(decode_attn_kernel<T, D, G, true>, (unsigned)grid, kAttnThreads, s, p, qt, lengths, kn,
+                                           vn, static_cast<T*>(out), early)
+                        : launch_dependent(decode_attn_kernel<T, D, G, false>, (unsigned)grid, kAttnThreads, s, p, qt, lengths, kn,
+                                           vn, static_cast<T*>(out), early);
   }
   if (e != cudaSuccess) return e;
   {
@@ -973,13 +967,13 @@ cudaError_t launch_typed(const DeviceProblem& p, const void* q, const int32_t* l
     // units of at most 16 items each (32, if a block per head would be more than the GPU holds at once): a warp per head.
     // Otherwise a block per head; up to 16 of them per SM the variant that loads ahead (its blocks are resident within a
     // few waves)
-    if (p.items_cap <= ((int64_t)p.view_U * G > 148 * 4 ? kDecodeFewItems : kDecodeFewItems / 2))
+    if (p.items_cap <= ((int64_t)p.view_U * G > 4 * kSms ? kDecodeFewItems : kDecodeFewItems / 2))
       e = launch_dependent(decode_combine_few_kernel<T, D, G>, (unsigned)((p.view_U * G + kCombineWarps - 1) / kCombineWarps),
                            kCombineThreads, s, p, lengths, fused, static_cast<T*>(out));
     else if (p.dec_tail != p.dec_shift)      // (fewer than 296 items after compression, so fewer units than that)
       e = launch_dependent(decode_combine_kernel<T, D, G, 8, true>, (unsigned)(p.view_U * G), kCombineThreads, s, p, lengths,
                            fused, static_cast<T*>(out));
-    else if ((int64_t)p.view_U * G <= 148 * 16)
+    else if ((int64_t)p.view_U * G <= 16 * kSms)
       e = launch_dependent(decode_combine_kernel<T, D, G, 8, false>, (unsigned)(p.view_U * G), kCombineThreads, s, p, lengths,
                            fused, static_cast<T*>(out));
     else

@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(256) na_combine_kernel(NaArgs a) {
 template <typename T, int D, int G>
 cudaError_t na_launch(const NaArgs& a, cudaStream_t s) {
   const int64_t total = (int64_t)a.n_units * a.splits;
-  const unsigned grid = (unsigned)(total < 148 * 8 ? total : 148 * 8);
+  const unsigned grid = (unsigned)(total < 8 * kSms ? total : 8 * kSms);
   {
     LaunchScope ls(K_DECODE_ATTN, s);
     na_attn_kernel<T, D, G><<<grid, kNaThreads, 0, s>>>(a);

@@ -6,7 +6,7 @@
 //   warp 0          TMA producer: K tiles of 128 keys (four stages), the block's Q rows (two buffers, one block ahead)
 //   warps 1, 6      tcgen05.mma issuers, alternate tiles; four accumulators of 128 columns in TMEM
 //   warps 2-5, 7-18 four epilogue groups, every fourth tile each
-// First walk: D[row, key] = Q K^T, a TMEM lane is a query row and keeps its own running (max, sum); the two groups'
+// First walk: D[row, key] = Q K^T, a TMEM lane is a query row and keeps its own running (max, sum); the four groups'
 // pairs meet in shared memory.  Second walk: D[key, row] = K Q^T, a lane is a key and sums its column.
 // Bound by the special-function unit: two exponentials per score at 16 a cycle and SM, 2048 cycles per tile and block.
 // Blocks are dealt out longest first, in both directions alternately, so that every CTA gets the same number of tiles;

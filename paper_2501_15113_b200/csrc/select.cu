@@ -546,7 +546,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_fast_kernel(DeviceProblem 
   }
   if (kmid == 0) return;
 
-  // pooled window sums in ascending position: ext = [3 left neighbours][32 own][3 right neighbours]
+  // pooled window sums in ascending position: ext = [3 left neighbours][EPT own][3 right neighbours]
   if (POOL_HALF > 0) {
     float ext[EPT + 2 * POOL_HALF];
 #pragma unroll
@@ -579,11 +579,11 @@ __global__ void __launch_bounds__(kThreads, 1) select_fast_kernel(DeviceProblem 
 
 // ---------------------------------------------------------------------------
 // Cluster variant for 32768 < N <= 262144 (and pooling kernel 1 or 7): a thread-block cluster of 2, 4 or 8 CTAs
-// owns a unit, CTA c keeps positions [32768 c, 32768 (c + 1)) in registers exactly as select_fast_kernel does, and
-// every block-wide count becomes a cluster-wide one: each warp leaves its count in a slot of every CTA's shared
-// memory (distributed shared memory), one cluster barrier, and every thread adds up all slots.  The slots are
-// double-buffered by step parity: a slot is rewritten two barriers after it was read.  Same results as the other
-// two kernels: exact k-th key, lower position first among equal keys, pooled sums added in ascending position.
+// owns a unit, CTA c keeps positions [32768 c, 32768 (c + 1)) in registers exactly as select_fast_kernel does.  A
+// refinement's histograms are read from all CTAs through distributed shared memory between two cluster barriers (all are
+// complete before they are read; none is cleared before all have read it), and every CTA adds them up for itself, so
+// that all refine the same range.  Same results as the other two kernels: exact k-th key, lower position first
+// among equal keys, pooled sums added in ascending position.
 constexpr int kMaxCS = 8;
 
 struct ClusterSmem {
