@@ -168,45 +168,53 @@ def test_shapes_and_edge_cases(case):
 
 
 # Small decode calls run as one launch of clusters (up to 16 CTAs a unit, up to two items a CTA), larger ones as attention
-# and combine kernels; the same cache is decoded whole (the kernels) and layer by layer (the clusters), or the other way
-# round, and gives the same bits.  Prompt lengths around the items' 64 ... 512 rows; grown past one item boundary.
+# and combine kernels; the same cache is decoded whole (the kernels) and layer by layer (the clusters) and gives the same
+# bits, fused steps and the paged layout included; a cache of one layer, whose whole call is a cluster launch, is compared with one that a
+# large reserve gives the kernels.  Prompt lengths around the items' 64 and 512 rows; grown past one item boundary.
 @pytest.mark.parametrize("kw", [dict(n=4, n_kv=4, d=64, seq_lens=[127], R=1, dtype="f32"),
-                                dict(n=8, n_kv=4, d=128, seq_lens=[513, 300], R=2, dtype="f32"),
+                                dict(n=8, n_kv=4, d=128, seq_lens=[513, 300], R=3, dtype="f32"),
+                                dict(n=16, n_kv=8, d=64, seq_lens=[510], R=6, dtype="f32"),
                                 dict(n=32, n_kv=32, d=128, seq_lens=[4095], R=10, dtype="bf16"),
                                 dict(n=32, n_kv=32, d=64, seq_lens=[4090], R=10, dtype="bf16"),
                                 dict(n=32, n_kv=4, d=128, seq_lens=[8190], R=20, dtype="bf16"),
-                                dict(n=8, n_kv=4, d=64, seq_lens=[2047, 900], R=3, dtype="bf16")])
+                                dict(n=8, n_kv=4, d=64, seq_lens=[1022, 900], R=3, dtype="bf16")])
 @pytest.mark.parametrize("page_rows", [0, 64])
 def test_cluster_decode_equals_the_two_kernels_bit_for_bit(kw, page_rows):
     tk = _tk()
     wl = small("cldec", N=0, L=16, s1=4, s2=64, k=300, nh=1, steps=4, **kw)
     qs, ks, vs = W.materialize(wl, DEV)
-    params = tk.params_from_workload(wl, max_new_tokens=8)
     R = wl.n_layers
 
-    def compress():
+    def compress(reserve=8):
+        params = tk.params_from_workload(wl, max_new_tokens=reserve)
         if not page_rows:
             return tk.taskkv_compress_ex(params, qs, ks, vs), None
         info, pages = tk.taskkv_plan_paged(params, page_rows)
         pool = tk.Pool(page_rows, pages + int(info.n_units), wl.head_dim, wl.dtype, DEV)
         return tk.taskkv_compress_paged(params, qs, ks, vs, pool), pool
 
+    def launches(want, call):
+        before = tk.lib.taskkv_launch_count()
+        out = call()
+        assert tk.lib.taskkv_launch_count() - before == want, "not the kernels this case is about"
+        return out
+
     (a, pa), (b, pb) = compress(), compress()
     P = _parity()
-    if not page_rows and R > 1:
-        # a reserve of 32 items makes the whole call's merge the block per head, not the warp per head
-        far = tk.taskkv_compress_ex(tk.params_from_workload(wl, max_new_tokens=32 * 512), qs, ks, vs)
-        q, _, _ = W.gen_decode_step(wl, 9, DEV)
-        assert torch.equal(far.taskkv_decode(q), a.taskkv_decode(q))
-        far.close()
+    # a reserve of 32 items makes the whole call's merge the block per head, not the warp per head
+    far, pf = compress(32 * 512)
     for s in range(4):
         q, kn, vn = W.gen_decode_step(wl, s, DEV)
-        whole = a.taskkv_decode_step(q, kn, vn)
-        parts = [b.taskkv_decode_step_ex(*(x[:, r:r + 1].contiguous() for x in (q, kn, vn)), r, 1) for r in range(R)]
+        whole = launches(2 if R > 1 else 1, lambda: a.taskkv_decode_step(q, kn, vn))
+        parts = launches(R, lambda: [b.taskkv_decode_step_ex(*(x[:, r:r + 1].contiguous() for x in (q, kn, vn)), r, 1)
+                                     for r in range(R)])
         assert torch.equal(whole, torch.cat(parts, dim=1))
-        again = [b.taskkv_decode_ex(q[:, r:r + 1].contiguous(), r, 1) for r in range(R)]   # the row just appended included
-        assert torch.equal(whole, torch.cat(again, dim=1))
-    assert a.status() == 0 and b.status() == 0 and a.lengths().tolist() == b.lengths().tolist()
+        again = launches(R, lambda: [b.taskkv_decode_ex(q[:, r:r + 1].contiguous(), r, 1) for r in range(R)])
+        assert torch.equal(whole, torch.cat(again, dim=1))                 # the row just appended included
+        assert torch.equal(whole, launches(2, lambda: far.taskkv_decode_step(q, kn, vn)))
+        assert torch.equal(whole, launches(2, lambda: far.taskkv_decode(q)))
+    for c in (a, b, far):
+        assert c.status() == 0 and c.lengths().tolist() == a.lengths().tolist()
     # the first layer of sequence 0 against 64-bit attention over the rows the cache holds
     G, d = wl.group, wl.head_dim
     for h in range(wl.n_kv_heads):
@@ -214,7 +222,7 @@ def test_cluster_decode_equals_the_two_kernels_bit_for_bit(kw, page_rows):
         sc = q[0, 0, h * G:(h + 1) * G].double().cpu() @ kc.T / d ** 0.5
         want = torch.softmax(sc, -1) @ vc
         assert (whole[0, 0, h * G:(h + 1) * G].double().cpu() - want).abs().max() < P.TOL_OUT[wl.dtype]
-    for c, p in ((a, pa), (b, pb)):
+    for c, p in ((a, pa), (b, pb), (far, pf)):
         c.close()
         if p:
             p.close()
@@ -299,6 +307,27 @@ def test_second_device_of_a_process_decodes_with_clusters_of_sixteen():
                                      (1, 16, 64, 32769), (2, 16, 128, 33000)])
 def test_windows_of_every_size(G, L, d, N, dtype):
     run_workload(small("winrows", n=4 * G, n_kv=4, d=d, N=N, L=L, s1=4, s2=32, k=40, dtype=dtype, nh=0, t=64, steps=1))
+
+
+# The scores against 64 bits, over windows that fill a tile and windows that do not: a score's exponent (up to ~16 in log2
+# units) is rounded to 2^-21, i.e. its exponential to 2^-21 ln 2 = 3.3e-7, a row's normaliser is a sum of such terms in a tree
+# (a few units of 6e-8), and the scale of the scores is rounded once (6e-8 of an exponent of up to 16): under 1e-6 in the
+# 2-norm.  Measured: 0.9e-7 to 3.2e-7.
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("G,L,d,N", [(1, 9, 64, 6001), (1, 9, 128, 33000), (1, 32, 128, 33000), (2, 17, 64, 3001), (2, 24, 128, 9001),
+                                     (2, 32, 128, 9001), (4, 17, 64, 9001), (4, 31, 128, 9001), (4, 32, 128, 9001)])
+def test_window_scores_error_against_64_bits(G, L, d, N, dtype):
+    tk = _tk()
+    wl = small("err64", n=8 * G, n_kv=8, d=d, N=N, L=L, s1=4, s2=32, k=40, dtype=dtype, nh=0, t=64, steps=1, variance=0.5)
+    qs, ks, vs = W.materialize(wl, DEV)
+    cache = tk.taskkv_compress_ex(tk.params_from_workload(wl, max_new_tokens=0), qs, ks, vs)
+    got = torch.from_numpy(cache.query(tk.Q_SCORES)).reshape(8, -1)[:, :N].double().to(DEV)
+    cache.close()
+    s = torch.einsum("hrd,hjd->hrj", qs[0][0].double().view(8, G * L, d), ks[0][0].double()) / d ** 0.5
+    last = N - L + torch.arange(G * L, device=DEV) % L
+    s.masked_fill_(torch.arange(N, device=DEV)[None] > last[:, None], -float("inf"))
+    want = torch.softmax(s, -1).mean(1)
+    assert float((got - want).norm() / want.norm()) < 1e-6
 
 
 # A key with an infinite element that every window row scores -inf weighs nothing, whatever fills the window's tile up: a zero
