@@ -11,10 +11,13 @@ Prints ONE JSON line.  `value` is decode attention steps per second (all layers
 per step), measured on the device with inputs resident in HBM; compression
 tokens per second is reported beside it, and `e2e` repeats the measurement
 through the host-buffer entry points with the copies inside the timed region.
-On one GPU the line also carries, under `workloads`, the same device-timed
-measurement of the other single-GPU workloads: the Llama-3-8B-shaped
+On one GPU the line also carries, under `workloads`, the times of the same
+device-timed measurement of the other single-GPU workloads: the Llama-3-8B-shaped
 grouped-query stack, the Mistral-7B-shaped ragged batch and the 15 points of
-the budget sweep (`--no-extra` skips them).
+the budget sweep (`--no-extra` skips them), [compress ms, decode ms per step]
+each.  Per-kernel times and the other records in full, which would make the line
+too long for readers that keep only the end of a log, go to stderr, a JSON object
+to a line.
 `--impl reference` times the CPU oracle on a bounded sample instead; that arm
 never builds or loads the CUDA library.
 """
@@ -254,6 +257,41 @@ def measure_workload(tk, W, wl, dev, steps, warmup, policy, peak, peak_kind, sam
 EXTRA_WORKLOADS = ["llama3", "mistral"] + [f"sweep:{h}:{k}" for h in (0, 1, 2, 4, 8) for k in (64, 256, 1024)]
 
 
+def digits(x, n):
+    """Floats rounded to n significant digits."""
+    if isinstance(x, dict):
+        return {k: digits(v, n) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [digits(v, n) for v in x]
+    return float(f"{x:.{n}g}") if isinstance(x, float) else x
+
+
+# records that go to stderr in full: the name that a figure of theirs gets in the line, and where it is
+DETAILS = {"per_pass": {}, "kernels": {},
+           "latency_mode": {"layer_by_layer_ms_per_token": "eager_ms_per_token", "layer_by_layer_graph_ms_per_token": "graph_ms_per_token"},
+           "layer_streamed_compress": {"layer_streamed_compress_ms": "total_ms"},
+           "compress_with_window_lse": {"compress_with_window_lse_ms": "compress_ms"},
+           "paged_cache": {"paged_compress_ms": "compress_ms", "paged_decode_ms_per_step": "decode_ms_per_step"},
+           "exact_semantic": {"exact_semantic_ms": "ms"}}
+
+
+def print_line(line):
+    """The JSON line on stdout, the records in full on stderr."""
+    out = {}
+    for key, v in line.items():
+        if key == "workloads":
+            for name, rec in v.items():
+                print(json.dumps({"workload": name, "record": rec}), file=sys.stderr)
+            out[key] = {name: rec.get("error") or digits([rec["compress_ms"], rec["decode_ms_per_step"]], 4)
+                        for name, rec in v.items()}
+        elif key in DETAILS and isinstance(v, dict):
+            print(json.dumps({key: v}), file=sys.stderr)
+            out.update({name: digits(v[x], 6) for name, x in DETAILS[key].items() if x in v})
+        else:
+            out[key] = v if key in ("value", "ms_per_step") else digits(v, 8)
+    print(json.dumps(out))
+
+
 def run_extra_workloads(tk, W, args, dev, peak, peak_kind, gpu):
     """The other single-GPU workloads, each measured like the headline one (3 warm-up and 3 timed passes, per-kernel
     pass, clocks sampled): the grouped-query stack, the ragged serving batch, and the 15 budget-sweep points."""
@@ -342,7 +380,7 @@ def run_ours(args):
     if rank == 0 and world == 1 and not args.no_extra:
         line["workloads"] = run_extra_workloads(tk, W, args, dev, peak, peak_kind, local)
     if rank == 0:
-        print(json.dumps(line))
+        print_line(line)
     if world > 1:
         import torch.distributed as dist
         dist.barrier()
