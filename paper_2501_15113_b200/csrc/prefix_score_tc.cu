@@ -8,12 +8,13 @@
 //   warps 2-5, 7-18 four epilogue groups, every fourth tile each
 // First walk: D[row, key] = Q K^T, a TMEM lane is a query row and keeps its own running (max, sum); the four groups'
 // pairs meet in shared memory.  Second walk: D[key, row] = K Q^T, a lane is a key and sums its column.
-// Bound by the special-function unit: two exponentials per score at 16 a cycle and SM, 2048 cycles per tile and block.
+// Bound by the special-function unit (two exponentials per score at 16 a cycle and SM, 2048 cycles per tile and block), so a
+// quarter of them is computed on the FMA pipe, and by the hand-overs between the warps.
 // Blocks are dealt out longest first, in both directions alternately, so that every CTA gets the same number of tiles;
 // the heads go in groups whose keys fit well into L2.  32 heads x 16384 rows, d = 128, both walks: as two launches of
 // the window kernel over (block, 2048 keys) items 4.19 ms (a CTA met the same two of a block's eight key ranges again
-// and again, a third more tiles for some than on average), like this with two epilogue groups 2.98 ms, with four 2.76 ms,
-// 1480 cycles per tile and walk: with two warps to a scheduler the special-function unit idles while they hand over.
+// and again, a third more tiles for some than on average), like this with two epilogue groups 2.98 ms, with four 2.76 ms:
+// with two warps to a scheduler the special-function unit idles while they hand over.  With the exponentials shared 2.5 ms.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -76,6 +77,19 @@ inline PrefixLayout make_prefix_layout(int D) {
   return l;
 }
 
+__device__ __forceinline__ float2 pair_of(const uint32_t* r, int i) {
+  return make_float2(__uint_as_float(r[i]), __uint_as_float(r[i + 1]));
+}
+// Weights of columns i, i + 1 of a tile.  Every fourth pair goes through the FMA pipe: the special-function unit alone is
+// busy for 1024 of a tile's cycles.  32 heads x 16384 rows, none / 2 / 4 / 5 / 6 / 8 of 16 pairs: 2.82 / 2.64 / 2.62 / 2.68 /
+// 2.71 / 2.92 ms for a call by itself (2.89 with the pairs' products and sums unpacked), and 2.91 / 2.84 / 2.84 / 2.89 / - /
+// 3.16 (2.98) in a row of calls, which the power limit slows down; the error against 64 bits stays where it was.
+constexpr int kFmaEvery = 4;
+__device__ __forceinline__ float2 weight2(int i, float2 x) {
+  if ((i >> 1) % kFmaEvery == 0) return ex2_fma(x);
+  return make_float2(ex2(x.x), ex2(x.y));
+}
+
 enum : int {
   B_FULL = 0, B_EMPTY = 4, B_QFULL = 8, B_QEMPTY = 10, B_TFULL = 12, B_TEMPTY = 16, B_STAT = 20, B_COUNT = 22
 };
@@ -117,6 +131,7 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
   const float scale2 = kLog2e * rsqrtf((float)D);
+  const float2 scale22 = make_float2(scale2, scale2);
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -255,11 +270,12 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
             m_run = cm;
           }
           if (m_run > -INFINITY) {
-            const float ms = -m_run * scale2;
-            float zs[4] = {0.f, 0.f, 0.f, 0.f};
+            const float2 ms = make_float2(-m_run * scale2, -m_run * scale2);
+            float2 zs[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
-            for (int i = 0; i < kCols; ++i) zs[i & 3] += ex2(fmaf(__uint_as_float(r[i]), scale2, ms));
-            z_run += (zs[0] + zs[1]) + (zs[2] + zs[3]);
+            for (int i = 0; i < kCols; i += 2)
+              zs[(i >> 1) & 1] = __fadd2_rn(zs[(i >> 1) & 1], weight2(i, __ffma2_rn(pair_of(r, i), scale22, ms)));
+            z_run += (zs[0].x + zs[0].y) + (zs[1].x + zs[1].y);
           }
         }
         done_with(acc);
@@ -284,7 +300,7 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
           const float2 o = sStat[(buf * kGroups + g) * kTile + i];
           if (o.x > -INFINITY) z += o.y * exp2f(o.x - M);
         }
-        myOff[i] = (z > 0.f && x.b * kTile + i < a.N) ? M + log2f(z) + 7.f : INFINITY;
+        myOff[i] = (z > 0.f && x.b * kTile + i < a.N) ? -(M + log2f(z) + 7.f) : -INFINITY;
       }
       __syncwarp();
       // ---- second walk: this thread's key, summed over the rows
@@ -296,7 +312,7 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
         if (!ok) break;
         tc_fence_after();
         const bool tail = t == T - 1;
-        float cs[4] = {0.f, 0.f, 0.f, 0.f};
+        float2 cs[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
         for (int c0 = 0; c0 < kTile; c0 += kCols) {
           uint32_t r[kCols];
@@ -311,13 +327,11 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
 #pragma unroll
           for (int i = 0; i < kCols; i += 4) {
             const float4 off = off4[i >> 2];
-            cs[0] += ex2(fmaf(__uint_as_float(r[i]), scale2, -off.x));
-            cs[1] += ex2(fmaf(__uint_as_float(r[i + 1]), scale2, -off.y));
-            cs[2] += ex2(fmaf(__uint_as_float(r[i + 2]), scale2, -off.z));
-            cs[3] += ex2(fmaf(__uint_as_float(r[i + 3]), scale2, -off.w));
+            cs[0] = __fadd2_rn(cs[0], weight2(i, __ffma2_rn(pair_of(r, i), scale22, make_float2(off.x, off.y))));
+            cs[1] = __fadd2_rn(cs[1], weight2(i + 2, __ffma2_rn(pair_of(r, i + 2), scale22, make_float2(off.z, off.w))));
           }
         }
-        out[t * kTile + row] = (cs[0] + cs[1]) + (cs[2] + cs[3]);
+        out[t * kTile + row] = (cs[0].x + cs[0].y) + (cs[1].x + cs[1].y);
         done_with(acc);
       }
     }

@@ -155,6 +155,36 @@ static __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
+// 2^x of a pair on the FMA pipe, for x <= 0 (and up to 127), where the special-function unit's 16 exponentials a cycle and
+// SM are what a kernel is bound by: n = round(x), 2^(x - n) by a polynomial of degree 6 on [-1/2, 1/2] (a least-squares fit
+// reweighted to equal relative errors, its constant term held at 1: 2e-9 before rounding, 8e-8 at most and 2.7e-8 in the mean
+// square in fp32 with these coefficients), times 2^n built as exponent bits.  Below 2^-126 the result is 0 (x = -inf
+// included), as with ex2; NaN stays NaN.  7 issue slots an exponential, since all but the clamp and the shift are packed.
+static __device__ __forceinline__ float max_nan(float a, float b) {
+  float y;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+  return y;
+}
+static __device__ __forceinline__ float2 ex2_fma(float2 x) {
+  const float2 magic = make_float2(12582912.f, 12582912.f), neg_magic = make_float2(-12582912.f, -12582912.f);   // 1.5 * 2^23
+  x.x = max_nan(x.x, -127.f);
+  x.y = max_nan(x.y, -127.f);
+  const float2 t = __fadd2_rn(x, magic);                    // the integer sits in the low bits
+  const float2 n = __fadd2_rn(t, neg_magic);
+  const float2 r = __ffma2_rn(n, make_float2(-1.f, -1.f), x);
+  float2 y = make_float2(1.53533619e-4f, 1.53533619e-4f);
+  y = __ffma2_rn(y, r, make_float2(1.33988750e-3f, 1.33988750e-3f));
+  y = __ffma2_rn(y, r, make_float2(9.61843692e-3f, 9.61843692e-3f));
+  y = __ffma2_rn(y, r, make_float2(5.55033237e-2f, 5.55033237e-2f));
+  y = __ffma2_rn(y, r, make_float2(2.40226477e-1f, 2.40226477e-1f));
+  y = __ffma2_rn(y, r, make_float2(6.93147182e-1f, 6.93147182e-1f));
+  y = __ffma2_rn(y, r, make_float2(1.f, 1.f));
+  // the magic number's bits leave the word with the shift: what remains is n + 127 as an exponent, 0 for n = -127
+  const float2 p = make_float2(__uint_as_float((__float_as_uint(t.x) << 23) + 0x3f800000u),
+                               __uint_as_float((__float_as_uint(t.y) << 23) + 0x3f800000u));
+  return __fmul2_rn(y, p);
+}
+
 // Shared-memory matrix descriptor: K-major operand, rows of 128 bytes, 128-byte
 // swizzle, 8-row groups 1024 bytes apart.
 static __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
