@@ -168,8 +168,8 @@ cudaError_t launch_lse_to_stat(const DeviceProblem& p, int u0, int n_units, cons
 cudaError_t launch_window_scores(const DeviceProblem& p, int dtype, int max_N, const WindowHostInfo& h,
                                  cudaStream_t s, int layer0 = 0, int n_layers = -1);
 bool window_tc_supported(const DeviceProblem& p, int dtype);
-cudaError_t launch_window_scores_tc(const DeviceProblem& p, const WindowHostInfo& h, cudaStream_t s, int layer0 = 0,
-                                    int n_layers = -1);
+cudaError_t launch_window_scores_tc(const DeviceProblem& p, int dtype, const WindowHostInfo& h, cudaStream_t s,
+                                    int layer0 = 0, int n_layers = -1);
 // Column sums of the causal attention matrix per 128-row block: q [heads][N][d], k [heads / group][N][d] ->
 // scores [heads][64 nb (nb + 1)], nb = ceil(N / 128), block b of a head at offset 64 b (b + 1).
 cudaError_t launch_prefix_scores(const void* q, const void* k, int d, int heads, int group, int N, float* scores,

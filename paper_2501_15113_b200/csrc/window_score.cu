@@ -2,7 +2,9 @@
 //   S = Q_win K^T / sqrt(d), causal mask on the last L keys, row softmax,
 //   C[j] = mean over the unit's G*L window rows of the normalised weights.
 //
-// Two-pass path on the CUDA cores for fp32 inputs (bf16 runs on the tensor cores):
+// Two-pass path on the CUDA cores for fp32 inputs with up to 32 window rows (the others run on the tensor cores; for few rows
+// splitting the keys into planes for them costs more than the products: 128 units of 3000 keys, 16 rows, d = 128, both passes
+// 191 us here and 207 there; 32 units of 6001 keys, 128 rows, d = 64, 252 here and 88 there):
 //   pass 1  per (unit, 256-key chunk): row maxima and exp-sums  -> partial stats
 //   reduce  per unit: combine chunks -> (row max, 1 / row sum); units of up to 32 chunks need no launch for it,
 //           their pass-2 blocks combine the chunks themselves
@@ -10,10 +12,8 @@
 // Scores are kept in log2 units (scaled by log2(e)/sqrt(d)) so exp is one ex2.
 //
 // Bound by the fp32 FMA rate (2 * rows * d flop per key and pass), so each pass is a register-tiled product: a thread
-// holds KPT keys x RPT rows (8x8 at 128 rows), fed by 16-byte shared-memory reads along d, and keeps its own running
-// (max, sum) per row, so that lanes meet once per chunk instead of twice per row and tile.  32 units of 6001 keys, 64
-// rows, d = 64, fp32 (3.1 GFLOP in both passes): with one key per thread and a warp reduction per row and tile
-// 0.57 + 0.32 ms, this form 0.12 + 0.10 ms; the whole compression with four decode steps 1.06 -> 0.42 ms.
+// holds KPT keys x RPT rows, fed by 16-byte shared-memory reads along d, and keeps its own running (max, sum) per row, so
+// that lanes meet once per chunk instead of twice per row and tile.
 #include "common.cuh"
 
 namespace taskkv {
@@ -29,7 +29,7 @@ constexpr int kFoldChunks = 32; // units of up to this many chunks are folded by
 // How a block's 256 threads cover 128 keys x ROWS window rows.
 template <int ROWS>
 struct WinTile {
-  static constexpr int RPT = ROWS == 128 ? 8 : 4;
+  static constexpr int RPT = 4;
   static constexpr int NTY = ROWS / RPT;
   static constexpr int NTX = kBlock / NTY;
   static constexpr int KPT = kTile / NTX;
@@ -314,9 +314,7 @@ template <int D>
 cudaError_t launch_generic(const DeviceProblem& p, int max_N, const WindowHostInfo& h, cudaStream_t s, int layer0,
                            int n_layers) {
   if (p.rows <= 16) return launch_generic_rows<D, 16>(p, max_N, h, s, layer0, n_layers);
-  if (p.rows <= 32) return launch_generic_rows<D, 32>(p, max_N, h, s, layer0, n_layers);
-  if (p.rows <= 64) return launch_generic_rows<D, 64>(p, max_N, h, s, layer0, n_layers);
-  return launch_generic_rows<D, 128>(p, max_N, h, s, layer0, n_layers);
+  return launch_generic_rows<D, 32>(p, max_N, h, s, layer0, n_layers);
 }
 
 }  // namespace
@@ -331,7 +329,8 @@ cudaError_t launch_lse_to_stat(const DeviceProblem& p, int u0, int n_units, cons
 cudaError_t launch_window_scores(const DeviceProblem& p, int dtype, int max_N, const WindowHostInfo& h,
                                  cudaStream_t s, int layer0, int n_layers) {
   if (n_layers < 0) { layer0 = 0; n_layers = p.R; }
-  if (window_tc_supported(p, dtype)) return launch_window_scores_tc(p, h, s, layer0, n_layers);
+  if ((dtype == TASKKV_F32 && p.rows > 32) || window_tc_supported(p, dtype))
+    return launch_window_scores_tc(p, dtype, h, s, layer0, n_layers);
   if (dtype != TASKKV_F32) return cudaErrorNotSupported;      // bf16 without the driver's tensor maps
   return p.d == 64 ? launch_generic<64>(p, max_N, h, s, layer0, n_layers) : launch_generic<128>(p, max_N, h, s, layer0, n_layers);
 }

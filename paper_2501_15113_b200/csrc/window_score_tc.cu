@@ -1,5 +1,5 @@
-// Observation-window scores (Eq. 12, Eq. 13) on the 5th-generation tensor cores,
-// for bf16 inputs.  Kernels for 32, 64 and 128 window rows (G*L); other windows are filled up with zero rows.
+// Observation-window scores (Eq. 12, Eq. 13) on the 5th-generation tensor cores, for bf16 inputs and, as sums of products of
+// bf16 planes, for fp32 ones.  Kernels for 32, 64 and 128 window rows (G*L); other windows are filled up with zero rows.
 //
 // The contraction S = Q_win K^T is 2*G*L*d flop per key (32-128 flop per byte of
 // K): too much for the CUDA cores next to an HBM-rate K stream, little for
@@ -84,9 +84,31 @@ static_assert(kEpiWarps == kTcParts, "one partial-statistic slot per epilogue wa
 constexpr int kThreads = 352;       // warp 0 producer; 1, 6 MMA issuers; 2-5 and 7-10 epilogue groups
 constexpr uint32_t kTmemCols = 512; // four accumulators of up to 128 columns
 
+// fp32 inputs (SPLIT): every row of 64 elements as three bf16 planes: the elements rounded to a grid of 2^-7 of the row's
+// largest power of two, the rest rounded to one of 2^-15, and what is left then, rounded to eight bits (2^-25 of the row's
+// largest).  A score is the sum of six of the nine products of planes (the others are below 2^-24 of its terms, with either
+// sign).  With more than 32 rows; up to 32 the CUDA cores are faster (window_score.cu).  Bound by the conversion with 64 rows (a
+// warp's chain, 1100 cycles for 64 rows x 64 elements), by the 24 products a 64 elements with 128 (2600 cycles of the 3300 a tile
+// takes at d = 64): 32 units of 6001 keys, 128 rows, d = 64, both passes 252 us on the CUDA cores, 88 here; one layer of
+// 8 x 8000 keys, 128 rows, d = 128, 159 and 60.  The leading product has an accumulator of its own, the other five share one:
+// the tensor cores truncate what does not fit an accumulator's 24 bits, but sums of products on one grid fit.  (Planes by
+// truncation and one accumulator for all products: error of C at d = 128 3e-6; leading products apart 4.3e-7; like this 1.6e-7;
+// fp32 on the CUDA cores 2.6e-7.)  Warps 0 and 11-13 read the fp32 rows and write the planes in the producer's place, warp 1
+// alone issues.
+constexpr int kSplitThreads = 448;
+constexpr int kCvtWarps = 4;
+constexpr int kPlanes = 3;
+constexpr int kSmallPairs = 5;      // smallest first
+__device__ constexpr int kPairQ[kSmallPairs] = {2, 0, 1, 1, 0};
+__device__ constexpr int kPairK[kSmallPairs] = {0, 2, 1, 0, 1};
+constexpr float kPlaneMax = 1.0e12f, kPlaneMin = 1.0e-12f;   // rows whose largest element is outside are scored in fp32
+constexpr int kOddRing = 8;         // tiles whose marks ("not to be had as planes") are kept
+
 // Work items of one launch (one pass over up to kMaxSeq sequences): (sequence, unit, chunk of chunk_keys keys),
 // numbered sequence-major, then unit-major: i = item_off[s] + unit * chunks[s] + chunk.  CTA c of a grid of g
-// CTAs takes the items c, c + g, c + 2g, ...  Short sequences share a launch so that every SM has work.
+// CTAs takes the items c, c + g, c + 2g, ..., fp32 ones c, 2g - 1 - c, 2g + c, ...: a unit's last chunk is short, and with few
+// items a CTA some would get nothing but full ones (128 units of 3000 keys, chunks of 2048 and 952: 32 tiles for half of them).
+// Short sequences share a launch so that every SM has work.
 constexpr int kMaxSeq = 8;
 struct TcMaps {
   CUtensorMap k[kMaxSeq];   // [units * N][d] of each sequence
@@ -120,9 +142,10 @@ struct Item {
   int krow0;                // first row of the unit in the K tensor map
   bool valid;
 };
+template <bool SPLIT>
 __device__ __forceinline__ Item decode_item(const TcArgs& a, int k) {
   Item it;
-  const int i = (int)blockIdx.x + k * (int)gridDim.x;
+  const int i = k * (int)gridDim.x + (SPLIT && (k & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
   it.valid = i < a.item_off[a.n_seq];
   it.seq = 0;
 #pragma unroll
@@ -141,27 +164,29 @@ __device__ __forceinline__ Item decode_item(const TcArgs& a, int k) {
 // window rows; what is left of the 227 KB goes to K stages (an even count, so that each stage is always
 // consumed by the same issuer).
 struct TcLayout {
-  int stages;
-  int tile_bytes, q_block_bytes;
+  int stages, q_bufs;
+  int tile_bytes, q_block_bytes;      // SPLIT: a stage is the planes of 64 elements of a tile's keys
   int off_q, off_stat, off_trans, off_bars;
   int total;
 };
 
-inline TcLayout make_layout(int D, int rows) {
+inline TcLayout make_layout(int D, int rows, bool split) {
   TcLayout l;
   const int KB = D / 64;
-  l.tile_bytes = KB * kTile * 128;
-  l.q_block_bytes = KB * rows * 128;
+  l.tile_bytes = (split ? kPlanes : KB) * kTile * 128;
+  l.q_block_bytes = (split ? kPlanes : 1) * KB * rows * 128;
   const int stat = kEpiWarps * rows * (int)sizeof(float2);
   // with 128 rows pass 1 puts the window rows on the TMEM lanes and needs no transposition
   const int trans = rows == 128 ? 0 : kEpiWarps * 32 * 33 * (int)sizeof(float);
   const int bars = 512;
   const int budget = 232448 - 1024;     // dynamic shared memory of one CTA minus the alignment slack
-  int stages = (budget - 2 * l.q_block_bytes - stat - trans - bars) / l.tile_bytes;
+  auto fit = [&](int q_bufs) { return (budget - q_bufs * l.q_block_bytes - stat - trans - bars) / l.tile_bytes; };
+  l.q_bufs = split && fit(2) < 2 ? 1 : 2;
+  int stages = fit(l.q_bufs);
   if (stages > kMaxStages) stages = kMaxStages;
-  l.stages = stages & ~1;
+  l.stages = split ? stages : stages & ~1;
   l.off_q = l.stages * l.tile_bytes;
-  l.off_stat = l.off_q + 2 * l.q_block_bytes;
+  l.off_stat = l.off_q + l.q_bufs * l.q_block_bytes;
   l.off_trans = l.off_stat + stat;
   l.off_bars = l.off_trans + trans;
   l.total = l.off_bars + bars + 1024;
@@ -173,13 +198,136 @@ enum : int {
   B_FULL = 0, B_EMPTY = 8, B_QFULL = 16, B_QEMPTY = 18, B_TFULL = 20, B_TEMPTY = 24, B_COUNT = 28
 };
 
+// `W` (32 or 64) scores of this thread's lane; SPLIT: the sum of the two accumulators.
+template <int W, bool SPLIT>
+__device__ __forceinline__ void load_scores(uint32_t taddr, uint32_t (&r)[W]) {
+  if constexpr (W == 64) tc_ld64(taddr, r);
+  else tc_ld32(taddr, r);
+  if constexpr (SPLIT) {
+    static_assert(W == 32, "the second accumulator's columns take registers, too");
+    uint32_t rest[W];
+    tc_ld32(taddr + 128u, rest);
+    tc_wait_ld();
+#pragma unroll
+    for (int i = 0; i < W; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) + __uint_as_float(rest[i]));
+  } else {
+    tc_wait_ld();
+  }
+}
+
+// Eight elements of a row whose largest (over 64 elements) is `top` as three planes of eight bf16.  False if the planes do not
+// hold them.
+__device__ __forceinline__ bool split8(const float4& lo, const float4& hi, float top, uint4 (&plane)[kPlanes]) {
+  float2 v[4] = {make_float2(lo.x, lo.y), make_float2(lo.z, lo.w), make_float2(hi.x, hi.y), make_float2(hi.z, hi.w)};
+  // 2^e <= top < 2^(e+1): adding and taking away 1.5 * 2^(e-7+23) rounds to a multiple of 2^(e-7), and so on
+  const uint32_t e23 = __float_as_uint(fmaxf(top, kPlaneMin)) & 0x7f800000u;
+  float2 odd = make_float2(0.f, 0.f);
+  const float2 neg_one = make_float2(-1.f, -1.f);
+  uint32_t w[kPlanes][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+#pragma unroll
+    for (int pl = 0; pl < kPlanes - 1; ++pl) {
+      const float m = __uint_as_float(e23 + ((16u - 8u * pl) << 23) + 0x00400000u);
+      const float2 b = __fadd2_rn(__fadd2_rn(v[i], make_float2(m, m)), make_float2(-m, -m));
+      v[i] = __ffma2_rn(b, neg_one, v[i]);
+      w[pl][i] = __byte_perm(__float_as_uint(b.x), __float_as_uint(b.y), 0x7632);
+    }
+    odd = __ffma2_rn(v[i], make_float2(0.f, 0.f), odd);            // NaN for what is not finite
+    const __nv_bfloat162 r = __floats2bfloat162_rn(v[i].x, v[i].y);
+    w[kPlanes - 1][i] = *reinterpret_cast<const uint32_t*>(&r);
+  }
+#pragma unroll
+  for (int pl = 0; pl < kPlanes; ++pl) plane[pl] = make_uint4(w[pl][0], w[pl][1], w[pl][2], w[pl][3]);
+  return odd.x == 0.f && odd.y == 0.f && top < kPlaneMax && (top > kPlaneMin || top == 0.f);
+}
+// 64 elements of rows of an fp32 matrix (`pitch` floats a row; src: the first of the batch's; rows from `there` on are zeros), by
+// the converting warps' threads (thread i), eight elements a thread and row: the c-th four of each half, so that neighbours read
+// neighbouring words (which element is where in a row of planes does not matter as long as keys and queries agree).
+constexpr int kCvtThreads = kCvtWarps * 32, kBatchRows = kCvtThreads / 8 * 4;
+struct Batch { float4 lo[4], hi[4]; };
+template <int B>
+__device__ __forceinline__ void load_batch(Batch& x, const float* __restrict__ src, int pitch, int there, int i) {
+#pragma unroll
+  for (int b = 0; b < B; ++b) {
+    const int row = (b * kCvtThreads + i) >> 3, c = i & 7;
+    x.lo[b] = x.hi[b] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (row < there) {
+      const float4* at = reinterpret_cast<const float4*>(src + (size_t)row * pitch) + c;
+      x.lo[b] = at[0];
+      x.hi[b] = at[8];
+    }
+  }
+}
+// ... as three planes in shared memory, rows of 128 bytes in the 128-byte swizzle, plane_pitch bytes apart (dst: the batch's
+// first row, a multiple of eight).  Returns whether planes hold all that this thread has.  (The rows' largest elements, over the
+// eight lanes that share a row, of all groups first: one group after the other a batch took a warp 1450 cycles, the shuffles'
+// and conversions' latencies in a row.)
+template <int B>
+__device__ __forceinline__ bool store_batch(const Batch& x, unsigned char* dst, int plane_pitch, int i) {
+  float top[B];
+#pragma unroll
+  for (int b = 0; b < B; ++b)
+    top[b] = fmaxf(fmaxf(fmaxf(fabsf(x.lo[b].x), fabsf(x.lo[b].y)), fmaxf(fabsf(x.lo[b].z), fabsf(x.lo[b].w))),
+                   fmaxf(fmaxf(fabsf(x.hi[b].x), fabsf(x.hi[b].y)), fmaxf(fabsf(x.hi[b].z), fabsf(x.hi[b].w))));
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+    float other[B];
+#pragma unroll
+    for (int b = 0; b < B; ++b) other[b] = __shfl_xor_sync(0xffffffffu, top[b], o);
+#pragma unroll
+    for (int b = 0; b < B; ++b) top[b] = fmaxf(top[b], other[b]);
+  }
+  bool fits = true;
+#pragma unroll
+  for (int b0 = 0; b0 < B; b0 += 2) {
+    uint4 plane[2][kPlanes];
+#pragma unroll
+    for (int b = 0; b < 2; ++b) fits = split8(x.lo[b0 + b], x.hi[b0 + b], top[b0 + b], plane[b]) && fits;
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int row = ((b0 + b) * kCvtThreads + i) >> 3, c = i & 7;
+#pragma unroll
+      for (int pl = 0; pl < kPlanes; ++pl)
+        *reinterpret_cast<uint4*>(dst + pl * plane_pitch + row * 128 + ((c ^ (row & 7)) << 4)) = plane[b][pl];
+    }
+  }
+  return fits;
+}
+// Asks for `rows` rows (of `bytes` bytes, one after the other) to be brought into L2.
+__device__ __forceinline__ void prefetch_rows(const void* src, int rows, int bytes) {
+  if (rows > 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(rows * bytes) : "memory");
+}
+// A tile with a row, of its keys or of the queries, that planes do not hold (too large, too small, not finite: products of
+// planes are NaN where the score is infinite): the tile is scored again in fp32, this thread's lane against `n` rows of `other`,
+// and put into the accumulators.  Rare, hence slow and a call of its own.
+template <int D>
+__device__ __noinline__ void rescore(uint32_t taddr, const float* __restrict__ mine, bool there, const float* __restrict__ other,
+                                     int n, int cols) {
+  for (int c0 = 0; c0 < cols; c0 += 32) {
+    uint32_t r[32], zero[32];
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+      float sum = 0.f;
+      if (there && c0 + c < n)
+        for (int x = 0; x < D; ++x) sum = fmaf(mine[x], other[(size_t)(c0 + c) * D + x], sum);
+      r[c] = __float_as_uint(sum);
+      zero[c] = 0u;
+    }
+    __syncwarp();
+    tc_st32(taddr + (uint32_t)c0, r);
+    tc_st32(taddr + 128u + (uint32_t)c0, zero);
+  }
+  tc_wait_st();
+}
+
 // ROWS (32, 64 or 128: columns of an accumulator) is a template argument also for the sake of registers: with 128 rows the
 // gather of another chunk of layers shares the SMs with this kernel, and how many of its blocks (6144 registers) fit beside
 // a CTA is decided here.  One kernel for all row counts took 168 registers a thread, which leaves room for one gather block:
 // 7.0 -> 7.5 ms for 32 layers of 131072 keys; this one takes 128, room for three.  FILLED: the window has ROWS rows; the
 // masks of the others cost full windows 0.5 us a layer of 8191 keys if they are only known at run time.
-template <int D, int ROWS, bool FILLED>
-__global__ void __launch_bounds__(kThreads, 1)
+template <int D, int ROWS, bool FILLED, bool SPLIT>
+__global__ void __launch_bounds__(SPLIT ? kSplitThreads : kThreads, 1)
 window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __grid_constant__ TcArgs a,
                  TcLayout lay) {
   constexpr int KB = D / 64;
@@ -195,6 +343,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + lay.off_bars);
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + B_COUNT);
   volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
+  volatile int* sOdd = s_abort + 1;                                 // [converting warps][kOddRing]  tile not in planes
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int rows = ROWS;                // the window's own rows: p.rows
@@ -204,14 +353,14 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
   auto BAR = [&](int i) { return bar0 + 8u * (uint32_t)i; };
 
   if (tid == 0) {
-    for (int i = 0; i < kMaxStages; ++i) { mbar_init(BAR(B_FULL + i), 1); mbar_init(BAR(B_EMPTY + i), 1); }
+    for (int i = 0; i < kMaxStages; ++i) { mbar_init(BAR(B_FULL + i), SPLIT ? kCvtWarps : 1); mbar_init(BAR(B_EMPTY + i), 1); }
     for (int i = 0; i < 4; ++i) {
       mbar_init(BAR(B_TFULL + i), 1);
       mbar_init(BAR(B_TEMPTY + i), 4);     // the four warps of the group that reads the accumulator
     }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(BAR(B_QFULL + i), 1);
-      mbar_init(BAR(B_QEMPTY + i), 2);     // both issuers release a Q block
+      mbar_init(BAR(B_QFULL + i), SPLIT ? kCvtWarps : 1);
+      mbar_init(BAR(B_QEMPTY + i), SPLIT ? 1 : 2);     // (both) issuers release a Q block
     }
     *s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -227,14 +376,82 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
   const float scale2 = kLog2e * rsqrtf((float)D);
   grid_dependency_wait();       // the setup above runs under the tail of the kernel before this one
 
-  if (warp == 0) {
+  if (SPLIT && (warp == 0 || warp > 10)) {
+    // ------------------------------------------------------------ converting warps.  A stage is two batches of 64 keys; the
+    // next batch's loads are on their way while one is converted, and tiles are asked into L2 two ahead.
+    const int me = warp == 0 ? 0 : warp - 10, i = me * 32 + lane;
+    int stage = 0, qb = 0, n = 0;
+    uint32_t phase = 0, qphase[2] = {0, 0};
+    bool ok = true;
+    auto hand_over = [&](int bar) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(BAR(bar));
+    };
+    for (int k = 0; k < a.steps && ok; ++k) {
+      const Item it = decode_item<SPLIT>(a, k);
+      if (!it.valid) continue;
+      const int u = a.u0[it.seq] + it.lu;
+      const int key0 = it.ch * a.chunk_keys, end = min(it.N, key0 + a.chunk_keys);
+      const int ntiles = (end - key0 + kTile - 1) / kTile;
+      const float* q = static_cast<const float*>(p.q_ptr[u]);
+      const float* kp = static_cast<const float*>(p.k_ptr[u]);
+      if (i == 0) prefetch_rows(kp + (size_t)key0 * D, min(2 * kTile, end - key0), D * 4);
+      constexpr int kQBatch = ROWS < kBatchRows ? ROWS / (kCvtThreads / 8) : 4, kQBatches = ROWS < kBatchRows ? 1 : ROWS / kBatchRows;
+      bool q_fits = true;
+#pragma unroll 1
+      for (int x = 0; x < KB * kQBatches; ++x) {
+        const int kb = x / kQBatches, r0 = x % kQBatches * kBatchRows;
+        Batch qx;
+        load_batch<kQBatch>(qx, q + (size_t)r0 * D + kb * 64, D, p.rows - r0, i);
+        if (x == 0) ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_QEMPTY + qb), qphase[qb] ^ 1, s_abort));
+        if (!ok) break;
+        q_fits = store_batch<kQBatch>(qx, sQ + (size_t)qb * lay.q_block_bytes + (kb * ROWS + r0) * 128, KB * ROWS * 128, i) && q_fits;
+      }
+      if (!ok) break;
+      hand_over(B_QFULL + qb);
+      qphase[qb] ^= 1;
+      if (lay.q_bufs == 2) qb ^= 1;
+      Batch x0, x1;
+      load_batch<4>(x0, kp + (size_t)key0 * D, D, it.N - key0, i);
+      bool fits = q_fits;
+      for (int c = 0; c < ntiles * KB; ++c) {
+        const int t = c / KB, kb = c % KB, at = key0 + t * kTile;
+        load_batch<4>(x1, kp + (size_t)(at + kBatchRows) * D + kb * 64, D, it.N - at - kBatchRows, i);
+        if (kb == 0 && i == 0) prefetch_rows(kp + (size_t)(at + 2 * kTile) * D, min(kTile, end - at - 2 * kTile), D * 4);
+        ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_EMPTY + stage), phase ^ 1, s_abort));
+        if (!ok) break;
+        unsigned char* dst = sK + (size_t)stage * lay.tile_bytes;
+        fits = store_batch<4>(x0, dst, kTile * 128, i) && fits;
+        const int t1 = (c + 1) / KB, at1 = key0 + t1 * kTile;
+        if (c + 1 < ntiles * KB) load_batch<4>(x0, kp + (size_t)at1 * D + (c + 1) % KB * 64, D, it.N - at1, i);
+        fits = store_batch<4>(x1, dst + kBatchRows * 128, kTile * 128, i) && fits;
+        if (kb == KB - 1) {
+          // (the tile whose entry this was is done: its accumulator has been used again since)
+          const bool all = __all_sync(0xffffffffu, fits);
+          if (lane == 0) sOdd[me * kOddRing + (n & (kOddRing - 1))] = all ? 0 : 1;
+          fits = q_fits;
+          ++n;
+        }
+        hand_over(B_FULL + stage);
+        if (++stage == S) { stage = 0; phase ^= 1; }
+      }
+    }
+    // drain, as below
+    for (int j = 0; j < S && ok; ++j) {
+      ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_EMPTY + stage), phase ^ 1, s_abort));
+      if (++stage == S) { stage = 0; phase ^= 1; }
+    }
+    for (int j = 0; j < lay.q_bufs && ok; ++j, qb = lay.q_bufs == 2 ? qb ^ 1 : qb)
+      ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_QEMPTY + qb), qphase[qb] ^ 1, s_abort));
+  } else if (!SPLIT && warp == 0) {
     // ------------------------------------------------------------ TMA producer (whole warp, one lane issues)
     {
       int stage = 0, qb = 0;
       uint32_t phase = 0, qphase[2] = {0, 0};
       bool ok = true;
       for (int k = 0; k < a.steps && ok; ++k) {
-        const Item it = decode_item(a, k);
+        const Item it = decode_item<SPLIT>(a, k);
         if (!it.valid) continue;
         const int N = it.N;
         const int key0 = it.ch * a.chunk_keys;
@@ -273,6 +490,59 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
       for (int i = 0; i < 2 && ok; ++i, qb ^= 1)
         ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_QEMPTY + qb), qphase[qb] ^ 1, s_abort));
     }
+  } else if (SPLIT && warp == 6) {
+  } else if (SPLIT && warp == 1) {
+    // ------------------------------------------------------------ MMA issuer for planes: tile n goes to accumulator n & 1,
+    // its leading products to columns 256 (n & 1), the others 128 columns on
+    int stage = 0, qb = 0, n = 0;
+    uint32_t sphase = 0, qphase[2] = {0, 0};
+    const uint32_t idesc = instr_desc(128, rows);
+    const uint64_t desc_hi = smem_desc(0);
+    bool ok = true;
+    for (int k = 0; k < a.steps && ok; ++k) {
+      const Item it = decode_item<SPLIT>(a, k);
+      if (!it.valid) continue;
+      const int key0 = it.ch * a.chunk_keys;
+      const int ntiles = (min(it.N, key0 + a.chunk_keys) - key0 + kTile - 1) / kTile;
+      ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_QFULL + qb), qphase[qb], s_abort));
+      if (!ok) break;
+      qphase[qb] ^= 1;
+      const uint32_t q_lo = smem_u32(sQ + (size_t)qb * lay.q_block_bytes) >> 4;
+      const bool swap = a.pass == 1 && rows == 128;   // D[row, key] instead of D[key, row]
+      for (int t = 0; t < ntiles && ok; ++t, ++n) {
+        const int acc = n & 1;
+        const uint32_t d_main = tmem_base + (uint32_t)acc * 256u, d_rest = d_main + 128u;
+        ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_TEMPTY + acc), ((uint32_t)(n >> 1) & 1u) ^ 1u, s_abort));
+        for (int kb = 0; kb < KB && ok; ++kb) {
+          ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_FULL + stage), sphase, s_abort));
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t k_lo = smem_u32(sK + (size_t)stage * lay.tile_bytes) >> 4;
+          if (elect_one()) {
+            auto product = [&](uint32_t d, int pq, int pk, int kk, uint32_t add) {
+              const uint64_t kd = desc_hi | (uint64_t)(k_lo + (uint32_t)((pk * kTile * 128 + kk * 32) >> 4));
+              const uint64_t qd = desc_hi | (uint64_t)(q_lo + (uint32_t)(((pq * KB + kb) * rows * 128 + kk * 32) >> 4));
+              if (swap) tc_mma(d, qd, kd, idesc, add);
+              else tc_mma(d, kd, qd, idesc, add);
+            };
+#pragma unroll
+            for (int x = 0; x < kSmallPairs; ++x)
+#pragma unroll
+              for (int kk = 0; kk < 4; ++kk) product(d_rest, kPairQ[x], kPairK[x], kk, (kb | x | kk) ? 1u : 0u);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) product(d_main, 0, 0, kk, (kb | kk) ? 1u : 0u);
+            tc_commit(BAR(B_EMPTY + stage));
+            if (kb == KB - 1) tc_commit(BAR(B_TFULL + acc));
+          }
+          __syncwarp();
+          if (++stage == S) { stage = 0; sphase ^= 1; }
+        }
+      }
+      if (!ok) break;
+      if (elect_one()) tc_commit(BAR(B_QEMPTY + qb));
+      __syncwarp();
+      if (lay.q_bufs == 2) qb ^= 1;
+    }
   } else if (warp == 1 || warp == 6) {
     // ------------------------------------------------------------ MMA issuers: D[key, row] = K Q^T, both passes.
     // Two elected threads: the issue -> commit -> hand-over chain of one tile overlaps with the other's.
@@ -290,7 +560,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
       const uint64_t desc_hi = smem_desc(0);    // everything but the start address
       bool ok = true;
       for (int k = 0; k < a.steps && ok; ++k) {
-        const Item it = decode_item(a, k);
+        const Item it = decode_item<SPLIT>(a, k);
         if (!it.valid) continue;
         const int N = it.N;
         const int key0 = it.ch * a.chunk_keys;
@@ -341,6 +611,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
     const int quad = warp & 3;                      // TMEM lane quadrant this warp may read
     float* myStat = reinterpret_cast<float*>(sStat) + ew * 2 * rows;
     float* myT = sTrans + ew * (32 * 33);
+    constexpr int kWide = SPLIT ? 32 : 64;          // columns per tensor-memory load where many are to be had
     int n = 0;
     bool ok = true;
     // pass 2: the rows' offsets max + log2(sum) + log2(rows) of a unit (one subtraction then turns a raw score
@@ -348,7 +619,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
     const float* stat_g = p.stat;
     float pre[4];
     auto fetch_stats = [&](int k) {
-      const Item nx = decode_item(a, k);
+      const Item nx = decode_item<SPLIT>(a, k);
       const float* st = stat_g + (size_t)(a.u0[nx.seq] + nx.lu) * (2 * p.rows_pad);
       if (rows == 32) {
         // the row's maximum and the weight 1 / (sum rows): with few rows to average over, the rounding of one offset that
@@ -364,7 +635,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
     };
     if (a.pass == 2) fetch_stats(0);
     for (int k = 0; k < a.steps && ok; ++k) {
-      const Item it = decode_item(a, k);
+      const Item it = decode_item<SPLIT>(a, k);
       if (!it.valid) continue;
       const int u = a.u0[it.seq] + it.lu;
       const int N = it.N;
@@ -423,36 +694,50 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
       for (int t = 0; t < ntiles; ++t, ++n) {
         if ((n & 1) != grp) continue;
         if (a.pass == 1 && (t >> sub_shift) != sub) end_part();
-        const int acc = n & 3;
-        const uint32_t accphase = (uint32_t)((n >> 2) & 1);
+        const int acc = SPLIT ? n & 1 : n & 3;
+        const uint32_t accphase = (uint32_t)((SPLIT ? n >> 1 : n >> 2) & 1);
         ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_TFULL + acc), accphase, s_abort));
         if (!ok) break;
         tc_fence_after();
-        const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)acc * 128u;
+        const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)acc * (SPLIT ? 256u : 128u);
         const int tbase = key0 + t * kTile;
+        if constexpr (SPLIT) {
+          int odd = 0;
+#pragma unroll
+          for (int w = 0; w < kCvtWarps; ++w) odd |= sOdd[w * kOddRing + (n & (kOddRing - 1))];
+          if (odd) {
+            // lane and column: row and key in pass 1 of 128 rows, key and row otherwise
+            const float* q = static_cast<const float*>(p.q_ptr[u]);
+            const float* kp = static_cast<const float*>(p.k_ptr[u]);
+            const int l = quad * 32 + lane;
+            const bool swap = a.pass == 1 && rows == 128;
+            const bool there = swap ? l < p.rows : tbase + l < N;
+            const float* mine = swap ? q + (size_t)(there ? l : 0) * D : kp + (size_t)(there ? tbase + l : 0) * D;
+            rescore<D>(taddr, mine, there, swap ? kp + (size_t)tbase * D : q, swap ? min(kTile, N - tbase) : p.rows, swap ? kTile : rows);
+          }
+        }
         const bool tail = (tbase + kTile - 1 > N - L);   // some key of the tile is masked for some row
         if (a.pass == 1 && rows == 128) {
           // a TMEM lane is a window row (quad * 32 + lane), the 128 columns are the keys of the tile
           const int pos = N - L + ((quad * 32 + lane) % L);   // last key this window row may see
 #pragma unroll
-          for (int cg = 0; cg < 2; ++cg) {               // 64 keys per TMEM load
-            uint32_t r[64];
-            tc_ld64(taddr + (uint32_t)(cg * 64), r);
-            tc_wait_ld();
-            float x[64];
+          for (int cg = 0; cg < kTile / kWide; ++cg) {   // kWide keys per TMEM load
+            uint32_t r[kWide];
+            load_scores<kWide, SPLIT>(taddr + (uint32_t)(cg * kWide), r);
+            float x[kWide];
             if (!tail) {
 #pragma unroll
-              for (int k = 0; k < 64; ++k) x[k] = __uint_as_float(r[k]);
+              for (int k = 0; k < kWide; ++k) x[k] = __uint_as_float(r[k]);
             } else {
 #pragma unroll
-              for (int k = 0; k < 64; ++k) {
-                const int j = tbase + cg * 64 + k;
+              for (int k = 0; k < kWide; ++k) {
+                const int j = tbase + cg * kWide + k;
                 x[k] = (j <= pos && j < N) ? __uint_as_float(r[k]) : -INFINITY;
               }
             }
             float cm4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-            for (int k = 0; k < 64; ++k) cm4[k & 3] = fmaxf(cm4[k & 3], x[k]);
+            for (int k = 0; k < kWide; ++k) cm4[k & 3] = fmaxf(cm4[k & 3], x[k]);
             const float cm = fmaxf(fmaxf(cm4[0], cm4[1]), fmaxf(cm4[2], cm4[3]));
             if (cm > m_run[0]) {
               z_run[0] *= ex2((m_run[0] - cm) * scale2);
@@ -462,7 +747,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
               const float ms = -m_run[0] * scale2;
               float zs[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-              for (int k = 0; k < 64; ++k) zs[k & 3] += ex2(fmaf(x[k], scale2, ms));
+              for (int k = 0; k < kWide; ++k) zs[k & 3] += ex2(fmaf(x[k], scale2, ms));
               z_run[0] += (zs[0] + zs[1]) + (zs[2] + zs[3]);
             }
           }
@@ -472,8 +757,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
           for (int rg = 0; rg < 4; ++rg) {
             if (rg * 32 < rows) {
               uint32_t r[32];
-              tc_ld32(taddr + (uint32_t)(rg * 32), r);
-              tc_wait_ld();
+              load_scores<32, SPLIT>(taddr + (uint32_t)(rg * 32), r);
               // transpose the warp's [32 keys][32 rows] block through shared memory
 #pragma unroll
               for (int c = 0; c < 32; ++c) myT[lane * 33 + c] = __uint_as_float(r[c]);
@@ -516,13 +800,12 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
           // such rows are left out, not given a weight of zero.
           if (rows >= 64 && !tail && FILLED) {
             // 64 columns per TMEM load: half the load / wait round trips of the 32-column walk below
-            for (int c0 = 0; c0 < rows; c0 += 64) {
-              uint32_t r[64];
-              tc_ld64(taddr + (uint32_t)c0, r);
-              tc_wait_ld();
+            for (int c0 = 0; c0 < rows; c0 += kWide) {
+              uint32_t r[kWide];
+              load_scores<kWide, SPLIT>(taddr + (uint32_t)c0, r);
               const float4* st4 = reinterpret_cast<const float4*>(myStat + c0);   // four rows per 16-byte load
 #pragma unroll
-              for (int c = 0; c < 64; c += 4) {
+              for (int c = 0; c < kWide; c += 4) {
                 const float4 off = st4[c >> 2];
                 cs[0] += ex2(fmaf(__uint_as_float(r[c]), scale2, -off.x));
                 cs[1] += ex2(fmaf(__uint_as_float(r[c + 1]), scale2, -off.y));
@@ -532,8 +815,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
             }
           } else if (rows == 32) {
             uint32_t r[32];
-            tc_ld32(taddr, r);
-            tc_wait_ld();
+            load_scores<32, SPLIT>(taddr, r);
             const float4* mx4 = reinterpret_cast<const float4*>(myStat);
             const float4* wt4 = reinterpret_cast<const float4*>(myStat + 32);
             uint32_t vm = FILLED ? 0xffffffffu : (1u << p.rows) - 1u;   // bit c: window row c sees this thread's key
@@ -561,8 +843,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
           } else
           for (int c0 = 0; c0 < (FILLED ? rows : p.rows); c0 += 32) {
             uint32_t r[32];
-            tc_ld32(taddr + (uint32_t)c0, r);
-            tc_wait_ld();
+            load_scores<32, SPLIT>(taddr + (uint32_t)c0, r);
             if (!tail) {
               const float4* st4 = reinterpret_cast<const float4*>(myStat + c0);   // four rows per 16-byte load
 #pragma unroll
@@ -681,14 +962,14 @@ inline int pick_chunk(int64_t units_times_keys, int n_sm, int least) {
   return chunk;
 }
 
-template <int D, int ROWS, bool FILLED>
+template <int D, int ROWS, bool FILLED, bool SPLIT>
 cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStream_t s, int layer0, int n_layers) {
   const int n_sm = sm_count();
   constexpr int rows = ROWS;
-  const TcLayout lay = make_layout(D, rows);
+  const TcLayout lay = make_layout(D, rows, SPLIT);
   if (lay.stages < 2) return cudaErrorInvalidValue;
   const int smem = lay.total;
-  cudaError_t e = cudaFuncSetAttribute(window_tc_kernel<D, ROWS, FILLED>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(window_tc_kernel<D, ROWS, FILLED, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const int per_seq_all = p.R * p.n_kv;
   const int first = layer0 * p.n_kv;               // the launch covers units [first, first + per_seq) of every sequence
@@ -710,7 +991,7 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
       if (i >= nb) {
         maps.k[i] = maps.k[0];
         maps.q[i] = maps.q[0];
-      } else {
+      } else if (!SPLIT) {                                      // (fp32 rows are read through the units' pointers)
         const char* kb = static_cast<const char*>(h.k[b]) + (size_t)skip * (size_t)N * D * sizeof(__nv_bfloat16);
         const char* qb = static_cast<const char*>(h.q[b]) + (size_t)skip * p.rows * D * sizeof(__nv_bfloat16);
         if (!make_tensor_map_2d(&maps.k[i], kb, D, (uint64_t)per_seq * (uint64_t)N, kTile)) return cudaErrorUnknown;
@@ -731,7 +1012,8 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
       const int items = a.item_off[nb], grid = items < n_sm ? items : n_sm;
       a.steps = (items + grid - 1) / grid;
       LaunchScope ls(K_WINDOW_TC, s);
-      return launch_dependent_smem(window_tc_kernel<D, ROWS, FILLED>, (unsigned)grid, kThreads, (size_t)smem, s, maps, p, a, lay);
+      return launch_dependent_smem(window_tc_kernel<D, ROWS, FILLED, SPLIT>, (unsigned)grid, SPLIT ? kSplitThreads : kThreads, (size_t)smem, s,
+                                  maps, p, a, lay);
     };
     if (h.lse) {
       // the caller already has the rows' normalisers: no pass 1
@@ -757,28 +1039,31 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
   return cudaSuccess;
 }
 
-template <int ROWS>
+template <int ROWS, bool SPLIT>
 cudaError_t launch_tc_rows(const DeviceProblem& p, const WindowHostInfo& h, cudaStream_t s, int layer0, int n_layers) {
   if (p.rows == ROWS)
-    return p.d == 64 ? launch_tc_d<64, ROWS, true>(p, h, s, layer0, n_layers) : launch_tc_d<128, ROWS, true>(p, h, s, layer0, n_layers);
-  return p.d == 64 ? launch_tc_d<64, ROWS, false>(p, h, s, layer0, n_layers) : launch_tc_d<128, ROWS, false>(p, h, s, layer0, n_layers);
+    return p.d == 64 ? launch_tc_d<64, ROWS, true, SPLIT>(p, h, s, layer0, n_layers)
+                     : launch_tc_d<128, ROWS, true, SPLIT>(p, h, s, layer0, n_layers);
+  return p.d == 64 ? launch_tc_d<64, ROWS, false, SPLIT>(p, h, s, layer0, n_layers)
+                   : launch_tc_d<128, ROWS, false, SPLIT>(p, h, s, layer0, n_layers);
 }
-
 }  // namespace
 
 bool window_tc_supported(const DeviceProblem& p, int dtype) {
   return dtype == TASKKV_BF16 && p.rows <= 128 && encode_fn() != nullptr;
 }
 
-cudaError_t launch_window_scores_tc(const DeviceProblem& p, const WindowHostInfo& h, cudaStream_t s, int layer0,
+cudaError_t launch_window_scores_tc(const DeviceProblem& p, int dtype, const WindowHostInfo& h, cudaStream_t s, int layer0,
                                     int n_layers) {
   if (n_layers < 0) { layer0 = 0; n_layers = p.R; }
+  if (dtype == TASKKV_F32)
+    return p.rows <= 64 ? launch_tc_rows<64, true>(p, h, s, layer0, n_layers) : launch_tc_rows<128, true>(p, h, s, layer0, n_layers);
   // 32 window rows and sequences short enough for a unit's scores to stay in tensor memory: K is read once
   if (window_res_supported(p, h)) return launch_window_scores_res(p, h, s, layer0, n_layers);
   switch (tc_rows(p.rows)) {
-    case 32: return launch_tc_rows<32>(p, h, s, layer0, n_layers);
-    case 64: return launch_tc_rows<64>(p, h, s, layer0, n_layers);
-    default: return launch_tc_rows<128>(p, h, s, layer0, n_layers);
+    case 32: return launch_tc_rows<32, false>(p, h, s, layer0, n_layers);
+    case 64: return launch_tc_rows<64, false>(p, h, s, layer0, n_layers);
+    default: return launch_tc_rows<128, false>(p, h, s, layer0, n_layers);
   }
 }
 

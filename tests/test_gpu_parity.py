@@ -297,9 +297,9 @@ def test_second_device_of_a_process_decodes_with_clusters_of_sixteen():
     assert torch.equal(outs[0], outs[1])
 
 
-# (query heads per KV head, window) -> 8 to 128 window rows: on the CUDA cores (fp32), or as the next larger tensor-core
-# tile with zero rows (bf16; up to 32768 keys the single-read kernel takes up to 32 rows); key counts around the 128-key tile, the
-# 256-key chunk and the 8192 keys up to which pass 2 folds the chunks' statistics itself.  (Four KV heads: two are always
+# (query heads per KV head, window) -> 8 to 128 window rows, up to 32 of them on the CUDA cores (fp32), or as the next larger
+# tensor-core tile with zero rows (bf16: up to 32768 keys the single-read kernel takes up to 32 rows); key counts around the 128-key
+# tile, the 256-key chunk and the 8192 keys up to which pass 2 folds the chunks' statistics itself.  (Four KV heads: two are always
 # equally far from their mean, so which of them is promoted would be a tie.)
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("G,L,d,N", [(1, 8, 64, 129), (2, 8, 128, 255), (1, 24, 64, 257), (2, 24, 128, 511),
@@ -328,6 +328,44 @@ def test_window_scores_error_against_64_bits(G, L, d, N, dtype):
     s.masked_fill_(torch.arange(N, device=DEV)[None] > last[:, None], -float("inf"))
     want = torch.softmax(s, -1).mean(1)
     assert float((got - want).norm() / want.norm()) < 1e-6
+
+
+# fp32 inputs with more than 32 window rows go through the tensor cores as planes of bf16 on a grid per row of 64 elements.  What planes do not hold is scored in
+# fp32: rows beyond their range (queries times 2^-45, keys times 2^45: the same scores), rows far below it (a key that is
+# almost zero, and one that is), infinite elements (a key that scores -inf).  One partial row or row half of such a kind in a
+# tile sends the whole tile there; lengths with and without a partial tile.  Tolerance: as derived above.
+@pytest.mark.parametrize("kind", ["plain", "scaled", "tiny", "infinite", "spread"])
+@pytest.mark.parametrize("G,L,d,N", [(1, 9, 64, 129), (1, 32, 128, 5000), (2, 24, 64, 4097), (2, 32, 128, 640), (4, 24, 128, 2049),
+                                     (4, 32, 64, 2500)])
+def test_fp32_window_scores_in_and_out_of_the_planes_range(G, L, d, N, kind):
+    tk = _tk()
+    wl = small("planes", n=8 * G, n_kv=8, d=d, N=N, L=L, s1=4, s2=32, k=40, dtype="f32", nh=0, t=64, steps=1, variance=0.5)
+    qs, ks, vs = W.materialize(wl, DEV)
+    q, k = qs[0][0], ks[0][0]
+    if kind == "scaled":
+        q *= 2.0 ** -45
+        k *= 2.0 ** 45
+    elif kind == "tiny":
+        k[:, N // 2] *= 1e-25
+        k[:, N // 3] = 0
+        k[:, 5, :32] *= 1e-30
+    elif kind == "spread":                  # elements from 1 to 2^-20 in every row, and rows of different size (six times: of the
+        k *= 2.0 ** -torch.arange(d, device=DEV).remainder(21).float()     # row's elements about two a 21 weigh in, so the
+        k[:, ::3] *= 6.0                                                   # exponents stay within the 16 of the bound)
+    elif kind == "infinite":
+        q[..., 3] = q[..., 3].abs() + 0.5
+        k[:, [5, N // 2, N - L - 1], 3] = -float("inf")
+    cache = tk.taskkv_compress_ex(tk.params_from_workload(wl, max_new_tokens=0), qs, ks, vs)
+    got = torch.from_numpy(cache.query(tk.Q_SCORES)).reshape(8, -1)[:, :N].double().to(DEV)
+    assert cache.status() == 0
+    cache.close()
+    s = torch.einsum("hrd,hjd->hrj", q.double().view(8, G * L, d), k.double()) / d ** 0.5
+    last = N - L + torch.arange(G * L, device=DEV) % L
+    s.masked_fill_(torch.arange(N, device=DEV)[None] > last[:, None], -float("inf"))
+    want = torch.softmax(s, -1).mean(1)
+    assert float((got - want).norm() / want.norm()) < 1e-6
+    if kind == "infinite":
+        assert not got[:, [5, N // 2, N - L - 1]].any()
 
 
 # A key with an infinite element that every window row scores -inf weighs nothing, whatever fills the window's tile up: a zero
