@@ -84,24 +84,26 @@ static_assert(kEpiWarps == kTcParts, "one partial-statistic slot per epilogue wa
 constexpr int kThreads = 352;       // warp 0 producer; 1, 6 MMA issuers; 2-5 and 7-10 epilogue groups
 constexpr uint32_t kTmemCols = 512; // four accumulators of up to 128 columns
 
-// fp32 inputs (SPLIT): every row of 64 elements as three bf16 planes: the elements rounded to a grid of 2^-7 of the row's
-// largest power of two, the rest rounded to one of 2^-15, and what is left then, rounded to eight bits (2^-25 of the row's
-// largest).  A score is the sum of six of the nine products of planes (the others are below 2^-24 of its terms, with either
-// sign).  With more than 32 rows; up to 32 the CUDA cores are faster (window_score.cu).  Bound by the conversion with 64 rows (a
-// warp's chain, 1100 cycles for 64 rows x 64 elements), by the 24 products a 64 elements with 128 (2600 cycles of the 3300 a tile
-// takes at d = 64): 32 units of 6001 keys, 128 rows, d = 64, both passes 252 us on the CUDA cores, 88 here; one layer of
-// 8 x 8000 keys, 128 rows, d = 128, 159 and 60.  The leading product has an accumulator of its own, the other five share one:
-// the tensor cores truncate what does not fit an accumulator's 24 bits, but sums of products on one grid fit.  (Planes by
-// truncation and one accumulator for all products: error of C at d = 128 3e-6; leading products apart 4.3e-7; like this 1.6e-7;
-// fp32 on the CUDA cores 2.6e-7.)  Warps 0 and 11-13 read the fp32 rows and write the planes in the producer's place, warp 1
-// alone issues.
+// fp32 inputs (SPLIT): every element as the sum of three bf16 planes, exactly, whatever the elements beside it are (split8).  A
+// score is the sum of six of the nine products of planes; the second plane is at most 2^-8 and the third 2^-17 of the element,
+// so the three left out are below 2^-24 of an element's own term, with either sign (2^-27.4 in the mean square).  The leading
+// product has an accumulator of its own, since the tensor cores truncate what does not fit an accumulator's 24 bits; the other
+// five share one.
+// Error of C against 64 bits, six shapes of 40 to 128 rows: 1.3e-7 to 1.8e-7, fp32 on the CUDA cores 1.9e-7 to 2.6e-7; powers of
+// two that scale a channel of the keys up and of the queries down (2^-20 to 2^20) change no bit of either.  (Planes on one grid
+// per row of 64 elements, which sum without truncation, are as good for rows whose elements are of one size, but keep the small
+// elements beside a large one in fewer bits: 1e-5 for one channel of 2^10, 1e-3 to 1e-2 for one of 2^20.)
+// With more than 32 rows; up to 32 the CUDA cores are faster (window_score.cu).  Bound by the conversion with 64 rows, by the 24
+// products a 64 elements with 128: 32 units of 6001 keys, d = 64, both passes and their reduction 64 rows 150 us on the CUDA
+// cores, 84 here, 128 rows 250 and 97; one layer of 8 x 8000 keys, 128 rows, d = 128, 156 and 67.  Warps 0 and 11-13 read the
+// fp32 rows and write the planes in the producer's place, warp 1 alone issues.
 constexpr int kSplitThreads = 448;
 constexpr int kCvtWarps = 4;
 constexpr int kPlanes = 3;
 constexpr int kSmallPairs = 5;      // smallest first
 __device__ constexpr int kPairQ[kSmallPairs] = {2, 0, 1, 1, 0};
 __device__ constexpr int kPairK[kSmallPairs] = {0, 2, 1, 0, 1};
-constexpr float kPlaneMax = 1.0e12f, kPlaneMin = 1.0e-12f;   // rows whose largest element is outside are scored in fp32
+constexpr float kPlaneMax = 7.2057594e16f;   // 2^56: tiles with a larger element, or an infinite one, are scored in fp32
 constexpr int kOddRing = 8;         // tiles whose marks ("not to be had as planes") are kept
 
 // Work items of one launch (one pass over up to kMaxSeq sequences): (sequence, unit, chunk of chunk_keys keys),
@@ -215,31 +217,27 @@ __device__ __forceinline__ void load_scores(uint32_t taddr, uint32_t (&r)[W]) {
   }
 }
 
-// Eight elements of a row whose largest (over 64 elements) is `top` as three planes of eight bf16.  False if the planes do not
-// hold them.
-__device__ __forceinline__ bool split8(const float4& lo, const float4& hi, float top, uint4 (&plane)[kPlanes]) {
+// Eight elements as three planes of eight bf16: x = b0 + b1 + b2 exactly (for |x| above 2^-100; below, to 2^-126).  Adding x to
+// 2^16 x leaves x rounded to a bf16's eight bits behind when 2^16 x is taken away again (Dekker's splitting), the rest of at
+// most 16 bits goes the same way, and what is left then has eight.
+__device__ __forceinline__ void split8(const float4& lo, const float4& hi, uint4 (&plane)[kPlanes]) {
   float2 v[4] = {make_float2(lo.x, lo.y), make_float2(lo.z, lo.w), make_float2(hi.x, hi.y), make_float2(hi.z, hi.w)};
-  // 2^e <= top < 2^(e+1): adding and taking away 1.5 * 2^(e-7+23) rounds to a multiple of 2^(e-7), and so on
-  const uint32_t e23 = __float_as_uint(fmaxf(top, kPlaneMin)) & 0x7f800000u;
-  float2 odd = make_float2(0.f, 0.f);
-  const float2 neg_one = make_float2(-1.f, -1.f);
+  const float2 up = make_float2(65536.f, 65536.f), down = make_float2(-65536.f, -65536.f), neg_one = make_float2(-1.f, -1.f);
   uint32_t w[kPlanes][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
 #pragma unroll
-    for (int pl = 0; pl < kPlanes - 1; ++pl) {
-      const float m = __uint_as_float(e23 + ((16u - 8u * pl) << 23) + 0x00400000u);
-      const float2 b = __fadd2_rn(__fadd2_rn(v[i], make_float2(m, m)), make_float2(-m, -m));
-      v[i] = __ffma2_rn(b, neg_one, v[i]);
+    for (int pl = 0; pl < kPlanes; ++pl) {
+      float2 b = v[i];
+      if (pl < kPlanes - 1) {
+        b = __ffma2_rn(b, down, __ffma2_rn(b, up, b));
+        v[i] = __ffma2_rn(b, neg_one, v[i]);
+      }
       w[pl][i] = __byte_perm(__float_as_uint(b.x), __float_as_uint(b.y), 0x7632);
     }
-    odd = __ffma2_rn(v[i], make_float2(0.f, 0.f), odd);            // NaN for what is not finite
-    const __nv_bfloat162 r = __floats2bfloat162_rn(v[i].x, v[i].y);
-    w[kPlanes - 1][i] = *reinterpret_cast<const uint32_t*>(&r);
   }
 #pragma unroll
   for (int pl = 0; pl < kPlanes; ++pl) plane[pl] = make_uint4(w[pl][0], w[pl][1], w[pl][2], w[pl][3]);
-  return odd.x == 0.f && odd.y == 0.f && top < kPlaneMax && (top > kPlaneMin || top == 0.f);
 }
 // 64 elements of rows of an fp32 matrix (`pitch` floats a row; src: the first of the batch's; rows from `there` on are zeros), by
 // the converting warps' threads (thread i), eight elements a thread and row: the c-th four of each half, so that neighbours read
@@ -260,30 +258,20 @@ __device__ __forceinline__ void load_batch(Batch& x, const float* __restrict__ s
   }
 }
 // ... as three planes in shared memory, rows of 128 bytes in the 128-byte swizzle, plane_pitch bytes apart (dst: the batch's
-// first row, a multiple of eight).  Returns whether planes hold all that this thread has.  (The rows' largest elements, over the
-// eight lanes that share a row, of all groups first: one group after the other a batch took a warp 1450 cycles, the shuffles'
-// and conversions' latencies in a row.)
+// first row, a multiple of eight).  Returns the largest |element| that this thread has (a NaN is not seen; it stays one).
 template <int B>
-__device__ __forceinline__ bool store_batch(const Batch& x, unsigned char* dst, int plane_pitch, int i) {
-  float top[B];
-#pragma unroll
-  for (int b = 0; b < B; ++b)
-    top[b] = fmaxf(fmaxf(fmaxf(fabsf(x.lo[b].x), fabsf(x.lo[b].y)), fmaxf(fabsf(x.lo[b].z), fabsf(x.lo[b].w))),
-                   fmaxf(fmaxf(fabsf(x.hi[b].x), fabsf(x.hi[b].y)), fmaxf(fabsf(x.hi[b].z), fabsf(x.hi[b].w))));
-#pragma unroll
-  for (int o = 4; o > 0; o >>= 1) {
-    float other[B];
-#pragma unroll
-    for (int b = 0; b < B; ++b) other[b] = __shfl_xor_sync(0xffffffffu, top[b], o);
-#pragma unroll
-    for (int b = 0; b < B; ++b) top[b] = fmaxf(top[b], other[b]);
-  }
-  bool fits = true;
+__device__ __forceinline__ float store_batch(const Batch& x, unsigned char* dst, int plane_pitch, int i) {
+  float top = 0.f;
 #pragma unroll
   for (int b0 = 0; b0 < B; b0 += 2) {
     uint4 plane[2][kPlanes];
 #pragma unroll
-    for (int b = 0; b < 2; ++b) fits = split8(x.lo[b0 + b], x.hi[b0 + b], top[b0 + b], plane[b]) && fits;
+    for (int b = 0; b < 2; ++b) {
+      const float4 lo = x.lo[b0 + b], hi = x.hi[b0 + b];
+      top = fmaxf(top, fmaxf(fmaxf(fmaxf(fabsf(lo.x), fabsf(lo.y)), fmaxf(fabsf(lo.z), fabsf(lo.w))),
+                             fmaxf(fmaxf(fabsf(hi.x), fabsf(hi.y)), fmaxf(fabsf(hi.z), fabsf(hi.w)))));
+      split8(lo, hi, plane[b]);
+    }
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
       const int row = ((b0 + b) * kCvtThreads + i) >> 3, c = i & 7;
@@ -292,14 +280,14 @@ __device__ __forceinline__ bool store_batch(const Batch& x, unsigned char* dst, 
         *reinterpret_cast<uint4*>(dst + pl * plane_pitch + row * 128 + ((c ^ (row & 7)) << 4)) = plane[b][pl];
     }
   }
-  return fits;
+  return top;
 }
 // Asks for `rows` rows (of `bytes` bytes, one after the other) to be brought into L2.
 __device__ __forceinline__ void prefetch_rows(const void* src, int rows, int bytes) {
   if (rows > 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(rows * bytes) : "memory");
 }
-// A tile with a row, of its keys or of the queries, that planes do not hold (too large, too small, not finite: products of
-// planes are NaN where the score is infinite): the tile is scored again in fp32, this thread's lane against `n` rows of `other`,
+// A tile with an element, of its keys or of the queries, that planes do not hold (too large for products and sums to stay finite,
+// or infinite itself: products of planes are NaN where the score is infinite): the tile is scored again in fp32, this thread's lane against `n` rows of `other`,
 // and put into the accumulators.  Rare, hence slow and a call of its own.
 template <int D>
 __device__ __noinline__ void rescore(uint32_t taddr, const float* __restrict__ mine, bool there, const float* __restrict__ other,
@@ -398,7 +386,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
       const float* kp = static_cast<const float*>(p.k_ptr[u]);
       if (i == 0) prefetch_rows(kp + (size_t)key0 * D, min(2 * kTile, end - key0), D * 4);
       constexpr int kQBatch = ROWS < kBatchRows ? ROWS / (kCvtThreads / 8) : 4, kQBatches = ROWS < kBatchRows ? 1 : ROWS / kBatchRows;
-      bool q_fits = true;
+      float q_top = 0.f;
 #pragma unroll 1
       for (int x = 0; x < KB * kQBatches; ++x) {
         const int kb = x / kQBatches, r0 = x % kQBatches * kBatchRows;
@@ -406,7 +394,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
         load_batch<kQBatch>(qx, q + (size_t)r0 * D + kb * 64, D, p.rows - r0, i);
         if (x == 0) ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_QEMPTY + qb), qphase[qb] ^ 1, s_abort));
         if (!ok) break;
-        q_fits = store_batch<kQBatch>(qx, sQ + (size_t)qb * lay.q_block_bytes + (kb * ROWS + r0) * 128, KB * ROWS * 128, i) && q_fits;
+        q_top = fmaxf(q_top, store_batch<kQBatch>(qx, sQ + (size_t)qb * lay.q_block_bytes + (kb * ROWS + r0) * 128, KB * ROWS * 128, i));
       }
       if (!ok) break;
       hand_over(B_QFULL + qb);
@@ -414,7 +402,7 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
       if (lay.q_bufs == 2) qb ^= 1;
       Batch x0, x1;
       load_batch<4>(x0, kp + (size_t)key0 * D, D, it.N - key0, i);
-      bool fits = q_fits;
+      float top = q_top;
       for (int c = 0; c < ntiles * KB; ++c) {
         const int t = c / KB, kb = c % KB, at = key0 + t * kTile;
         load_batch<4>(x1, kp + (size_t)(at + kBatchRows) * D + kb * 64, D, it.N - at - kBatchRows, i);
@@ -422,15 +410,15 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
         ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_EMPTY + stage), phase ^ 1, s_abort));
         if (!ok) break;
         unsigned char* dst = sK + (size_t)stage * lay.tile_bytes;
-        fits = store_batch<4>(x0, dst, kTile * 128, i) && fits;
+        top = fmaxf(top, store_batch<4>(x0, dst, kTile * 128, i));
         const int t1 = (c + 1) / KB, at1 = key0 + t1 * kTile;
         if (c + 1 < ntiles * KB) load_batch<4>(x0, kp + (size_t)at1 * D + (c + 1) % KB * 64, D, it.N - at1, i);
-        fits = store_batch<4>(x1, dst + kBatchRows * 128, kTile * 128, i) && fits;
+        top = fmaxf(top, store_batch<4>(x1, dst + kBatchRows * 128, kTile * 128, i));
         if (kb == KB - 1) {
           // (the tile whose entry this was is done: its accumulator has been used again since)
-          const bool all = __all_sync(0xffffffffu, fits);
+          const bool all = __all_sync(0xffffffffu, top < kPlaneMax);
           if (lane == 0) sOdd[me * kOddRing + (n & (kOddRing - 1))] = all ? 0 : 1;
-          fits = q_fits;
+          top = q_top;
           ++n;
         }
         hand_over(B_FULL + stage);

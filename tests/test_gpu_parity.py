@@ -330,11 +330,11 @@ def test_window_scores_error_against_64_bits(G, L, d, N, dtype):
     assert float((got - want).norm() / want.norm()) < 1e-6
 
 
-# fp32 inputs with more than 32 window rows go through the tensor cores as planes of bf16 on a grid per row of 64 elements.  What planes do not hold is scored in
-# fp32: rows beyond their range (queries times 2^-45, keys times 2^45: the same scores), rows far below it (a key that is
-# almost zero, and one that is), infinite elements (a key that scores -inf).  One partial row or row half of such a kind in a
-# tile sends the whole tile there; lengths with and without a partial tile.  Tolerance: as derived above.
-@pytest.mark.parametrize("kind", ["plain", "scaled", "tiny", "infinite", "spread"])
+# fp32 inputs with more than 32 window rows go through the tensor cores as planes of bf16 (elements below 2^56): queries times
+# 2^-45 and keys times 2^45 (the same scores), a key that is almost zero, and one that is.  What planes do not hold is scored
+# in fp32: keys times 2^60 ("beyond"), infinite elements (a key that scores -inf).  One such element in a tile sends the whole
+# tile there; lengths with and without a partial tile.  Tolerance: as derived above.
+@pytest.mark.parametrize("kind", ["plain", "scaled", "beyond", "tiny", "infinite", "spread"])
 @pytest.mark.parametrize("G,L,d,N", [(1, 9, 64, 129), (1, 32, 128, 5000), (2, 24, 64, 4097), (2, 32, 128, 640), (4, 24, 128, 2049),
                                      (4, 32, 64, 2500)])
 def test_fp32_window_scores_in_and_out_of_the_planes_range(G, L, d, N, kind):
@@ -345,6 +345,9 @@ def test_fp32_window_scores_in_and_out_of_the_planes_range(G, L, d, N, kind):
     if kind == "scaled":
         q *= 2.0 ** -45
         k *= 2.0 ** 45
+    elif kind == "beyond":
+        q *= 2.0 ** -60
+        k *= 2.0 ** 60
     elif kind == "tiny":
         k[:, N // 2] *= 1e-25
         k[:, N // 3] = 0
@@ -366,6 +369,62 @@ def test_fp32_window_scores_in_and_out_of_the_planes_range(G, L, d, N, kind):
     assert float((got - want).norm() / want.norm()) < 1e-6
     if kind == "infinite":
         assert not got[:, [5, N // 2, N - L - 1]].any()
+
+
+# A channel of the keys times a power of two and the queries' channel divided by it: every product, and hence every sum and its
+# rounding, is what it was, so the scores are the same bits however far the elements of a row are apart (here all of them stay
+# within fp32's and the planes' range).
+@pytest.mark.parametrize("G,L,d,N", [(1, 40, 64, 1500), (2, 32, 128, 641), (4, 24, 64, 2049), (4, 32, 128, 1100)])
+def test_fp32_window_scores_do_not_depend_on_the_scales_of_channels(G, L, d, N):
+    tk = _tk()
+    wl = small("channels", n=4 * G, n_kv=4, d=d, N=N, L=L, s1=4, s2=32, k=40, dtype="f32", nh=0, t=64, steps=1, variance=0.5)
+    qs, ks, vs = W.materialize(wl, DEV)
+    ch = torch.arange(d, device=DEV)
+    scales = [torch.ones(d, device=DEV)]
+    scales += [torch.where(ch == 5, 2.0 ** e, 1.0) for e in (6, 10, 14, 20, -6, -10, -20)]                # one channel
+    scales += [2.0 ** -(ch * 7 % (e + 1)).float() for e in (10, 16, 20, 30)]                              # all of them, spread
+    scales += [2.0 ** (e * ((ch % 8 == 3).float() - (ch % 8 == 6).float())) for e in (6, 10, 16, 40)]     # some up, some down
+    got = []
+    for x in scales:
+        cache = tk.taskkv_compress_ex(tk.params_from_workload(wl, max_new_tokens=0), [t / x for t in qs], [t * x for t in ks], vs)
+        got.append(torch.from_numpy(cache.query(tk.Q_SCORES)).reshape(4, -1)[:, :N].clone())
+        assert cache.status() == 0
+        cache.close()
+    for i in range(1, len(scales)):
+        assert torch.equal(got[i], got[0]), i
+
+
+# Elements of a row that differ in size by themselves, a large channel of the keys that no query uses, keys with a common large
+# channel, and scores that are differences of large terms: the error against 64 bits.  An fp32 sum's error is up to 2^-24 of
+# its partial sums a term, so for these inputs the bound above (exponents of up to 16) is taken four times.
+@pytest.mark.parametrize("kind", ["elements", "unused", "offset", "differences"])
+@pytest.mark.parametrize("G,L,d,N", [(1, 40, 64, 6001), (2, 32, 128, 4097), (4, 24, 128, 2049), (4, 32, 64, 6001)])
+def test_fp32_window_scores_of_elements_of_different_size(G, L, d, N, kind):
+    tk = _tk()
+    wl = small("sizes", n=4 * G, n_kv=4, d=d, N=N, L=L, s1=4, s2=32, k=40, dtype="f32", nh=0, t=64, steps=1, variance=0.5)
+    qs, ks, vs = W.materialize(wl, DEV)
+    q, k = qs[0][0], ks[0][0]
+    if kind == "elements":
+        g = torch.Generator(device=DEV).manual_seed(3)
+        k *= 2.0 ** torch.randint(-8, 2, k.shape, generator=g, device=DEV).float()
+    elif kind == "unused":
+        k[..., 9] *= 1000.0
+        q[..., 9] *= 1e-6
+    elif kind == "offset":
+        k[..., 17] += 20.0
+    else:
+        k[..., 1] = k[..., 0] + 0.01 * k[..., 1]
+        q[..., 1] = -q[..., 0]
+        k[..., :2] *= 20.0
+    cache = tk.taskkv_compress_ex(tk.params_from_workload(wl, max_new_tokens=0), qs, ks, vs)
+    got = torch.from_numpy(cache.query(tk.Q_SCORES)).reshape(4, -1)[:, :N].double().to(DEV)
+    assert cache.status() == 0
+    cache.close()
+    s = torch.einsum("hrd,hjd->hrj", q.double().view(4, G * L, d), k.double()) / d ** 0.5
+    last = N - L + torch.arange(G * L, device=DEV) % L
+    s.masked_fill_(torch.arange(N, device=DEV)[None] > last[:, None], -float("inf"))
+    want = torch.softmax(s, -1).mean(1)
+    assert float((got - want).norm() / want.norm()) < 4e-6
 
 
 # A key with an infinite element that every window row scores -inf weighs nothing, whatever fills the window's tile up: a zero
