@@ -159,9 +159,11 @@ inline UnitRange layer_range(const DeviceProblem& p, int batch, int layer0, int 
   return UnitRange{layer0 * p.n_kv, n_layers * p.n_kv, p.R * p.n_kv, batch * n_layers * p.n_kv};
 }
 
-// Row statistics from caller-supplied normalisers (replaces pass 1): units [u0, u0 + n_units) of one sequence.
-cudaError_t launch_lse_to_stat(const DeviceProblem& p, int u0, int n_units, const float* lse, bool tensor_core_format,
-                               cudaStream_t s);
+// Row statistics from caller-supplied normalisers (replaces pass 1): units [u0, u0 + n_units) of one sequence, as the kernel that
+// reads them has them: pairs (lse log2(e), 1 / rows), one array after the other; offsets lse log2(e) + log2(rows); on the CUDA
+// cores pairs (reference, 1 / sum relative to it) = (lse log2(e), 1).
+enum LseFormat : int { LSE_PAIR, LSE_OFFSET, LSE_CUDA_CORES };
+cudaError_t launch_lse_to_stat(const DeviceProblem& p, int u0, int n_units, const float* lse, LseFormat format, cudaStream_t s);
 
 // kernel launchers (one per translation unit).  Where a launcher takes (layer0, n_layers) it works on those layers
 // of every sequence; n_layers < 0 means all of them.

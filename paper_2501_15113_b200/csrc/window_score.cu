@@ -253,19 +253,20 @@ __global__ void __launch_bounds__(kBlock) window_reduce_kernel(DeviceProblem p, 
 }
 
 // Caller-supplied normalisers lse_i = ln sum_j exp(s_ij) of the window rows, in place of pass 1.  A unit's G*L rows
-// are contiguous in [R][n][L].  Tensor-core path: one offset per row, lse * log2(e) + log2(rows),
-// up to 32 rows the pair (lse * log2(e), 1 / rows), one array after the other; here: the pair
-// (reference, 1 / sum relative to it) = (lse * log2(e), 1).
-__global__ void lse_to_stat_kernel(DeviceProblem p, int u0, const float* __restrict__ lse, int tc_format) {
+// are contiguous in [R][n][L].
+__global__ void lse_to_stat_kernel(DeviceProblem p, int u0, const float* __restrict__ lse, LseFormat format) {
   const int lu = blockIdx.x, row = threadIdx.x;
   if (row >= p.rows) return;
   const float v = lse[(size_t)lu * p.rows + row] * kLog2e;
-  const size_t u = (size_t)(u0 + lu);
-  if (tc_format && p.rows <= 32) {
-    p.stat[u * (2 * p.rows_pad) + row] = v;
-    p.stat[u * (2 * p.rows_pad) + p.rows_pad + row] = 1.0f / (float)p.rows;
-  } else if (tc_format) p.stat[u * (2 * p.rows_pad) + row] = v + log2f((float)p.rows);
-  else reinterpret_cast<float2*>(p.stat)[u * p.rows_pad + row] = make_float2(v, 1.0f);
+  float* st = p.stat + (size_t)(u0 + lu) * (2 * p.rows_pad);
+  if (format == LSE_PAIR) {
+    st[row] = v;
+    st[p.rows_pad + row] = 1.0f / (float)p.rows;
+  } else if (format == LSE_OFFSET) {
+    st[row] = v + log2f((float)p.rows);
+  } else {
+    reinterpret_cast<float2*>(st)[row] = make_float2(v, 1.0f);
+  }
 }
 
 template <int D, int ROWS>
@@ -287,7 +288,7 @@ cudaError_t launch_generic_rows(const DeviceProblem& p, int max_N, const WindowH
     const int per_seq = p.R * p.n_kv;
     const size_t lse_skip = (size_t)(layer0 - h.base_layer) * p.n_heads * p.L;
     for (int b = 0; b < h.batch; ++b) {
-      e = launch_lse_to_stat(p, b * per_seq + ur.first, ur.count, static_cast<const float*>(h.lse[b]) + lse_skip, false, s);
+      e = launch_lse_to_stat(p, b * per_seq + ur.first, ur.count, static_cast<const float*>(h.lse[b]) + lse_skip, LSE_CUDA_CORES, s);
       if (e != cudaSuccess) return e;
     }
   } else {
@@ -319,10 +320,9 @@ cudaError_t launch_generic(const DeviceProblem& p, int max_N, const WindowHostIn
 
 }  // namespace
 
-cudaError_t launch_lse_to_stat(const DeviceProblem& p, int u0, int n_units, const float* lse, bool tensor_core_format,
-                               cudaStream_t s) {
+cudaError_t launch_lse_to_stat(const DeviceProblem& p, int u0, int n_units, const float* lse, LseFormat format, cudaStream_t s) {
   LaunchScope ls(K_WINDOW_REDUCE, s);
-  lse_to_stat_kernel<<<n_units, 128, 0, s>>>(p, u0, lse, tensor_core_format ? 1 : 0);
+  lse_to_stat_kernel<<<n_units, 128, 0, s>>>(p, u0, lse, format);
   return cudaGetLastError();
 }
 

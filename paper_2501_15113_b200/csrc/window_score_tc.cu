@@ -200,6 +200,11 @@ enum : int {
   B_FULL = 0, B_EMPTY = 8, B_QFULL = 16, B_QEMPTY = 18, B_TFULL = 20, B_TEMPTY = 24, B_COUNT = 28
 };
 
+// What pass 2 knows of a row: its maximum and the weight 1 / (sum rows), or one offset max + log2(sum) + log2(rows), with which a
+// score costs one load and one addition less.  An offset is rounded to 2^-24 of itself: with 64 or 128 rows of bf16 to average
+// over that does not show, with up to 32, and beside the error of fp32 scores, it would.
+__host__ __device__ constexpr bool stat_pairs(int rows, bool split) { return split || rows == 32; }
+
 // `W` (32 or 64) scores of this thread's lane; SPLIT: the sum of the two accumulators.
 template <int W, bool SPLIT>
 __device__ __forceinline__ void load_scores(uint32_t taddr, uint32_t (&r)[W]) {
@@ -319,6 +324,7 @@ __global__ void __launch_bounds__(SPLIT ? kSplitThreads : kThreads, 1)
 window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __grid_constant__ TcArgs a,
                  TcLayout lay) {
   constexpr int KB = D / 64;
+  constexpr bool PAIR = stat_pairs(ROWS, SPLIT);
   extern __shared__ unsigned char smem_raw[];
   // 1024-byte alignment: the swizzle pattern is a function of the address bits
   // (offset added to the array itself: a round trip through an integer would turn every access below into a
@@ -602,23 +608,19 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
     constexpr int kWide = SPLIT ? 32 : 64;          // columns per tensor-memory load where many are to be had
     int n = 0;
     bool ok = true;
-    // pass 2: the rows' offsets max + log2(sum) + log2(rows) of a unit (one subtraction then turns a raw score
-    // into its share of C), lane i holding rows i, i + 32, ...; loaded one item ahead
+    // pass 2: the rows' pairs or offsets (which turn a raw score into its share of C) of a unit, lane i holding rows i, i + 32,
+    // ...; loaded one item ahead
     const float* stat_g = p.stat;
-    float pre[4];
+    float pre[4], pre_w[PAIR ? 4 : 1];
     auto fetch_stats = [&](int k) {
       const Item nx = decode_item<SPLIT>(a, k);
       const float* st = stat_g + (size_t)(a.u0[nx.seq] + nx.lu) * (2 * p.rows_pad);
-      if (rows == 32) {
-        // the row's maximum and the weight 1 / (sum rows): with few rows to average over, the rounding of one offset that
-        // holds both would show in the result
-        const bool there = nx.valid && lane < p.rows;
-        pre[0] = there ? st[lane] : 0.f;
-        pre[1] = there ? st[p.rows_pad + lane] : 0.f;
-      } else {
 #pragma unroll
-        for (int q = 0; q < 4; ++q)               // a row that is not there weighs nothing
-          pre[q] = (nx.valid && q * 32 + lane < p.rows) ? st[q * 32 + lane] : INFINITY;
+      for (int q = 0; q < 4; ++q) {               // a row that is not there weighs nothing
+        if (q * 32 >= rows) break;
+        const bool there = nx.valid && q * 32 + lane < p.rows;
+        pre[q] = there ? st[q * 32 + lane] : PAIR ? 0.f : INFINITY;
+        if (PAIR) pre_w[PAIR ? q : 0] = there ? st[p.rows_pad + q * 32 + lane] : 0.f;
       }
     };
     if (a.pass == 2) fetch_stats(0);
@@ -637,7 +639,10 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
         __syncwarp();                       // the previous item's readers of myStat are done
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-          if (q * 32 + lane < (rows == 32 ? 64 : rows)) myStat[q * 32 + lane] = pre[q];
+          if (q * 32 < rows) {
+            myStat[q * 32 + lane] = pre[q];
+            if (PAIR) myStat[rows + q * 32 + lane] = pre_w[PAIR ? q : 0];
+          }
         __syncwarp();
         fetch_stats(k + 1);                 // in flight while this item's tiles are worked on
       }
@@ -792,20 +797,33 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
               uint32_t r[kWide];
               load_scores<kWide, SPLIT>(taddr + (uint32_t)c0, r);
               const float4* st4 = reinterpret_cast<const float4*>(myStat + c0);   // four rows per 16-byte load
+              const float4* wt4 = reinterpret_cast<const float4*>(myStat + rows + c0);
 #pragma unroll
               for (int c = 0; c < kWide; c += 4) {
                 const float4 off = st4[c >> 2];
-                cs[0] += ex2(fmaf(__uint_as_float(r[c]), scale2, -off.x));
-                cs[1] += ex2(fmaf(__uint_as_float(r[c + 1]), scale2, -off.y));
-                cs[2] += ex2(fmaf(__uint_as_float(r[c + 2]), scale2, -off.z));
-                cs[3] += ex2(fmaf(__uint_as_float(r[c + 3]), scale2, -off.w));
+                const float e0 = ex2(fmaf(__uint_as_float(r[c]), scale2, -off.x));
+                const float e1 = ex2(fmaf(__uint_as_float(r[c + 1]), scale2, -off.y));
+                const float e2 = ex2(fmaf(__uint_as_float(r[c + 2]), scale2, -off.z));
+                const float e3 = ex2(fmaf(__uint_as_float(r[c + 3]), scale2, -off.w));
+                if constexpr (PAIR) {
+                  const float4 w = wt4[c >> 2];
+                  cs[0] = fmaf(e0, w.x, cs[0]);
+                  cs[1] = fmaf(e1, w.y, cs[1]);
+                  cs[2] = fmaf(e2, w.z, cs[2]);
+                  cs[3] = fmaf(e3, w.w, cs[3]);
+                } else {
+                  cs[0] += e0;
+                  cs[1] += e1;
+                  cs[2] += e2;
+                  cs[3] += e3;
+                }
               }
             }
           } else if (rows == 32) {
             uint32_t r[32];
             load_scores<32, SPLIT>(taddr, r);
             const float4* mx4 = reinterpret_cast<const float4*>(myStat);
-            const float4* wt4 = reinterpret_cast<const float4*>(myStat + 32);
+            const float4* wt4 = reinterpret_cast<const float4*>(myStat + rows);
             uint32_t vm = FILLED ? 0xffffffffu : (1u << p.rows) - 1u;   // bit c: window row c sees this thread's key
             if (tail) {
               const int need = j < N ? j - (N - L) : L;        // the residue c % L the row must reach (L: none does)
@@ -834,13 +852,17 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
             load_scores<32, SPLIT>(taddr + (uint32_t)c0, r);
             if (!tail) {
               const float4* st4 = reinterpret_cast<const float4*>(myStat + c0);   // four rows per 16-byte load
+              const float4* wt4 = reinterpret_cast<const float4*>(myStat + rows + c0);
 #pragma unroll
               for (int c = 0; c < 32; c += 4) {
-                const float4 off = st4[c >> 2];
-                const float o4[4] = {off.x, off.y, off.z, off.w};
+                const float4 off = st4[c >> 2], w = PAIR ? wt4[c >> 2] : make_float4(1.f, 1.f, 1.f, 1.f);
+                const float o4[4] = {off.x, off.y, off.z, off.w}, w4[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                  if (FILLED || c0 + c + i < p.rows) cs[i] += ex2(fmaf(__uint_as_float(r[c + i]), scale2, -o4[i]));
+                  if (FILLED || c0 + c + i < p.rows) {
+                    const float e = ex2(fmaf(__uint_as_float(r[c + i]), scale2, -o4[i]));
+                    cs[i] = PAIR ? fmaf(e, w4[i], cs[i]) : cs[i] + e;
+                  }
               }
             } else {
               // window row c0 + c sees keys up to N - L + (c0 + c) % L.  The residue is counted along (one
@@ -851,7 +873,10 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
               for (int c = 0; c < 32; ++c) {
                 const float off = myStat[c0 + c];
                 const bool vis = (j < N) && (need <= res) && (FILLED || c0 + c < p.rows);
-                if (vis) cs[c & 3] += ex2(fmaf(__uint_as_float(r[c]), scale2, -off));
+                if (vis) {
+                  const float e = ex2(fmaf(__uint_as_float(r[c]), scale2, -off));
+                  cs[c & 3] = PAIR ? fmaf(e, myStat[rows + c0 + c], cs[c & 3]) : cs[c & 3] + e;
+                }
                 res = (res + 1 == L) ? 0 : res + 1;
               }
             }
@@ -885,10 +910,10 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
   if (tid == 0 && *s_abort) set_status(p.status, TASKKV_ETIMEOUT);
 }
 
-// Folds the partial statistics of one unit -> one offset per row.  One block per unit; 8 to 32 threads share a row, each
+// Folds the partial statistics of one unit -> a pair or an offset per row.  One block per unit; 8 to 32 threads share a row, each
 // taking every 8th to 32nd slot in order with four loads ahead of the dependent updates, and their results are
 // joined in order: the outcome depends on the unit's own length alone.
-__global__ void __launch_bounds__(1024) window_tc_reduce_kernel(DeviceProblem p, UnitRange ur, int fine) {
+__global__ void __launch_bounds__(1024) window_tc_reduce_kernel(DeviceProblem p, UnitRange ur, int fine, int pairs) {
   __shared__ float2 tmp[1024];
   const int u = ur.unit(blockIdx.x);
   const int N = p.unit_N[u];
@@ -929,11 +954,10 @@ __global__ void __launch_bounds__(1024) window_tc_reduce_kernel(DeviceProblem p,
   if (part == 0 && there) {
     for (int q = 1; q < P; ++q) fold_stat(acc, tmp[q * rows + row]);
     float* st = p.stat + (size_t)u * (2 * p.rows_pad);
-    if (rows == 32) {
+    if (pairs) {
       st[row] = acc.y > 0.f ? acc.x : 0.f;
       st[p.rows_pad + row] = acc.y > 0.f ? 1.0f / (acc.y * (float)p.rows) : 0.f;
     } else {
-      // one offset per row: score * scale - (max + log2(sum) + log2(rows)) is log2 of the row's share of C
       st[row] = acc.y > 0.f ? acc.x + log2f(acc.y) + log2f((float)p.rows) : INFINITY;
     }
   }
@@ -1008,7 +1032,7 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
       const size_t lse_skip = (size_t)(layer0 - h.base_layer) * p.n_heads * p.L;
       for (int i = 0; i < nb; ++i) {
         e = launch_lse_to_stat(p, (b0 + i) * per_seq_all + first, per_seq,
-                               static_cast<const float*>(h.lse[b0 + i]) + lse_skip, true, s);
+                               static_cast<const float*>(h.lse[b0 + i]) + lse_skip, stat_pairs(ROWS, SPLIT) ? LSE_PAIR : LSE_OFFSET, s);
         if (e != cudaSuccess) return e;
       }
     } else {
@@ -1016,7 +1040,7 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
       if (e != cudaSuccess) return e;
       LaunchScope ls(K_WINDOW_REDUCE, s);
       const UnitRange ur{b0 * per_seq_all + first, per_seq, per_seq_all, nb * per_seq};
-      e = launch_dependent(window_tc_reduce_kernel, (unsigned)(nb * per_seq), 1024, s, p, ur, a.fine);
+      e = launch_dependent(window_tc_reduce_kernel, (unsigned)(nb * per_seq), 1024, s, p, ur, a.fine, stat_pairs(ROWS, SPLIT) ? 1 : 0);
       if (e != cudaSuccess) return e;
     }
     e = launch_pass(2, 4 * kTile);

@@ -427,6 +427,31 @@ def test_fp32_window_scores_of_elements_of_different_size(G, L, d, N, kind):
     assert float((got - want).norm() / want.norm()) < 4e-6
 
 
+# Scores that are exact (one channel, a few bits) and far from zero, on every row and key alike: what is left is the rounding of the
+# row's statistics.  An exponential is good to 2^-22 and the row's sum and weight to a few units of 2^-24, under 4e-7 in all; a
+# statistic that holds maximum and sum in one word of fp32 is rounded to 2^-24 of itself, which at 50 is 2e-6.
+@pytest.mark.parametrize("shift", [37.0, 301.0])
+@pytest.mark.parametrize("G,L,d,N", [(1, 40, 64, 6001), (2, 32, 128, 4097), (4, 24, 128, 2049), (4, 32, 64, 6001)])
+def test_fp32_window_scores_far_from_zero(G, L, d, N, shift):
+    tk = _tk()
+    wl = small("far", n=4 * G, n_kv=4, d=d, N=N, L=L, s1=4, s2=32, k=40, dtype="f32", nh=0, t=64, steps=1)
+    qs, ks, vs = W.materialize(wl, DEV)
+    q, k = qs[0][0], ks[0][0]
+    q.zero_()
+    k.zero_()
+    q[..., 0] = 8.0
+    k[..., 0] = shift + torch.arange(N, device=DEV).remainder(7) * 0.125
+    cache = tk.taskkv_compress_ex(tk.params_from_workload(wl, max_new_tokens=0), qs, ks, vs)
+    got = torch.from_numpy(cache.query(tk.Q_SCORES)).reshape(4, -1)[:, :N].double().to(DEV)
+    assert cache.status() == 0
+    cache.close()
+    s = torch.einsum("hrd,hjd->hrj", q.double().view(4, G * L, d), k.double()) / d ** 0.5
+    last = N - L + torch.arange(G * L, device=DEV) % L
+    s.masked_fill_(torch.arange(N, device=DEV)[None] > last[:, None], -float("inf"))
+    want = torch.softmax(s, -1).mean(1)
+    assert float((got - want).norm() / want.norm()) < 4e-7
+
+
 # A key with an infinite element that every window row scores -inf weighs nothing, whatever fills the window's tile up: a zero
 # query times infinity is NaN.  (G, L): 9 rows in the single-read kernel and in a tile of 32, 48 in one of 64, 96 in one of
 # 128, and full tiles; with and without the caller's normalisers (which take the two-pass kernel's second pass alone).
