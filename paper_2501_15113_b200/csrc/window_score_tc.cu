@@ -104,6 +104,7 @@ constexpr int kSmallPairs = 5;      // smallest first
 __device__ constexpr int kPairQ[kSmallPairs] = {2, 0, 1, 1, 0};
 __device__ constexpr int kPairK[kSmallPairs] = {0, 2, 1, 0, 1};
 constexpr float kPlaneMax = 7.2057594e16f;   // 2^56: tiles with a larger element, or an infinite one, are scored in fp32
+constexpr int kStageDepth = 8, kStagePitch = kStageDepth + 4;     // floats of a row staged by rescore(): 16-byte writes hit all banks
 constexpr int kOddRing = 8;         // tiles whose marks ("not to be had as planes") are kept
 
 // Work items of one launch (one pass over up to kMaxSeq sequences): (sequence, unit, chunk of chunk_keys keys),
@@ -168,7 +169,7 @@ __device__ __forceinline__ Item decode_item(const TcArgs& a, int k) {
 struct TcLayout {
   int stages, q_bufs;
   int tile_bytes, q_block_bytes;      // SPLIT: a stage is the planes of 64 elements of a tile's keys
-  int off_q, off_stat, off_trans, off_bars;
+  int off_q, off_stat, off_trans, off_stage, off_bars;
   int total;
 };
 
@@ -180,9 +181,10 @@ inline TcLayout make_layout(int D, int rows, bool split) {
   const int stat = kEpiWarps * rows * (int)sizeof(float2);
   // with 128 rows pass 1 puts the window rows on the TMEM lanes and needs no transposition
   const int trans = rows == 128 ? 0 : kEpiWarps * 32 * 33 * (int)sizeof(float);
+  const int stage = split ? kEpiWarps * 32 * kStagePitch * (int)sizeof(float) : 0;
   const int bars = 512;
   const int budget = 232448 - 1024;     // dynamic shared memory of one CTA minus the alignment slack
-  auto fit = [&](int q_bufs) { return (budget - q_bufs * l.q_block_bytes - stat - trans - bars) / l.tile_bytes; };
+  auto fit = [&](int q_bufs) { return (budget - q_bufs * l.q_block_bytes - stat - trans - stage - bars) / l.tile_bytes; };
   l.q_bufs = split && fit(2) < 2 ? 1 : 2;
   int stages = fit(l.q_bufs);
   if (stages > kMaxStages) stages = kMaxStages;
@@ -190,7 +192,8 @@ inline TcLayout make_layout(int D, int rows, bool split) {
   l.off_q = l.stages * l.tile_bytes;
   l.off_stat = l.off_q + l.q_bufs * l.q_block_bytes;
   l.off_trans = l.off_stat + stat;
-  l.off_bars = l.off_trans + trans;
+  l.off_stage = l.off_trans + trans;
+  l.off_bars = l.off_stage + stage;
   l.total = l.off_bars + bars + 1024;
   return l;
 }
@@ -292,24 +295,61 @@ __device__ __forceinline__ void prefetch_rows(const void* src, int rows, int byt
   if (rows > 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(rows * bytes) : "memory");
 }
 // A tile with an element, of its keys or of the queries, that planes do not hold (too large for products and sums to stay finite,
-// or infinite itself: products of planes are NaN where the score is infinite): the tile is scored again in fp32, this thread's lane against `n` rows of `other`,
-// and put into the accumulators.  Rare, hence slow and a call of its own.
+// or infinite itself: products of planes are NaN where the score is infinite): the tile is scored again in fp32, this thread's
+// lane against `n` rows of `other`, and put into the accumulators.  A call of its own: a few elements at a time, of the lane's
+// row in registers and of 32 other rows in the warp's shared memory (`stage`), from where a load serves all lanes; the next ones
+// are on their way meanwhile.  Eight elements, since what the call needs in registers the code around it spills (sixteen: ordinary
+// calls 6 to 20 % slower).  32 units of 6001 keys, d = 64, all tiles scored like this, both passes: 64 rows 0.35 ms, 128 rows
+// 0.56; on the CUDA cores alone 0.15 and 0.25; with a load of either side from global memory for every product 7.9 and 14.
 template <int D>
 __device__ __noinline__ void rescore(uint32_t taddr, const float* __restrict__ mine, bool there, const float* __restrict__ other,
-                                     int n, int cols) {
-  for (int c0 = 0; c0 < cols; c0 += 32) {
-    uint32_t r[32], zero[32];
+                                     int n, int cols, float* stage) {
+  constexpr int V = kStageDepth / 4;
+  const int lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int c0 = 0; c0 < cols && c0 < n; c0 += 32) {
+    float sum[32];
 #pragma unroll
-    for (int c = 0; c < 32; ++c) {
-      float sum = 0.f;
-      if (there && c0 + c < n)
-        for (int x = 0; x < D; ++x) sum = fmaf(mine[x], other[(size_t)(c0 + c) * D + x], sum);
-      r[c] = __float_as_uint(sum);
-      zero[c] = 0u;
+    for (int c = 0; c < 32; ++c) sum[c] = 0.f;
+    const float* theirs = other + (size_t)min(c0 + lane, n - 1) * D;
+    float4 m[V], o[V];
+#pragma unroll
+    for (int i = 0; i < V; ++i) { m[i] = reinterpret_cast<const float4*>(mine)[i]; o[i] = reinterpret_cast<const float4*>(theirs)[i]; }
+#pragma unroll 1
+    for (int x = 0; x < D; x += kStageDepth) {
+      __syncwarp();                                   // the rows staged before have been read
+#pragma unroll
+      for (int i = 0; i < V; ++i) *reinterpret_cast<float4*>(stage + lane * kStagePitch + 4 * i) = o[i];
+      __syncwarp();
+      const int next = x + kStageDepth < D ? x + kStageDepth : x;
+      float4 m1[V];
+#pragma unroll
+      for (int i = 0; i < V; ++i) {
+        m1[i] = reinterpret_cast<const float4*>(mine + next)[i];
+        o[i] = reinterpret_cast<const float4*>(theirs + next)[i];
+      }
+#pragma unroll
+      for (int c = 0; c < 32; ++c) {
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+          const float4 v = *reinterpret_cast<const float4*>(stage + c * kStagePitch + 4 * i);
+          sum[c] = fmaf(m[i].x, v.x, sum[c]);
+          sum[c] = fmaf(m[i].y, v.y, sum[c]);
+          sum[c] = fmaf(m[i].z, v.z, sum[c]);
+          sum[c] = fmaf(m[i].w, v.w, sum[c]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < V; ++i) m[i] = m1[i];
     }
+    uint32_t r[32];
+#pragma unroll
+    for (int c = 0; c < 32; ++c) r[c] = there && c0 + c < n ? __float_as_uint(sum[c]) : 0u;
     __syncwarp();
     tc_st32(taddr + (uint32_t)c0, r);
-    tc_st32(taddr + 128u + (uint32_t)c0, zero);
+#pragma unroll
+    for (int c = 0; c < 32; ++c) r[c] = 0u;
+    tc_st32(taddr + 128u + (uint32_t)c0, r);
   }
   tc_wait_st();
 }
@@ -706,7 +746,8 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
             const bool swap = a.pass == 1 && rows == 128;
             const bool there = swap ? l < p.rows : tbase + l < N;
             const float* mine = swap ? q + (size_t)(there ? l : 0) * D : kp + (size_t)(there ? tbase + l : 0) * D;
-            rescore<D>(taddr, mine, there, swap ? kp + (size_t)tbase * D : q, swap ? min(kTile, N - tbase) : p.rows, swap ? kTile : rows);
+            rescore<D>(taddr, mine, there, swap ? kp + (size_t)tbase * D : q, swap ? min(kTile, N - tbase) : p.rows, swap ? kTile : rows,
+                       reinterpret_cast<float*>(smem + lay.off_stage) + ew * (32 * kStagePitch));
           }
         }
         const bool tail = (tbase + kTile - 1 > N - L);   // some key of the tile is masked for some row

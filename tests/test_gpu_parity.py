@@ -452,6 +452,29 @@ def test_fp32_window_scores_far_from_zero(G, L, d, N, shift):
     assert float((got - want).norm() / want.norm()) < 4e-7
 
 
+# A call all of whose tiles hold an element that planes do not (queries times 2^60, keys times 2^-60: the same scores) costs no
+# more than a few ordinary ones.  (In plain loops over global memory it cost fifty to a hundred.)
+@pytest.mark.parametrize("G,d", [(2, 64), (4, 128)])
+def test_fp32_window_scores_beyond_the_planes_range_are_not_slow(G, d):
+    tk = _tk()
+    wl = small("slow", n=16 * G, n_kv=16, d=d, N=6001, L=32, s1=4, s2=32, k=40, dtype="f32", nh=0, t=64, steps=1)
+    qs, ks, vs = W.materialize(wl, DEV)
+    params = tk.params_from_workload(wl, max_new_tokens=0)
+    best = []
+    for q, k in ((qs, ks), ([t * 2.0 ** 60 for t in qs], [t * 2.0 ** -60 for t in ks])):
+        ms = []
+        for _ in range(6):
+            begin, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            begin.record()
+            cache = tk.taskkv_compress_ex(params, q, k, vs)
+            end.record()
+            torch.cuda.synchronize()
+            ms.append(begin.elapsed_time(end))
+            cache.close()
+        best.append(min(ms))
+    assert best[1] < 8 * best[0], best
+
+
 # A key with an infinite element that every window row scores -inf weighs nothing, whatever fills the window's tile up: a zero
 # query times infinity is NaN.  (G, L): 9 rows in the single-read kernel and in a tile of 32, 48 in one of 64, 96 in one of
 # 128, and full tiles; with and without the caller's normalisers (which take the two-pass kernel's second pass alone).
