@@ -1198,10 +1198,14 @@ STREAM_CASES = [
     # whose tile counts are odd (9 and 19 tiles), while the per-layer launches give every CTA one item: the partial
     # row statistics must not depend on what a CTA worked on before
     dict(n=16, n_kv=8, d=64, N=0, L=32, s1=4, s2=64, k=70, dtype="bf16", R=8, seq_lens=[2400, 1150, 3300], nh=1),
+    # fp32 as planes of bf16: 48 rows in a tile of 64, and 128 rows of which a call has several items per CTA
+    dict(n=8, n_kv=4, d=128, N=0, L=24, s1=4, s2=32, k=50, dtype="f32", R=3, seq_lens=[900, 2500], nh=1),
+    dict(n=16, n_kv=4, d=64, N=0, L=32, s1=4, s2=64, k=70, dtype="f32", R=8, seq_lens=[2400, 1150, 3300], nh=1),
 ]
 
 
-@pytest.mark.parametrize("case", STREAM_CASES, ids=["bf16_gqa_ragged", "bf16_mha", "f32", "bf16_64rows_many_items"])
+@pytest.mark.parametrize("case", STREAM_CASES, ids=["bf16_gqa_ragged", "bf16_mha", "f32", "bf16_64rows_many_items", "f32_48rows",
+                                               "f32_128rows_many_items"])
 def test_layers_streamed_into_one_cache_equal_the_all_layer_call(case):
     """taskkv_cache_create + one taskkv_compress_layer per layer, in a scrambled order and with every layer's
     tensors in allocations of their own, against taskkv_compress_ex over all layers: semantic vectors, distances,
@@ -1445,7 +1449,9 @@ def test_random_shapes(seed):
     dict(n=4, n_kv=4, d=64, N=1500, L=16, s1=4, s2=32, k=77, dtype="f32"),               # CUDA-core path
     dict(n=4, n_kv=4, d=64, N=1500, L=9, s1=4, s2=32, k=77, dtype="bf16"),               # 9 rows in a tile of 32
     dict(n=8, n_kv=4, d=128, N=1500, L=24, s1=4, s2=32, k=77, dtype="bf16"),             # 48 rows in a tile of 64
-], ids=["tc32", "tc128_ragged", "f32", "tc9", "tc48"])
+    dict(n=8, n_kv=4, d=128, N=1500, L=24, s1=4, s2=32, k=77, dtype="f32"),              # 48 rows as planes
+    dict(n=8, n_kv=2, d=64, N=0, L=32, s1=4, s2=64, k=150, dtype="f32", R=2, seq_lens=[3000, 1777], nh=1),    # 128 rows as planes
+], ids=["tc32", "tc128_ragged", "f32", "tc9", "tc48", "f32_48", "f32_128_ragged"])
 def test_compress_with_supplied_window_lse(case):
     """With the window rows' log-sum-exp handed in (here: the oracle's, rounded to fp32) pass 1 is skipped; scores,
     selections, classes, rows and decode outputs must match the oracle exactly as in the full computation."""
@@ -1573,7 +1579,9 @@ def test_host_buffer_calls_return_the_sticky_device_status():
     dict(G=2, splits=[(0, 3), (3, 8)], dtype="bf16", frac=0.0),          # uneven shards, 64 window rows
     dict(G=4, splits=[(0, 2), (2, 4), (4, 8)], dtype="bf16", frac=0.35),  # three shards, 128 rows, budget as a fraction
     dict(G=1, splits=[(0, 4), (4, 8)], dtype="f32", frac=0.0),            # CUDA-core path
-], ids=["g2_uneven", "g4_three_budget_frac", "f32"])
+    dict(G=2, splits=[(0, 3), (3, 8)], dtype="f32", frac=0.0),            # fp32 as planes, 64 and 128 window rows
+    dict(G=4, splits=[(0, 2), (2, 4), (4, 8)], dtype="f32", frac=0.35),
+], ids=["g2_uneven", "g4_three_budget_frac", "f32", "f32_g2_uneven", "f32_g4_three_budget_frac"])
 def test_head_sharded_compression_equals_the_unsharded_call(case):
     """Every shard runs Eq. 12-15 for its own heads (taskkv_compress_shard_begin), the semantic vectors of all shards
     are put side by side in head order (what the ranks' all-gather produces), and every shard finishes with the
@@ -1662,7 +1670,9 @@ def test_head_sharded_compression_equals_the_unsharded_call(case):
     dict(n=16, n_kv=4, d=128, N=0, L=32, s1=4, s2=64, k=120, dtype="bf16", R=3, seq_lens=[2100, 1300], nh=1, P=64),
     dict(n=8, n_kv=8, d=128, N=0, L=32, s1=4, s2=64, k=150, dtype="bf16", R=2, seq_lens=[5000], nh=2, P=256),
     dict(n=4, n_kv=4, d=64, N=0, L=16, s1=4, s2=32, k=60, dtype="f32", R=2, seq_lens=[900, 700], nh=1, P=128),
-], ids=["bf16_gqa_p64", "bf16_mha_p256", "f32_p128"])
+    dict(n=16, n_kv=4, d=64, N=0, L=32, s1=4, s2=32, k=60, dtype="f32", R=2, seq_lens=[2500, 700], nh=1, P=64),
+    dict(n=8, n_kv=4, d=128, N=0, L=24, s1=4, s2=32, k=60, dtype="f32", R=2, seq_lens=[900, 1700], nh=1, P=128),
+], ids=["bf16_gqa_p64", "bf16_mha_p256", "f32_p128", "f32_128rows_p64", "f32_48rows_p128"])
 def test_paged_cache_equals_the_contiguous_cache(case):
     """The same compression with the rows in pages: classes, lengths and retained positions are the contiguous
     cache's, every unit's rows read back through its page table are the same bytes, and so are the decode outputs of
