@@ -303,7 +303,9 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
         myOff[i] = (z > 0.f && x.b * kTile + i < a.N) ? -(M + log2f(z) + 7.f) : -INFINITY;
       }
       __syncwarp();
-      // ---- second walk: this thread's key, summed over the rows
+      // ---- second walk: this thread's key, summed over the rows (of which the last block may have fewer; what stands in their
+      // place is another head's query or zero, and its score at a key with an infinite element may be NaN: left out)
+      const int rows_here = min(kTile, a.N - x.b * kTile);
       float* out = a.scores + (int64_t)x.head * 64 * a.nb * (a.nb + 1) + (int64_t)64 * x.b * (x.b + 1);
       for (int t = 0; t < T; ++t, ++n) {
         if ((n & (kGroups - 1)) != grp) continue;
@@ -313,22 +315,41 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
         tc_fence_after();
         const bool tail = t == T - 1;
         float2 cs[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        if (rows_here == kTile) {
 #pragma unroll
-        for (int c0 = 0; c0 < kTile; c0 += kCols) {
-          uint32_t r[kCols];
-          tc_ld32(lane_addr + (uint32_t)(acc * 128 + c0), r);
-          tc_wait_ld();
-          if (tail) {                               // key i is seen by rows i .. 127 of the block
+          for (int c0 = 0; c0 < kTile; c0 += kCols) {
+            uint32_t r[kCols];
+            tc_ld32(lane_addr + (uint32_t)(acc * 128 + c0), r);
+            tc_wait_ld();
+            if (tail) {                               // key i is seen by rows i .. 127 of the block
+#pragma unroll
+              for (int i = 0; i < kCols; ++i)
+                if (c0 + i < row) r[i] = __float_as_uint(-INFINITY);
+            }
+            const float4* off4 = reinterpret_cast<const float4*>(myOff + c0);
+#pragma unroll
+            for (int i = 0; i < kCols; i += 4) {
+              const float4 off = off4[i >> 2];
+              cs[0] = __fadd2_rn(cs[0], weight2(i, __ffma2_rn(pair_of(r, i), scale22, make_float2(off.x, off.y))));
+              cs[1] = __fadd2_rn(cs[1], weight2(i + 2, __ffma2_rn(pair_of(r, i + 2), scale22, make_float2(off.z, off.w))));
+            }
+          }
+        } else {
+#pragma unroll 1
+          for (int c0 = 0; c0 < kTile; c0 += kCols) {
+            uint32_t r[kCols];
+            tc_ld32(lane_addr + (uint32_t)(acc * 128 + c0), r);
+            tc_wait_ld();
 #pragma unroll
             for (int i = 0; i < kCols; ++i)
-              if (c0 + i < row) r[i] = __float_as_uint(-INFINITY);
-          }
-          const float4* off4 = reinterpret_cast<const float4*>(myOff + c0);
+              if ((tail && c0 + i < row) || c0 + i >= rows_here) r[i] = __float_as_uint(-INFINITY);
+            const float4* off4 = reinterpret_cast<const float4*>(myOff + c0);
 #pragma unroll
-          for (int i = 0; i < kCols; i += 4) {
-            const float4 off = off4[i >> 2];
-            cs[0] = __fadd2_rn(cs[0], weight2(i, __ffma2_rn(pair_of(r, i), scale22, make_float2(off.x, off.y))));
-            cs[1] = __fadd2_rn(cs[1], weight2(i + 2, __ffma2_rn(pair_of(r, i + 2), scale22, make_float2(off.z, off.w))));
+            for (int i = 0; i < kCols; i += 4) {
+              const float4 off = off4[i >> 2];
+              cs[0] = __fadd2_rn(cs[0], weight2(i, __ffma2_rn(pair_of(r, i), scale22, make_float2(off.x, off.y))));
+              cs[1] = __fadd2_rn(cs[1], weight2(i + 2, __ffma2_rn(pair_of(r, i + 2), scale22, make_float2(off.z, off.w))));
+            }
           }
         }
         out[t * kTile + row] = (cs[0].x + cs[0].y) + (cs[1].x + cs[1].y);

@@ -1529,6 +1529,31 @@ def test_exact_semantic_vector(case):
             assert np.abs(P.to64(sem[r, h]) - want_v).max() < bound
 
 
+# Keys that every row scores -inf have a column mean of zero and change nothing else, in whole and ragged blocks of rows; the
+# rows that fill the last block up (the next head's, or zeros, whose score at such a key is NaN) take no part.  Tolerance: as for
+# the window's scores above.
+@pytest.mark.parametrize("n,n_kv,d,N", [(2, 2, 64, 9), (4, 2, 128, 300), (2, 1, 64, 384), (2, 2, 128, 1000)])
+def test_exact_semantic_key_that_every_row_scores_minus_infinity(n, n_kv, d, N):
+    tk = _tk()
+    g = torch.Generator(device="cpu").manual_seed(N)
+    std = float(d) ** -0.25
+    q = torch.randn(1, n, N, d, generator=g) * std
+    q[..., 3] = q[..., 3].abs() + 0.5
+    k = torch.randn(1, n_kv, N, d, generator=g) * std
+    dead = [1, N // 2, N - 1]
+    k[:, :, dead, 3] = -float("inf")
+    q, k = q.bfloat16().to(DEV), k.bfloat16().to(DEV)
+    v = torch.randn(1, n_kv, N, d, generator=g).bfloat16().to(DEV)
+    sem, c = tk.taskkv_exact_semantic(q, k, v)
+    s = torch.einsum("hgid,hjd->hgij", q[0].double().view(n_kv, n // n_kv, N, d), k[0].double()) / d ** 0.5
+    s.masked_fill_(torch.ones(N, N, dtype=torch.bool, device=DEV).triu(1), -float("inf"))
+    want = torch.softmax(s, -1).mean((1, 2))
+    assert not c[0][:, dead].any()
+    assert float((c[0].double() - want).norm() / want.norm()) < 1e-6
+    want_v = torch.einsum("hj,hjd->hd", want, v[0].double())
+    assert float((sem[0].double() - want_v).abs().max()) < 1e-6
+
+
 # ---------------------------------------------------------------------------
 # Error reporting across the boundary
 # ---------------------------------------------------------------------------
