@@ -158,8 +158,8 @@ static __device__ __forceinline__ float ex2(float x) {
 // 2^x of a pair on the FMA pipe, for x <= 0 (and up to 127), where the special-function unit's 16 exponentials a cycle and
 // SM are what a kernel is bound by: n = round(x), 2^(x - n) by a polynomial of degree 6 on [-1/2, 1/2] (a least-squares fit
 // reweighted to equal relative errors, its constant term held at 1: 2e-9 before rounding, 8e-8 at most and 2.7e-8 in the mean
-// square in fp32 with these coefficients), times 2^n built as exponent bits.  Below 2^-126 the result is 0 (x = -inf
-// included), as with ex2; NaN stays NaN.  7 issue slots an exponential, since all but the clamp and the shift are packed.
+// square in fp32 with these coefficients), times 2^n built as exponent bits.  Below x = -126.5 the result is 0 (x = -inf
+// included), from there to -126 it is subnormal, where ex2 gives 0 below -126; NaN stays NaN.  7 issue slots an exponential, since all but the clamp and the shift are packed.
 static __device__ __forceinline__ float max_nan(float a, float b) {
   float y;
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));

@@ -1554,6 +1554,36 @@ def test_exact_semantic_key_that_every_row_scores_minus_infinity(n, n_kv, d, N):
     assert float((sem[0].double() - want_v).abs().max()) < 1e-6
 
 
+def test_exact_semantic_one_exponential_at_a_time():
+    """The last of nine keys is seen by the last row alone, and both sit where the exact vector's exponentials go through the FMA
+    pipe, so that its column mean is one of them: 2^x / (8 + 2^x) / 9 with x swept over the exponential's whole range, a head per
+    value.  The argument, x - log2(row sum) - 7, is rounded twice at up to 16 for x in [-2, 0] (2 x 2^-21 ln 2) after a sum and a
+    logarithm of a few units of 2^-23: under 1.5e-6, which leaves the polynomial's 8e-8 no room for another coefficient's last
+    digits.  Further down the score's own 64 products are summed to 2^-21 of up to 115: 4e-5."""
+    tk = _tk()
+    H, d = 4096, 64
+    g = torch.Generator(device="cpu").manual_seed(5)
+    x = torch.cat([torch.linspace(-2.0, 0.0, H // 2), torch.linspace(-130.0, -2.0, H // 2)])
+    q = torch.ones(1, H, 9, d, dtype=torch.bfloat16)
+    k = torch.zeros(1, H, 9, d, dtype=torch.bfloat16)
+    k[0, :, 8] = ((x * 8.0 / 1.4426950408889634 / d)[:, None] * (0.5 + torch.rand(H, d, generator=g))).bfloat16()
+    k[0, H - 1, 8] = 0.0
+    k[0, H - 1, 8, 5] = -float("inf")
+    k[0, H - 2, 8, 5] = float("nan")
+    v = torch.zeros_like(k)
+    _, c = tk.taskkv_exact_semantic(q.to(DEV), k.to(DEV), v.to(DEV))
+    got = c[0, :, 8].double().cpu()
+    w = torch.exp2(k[0, :, 8].double().sum(-1) / 8.0 * 1.4426950408889634)
+    want = w / (8.0 + w) / 9.0
+    assert got[H - 1] == 0.0 and torch.isnan(got[H - 2])
+    y = torch.log2(w)
+    near, deep, gone = y > -2.0, (y <= -2.0) & (y > -115.0), y < -118.0
+    assert near.sum() > 1000 and deep.sum() > 1000 and gone.sum() > 50
+    assert float((got / want - 1.0)[near].abs().max()) < 1.5e-6
+    assert float((got / want - 1.0)[deep].abs().max()) < 4e-5
+    assert bool(((got >= 0.0) & (got < 2.0 ** -120))[gone].all())
+
+
 # ---------------------------------------------------------------------------
 # Error reporting across the boundary
 # ---------------------------------------------------------------------------
