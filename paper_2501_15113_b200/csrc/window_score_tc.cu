@@ -252,10 +252,9 @@ __device__ __forceinline__ void split8(const float4& lo, const float4& hi, uint4
 // neighbouring words (which element is where in a row of planes does not matter as long as keys and queries agree).
 constexpr int kCvtThreads = kCvtWarps * 32, kBatchRows = kCvtThreads / 8 * 4;
 struct Batch { float4 lo[4], hi[4]; };
-template <int B>
 __device__ __forceinline__ void load_batch(Batch& x, const float* __restrict__ src, int pitch, int there, int i) {
 #pragma unroll
-  for (int b = 0; b < B; ++b) {
+  for (int b = 0; b < 4; ++b) {
     const int row = (b * kCvtThreads + i) >> 3, c = i & 7;
     x.lo[b] = x.hi[b] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (row < there) {
@@ -267,11 +266,10 @@ __device__ __forceinline__ void load_batch(Batch& x, const float* __restrict__ s
 }
 // ... as three planes in shared memory, rows of 128 bytes in the 128-byte swizzle, plane_pitch bytes apart (dst: the batch's
 // first row, a multiple of eight).  Returns the largest |element| that this thread has (a NaN is not seen; it stays one).
-template <int B>
 __device__ __forceinline__ float store_batch(const Batch& x, unsigned char* dst, int plane_pitch, int i) {
   float top = 0.f;
 #pragma unroll
-  for (int b0 = 0; b0 < B; b0 += 2) {
+  for (int b0 = 0; b0 < 4; b0 += 2) {
     uint4 plane[2][kPlanes];
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
@@ -370,8 +368,8 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
   // (offset added to the array itself: a round trip through an integer would turn every access below into a
   // generic-address load or store)
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  unsigned char* sK = smem;                                         // [stages][KB][128 keys][128 B]
-  unsigned char* sQ = smem + lay.off_q;                             // [2][KB][rows][128 B]
+  unsigned char* sK = smem;                                         // [stages][KB][128 keys][128 B]; SPLIT: [stages][planes][128 keys][128 B]
+  unsigned char* sQ = smem + lay.off_q;                             // [2][KB][rows][128 B]; SPLIT: [q_bufs][planes][KB][rows][128 B]
   float2* sStat = reinterpret_cast<float2*>(smem + lay.off_stat);   // [8 warps][rows]
   float* sTrans = reinterpret_cast<float*>(smem + lay.off_trans);   // [8 warps][32][33]
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + lay.off_bars);
@@ -431,35 +429,36 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
       const float* q = static_cast<const float*>(p.q_ptr[u]);
       const float* kp = static_cast<const float*>(p.k_ptr[u]);
       if (i == 0) prefetch_rows(kp + (size_t)key0 * D, min(2 * kTile, end - key0), D * 4);
-      constexpr int kQBatch = ROWS < kBatchRows ? ROWS / (kCvtThreads / 8) : 4, kQBatches = ROWS < kBatchRows ? 1 : ROWS / kBatchRows;
+      constexpr int kQBatches = SPLIT ? ROWS / kBatchRows : 1;
+      static_assert(!SPLIT || ROWS % kBatchRows == 0, "the queries' rows are converted in whole batches");
       float q_top = 0.f;
 #pragma unroll 1
       for (int x = 0; x < KB * kQBatches; ++x) {
         const int kb = x / kQBatches, r0 = x % kQBatches * kBatchRows;
         Batch qx;
-        load_batch<kQBatch>(qx, q + (size_t)r0 * D + kb * 64, D, p.rows - r0, i);
+        load_batch(qx, q + (size_t)r0 * D + kb * 64, D, p.rows - r0, i);
         if (x == 0) ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_QEMPTY + qb), qphase[qb] ^ 1, s_abort));
         if (!ok) break;
-        q_top = fmaxf(q_top, store_batch<kQBatch>(qx, sQ + (size_t)qb * lay.q_block_bytes + (kb * ROWS + r0) * 128, KB * ROWS * 128, i));
+        q_top = fmaxf(q_top, store_batch(qx, sQ + (size_t)qb * lay.q_block_bytes + (kb * ROWS + r0) * 128, KB * ROWS * 128, i));
       }
       if (!ok) break;
       hand_over(B_QFULL + qb);
       qphase[qb] ^= 1;
       if (lay.q_bufs == 2) qb ^= 1;
       Batch x0, x1;
-      load_batch<4>(x0, kp + (size_t)key0 * D, D, it.N - key0, i);
+      load_batch(x0, kp + (size_t)key0 * D, D, it.N - key0, i);
       float top = q_top;
       for (int c = 0; c < ntiles * KB; ++c) {
         const int t = c / KB, kb = c % KB, at = key0 + t * kTile;
-        load_batch<4>(x1, kp + (size_t)(at + kBatchRows) * D + kb * 64, D, it.N - at - kBatchRows, i);
+        load_batch(x1, kp + (size_t)(at + kBatchRows) * D + kb * 64, D, it.N - at - kBatchRows, i);
         if (kb == 0 && i == 0) prefetch_rows(kp + (size_t)(at + 2 * kTile) * D, min(kTile, end - at - 2 * kTile), D * 4);
         ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_EMPTY + stage), phase ^ 1, s_abort));
         if (!ok) break;
         unsigned char* dst = sK + (size_t)stage * lay.tile_bytes;
-        top = fmaxf(top, store_batch<4>(x0, dst, kTile * 128, i));
+        top = fmaxf(top, store_batch(x0, dst, kTile * 128, i));
         const int t1 = (c + 1) / KB, at1 = key0 + t1 * kTile;
-        if (c + 1 < ntiles * KB) load_batch<4>(x0, kp + (size_t)at1 * D + (c + 1) % KB * 64, D, it.N - at1, i);
-        top = fmaxf(top, store_batch<4>(x1, dst + kBatchRows * 128, kTile * 128, i));
+        if (c + 1 < ntiles * KB) load_batch(x0, kp + (size_t)at1 * D + (c + 1) % KB * 64, D, it.N - at1, i);
+        top = fmaxf(top, store_batch(x1, dst + kBatchRows * 128, kTile * 128, i));
         if (kb == KB - 1) {
           // (the tile whose entry this was is done: its accumulator has been used again since)
           const bool all = __all_sync(0xffffffffu, top < kPlaneMax);
@@ -1033,6 +1032,7 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
   for (int b0 = 0; b0 < h.batch; b0 += kMaxSeq) {
     const int nb = h.batch - b0 < kMaxSeq ? h.batch - b0 : kMaxSeq;
     TcMaps maps;
+    if (SPLIT) maps = TcMaps{};                              // fp32 rows are read through the units' pointers
     TcArgs a;
     int64_t keys = 0;
     for (int i = 0; i < nb; ++i) keys += (int64_t)per_seq * h.seq_lens[b0 + i];
@@ -1041,10 +1041,11 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
     for (int i = 0; i < kMaxSeq; ++i) {
       const int b = b0 + (i < nb ? i : 0);                  // unused slots repeat the first sequence
       const int N = h.seq_lens[b];
-      if (i >= nb) {
+      if (SPLIT) {
+      } else if (i >= nb) {
         maps.k[i] = maps.k[0];
         maps.q[i] = maps.q[0];
-      } else if (!SPLIT) {                                      // (fp32 rows are read through the units' pointers)
+      } else {
         const char* kb = static_cast<const char*>(h.k[b]) + (size_t)skip * (size_t)N * D * sizeof(__nv_bfloat16);
         const char* qb = static_cast<const char*>(h.q[b]) + (size_t)skip * p.rows * D * sizeof(__nv_bfloat16);
         if (!make_tensor_map_2d(&maps.k[i], kb, D, (uint64_t)per_seq * (uint64_t)N, kTile)) return cudaErrorUnknown;
