@@ -219,11 +219,12 @@ taskkv_status make_plan(const taskkv_params* p, HostPlan& hp, int32_t page_rows 
   hp.c_total = c_total;
   hp.rows = G * p->window;
   hp.rows_pad = (hp.rows + 15) / 16 * 16;
-  // partial-statistic slots per unit: one per 256-key chunk on the CUDA-core path, one per epilogue warp and 2048 keys on
-  // the tensor-core path
+  // partial-statistic slots per unit: one per 256-key chunk on the CUDA-core path, one per epilogue warp and 2048 keys (512
+  // where fp32 rows take tiles of 64, window_score_tc.cu) on the tensor-core path
   {
     const int generic = (hp.max_N + kScoreChunk - 1) / kScoreChunk;
-    const int tc = (hp.max_N + kTcChunk - 1) / kTcChunk * kTcParts;
+    const int part = p->dtype == TASKKV_F32 && hp.rows > 32 && hp.rows <= 64 ? kTcChunk / 4 : kTcChunk;
+    const int tc = (hp.max_N + part - 1) / part * kTcParts;
     hp.chunks_max = generic > tc ? generic : tc;
   }
 

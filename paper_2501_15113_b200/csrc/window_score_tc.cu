@@ -122,7 +122,7 @@ struct TcArgs {
   int n_seq;                // sequences in this launch
   int n_local;              // units per sequence (layers * kv heads)
   int chunk_keys;           // keys per work item (multiple of 512)
-  int fine;                 // 128 rows, items shorter than 2048 keys: pass 1 stores every 512 keys
+  int fine;                 // fine parts and items shorter than 2048 keys: pass 1 stores every 512 keys
   int steps;                // items of the busiest CTA
   int u0[kMaxSeq];          // first unit of each sequence
   int N[kMaxSeq];           // sequence length
@@ -207,6 +207,12 @@ enum : int {
 // score costs one load and one addition less.  An offset is rounded to 2^-24 of itself: with 64 or 128 rows of bf16 to average
 // over that does not show, with up to 32, and beside the error of fp32 scores, it would.
 __host__ __device__ constexpr bool stat_pairs(int rows, bool split) { return split || rows == 32; }
+
+// Whether pass 1's items may be shorter than 2048 keys, down to the 512 of one part.  Four times the slots of a row: with 128
+// rows a slot is two warps' and there is room; fp32 rows get it (partial_slots), since a tile of theirs takes two to three times
+// as long and a call of few units waits for one CTA's walk over 16 of them (8 units of 2500 keys, 64 rows: 73 us a call
+// with 2048, 53 with 512 at d = 64, 98 and 67 at d = 128; on the CUDA cores 56 and 77).
+__host__ __device__ constexpr bool fine_parts(int rows, bool split) { return split || rows == 128; }
 
 // `W` (32 or 64) scores of this thread's lane; SPLIT: the sum of the two accumulators.
 template <int W, bool SPLIT>
@@ -689,35 +695,35 @@ window_tc_kernel(const __grid_constant__ TcMaps maps, DeviceProblem p, const __g
       // at the item's start it is the even ones.  The partial statistics below are filed under that parity, not under
       // the group, so that a slot always holds the same tiles (and keys) whatever else the CTA worked on before:
       // results do not depend on how a problem is cut into launches -- nor on the length of the items: what is stored
-      // covers 16 tiles of the unit, and with 128 rows those are folded from four parts of 4 tiles each, here (long
+      // covers 16 tiles of the unit, and with fine parts those are folded from four parts of 4 tiles each, here (long
       // items) or, where items are shorter than 16 tiles (a.fine), from the stored parts by the reduction.
       const int par = grp ^ (n & 1);                 // parity, within the item, of the tiles this warp takes
-      const int sub_shift = rows == 128 ? 2 : 4;     // log2 of the tiles per part
+      constexpr int sub_shift = fine_parts(ROWS, SPLIT) ? 2 : 4;     // log2 of the tiles per part
       int sub = 0;                                   // the part this warp is working on, counted from the item's first
-      float2 group = make_float2(-INFINITY, 0.f);
+      constexpr int kGroupRows = ROWS == 128 ? 1 : ROWS / 32;        // rows of this lane
+      float2 group[kGroupRows];
+#pragma unroll
+      for (int rg = 0; rg < kGroupRows; ++rg) group[rg] = make_float2(-INFINITY, 0.f);
       auto end_part = [&]() {
         // slot (part of the unit, part of the warps): (tile parity, lane quadrant); with 128 rows a quadrant is a set of
         // rows, so there it is the tile parity alone
         float2* base = reinterpret_cast<float2*>(p.stat_part) + (size_t)u * p.chunks_max * p.rows_pad;
         const int tile0 = key0 / kTile;
-        if (rows == 128) {
-          const bool there = quad * 32 + lane < p.rows;
-          const float2 mine = make_float2(m_run[0] * scale2, z_run[0]);
-          if (a.fine) {
-            if (there) base[(size_t)(((tile0 >> 2) + sub) * 2 + par) * p.rows_pad + quad * 32 + lane] = mine;
-          } else {
-            fold_stat(group, mine);
-            if ((sub & 3) == 3 || sub == ((ntiles + 3) >> 2) - 1) {
-              if (there) base[(size_t)(((tile0 >> 4) + (sub >> 2)) * 2 + par) * p.rows_pad + quad * 32 + lane] = group;
-              group = make_float2(-INFINITY, 0.f);
-            }
-          }
-        } else {
+        const bool last = (sub & 3) == 3 || sub == ((ntiles + 3) >> 2) - 1;
 #pragma unroll
-          for (int rg = 0; rg < 4; ++rg)
-            if (rg * 32 + lane < p.rows)
-              base[(size_t)(((tile0 >> 4) + sub) * kTcParts + par * 4 + quad) * p.rows_pad + rg * 32 + lane] =
-                  make_float2(m_run[rg] * scale2, z_run[rg]);
+        for (int rg = 0; rg < kGroupRows; ++rg) {
+          const int row = (rows == 128 ? quad : rg) * 32 + lane;
+          const int slots = rows == 128 ? 2 : kTcParts, slot = rows == 128 ? par : par * 4 + quad;
+          float2 mine = make_float2(m_run[rg] * scale2, z_run[rg]);
+          int part = (tile0 >> sub_shift) + sub;
+          if (fine_parts(ROWS, SPLIT) && !a.fine) {
+            fold_stat(group[rg], mine);
+            if (!last) continue;
+            mine = group[rg];
+            group[rg] = make_float2(-INFINITY, 0.f);
+            part = (tile0 >> 4) + (sub >> 2);
+          }
+          if (row < p.rows) base[(size_t)(part * slots + slot) * p.rows_pad + row] = mine;
         }
 #pragma unroll
         for (int rg = 0; rg < 4; ++rg) { m_run[rg] = -INFINITY; z_run[rg] = 0.f; }
@@ -958,7 +964,8 @@ __global__ void __launch_bounds__(1024) window_tc_reduce_kernel(DeviceProblem p,
   const int u = ur.unit(blockIdx.x);
   const int N = p.unit_N[u];
   const int rows = tc_rows(p.rows), P = 1024 / rows;
-  const int slots = (N + 16 * kTile - 1) / (16 * kTile) * (rows == 128 ? 2 : kTcParts);
+  const int per = rows == 128 ? 2 : kTcParts;          // warps (or pairs of them) that a part has a slot for
+  const int slots = (N + 16 * kTile - 1) / (16 * kTile) * per;
   const int row = threadIdx.x % rows, part = threadIdx.x / rows;
   const float2* src = reinterpret_cast<const float2*>(p.stat_part) + (size_t)u * p.chunks_max * p.rows_pad + row;
   float2 acc = make_float2(-INFINITY, 0.f);
@@ -966,14 +973,14 @@ __global__ void __launch_bounds__(1024) window_tc_reduce_kernel(DeviceProblem p,
   grid_dependency_wait();
   if (!there) {
   } else if (fine) {
-    // 128 rows: slot (group, parity) is folded from up to four stored parts
+    // slot (group, warps) is folded from up to four stored parts
     const int parts = (N + 4 * kTile - 1) / (4 * kTile);
     for (int c = part; c < slots; c += P) {
       float2 o[4], g = make_float2(-INFINITY, 0.f);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int q = (c >> 1) * 4 + i;
-        o[i] = q < parts ? src[(size_t)(q * 2 + (c & 1)) * p.rows_pad] : make_float2(-INFINITY, 0.f);
+        const int q = c / per * 4 + i;
+        o[i] = q < parts ? src[(size_t)(q * per + c % per) * p.rows_pad] : make_float2(-INFINITY, 0.f);
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) fold_stat(g, o[i]);
@@ -1005,7 +1012,7 @@ __global__ void __launch_bounds__(1024) window_tc_reduce_kernel(DeviceProblem p,
 
 // Keys per work item.  Every item costs a Q load and, in pass 2, a statistics load, so long items are better as long as
 // the CTAs still get a dozen items each; a launch with fewer takes shorter ones, down to the 512 keys of one partial
-// (2048 with fewer than 128 rows, in pass 1), so that a single layer of a short prompt still reaches every SM: 8 units of
+// (2048 in pass 1 without fine parts), so that a single layer of a short prompt still reaches every SM: 8 units of
 // 8191 keys, 128 rows, took 23.2 us a pass on 32 CTAs of 16 tiles, 15.3 on 128 of 4.
 inline int pick_chunk(int64_t units_times_keys, int n_sm, int least) {
   if (units_times_keys / 4096 >= (int64_t)12 * n_sm) return 4096;
@@ -1057,7 +1064,7 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
     auto launch_pass = [&](int pass, int least) -> cudaError_t {
       a.pass = pass;
       a.chunk_keys = pick_chunk(keys, n_sm, least);
-      a.fine = pass == 1 && rows == 128 && a.chunk_keys < 16 * kTile ? 1 : 0;
+      a.fine = pass == 1 && fine_parts(ROWS, SPLIT) && a.chunk_keys < 16 * kTile ? 1 : 0;
       a.item_off[0] = 0;
       for (int i = 0; i < kMaxSeq; ++i) {
         a.chunks[i] = (a.N[i] + a.chunk_keys - 1) / a.chunk_keys;
@@ -1078,7 +1085,7 @@ cudaError_t launch_tc_d(const DeviceProblem& p, const WindowHostInfo& h, cudaStr
         if (e != cudaSuccess) return e;
       }
     } else {
-      e = launch_pass(1, rows == 128 ? 4 * kTile : kTcChunk);
+      e = launch_pass(1, fine_parts(ROWS, SPLIT) ? 4 * kTile : kTcChunk);
       if (e != cudaSuccess) return e;
       LaunchScope ls(K_WINDOW_REDUCE, s);
       const UnitRange ur{b0 * per_seq_all + first, per_seq, per_seq_all, nb * per_seq};

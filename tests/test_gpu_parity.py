@@ -475,6 +475,54 @@ def test_fp32_window_scores_beyond_the_planes_range_are_not_slow(G, d):
     assert best[1] < 8 * best[0], best
 
 
+# The items of pass 1 are as short as a call needs to reach every SM (512 to 4096 keys); what is kept of a unit is folded in one
+# order whatever they are: 256 units (items of 2048 keys) against one layer's 16 (items of 512), bit for bit.
+@pytest.mark.parametrize("G,L,d,N", [(2, 24, 64, 3661), (4, 32, 64, 3661), (2, 32, 128, 3600)])
+def test_fp32_window_scores_do_not_depend_on_the_items(G, L, d, N):
+    tk = _tk()
+    R, H = 16, 16
+    g = torch.Generator(device=DEV).manual_seed(G * d)
+    q = torch.randn(R, G * H, L, d, generator=g, device=DEV)
+    k = torch.randn(R, H, N, d, generator=g, device=DEV)
+
+    def scores(layers):
+        p = tk.Params(n_layers=len(layers), n_heads=G * H, n_kv_heads=H, head_dim=d, seq_lens=[N], sink=4, recent=32,
+                      mid_budget=[40] * len(layers), window=L, dtype="f32", top_t=64, beta=0.25, m_top=1, max_new_tokens=0)
+        cache = tk.taskkv_compress_ex(p, [q[layers].contiguous()], [k[layers].contiguous()], [k[layers].contiguous()])
+        got = cache.query(tk.Q_SCORES).reshape(len(layers), H, -1)[:, :, :N].copy()
+        assert cache.status() == 0
+        cache.close()
+        return got
+
+    whole = scores(list(range(R)))
+    for r in (0, 7, R - 1):
+        assert np.array_equal(whole[r], scores([r])[0])
+
+
+# A call of few units reaches every SM: the passes over one unit of 2500 keys take about as long as over one of 512 (items of
+# 2048 keys in pass 1 made one CTA walk 16 tiles: 2.4 times as long).
+def test_fp32_window_scores_of_few_units_are_cut_into_short_items():
+    tk = _tk()
+    took = []
+    for N in (512, 2500):
+        wl = small("few", n=2, n_kv=1, d=64, N=N, L=32, s1=4, s2=32, k=40, dtype="f32", nh=0, t=64, steps=1, promote=False)
+        qs, ks, vs = W.materialize(wl, DEV)
+        params = tk.params_from_workload(wl, max_new_tokens=0)
+        for _ in range(3):
+            tk.taskkv_compress_ex(params, qs, ks, vs).close()
+        torch.cuda.synchronize()
+        tk.taskkv_timing_enable(True)
+        tk.taskkv_timing_collect()
+        for _ in range(20):
+            tk.taskkv_compress_ex(params, qs, ks, vs).close()
+        torch.cuda.synchronize()
+        ms = [t for name, t in tk.taskkv_timing_collect() if name == "window_tc"]
+        tk.taskkv_timing_enable(False)
+        assert len(ms) == 40
+        took.append(float(np.median(ms[0::2]) + np.median(ms[1::2])))
+    assert took[1] < 1.6 * took[0], took
+
+
 # A key with an infinite element that every window row scores -inf weighs nothing, whatever fills the window's tile up: a zero
 # query times infinity is NaN.  (G, L): 9 rows in the single-read kernel and in a tile of 32, 48 in one of 64, 96 in one of
 # 128, and full tiles; with and without the caller's normalisers (which take the two-pass kernel's second pass alone).
