@@ -94,7 +94,9 @@ enum : int {
   B_FULL = 0, B_EMPTY = 4, B_QFULL = 8, B_QEMPTY = 10, B_TFULL = 12, B_TEMPTY = 16, B_STAT = 20, B_COUNT = 22
 };
 
-template <int D>
+// RAGGED: the last block of a head has fewer than 128 rows.  (A template argument, since the code for such blocks costs the whole
+// ones 0.5 to 1 % in the same kernel.)
+template <int D, bool RAGGED>
 __global__ void __launch_bounds__(kThreads, 1)
 prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_constant__ PrefixArgs a, PrefixLayout lay) {
   constexpr int KB = D / 64;
@@ -315,7 +317,7 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
         tc_fence_after();
         const bool tail = t == T - 1;
         float2 cs[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        if (rows_here == kTile) {
+        if (!RAGGED || rows_here == kTile) {
 #pragma unroll
           for (int c0 = 0; c0 < kTile; c0 += kCols) {
             uint32_t r[kCols];
@@ -335,14 +337,22 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
             }
           }
         } else {
-#pragma unroll 1
+#pragma unroll
           for (int c0 = 0; c0 < kTile; c0 += kCols) {
+            if (c0 >= rows_here) break;
             uint32_t r[kCols];
             tc_ld32(lane_addr + (uint32_t)(acc * 128 + c0), r);
             tc_wait_ld();
+            if (tail) {
 #pragma unroll
-            for (int i = 0; i < kCols; ++i)
-              if ((tail && c0 + i < row) || c0 + i >= rows_here) r[i] = __float_as_uint(-INFINITY);
+              for (int i = 0; i < kCols; ++i)
+                if (c0 + i < row) r[i] = __float_as_uint(-INFINITY);
+            }
+            if (c0 + kCols > rows_here) {
+#pragma unroll
+              for (int i = 0; i < kCols; ++i)
+                if (c0 + i >= rows_here) r[i] = __float_as_uint(-INFINITY);
+            }
             const float4* off4 = reinterpret_cast<const float4*>(myOff + c0);
 #pragma unroll
             for (int i = 0; i < kCols; i += 4) {
@@ -370,12 +380,12 @@ prefix_score_kernel(const __grid_constant__ PrefixMaps maps, const __grid_consta
   if (tid == 0 && *s_abort) set_status(a.status, TASKKV_ETIMEOUT);
 }
 
-template <int D>
+template <int D, bool RAGGED>
 cudaError_t launch_prefix_d(const void* q, const void* k, int heads, int group, int N, float* scores, int32_t* status,
                             cudaStream_t s) {
   const int n_sm = sm_count();
   const PrefixLayout lay = make_prefix_layout(D);
-  cudaError_t e = cudaFuncSetAttribute(prefix_score_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, lay.total);
+  cudaError_t e = cudaFuncSetAttribute(prefix_score_kernel<D, RAGGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, lay.total);
   if (e != cudaSuccess) return e;
   PrefixMaps maps;
   if (!make_tensor_map_2d(&maps.k, k, D, (uint64_t)(heads / group) * (uint64_t)N, kTile)) return cudaErrorUnknown;
@@ -397,7 +407,7 @@ cudaError_t launch_prefix_d(const void* q, const void* k, int heads, int group, 
   a.scores = scores;
   a.status = status;
   LaunchScope ls(K_WINDOW_TC, s);
-  prefix_score_kernel<D><<<grid, kThreads, lay.total, s>>>(maps, a, lay);
+  prefix_score_kernel<D, RAGGED><<<grid, kThreads, lay.total, s>>>(maps, a, lay);
   return cudaGetLastError();
 }
 
@@ -405,8 +415,11 @@ cudaError_t launch_prefix_d(const void* q, const void* k, int heads, int group, 
 
 cudaError_t launch_prefix_scores(const void* q, const void* k, int d, int heads, int group, int N, float* scores,
                                  int32_t* status, cudaStream_t s) {
-  return d == 64 ? launch_prefix_d<64>(q, k, heads, group, N, scores, status, s)
-                 : launch_prefix_d<128>(q, k, heads, group, N, scores, status, s);
+  if (N % kTile)
+    return d == 64 ? launch_prefix_d<64, true>(q, k, heads, group, N, scores, status, s)
+                   : launch_prefix_d<128, true>(q, k, heads, group, N, scores, status, s);
+  return d == 64 ? launch_prefix_d<64, false>(q, k, heads, group, N, scores, status, s)
+                 : launch_prefix_d<128, false>(q, k, heads, group, N, scores, status, s);
 }
 
 }  // namespace taskkv
