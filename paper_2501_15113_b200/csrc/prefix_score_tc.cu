@@ -8,13 +8,15 @@
 //   warps 2-5, 7-18 four epilogue groups, every fourth tile each
 // First walk: D[row, key] = Q K^T, a TMEM lane is a query row and keeps its own running (max, sum); the four groups'
 // pairs meet in shared memory.  Second walk: D[key, row] = K Q^T, a lane is a key and sums its column.
-// Bound by the special-function unit (two exponentials per score at 16 a cycle and SM, 2048 cycles per tile and block), so a
-// quarter of them is computed on the FMA pipe, and by the hand-overs between the warps.
+// Two exponentials per score at 16 a cycle and SM are 2048 cycles per tile and block on the special-function unit, so a quarter of
+// them is computed on the FMA pipe.  That unit is then 67 % busy and the tensor pipe 43 %; what the warps wait for most is their
+// tensor-memory loads, one 32-column step after the other, and each other.
 // Blocks are dealt out longest first, in both directions alternately, so that every CTA gets the same number of tiles;
 // the heads go in groups whose keys fit well into L2.  32 heads x 16384 rows, d = 128, both walks: as two launches of
 // the window kernel over (block, 2048 keys) items 4.19 ms (a CTA met the same two of a block's eight key ranges again
 // and again, a third more tiles for some than on average), like this with two epilogue groups 2.98 ms, with four 2.76 ms:
-// with two warps to a scheduler the special-function unit idles while they hand over.  With the exponentials shared 2.5 ms.
+// with two warps to a scheduler the special-function unit idles while they hand over.  With the exponentials shared 2.82 -> 2.62 ms
+// for a call by itself, 2.91 -> 2.84 in a row of calls, which the power limit slows down (weight2).
 #include <cuda.h>
 
 #include "common.cuh"

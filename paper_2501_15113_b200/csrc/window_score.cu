@@ -2,9 +2,10 @@
 //   S = Q_win K^T / sqrt(d), causal mask on the last L keys, row softmax,
 //   C[j] = mean over the unit's G*L window rows of the normalised weights.
 //
-// Two-pass path on the CUDA cores for fp32 inputs with up to 32 window rows (the others run on the tensor cores; for few rows
-// splitting the keys into planes for them costs more than the products: 128 units of 3000 keys, 16 rows, d = 128, both passes
-// 191 us here and 207 there; 32 units of 6001 keys, 128 rows, d = 64, 252 here and 88 there):
+// Two-pass path on the CUDA cores for fp32 inputs with up to 32 window rows; the others run on the tensor cores, where splitting
+// the keys into planes costs the same whatever the rows.  Both passes here and there: 128 units of 3000 keys, d = 128, 16 rows 189
+// and 189 us, 24 rows 281 and 191, 32 rows 286 and 193; 32 units of 6001 keys, d = 64, 24 and 32 rows 90 and 83, 64 rows 150 and
+// 83, 128 rows 250 and 93.  So the kernels are level at 16 rows, and the line at 32 is higher than these figures put it:
 //   pass 1  per (unit, 256-key chunk): row maxima and exp-sums  -> partial stats
 //   reduce  per unit: combine chunks -> (row max, 1 / row sum); units of up to 32 chunks need no launch for it,
 //           their pass-2 blocks combine the chunks themselves

@@ -89,14 +89,16 @@ constexpr uint32_t kTmemCols = 512; // four accumulators of up to 128 columns
 // so the three left out are below 2^-24 of an element's own term, with either sign (2^-27.4 in the mean square).  The leading
 // product has an accumulator of its own, since the tensor cores truncate what does not fit an accumulator's 24 bits; the other
 // five share one.
-// Error of C against 64 bits, six shapes of 40 to 128 rows: 1.3e-7 to 1.8e-7, fp32 on the CUDA cores 1.9e-7 to 2.6e-7; powers of
-// two that scale a channel of the keys up and of the queries down (2^-20 to 2^20) change no bit of either.  (Planes on one grid
-// per row of 64 elements, which sum without truncation, are as good for rows whose elements are of one size, but keep the small
-// elements beside a large one in fewer bits: 1e-5 for one channel of 2^10, 1e-3 to 1e-2 for one of 2^20.)
-// With more than 32 rows; up to 32 the CUDA cores are faster (window_score.cu).  Bound by the conversion with 64 rows, by the 24
-// products a 64 elements with 128: 32 units of 6001 keys, d = 64, both passes and their reduction 64 rows 150 us on the CUDA
-// cores, 84 here, 128 rows 250 and 97; one layer of 8 x 8000 keys, 128 rows, d = 128, 156 and 67.  Warps 0 and 11-13 read the
-// fp32 rows and write the planes in the producer's place, warp 1 alone issues.
+// Error of C against 64 bits, six shapes of 40 to 128 rows: 1.0e-7 to 1.4e-7, fp32 on the CUDA cores 1.9e-7 to 2.6e-7; powers of
+// two that scale a channel of the keys up and of the queries down (2^-40 to 2^40) change no bit.  (Planes on one grid per row of
+// 64 elements, which sum without truncation, are as good for rows whose elements are of one size, but keep the small elements
+// beside a large one in fewer bits: 1e-5 for one channel of 2^10, 1e-3 to 1e-2 for one of 2^20.)
+// With more than 32 rows (window_score.cu).  Bound by neither pipe nor issue slots, which are 35 % (tensor, 128 rows; 20 % with 64)
+// and 38 % busy, but by a stage's way around: the converting warps' loads and arithmetic, the products, the stage given back, with
+// room for two stages.  Both passes and their reduction, 32 units of 6001 keys, d = 64: 64 rows 150 us on the CUDA cores, 83 here,
+// 128 rows 250 and 93; one layer of 8 x 8000 keys, d = 128: 64 rows 103 and 54, 128 rows 156 and 63.  128 registers a thread (14
+// warps are given those of 16), of which a few words spill in the converting warps.  Warps 0 and 11-13 read the fp32 rows and
+// write the planes in the producer's place, warp 1 alone issues.
 constexpr int kSplitThreads = 448;
 constexpr int kCvtWarps = 4;
 constexpr int kPlanes = 3;
@@ -209,7 +211,7 @@ enum : int {
 __host__ __device__ constexpr bool stat_pairs(int rows, bool split) { return split || rows == 32; }
 
 // Whether pass 1's items may be shorter than 2048 keys, down to the 512 of one part.  Four times the slots of a row: with 128
-// rows a slot is two warps' and there is room; fp32 rows get it (partial_slots), since a tile of theirs takes two to three times
+// rows a slot is two warps' and there is room; fp32 rows get it (partial_slots), since a tile of theirs takes several times
 // as long and a call of few units waits for one CTA's walk over 16 of them (8 units of 2500 keys, 64 rows: 73 us a call
 // with 2048, 53 with 512 at d = 64, 98 and 67 at d = 128; on the CUDA cores 56 and 77).
 __host__ __device__ constexpr bool fine_parts(int rows, bool split) { return split || rows == 128; }
